@@ -1,0 +1,791 @@
+// The passes of the plane path with the grid size known at compile time
+// (2,3,5-smooth n from 24 to 160): the z passes and the plane pass of one
+// evaluation, or of one preconditioning pass.
+//
+// What bounds the generic passes (k_zfwd, k_plane, k_zinv_epi) on these grids is
+// neither memory (the spectra stay in L2) nor arithmetic but instructions and
+// barriers: index arithmetic with run-time sizes, staging copies and a trip
+// through shared memory per field and stage took 390 + 505 + 684 instructions
+// per grid point at 75^3 (two fields), issued at 1.6 per cycle, and the plane
+// pass of a small grid left most SMs idle.  Here every size, stride and radix is
+// a constant; the first stage reads its inputs from memory into registers, the
+// G-space terms sit between the last forward and the first inverse stage in
+// registers, the last inverse stage stores to memory; all fields of a z pass go
+// through each stage together (three barriers instead of a dozen); and the plane
+// of a small grid is spread over a cluster of up to four blocks.
+//
+// The transforms keep the generic passes' radices (the same search, evaluated
+// at compile time), twiddles and operation order, so a spectrum or a potential
+// has the same bits: the rounding of the psi transform, amplified by G^2, is
+// the largest error of an FP32 potential.
+#pragma once
+#include <cooperative_groups.h>
+#include "passes.cuh"
+
+namespace ofdft {
+
+// ---------------------------------------------------------------------------
+// Radices at compile time: the first factorisation with the fewest passes in
+// the order of factor_radices, and that of factor_radices_balanced.
+struct CFac { int c; int r[4]; };
+constexpr int kCand[10] = {16, 12, 10, 9, 8, 6, 5, 4, 3, 2};
+constexpr bool is_cand(int n) {
+  for (int c : kCand) if (c == n) return true;
+  return false;
+}
+// the k-th (k = 0 first) factorisation into three at most; bal: the smallest largest radix
+constexpr CFac cfac(int n, bool bal) {
+  CFac best{0, {0, 0, 0, 0}};
+  int bmax = 1 << 30;
+  if (is_cand(n)) return CFac{1, {n, 0, 0, 0}};
+  for (int a : kCand) {
+    if (n % a) continue;
+    const int b = n / a;
+    if (!is_cand(b)) continue;
+    const int mx = a > b ? a : b;
+    if (!bal) return CFac{2, {a, b, 0, 0}};
+    if (mx < bmax) { bmax = mx; best = CFac{2, {a, b, 0, 0}}; }
+  }
+  if (best.c) return best;
+  for (int a : kCand) {
+    if (n % a) continue;
+    for (int b : kCand) {
+      if ((n / a) % b) continue;
+      const int d = n / a / b;
+      if (!is_cand(d)) continue;
+      int mx = a > b ? a : b;
+      if (d > mx) mx = d;
+      if (!bal) return CFac{3, {a, b, d, 0}};
+      if (mx < bmax) { bmax = mx; best = CFac{3, {a, b, d, 0}}; }
+    }
+  }
+  return best;
+}
+constexpr int cdiv(int a, int b) { return (a + b - 1) / b; }
+// threads for `items` items, at most `most`, in as few and as full rounds as possible
+constexpr int fit_threads(int items, int most, int least) {
+  const int rounds = cdiv(items, most);
+  int nt = cdiv(cdiv(items, rounds), 32) * 32;
+  return nt < least ? least : nt;
+}
+
+// z passes: rows per block, transform length (half for even n, full for odd n:
+// two rows per transform), radices, threads, pitches.
+template <int N> struct CZ {
+  static constexpr bool ODD = N & 1;
+  static constexpr int H = N / 2, NH = H + 1;
+  static constexpr int R = N <= 50 ? 8 : 16;            // at least 152 blocks from n = 36 up
+  static constexpr int L = ODD ? N : H;
+  static constexpr int LINES = ODD ? R / 2 : R;         // transforms per block and field
+  static constexpr CFac F = cfac(L, !ODD);
+  static constexpr int F0 = F.r[0], F1 = F.r[1], F2 = F.c == 3 ? F.r[2] : 1;
+  static constexpr int NT = N <= 50 ? 128 : 256;
+  // element e of a line sits at e + e / F0 (even F0: the first stage writes
+  // with stride F0); odd pitch, so that lines differ in bank
+  static constexpr int pad(int e) { return (F0 & 1) ? e : e + e / F0; }
+  static constexpr int XP = (pad(L - 1) + 1) | 1;
+  static constexpr int SP = (ODD ? (N + 1) / 2 : NH) | 1;   // spectrum row pitch (odd n: two rows hold a line of L <= 2 SP)
+  static constexpr int BP = (ODD ? 2 : 1) * SP;             // the same region as lines: pitch
+  static constexpr int GRID = cdiv(N * N, R);
+};
+
+// ---------------------------------------------------------------------------
+// Block sums of 8 per-thread values without a tree of barriers: each warp
+// halves columns and lanes together (lane bits 4..2 choose the column, 7
+// additions), two more steps finish the warp, one barrier, and the first warp
+// adds the warps' sums.  Fixed order.  Floats as (hi, lo) pairs (tree_add).
+__device__ __forceinline__ float2 shfl_xor_v(float2 v, int m) {
+  return make_float2(__shfl_xor_sync(0xffffffffu, v.x, m), __shfl_xor_sync(0xffffffffu, v.y, m));
+}
+__device__ __forceinline__ double shfl_xor_v(double v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
+
+// scr: [warps][8]; dst[c] (c < ncol) by thread c of the first warp.  Begins
+// with a barrier (scr may alias data still being read); no barrier at the end.
+template <typename V>
+__device__ __forceinline__ void block_sum8(V (&v)[8], V* scr, V* dst, int ncol) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  V w4[4], w2[2], w1;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const bool hi = lane & 16;
+    const V keep = hi ? v[i + 4] : v[i], send = hi ? v[i] : v[i + 4];
+    w4[i] = tree_add(keep, shfl_xor_v(send, 16));
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const bool hi = lane & 8;
+    const V keep = hi ? w4[i + 2] : w4[i], send = hi ? w4[i] : w4[i + 2];
+    w2[i] = tree_add(keep, shfl_xor_v(send, 8));
+  }
+  {
+    const bool hi = lane & 4;
+    const V keep = hi ? w2[1] : w2[0], send = hi ? w2[0] : w2[1];
+    w1 = tree_add(keep, shfl_xor_v(send, 4));
+  }
+  w1 = tree_add(w1, shfl_xor_v(w1, 2));
+  w1 = tree_add(w1, shfl_xor_v(w1, 1));
+  const int col = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+  __syncthreads();
+  if ((lane & 3) == 0) scr[wid * 8 + col] = w1;
+  __syncthreads();
+  if (wid == 0) {
+    const int c = lane & 7;
+    V s{};
+    for (int w = lane >> 3; w < nw; w += 4) s = tree_add(s, scr[w * 8 + c]);
+    s = tree_add(s, shfl_xor_v(s, 8));
+    s = tree_add(s, shfl_xor_v(s, 16));
+    if (lane < ncol) dst[lane] = s;
+  }
+}
+template <typename T> __device__ __forceinline__ typename TreeVal<T>::type short_val(const AccShort<T>& a) {
+  if constexpr (sizeof(T) == 4) return make_float2(a.s, 0.0f);
+  else return a.s;
+}
+
+// finalize_eval with block_sum8: by the last block of the epilogue.
+template <typename T>
+static __device__ void finalize_eval8(const FinArgs<T>& f, typename TreeVal<T>::type* scr) {
+  using V = typename TreeVal<T>::type;
+  __shared__ V tot[16];
+  const int nt = blockDim.x;
+  V g[8], e[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) { g[q] = V{}; e[q] = V{}; }
+  for (int b = threadIdx.x; b < f.ng; b += nt) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) g[q] = tree_add(g[q], __ldcg(f.pg + (size_t)b * 4 + q));
+  }
+  for (int b0 = threadIdx.x; b0 < f.ne; b0 += 4 * nt) {
+    V x[4][8];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int b = b0 + u * nt;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) x[u][q] = b < f.ne ? __ldcg(f.pe + (size_t)b * 8 + q) : V{};
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int q = 0; q < 8; ++q) e[q] = tree_add(e[q], x[u][q]);
+  }
+  block_sum8(e, scr, tot + 4, 8);
+  block_sum8(g, scr, tot, 4);
+  __syncthreads();
+  if (threadIdx.x < 12) f.out[threadIdx.x] = tree_get(tot[threadIdx.x]);
+}
+
+// ---------------------------------------------------------------------------
+// The stages of a z pass after the first, in shared memory, all lines of the
+// block at once: data in xa (padded), the result as natural elements: get(line, e)
+// of the result's buffer is xa[line XP + pad(e)] for two stages and
+// xb[line BP + e] for three.  Ends with a barrier.
+template <typename T, int N, int DIR>
+__device__ __forceinline__ void cz_stages(cplx<T>* xa, cplx<T>* xb, int lines, const cplx<T>* __restrict__ tw) {
+  using Z = CZ<N>;
+  constexpr int L = Z::L, F0 = Z::F0, F1 = Z::F1, F2 = Z::F2;
+  if constexpr (Z::F.c == 2) {
+    for (int it = threadIdx.x; it < lines * F0; it += Z::NT) {
+      const int ln = it / F0, j = it - ln * F0;
+      cplx<T>* x = xa + ln * Z::XP;
+      cplx<T> v[F1];
+#pragma unroll
+      for (int r = 0; r < F1; ++r) v[r] = x[Z::pad(r * F0) + j];
+#pragma unroll
+      for (int r = 1; r < F1; ++r) {
+        cplx<T> w = tw[j * r];
+        if (DIR > 0) w.y = -w.y;
+        v[r] = cmul(v[r], w);
+      }
+      Codelet<cplx<T>, F1, DIR>::run(v);
+#pragma unroll
+      for (int r = 0; r < F1; ++r) x[Z::pad(r * F0) + j] = v[r];
+    }
+    __syncthreads();
+  } else {
+    constexpr int M1 = L / F1, M2 = L / F2;
+    for (int it = threadIdx.x; it < lines * M1; it += Z::NT) {
+      const int ln = it / M1, j = it - ln * M1;
+      const cplx<T>* x = xa + ln * Z::XP;
+      cplx<T> v[F1];
+#pragma unroll
+      for (int r = 0; r < F1; ++r) v[r] = x[Z::pad(j + r * M1)];
+      const int jq = j / F0, k = j - jq * F0;
+#pragma unroll
+      for (int r = 1; r < F1; ++r) {
+        cplx<T> w = tw[k * r * F2];
+        if (DIR > 0) w.y = -w.y;
+        v[r] = cmul(v[r], w);
+      }
+      Codelet<cplx<T>, F1, DIR>::run(v);
+      cplx<T>* y = xb + ln * Z::BP + jq * F0 * F1 + k;
+#pragma unroll
+      for (int r = 0; r < F1; ++r) y[r * F0] = v[r];
+    }
+    __syncthreads();
+    for (int it = threadIdx.x; it < lines * M2; it += Z::NT) {
+      const int ln = it / M2, j = it - ln * M2;
+      cplx<T>* y = xb + ln * Z::BP + j;
+      cplx<T> v[F2];
+#pragma unroll
+      for (int r = 0; r < F2; ++r) v[r] = y[r * M2];
+#pragma unroll
+      for (int r = 1; r < F2; ++r) {
+        cplx<T> w = tw[j * r];
+        if (DIR > 0) w.y = -w.y;
+        v[r] = cmul(v[r], w);
+      }
+      Codelet<cplx<T>, F2, DIR>::run(v);
+#pragma unroll
+      for (int r = 0; r < F2; ++r) y[r * M2] = v[r];
+    }
+    __syncthreads();
+  }
+}
+template <typename T, int N>
+__device__ __forceinline__ cplx<T> cz_get(const cplx<T>* xa, const cplx<T>* xb, int ln, int e) {
+  using Z = CZ<N>;
+  if constexpr (Z::F.c == 2) return xa[ln * Z::XP + Z::pad(e)];
+  else return xb[ln * Z::BP + e];
+}
+
+// shared memory: tw[L] | twn[NH] | xa[nf][LINES][XP] | xb[nf][LINES][BP] (three stages)
+template <typename T, int N> __host__ __device__ constexpr size_t czfwd_bytes(int nf) {
+  using Z = CZ<N>;
+  return ((size_t)Z::L + Z::NH + (size_t)nf * Z::LINES * (Z::XP + (Z::F.c == 3 ? Z::BP : 0))) * sizeof(cplx<T>);
+}
+// Forward z pass: prologue (n, n^a, psi from rho or from psi + t d) and the
+// real-to-complex transform of R rows of every active field, plane layout.
+template <typename T, int N>
+__global__ void __launch_bounds__(CZ<N>::NT, (sizeof(T) == 4 ? 1024 : 512) / CZ<N>::NT)
+k_zfwd_c(ProArgs<T> a, Spectra<T> sp, const cplx<T>* __restrict__ tw_l, const cplx<T>* __restrict__ tw_n) {
+  using Z = CZ<N>;
+  using C = cplx<T>;
+  constexpr int R = Z::R, L = Z::L, H = Z::H, NH = Z::NH, F0 = Z::F0, M0 = L / F0, NN = N * N;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* tw = reinterpret_cast<C*>(smem_raw);
+  C* twn = tw + L;
+  C* xa = twn + NH;
+  C* xb = xa + sp.nact * Z::LINES * Z::XP;
+  const int row0 = blockIdx.x * R;
+  const int rows = min(R, NN - row0);
+  const int lines = Z::ODD ? (rows + 1) >> 1 : rows;
+  for (int q = threadIdx.x; q < L + NH; q += Z::NT) tw[q] = q < L ? tw_l[q] : tw_n[q - L];
+  const T* src = (a.mode == 0 ? a.rho : a.psi) + (size_t)row0 * N;
+  const bool has_d = a.mode != 0 && a.d != nullptr;
+  const T* dsrc = has_d ? a.d + (size_t)row0 * N : src;
+  const T tstep = a.dsc ? (T)a.dsc[2] : a.t;
+  const T scale = a.dsc ? (T)a.dsc[0] : a.scale, alpha = a.alpha, nmin = (T)kNmin;
+  const T shift = a.dsc ? (T)a.dsc[1] : a.psi_shift;
+  // the field's value from the density (mode 0) or psi_t
+  auto val = [&](int fid, T x) -> T {
+    if (fid == 2) {
+      if (a.mode == 0) x = sqrt(fmax(x, (T)0));
+      return x - shift;
+    }
+    const T nv = a.mode == 0 ? x : scale * x * x;
+    return fid == 0 ? nv : pow_t<T>(fmax(nv, nmin), alpha);
+  };
+  // stage 0: the line's elements j + s M0 from memory, radix F0
+  for (int it = threadIdx.x; it < sp.nact * Z::LINES * M0; it += Z::NT) {
+    const int fl = it / M0, j = it - fl * M0;
+    const int f = fl / Z::LINES, ln = fl - f * Z::LINES;
+    if (ln >= lines) continue;
+    const int fid = sp.idx[f];
+    C v[F0];
+    if constexpr (Z::ODD) {
+      const bool two = 2 * ln + 1 < rows;
+      const T* p0 = src + 2 * ln * N + j;
+      const T* d0 = dsrc + 2 * ln * N + j;
+#pragma unroll
+      for (int s = 0; s < F0; ++s) v[s] = mk<T>(__ldg(p0 + s * M0), two ? __ldg(p0 + N + s * M0) : (T)0);
+      if (has_d) {
+#pragma unroll
+        for (int s = 0; s < F0; ++s) {
+          v[s].x = v[s].x + tstep * __ldg(d0 + s * M0);
+          if (two) v[s].y = v[s].y + tstep * __ldg(d0 + N + s * M0);
+        }
+      }
+#pragma unroll
+      for (int s = 0; s < F0; ++s) v[s] = mk<T>(val(fid, v[s].x), two ? val(fid, v[s].y) : (T)0);
+    } else {
+      const C* p0 = reinterpret_cast<const C*>(src + ln * N) + j;
+      const C* d0 = reinterpret_cast<const C*>(dsrc + ln * N) + j;
+#pragma unroll
+      for (int s = 0; s < F0; ++s) v[s] = __ldg(p0 + s * M0);
+      if (has_d) {
+#pragma unroll
+        for (int s = 0; s < F0; ++s) {
+          const C d = __ldg(d0 + s * M0);
+          v[s].x = v[s].x + tstep * d.x; v[s].y = v[s].y + tstep * d.y;
+        }
+      }
+#pragma unroll
+      for (int s = 0; s < F0; ++s) v[s] = mk<T>(val(fid, v[s].x), val(fid, v[s].y));
+    }
+    Codelet<C, F0, -1>::run(v);
+    C* x = xa + fl * Z::XP + Z::pad(j * F0);
+#pragma unroll
+    for (int s = 0; s < F0; ++s) x[s] = v[s];
+  }
+  __syncthreads();
+  cz_stages<T, N, -1>(xa, xb, sp.nact * Z::LINES, tw);
+  // the rows' half spectra; consecutive threads take consecutive rows of one kz
+  for (int q = threadIdx.x; q < sp.nact * NH * R; q += Z::NT) {
+    const int fk = q / R, r = q - fk * R;
+    const int f = fk / NH, k = fk - f * NH;
+    if (r >= rows) continue;
+    C o;
+    if constexpr (Z::ODD) {
+      // X_a[k] = (Z[k] + Z*[n-k]) / 2, X_b[k] = -i (Z[k] - Z*[n-k]) / 2
+      const int ln = f * Z::LINES + (r >> 1);
+      const C zk = cz_get<T, N>(xa, xb, ln, k);
+      const C zc = cconj(cz_get<T, N>(xa, xb, ln, k == 0 ? 0 : N - k));
+      if ((r & 1) == 0) {
+        o = mk<T>((T)0.5 * (zk.x + zc.x), (T)0.5 * (zk.y + zc.y));
+      } else {
+        const C dd = csub(zk, zc);
+        o = mk<T>((T)0.5 * dd.y, (T)-0.5 * dd.x);
+      }
+    } else {
+      // X[k] = (Z[k] + Z*[h-k])/2 - (i/2) W^k (Z[k] - Z*[h-k]),  k = 0..h
+      const int ln = f * Z::LINES + r;
+      const C zk = cz_get<T, N>(xa, xb, ln, k == H ? 0 : k);
+      const C zc = cconj(cz_get<T, N>(xa, xb, ln, k == 0 ? 0 : H - k));
+      const C e = cadd(zk, zc);
+      const C wo = cmul(twn[k], csub(zk, zc));
+      o = mk<T>((T)0.5 * (e.x + wo.y), (T)0.5 * (e.y - wo.x));
+    }
+    sp.s[sp.idx[f]][(size_t)k * NN + row0 + r] = o;
+  }
+}
+
+// shared memory: tw[L] | twn[NH] | stg[nf][R][SP] | xa[nf][LINES][XP]
+template <typename T, int N> __host__ __device__ constexpr size_t czinv_bytes(int nf) {
+  using Z = CZ<N>;
+  const size_t b = ((size_t)Z::L + Z::NH + (size_t)nf * (Z::R * Z::SP + Z::LINES * Z::XP)) * sizeof(cplx<T>);
+  const size_t s = (size_t)(Z::NT / 32) * 8 * 8;
+  return b > s ? b : s;
+}
+// Inverse z pass: complex-to-real transform of R rows of every active field
+// (plane layout) and the pointwise functional, or (mode 3) the
+// preconditioning pass's output.
+template <typename T, int N>
+__global__ void __launch_bounds__(CZ<N>::NT, (sizeof(T) == 4 ? 1024 : 512) / CZ<N>::NT)
+k_zinv_c(Spectra<T> sp, EpiArgs<T> a, const cplx<T>* __restrict__ tw_l, const cplx<T>* __restrict__ tw_n) {
+  using Z = CZ<N>;
+  using C = cplx<T>;
+  constexpr int R = Z::R, L = Z::L, H = Z::H, NH = Z::NH, F0 = Z::F0, M0 = L / F0, NN = N * N;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* tw = reinterpret_cast<C*>(smem_raw);
+  C* twn = tw + L;
+  C* stg = twn + NH;
+  C* xa = stg + sp.nact * R * Z::SP;
+  const int row0 = blockIdx.x * R;
+  const int rows = min(R, NN - row0);
+  const size_t off = (size_t)row0 * N;
+  for (int q = threadIdx.x; q < sp.nact * NH * R; q += Z::NT) {
+    const int fk = q / R, r = q - fk * R;
+    const int f = fk / NH, k = fk - f * NH;
+    if (r < rows) cp_async_c(stg + (f * R + r) * Z::SP + k, sp.s[sp.idx[f]] + (size_t)k * NN + row0 + r, true);
+  }
+  cp_async_commit();
+  for (int q = threadIdx.x; q < L + NH; q += Z::NT) tw[q] = q < L ? tw_l[q] : tw_n[q - L];
+  cp_async_wait<0>();
+  __syncthreads();
+  // stage 0: Z at j + s M0 from the staged spectra, radix F0
+  for (int it = threadIdx.x; it < sp.nact * Z::LINES * M0; it += Z::NT) {
+    const int fl = it / M0, j = it - fl * M0;
+    C v[F0];
+    if constexpr (Z::ODD) {
+      // Z[k] = A[k] + i B[k], rows 2 ln and 2 ln + 1, A[n-k] = A*[k] (the
+      // imaginary parts at k = 0 dropped)
+      const int f = fl / Z::LINES, ln = fl - f * Z::LINES;
+      const C* in = stg + (f * R + 2 * ln) * Z::SP;
+      const bool two = 2 * ln + 1 < rows;
+#pragma unroll
+      for (int s = 0; s < F0; ++s) {
+        const int k = j + s * M0;
+        const bool lo = k < NH;
+        const int kk = lo ? k : N - k;
+        C A = in[kk];
+        C B = two ? in[Z::SP + kk] : mk<T>((T)0, (T)0);
+        if (k == 0) { A.y = 0; B.y = 0; }
+        if (!lo) { A.y = -A.y; B.y = -B.y; }
+        v[s] = mk<T>(A.x - B.y, A.y + B.x);
+      }
+    } else {
+      // Z[k] = (X[k] + X*[h-k]) + i W^-k (X[k] - X*[h-k])
+      const C* in = stg + fl * Z::SP;
+#pragma unroll
+      for (int s = 0; s < F0; ++s) {
+        const int k = j + s * M0;
+        const C xk = in[k];
+        const C xc = cconj(in[H - k]);
+        const C e = cadd(xk, xc);
+        const C o = cmul(cconj(twn[k]), csub(xk, xc));
+        v[s] = mk<T>(e.x - o.y, e.y + o.x);
+      }
+    }
+    Codelet<C, F0, +1>::run(v);
+    C* x = xa + fl * Z::XP + Z::pad(j * F0);
+#pragma unroll
+    for (int s = 0; s < F0; ++s) x[s] = v[s];
+  }
+  __syncthreads();                                       // (the staged spectra are free)
+  cz_stages<T, N, +1>(xa, stg, sp.nact * Z::LINES, tw);
+  // real value i of row r, field f: element i / 2 (even n; pairs of reals) or
+  // the row's component of element i (odd n)
+  auto real_at = [&](int f, int r, int i) -> T {
+    if constexpr (Z::ODD) {
+      const C z = cz_get<T, N>(xa, stg, f * Z::LINES + (r >> 1), i);
+      return (r & 1) ? z.y : z.x;
+    } else {
+      const C z = cz_get<T, N>(xa, stg, f * Z::LINES + r, i >> 1);
+      return (i & 1) ? z.y : z.x;
+    }
+  };
+  if (a.mode == 3) {
+    for (int q = threadIdx.x; q < rows * N; q += Z::NT) {
+      const int r = q / N, i = q - r * N;
+      const T v = real_at(0, r, i);
+      a.out[off + q] = v;
+      if (a.pyout) a.pyout[off + q] = v - __ldg(a.pold + off + q);
+    }
+    return;
+  }
+  int slot[3] = {-1, -1, -1};
+  for (int f = 0; f < sp.nact; ++f) slot[sp.idx[f]] = f;
+  const EpiPoint<T> ep(sp, a);
+  AccShort<T> acc[8];
+  const T* src = (a.mode == 0 ? a.rho : a.psi) + off;
+  const T* dsrc = a.mode == 1 ? a.d + off : nullptr;
+#pragma unroll 2
+  for (int q = threadIdx.x; q < rows * N; q += Z::NT) {
+    const int r = q / N, i = q - r * N;
+    const T x = __ldg(src + q), d = dsrc ? __ldg(dsrc + q) : (T)0;
+    ep.point(a, x, d, slot[0] >= 0 ? real_at(slot[0], r, i) : (T)0, slot[1] >= 0 ? real_at(slot[1], r, i) : (T)0,
+             slot[2] >= 0 ? real_at(slot[2], r, i) : (T)0, off + q, acc);
+  }
+  using V = typename TreeVal<T>::type;
+  V v[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) v[c] = short_val<T>(acc[c]);
+  V* scr = reinterpret_cast<V*>(smem_raw);
+  block_sum8(v, scr, a.partials + (size_t)blockIdx.x * 8, 8);
+  if (arrive_last(a.counter)) {
+    finalize_eval8<T>(a.fin, scr);
+    if (threadIdx.x == 0) *a.counter = 0u;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Plane pass on clusters of CL blocks: y and x transforms, G-space terms and
+// the inverses of one kz plane of one field.  Block c of the cluster holds the
+// rows ROWS c .. of the plane (as k_plane's shared-memory plane, pitch N + 1).
+// CL = 1: columns in place.  CL > 1: block c transforms the columns COLS c ..;
+// the first stage along x reads its rows from the cluster's blocks through
+// distributed shared memory into a column buffer of its own, the last inverse
+// stage writes the rows back; two cluster barriers in all.
+template <typename T, int N, int CL> struct CP {
+  static constexpr CFac F = cfac(N, false);
+  static constexpr int NP = F.c, F0 = F.r[0], F1 = F.r[1], F2 = NP == 3 ? F.r[2] : 1;
+  static constexpr int ROWS = cdiv(N, CL), P = N + 1;
+  static constexpr int CPT = CL == 1 ? P : (ROWS | 1);       // column buffer pitch
+  static constexpr int NH = N / 2 + 1;
+  static constexpr int NT = fit_threads(ROWS * (N / F0), sizeof(T) == 4 ? 1024 : 512, 128);
+  static constexpr size_t BYTES = ((size_t)ROWS * P + (CL == 1 ? 0 : (size_t)N * CPT) + N) * sizeof(cplx<T>);
+};
+
+// One in-place butterfly with its twiddles (ip_stage's arithmetic).
+template <typename T, int N, int R, int DIR, int LSUB>
+__device__ __forceinline__ void cp_bfly(cplx<T> (&v)[R], int j, const cplx<T>* __restrict__ tw) {
+  constexpr int m = LSUB / R, tstep = N / LSUB;
+  if constexpr (DIR > 0 && m > 1) {
+#pragma unroll
+    for (int r = 1; r < R; ++r) {
+      cplx<T> w = tw[j * r * tstep];
+      w.y = -w.y;
+      v[r] = cmul(v[r], w);
+    }
+  }
+  Codelet<cplx<T>, R, DIR>::run(v);
+  if constexpr (DIR < 0 && m > 1) {
+#pragma unroll
+    for (int r = 1; r < R; ++r) v[r] = cmul(v[r], tw[j * r * tstep]);
+  }
+}
+
+// A stage along the rows held by the block, in shared memory.
+template <typename T, int N, int CL, int R, int DIR, int LSUB>
+__device__ __forceinline__ void cp_rows(cplx<T>* a, int nr, const cplx<T>* __restrict__ tw) {
+  using Q = CP<T, N, CL>;
+  constexpr int m = LSUB / R, PER = N / R;
+  for (int it = threadIdx.x; it < Q::ROWS * PER; it += Q::NT) {
+    int ln, t;
+    if constexpr (m >= 16) { ln = it / PER; t = it - ln * PER; }
+    else { t = it / Q::ROWS; ln = it - t * Q::ROWS; }
+    if (ln >= nr) continue;
+    const int b = t / m, j = t - b * m;
+    cplx<T>* x = a + ln * Q::P + b * LSUB + j;
+    cplx<T> v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = x[r * m];
+    cp_bfly<T, N, R, DIR, LSUB>(v, j, tw);
+#pragma unroll
+    for (int r = 0; r < R; ++r) x[r * m] = v[r];
+  }
+  __syncthreads();
+}
+// A stage along the block's columns, in the column buffer.
+template <typename T, int N, int CL, int R, int DIR, int LSUB>
+__device__ __forceinline__ void cp_cols(cplx<T>* b0, int nc, const cplx<T>* __restrict__ tw) {
+  using Q = CP<T, N, CL>;
+  constexpr int m = LSUB / R, PER = N / R;
+  for (int it = threadIdx.x; it < Q::ROWS * PER; it += Q::NT) {
+    const int t = it / Q::ROWS, col = it - t * Q::ROWS;
+    if (col >= nc) continue;
+    const int b = t / m, j = t - b * m;
+    cplx<T>* x = b0 + (b * LSUB + j) * Q::CPT + col;
+    cplx<T> v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = x[r * m * Q::CPT];
+    cp_bfly<T, N, R, DIR, LSUB>(v, j, tw);
+#pragma unroll
+    for (int r = 0; r < R; ++r) x[r * m * Q::CPT] = v[r];
+  }
+  __syncthreads();
+}
+
+template <typename T, int N, int CL>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(CP<T, N, CL>::NT, 1)
+k_plane_c(Spectra<T> sp, GArgs<T> g, const cplx<T>* __restrict__ tw_g) {
+  namespace cg = cooperative_groups;
+  using Q = CP<T, N, CL>;
+  using C = cplx<T>;
+  constexpr int F0 = Q::F0, F1 = Q::F1, F2 = Q::F2, P = Q::P, NN = N * N, M0 = N / F0;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* a = reinterpret_cast<C*>(smem_raw);
+  C* bc = CL == 1 ? a : a + Q::ROWS * P;
+  C* tw = (CL == 1 ? a + Q::ROWS * P : bc + N * Q::CPT);
+  const int c = CL == 1 ? 0 : (int)(blockIdx.x % CL);
+  const int kz = blockIdx.x / CL;
+  const int row0 = c * Q::ROWS;                          // first row, and first column, of this block
+  const int nr = min(Q::ROWS, N - row0);
+  const int fid = sp.idx[blockIdx.y];
+  C* gpl = sp.s[fid] + (size_t)kz * NN + (size_t)row0 * N;
+  for (int q = threadIdx.x; q < N; q += Q::NT) tw[q] = tw_g[q];
+  __syncthreads();
+  // along ky: stage 0 from memory
+  for (int it = threadIdx.x; it < Q::ROWS * M0; it += Q::NT) {
+    const int ln = it / M0, j = it - ln * M0;
+    if (ln >= nr) continue;
+    const C* x = gpl + ln * N + j;
+    C v[F0];
+#pragma unroll
+    for (int r = 0; r < F0; ++r) v[r] = __ldcg(x + r * M0);
+    cp_bfly<T, N, F0, -1, N>(v, j, tw);
+    C* y = a + ln * P + j;
+#pragma unroll
+    for (int r = 0; r < F0; ++r) y[r * M0] = v[r];
+  }
+  __syncthreads();
+  cp_rows<T, N, CL, F1, -1, M0>(a, nr, tw);
+  if constexpr (Q::NP == 3) cp_rows<T, N, CL, F2, -1, F2>(a, nr, tw);
+  // along kx
+  if constexpr (CL == 1) {
+    cp_cols<T, N, CL, F0, -1, N>(a, N, tw);
+  } else {
+    cg::cluster_group cl = cg::this_cluster();
+    cl.sync();
+    const C* part[CL];
+#pragma unroll
+    for (int o = 0; o < CL; ++o) part[o] = cl.map_shared_rank(a, o);
+    for (int it = threadIdx.x; it < Q::ROWS * M0; it += Q::NT) {
+      const int j = it / Q::ROWS, col = it - j * Q::ROWS;
+      if (col >= nr) continue;
+      C v[F0];
+#pragma unroll
+      for (int r = 0; r < F0; ++r) {
+        const int row = j + r * M0, o = row / Q::ROWS;
+        const C* src = part[0];
+#pragma unroll
+        for (int u = 1; u < CL; ++u) if (o == u) src = part[u];
+        v[r] = src[(row - o * Q::ROWS) * P + row0 + col];
+      }
+      cp_bfly<T, N, F0, -1, N>(v, j, tw);
+      C* y = bc + j * Q::CPT + col;
+#pragma unroll
+      for (int r = 0; r < F0; ++r) y[r * M0 * Q::CPT] = v[r];
+    }
+    __syncthreads();
+  }
+  if constexpr (Q::NP == 3) cp_cols<T, N, CL, F1, -1, M0>(bc, nr, tw);
+  // last forward stage, G-space terms, first inverse stage, in registers
+  constexpr int RL = Q::NP == 3 ? F2 : F1;               // position b RL + r
+  const T tp2 = g.tp2, invN = g.invN, Om = g.Om, halfOm = g.halfOm, g2cut = g.g2cut_loc;
+  const bool with_loc = fid == 0 && g.vloc != nullptr;
+  const T w = (kz == 0 || 2 * kz == N) ? (T)1 : (T)2;
+  const C* vpl = with_loc ? g.vloc + (size_t)kz * NN : nullptr;
+  // frequency at a position of the in-place transforms
+  auto freq = [](int p) {
+    const int k0 = p / M0, rest = p - k0 * M0;
+    if constexpr (Q::NP == 2) return k0 + F0 * rest;
+    else { const int k1 = rest / F2; return k0 + F0 * k1 + F0 * F1 * (rest - k1 * F2); }
+  };
+  auto sgn = [](int k) { return k <= (N - 1) / 2 ? k : k - N; };
+  AccShort<T> e0, e1;                                    // (E_H, E_loc) or (E_NL, E_vW), before the factors
+  for (int it = threadIdx.x; it < Q::ROWS * (N / RL); it += Q::NT) {
+    const int b = it / Q::ROWS, col = it - b * Q::ROWS;
+    if (col >= nr) continue;
+    C* x = bc + b * RL * Q::CPT + col;
+    C v[RL];
+#pragma unroll
+    for (int r = 0; r < RL; ++r) v[r] = x[r * Q::CPT];
+    Codelet<C, RL, -1>::run(v);
+    const int py = row0 + col, my = sgn(freq(py));
+    const int mk2 = my * my + kz * kz;
+    const int kx0 = freq(b * RL);
+    constexpr int KS = N / RL;                           // frequency step of the last stage
+#pragma unroll
+    for (int r = 0; r < RL; ++r) {
+      const int mx = sgn(kx0 + KS * r);
+      const int m2 = mx * mx + mk2;
+      const T vr = v[r].x * invN, vi = v[r].y * invN;    // f~(G)
+      const T a2 = vr * vr + vi * vi;
+      if (fid == 0) {
+        T orr = 0, oi = 0;
+        if (g.hartree && m2 > 0) {
+          const T cc = __ldg(g.cou + m2);                // 4 pi / G^2
+          e0.add(cc * a2);
+          orr = cc * vr; oi = cc * vi;
+        }
+        if (with_loc && tp2 * (T)m2 <= g2cut) {          // zero beyond the cutoff
+          const C vl = __ldg(vpl + (b * RL + r) * N + py);
+          e1.add(vr * vl.x + vi * vl.y);
+          orr += vl.x; oi += vl.y;
+        }
+        v[r] = mk<T>(orr, oi);
+      } else if (fid == 1) {
+        const T k = __ldg(g.K + m2);
+        e0.add(k * a2);
+        v[r] = mk<T>(k * vr, k * vi);
+      } else if (g.prec != nullptr) {
+        const T pg = __ldg(g.prec + m2);
+        v[r] = mk<T>(pg * vr, pg * vi);
+      } else {
+        const T G2 = tp2 * (T)m2;
+        e1.add(G2 * a2);
+        if (sp.merged) {
+          const T k = __ldg(g.K + m2);
+          e0.add(k * a2);
+          const T cc = k + (T)0.5 * G2;
+          v[r] = mk<T>(cc * vr, cc * vi);
+        } else {
+          v[r] = mk<T>(G2 * vr, G2 * vi);
+        }
+      }
+    }
+    Codelet<C, RL, +1>::run(v);
+#pragma unroll
+    for (int r = 0; r < RL; ++r) x[r * Q::CPT] = v[r];
+  }
+  __syncthreads();
+  // inverse along kx
+  if constexpr (Q::NP == 3) cp_cols<T, N, CL, F1, 1, M0>(bc, nr, tw);
+  if constexpr (CL == 1) {
+    cp_cols<T, N, CL, F0, 1, N>(a, N, tw);
+  } else {
+    cg::cluster_group cl = cg::this_cluster();
+    C* part[CL];
+#pragma unroll
+    for (int o = 0; o < CL; ++o) part[o] = cl.map_shared_rank(a, o);
+    for (int it = threadIdx.x; it < Q::ROWS * M0; it += Q::NT) {
+      const int j = it / Q::ROWS, col = it - j * Q::ROWS;
+      if (col >= nr) continue;
+      const C* y = bc + j * Q::CPT + col;
+      C v[F0];
+#pragma unroll
+      for (int r = 0; r < F0; ++r) v[r] = y[r * M0 * Q::CPT];
+      cp_bfly<T, N, F0, 1, N>(v, j, tw);
+#pragma unroll
+      for (int r = 0; r < F0; ++r) {
+        const int row = j + r * M0, o = row / Q::ROWS;
+        C* dst = part[0];
+#pragma unroll
+        for (int u = 1; u < CL; ++u) if (o == u) dst = part[u];
+        dst[(row - o * Q::ROWS) * P + row0 + col] = v[r];
+      }
+    }
+    cl.sync();                                           // (no remote access after this)
+  }
+  // inverse along ky: the last stage to memory
+  if constexpr (Q::NP == 3) cp_rows<T, N, CL, F2, 1, F2>(a, nr, tw);
+  cp_rows<T, N, CL, F1, 1, M0>(a, nr, tw);
+  for (int it = threadIdx.x; it < Q::ROWS * M0; it += Q::NT) {
+    const int ln = it / M0, j = it - ln * M0;
+    if (ln >= nr) continue;
+    const C* y = a + ln * P + j;
+    C v[F0];
+#pragma unroll
+    for (int r = 0; r < F0; ++r) v[r] = y[r * M0];
+    cp_bfly<T, N, F0, 1, N>(v, j, tw);
+    C* x = gpl + ln * N + j;
+#pragma unroll
+    for (int r = 0; r < F0; ++r) x[r * M0] = v[r];
+  }
+  if (g.prec != nullptr) return;                         // (the whole grid alike: no sums)
+  using V = typename TreeVal<T>::type;
+  AccShort<T> acc[4];
+  if (fid == 0) { acc[0].s = w * halfOm * e0.s; acc[1].s = w * Om * e1.s; }
+  else { acc[2].s = w * Om * e0.s; acc[3].s = w * halfOm * e1.s; }
+  V v8[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) v8[q] = q < 4 ? short_val<T>(acc[q]) : V{};
+  const size_t bi = (size_t)blockIdx.y * gridDim.x + blockIdx.x;
+  block_sum8(v8, reinterpret_cast<V*>(smem_raw), g.partials + bi * 4, 4);
+}
+
+// ---------------------------------------------------------------------------
+// The kernels of one grid size: function pointers and launch shapes, or
+// nothing when n has none (see cpass_kernels).
+template <typename T> struct CPass {
+  using ZF = void (*)(ProArgs<T>, Spectra<T>, const cplx<T>*, const cplx<T>*);
+  using ZI = void (*)(Spectra<T>, EpiArgs<T>, const cplx<T>*, const cplx<T>*);
+  using PL = void (*)(Spectra<T>, GArgs<T>, const cplx<T>*);
+  int n, rows, zthreads, zgrid;
+  CFac fz, fp;
+  ZF zfwd; ZI zinv;
+  size_t zf_bytes[4], zi_bytes[4];      // by number of fields
+  // the plane pass with one field, and with more
+  struct { PL kern; int cl, threads; size_t bytes; } pl[2];
+};
+
+// Cluster size for nf fields: the largest of 4, 2, 1 whose blocks fit about one
+// wave of the 152 SMs (more blocks than SMs would only queue behind a cluster
+// that is waiting), and whose two buffers fit a block.
+template <typename T, int N> constexpr int cp_cluster(int nf) {
+  constexpr size_t lim = 225 * 1024;
+  const int nh = N / 2 + 1;
+  if (nf * nh * 4 <= 168 && CP<T, N, 4>::BYTES <= lim) return 4;
+  if (nf * nh * 2 <= 168 && CP<T, N, 2>::BYTES <= lim) return 2;
+  return CP<T, N, 1>::BYTES <= lim ? 1 : (CP<T, N, 4>::BYTES <= lim ? 4 : 0);
+}
+
+template <typename T, int N> CPass<T> make_cpass() {
+  using Z = CZ<N>;
+  CPass<T> p{};
+  p.n = N; p.rows = Z::R; p.zthreads = Z::NT; p.zgrid = Z::GRID;
+  p.fz = Z::F; p.fp = cfac(N, false);
+  p.zfwd = k_zfwd_c<T, N>;
+  p.zinv = k_zinv_c<T, N>;
+  for (int f = 0; f < 4; ++f) { p.zf_bytes[f] = czfwd_bytes<T, N>(f); p.zi_bytes[f] = czinv_bytes<T, N>(f); }
+  constexpr int c1 = cp_cluster<T, N>(1), c2 = cp_cluster<T, N>(2);
+  if constexpr (c1 > 0) { p.pl[0].kern = k_plane_c<T, N, c1>; p.pl[0].cl = c1; p.pl[0].threads = CP<T, N, c1>::NT; p.pl[0].bytes = CP<T, N, c1>::BYTES; }
+  if constexpr (c2 > 0) { p.pl[1].kern = k_plane_c<T, N, c2>; p.pl[1].cl = c2; p.pl[1].threads = CP<T, N, c2>::NT; p.pl[1].bytes = CP<T, N, c2>::BYTES; }
+  return p;
+}
+
+// nullptr when the grid has no compile-time passes
+template <typename T> const CPass<T>* cpass_kernels(int n);
+
+}  // namespace ofdft

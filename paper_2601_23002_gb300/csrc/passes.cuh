@@ -43,50 +43,59 @@ template <typename T> struct Spectra {
 
 // ---------------------------------------------------------------------------
 // Finite-temperature Thomas-Fermi pointwise: eta(y) and p(y) from the
-// piecewise Chebyshev tables (see gen_fd_fits.py); f_TF = n T (eta - p),
+// piecewise polynomials (see gen_fd_fits.py); f_TF = n T (eta - p),
 // v_TF = T eta.
+
+// Interval and local variable of a table over 2^LG equal intervals per binade
+// from 2^elo: both come from the argument's bits (the interval from exponent
+// and leading mantissa bits, t = mantissa - the interval's middle, exact).
+// False outside the table (negative values, infinities and NaN included).
+static __device__ __forceinline__ bool binade_cell(double y, int elo, int nint, int& i, double& t) {
+  constexpr int LG = BIN64_LG;
+  const int hi = __double2hiint(y), lo = __double2loint(y);
+  i = (hi >> (20 - LG)) - ((1023 + elo) << LG);
+  const int keep = hi & (0xFFFFF & ~((1 << (20 - LG)) - 1));
+  t = __hiloint2double((hi & 0xFFFFF) | 0x3FF00000, lo) - __hiloint2double(keep | 0x3FF00000 | (1 << (19 - LG)), 0);
+  return (unsigned)i < (unsigned)nint;
+}
+// The two polynomials of a table row (coefficient pairs) at t.
+static __device__ __forceinline__ void binade_poly(const double* __restrict__ row, double t, double& a, double& b) {
+  const double2* c = reinterpret_cast<const double2*>(row);
+  double2 k[BIN64_NC];
+#pragma unroll
+  for (int q = 0; q < BIN64_NC; ++q) k[q] = __ldg(c + q);
+  a = k[BIN64_NC - 1].x;
+  b = k[BIN64_NC - 1].y;
+#pragma unroll
+  for (int q = BIN64_NC - 2; q >= 0; --q) { a = fma(a, t, k[q].x); b = fma(b, t, k[q].y); }
+}
+
+// FP64: 16 FP64 multiply-adds and one subtraction, no logarithm.  The FP64
+// pipe (1/58 of the FP32 rate) bounds every FP64 evaluation, so the table is
+// short in operations rather than in bytes (its hot intervals stay in L1).
 static __device__ __forceinline__ void fd_eta_p(double y, double& eta, double& p) {
-  const double s = log(y);
-  const double lngamma32 = -0.12078223763524522234551844578164;  // ln Gamma(3/2)
-  if (s < FD_S_LO) {
+  int i;
+  double t;
+  if (binade_cell(y, FD64_ELO, FD64_NINT, i, t)) {
+    binade_poly(fd64_tab[i], t, eta, p);
+  } else if (y < 1.0) {
     const double u = y * 1.1283791670955125738961589031215;      // y / Gamma(3/2)
-    eta = s - lngamma32 + u * 0.35355339059327376220042218105242;   // + u / 2^(3/2)
-    p = 1.0 + u * 0.17677669529663688110021109052621;               // 1 + u / 2^(5/2)
-  } else if (s >= FD_S_HI) {
-    const double e0 = pow(1.5 * y, 2.0 / 3.0);
-    eta = e0 * (1.0 - 0.82246703342411321823620758332301 / (e0 * e0));   // pi^2/12
-    p = 0.4 * eta * (1.0 + 4.9348022005446793094172454999381 / (eta * eta));  // pi^2/2
+    eta = log(u) + u * (FD_A1 + u * (FD_A2 + u * FD_A3));
+    p = 1.0 + u * (FD_B1 + u * (FD_B2 + u * FD_B3));
   } else {
-    const double r = (s - FD_S_LO) / FD64_W;
-    int i = (int)r;
-    i = i < 0 ? 0 : (i >= FD64_NINT ? FD64_NINT - 1 : i);
-    const double x = 2.0 * (r - (double)i) - 1.0;
-    double ce[FD64_NC], cp[FD64_NC];
-    static_assert(FD64_NC % 2 == 0, "16-byte loads");
-    const double2* e2 = reinterpret_cast<const double2*>(fd64_eta[i]);
-    const double2* p2 = reinterpret_cast<const double2*>(fd64_p[i]);
-#pragma unroll
-    for (int k = 0; k < FD64_NC / 2; ++k) {
-      const double2 ev = __ldg(e2 + k), pv = __ldg(p2 + k);
-      ce[2 * k] = ev.x; ce[2 * k + 1] = ev.y; cp[2 * k] = pv.x; cp[2 * k + 1] = pv.y;
-    }
-    double b1 = 0, b2 = 0, c1 = 0, c2 = 0;
-#pragma unroll
-    for (int k = FD64_NC - 1; k >= 1; --k) {
-      const double t = fma(2.0 * x, b1, ce[k] - b2); b2 = b1; b1 = t;
-      const double u = fma(2.0 * x, c1, cp[k] - c2); c2 = c1; c1 = u;
-    }
-    eta = fma(x, b1, ce[0] - b2);
-    p = fma(x, c1, cp[0] - c2);
+    // Sommerfeld: mu / E_F and p / (0.4 e0) through (T/E_F)^4
+    const double c = cbrt(1.5 * y), e0 = c * c, r2 = 1.0 / (e0 * e0);
+    eta = e0 * (1.0 - r2 * (0.82246703342411321823620758332301 + r2 * 1.2176136379250302));       // pi^2/12, pi^4/80
+    p = 0.4 * e0 * (1.0 + r2 * (4.1123351671205660911810379166151 - r2 * 6.0880681896251510));    // 5 pi^2/12, pi^4/16
   }
 }
 
-static __device__ __forceinline__ void fd_eta_p(float y, float& eta, float& p) {
-  const float s = __logf(y);      // a few ulp: far below the fit's use of s
-  const float lngamma32 = -0.120782237635245222f;
+// FP32: s = ln y is given (from a base-2 logarithm the caller also uses for
+// the exchange-correlation terms).
+static __device__ __forceinline__ void fd_eta_p_s(float y, float s, float& eta, float& p) {
   if (s < (float)FD_S_LO) {
     const float u = y * 1.12837916709551257f;
-    eta = s - lngamma32 + u * 0.353553390593273762f;
+    eta = s + 0.120782237635245222f + u * 0.353553390593273762f;    // - ln Gamma(3/2)
     p = 1.0f + u * 0.176776695296636881f;
   } else if (s >= (float)FD_S_HI) {
     const float e0 = powf(1.5f * y, 2.0f / 3.0f);
@@ -98,23 +107,18 @@ static __device__ __forceinline__ void fd_eta_p(float y, float& eta, float& p) {
     i = i < 0 ? 0 : (i >= FD32_NINT ? FD32_NINT - 1 : i);
     const float x = 2.0f * (r - (float)i) - 1.0f;
     // each interval's 8 coefficients as two 16-byte loads per table
-    float ce[FD32_NC], cp[FD32_NC];
     static_assert(FD32_NC == 8, "two float4 per interval");
     const float4* e4 = reinterpret_cast<const float4*>(fd32_eta[i]);
     const float4* p4 = reinterpret_cast<const float4*>(fd32_p[i]);
     const float4 ea = __ldg(e4), eb = __ldg(e4 + 1), pa = __ldg(p4), pb = __ldg(p4 + 1);
-    ce[0] = ea.x; ce[1] = ea.y; ce[2] = ea.z; ce[3] = ea.w; ce[4] = eb.x; ce[5] = eb.y; ce[6] = eb.z; ce[7] = eb.w;
-    cp[0] = pa.x; cp[1] = pa.y; cp[2] = pa.z; cp[3] = pa.w; cp[4] = pb.x; cp[5] = pb.y; cp[6] = pb.z; cp[7] = pb.w;
-    float b1 = 0, b2 = 0, c1 = 0, c2 = 0;
-#pragma unroll
-    for (int k = FD32_NC - 1; k >= 1; --k) {
-      const float t = fmaf(2.0f * x, b1, ce[k] - b2); b2 = b1; b1 = t;
-      const float u = fmaf(2.0f * x, c1, cp[k] - c2); c2 = c1; c1 = u;
-    }
-    eta = fmaf(x, b1, ce[0] - b2);
-    p = fmaf(x, c1, cp[0] - c2);
+    eta = fmaf(fmaf(fmaf(eb.w, x, eb.z), x, eb.y), x, eb.x);
+    eta = fmaf(fmaf(fmaf(fmaf(eta, x, ea.w), x, ea.z), x, ea.y), x, ea.x);
+    p = fmaf(fmaf(fmaf(pb.w, x, pb.z), x, pb.y), x, pb.x);
+    p = fmaf(fmaf(fmaf(fmaf(p, x, pa.w), x, pa.z), x, pa.y), x, pa.x);
   }
 }
+// (__logf: a few ulp, far below the fit's use of s)
+static __device__ __forceinline__ void fd_eta_p(float y, float& eta, float& p) { fd_eta_p_s(y, __logf(y), eta, p); }
 
 // Perdew-Zunger LDA, unpolarised: returns e_xc per electron, v_xc.
 // PZ81 joins its two correlation branches at r_s = 1 by continuity of e_c and
@@ -127,55 +131,67 @@ constexpr double kPzDen1 = 1.0 + kPzB1 + kPzB2;
 constexpr double kPzD = -kPzG * (0.5 * kPzB1 + kPzB2) / (kPzDen1 * kPzDen1) - kPzA - kPzC;
 constexpr double kPzB = kPzG / kPzDen1 - kPzD;
 
-template <typename T>
-__device__ __forceinline__ void pz81(T n, T& exc, T& vxc) {
-  const T third = (T)(1.0 / 3.0);
-  const T cbn = cbrt(n);
+// FP64: the polynomials of xc64_tab in u = n / n_1 (16 multiply-adds instead of
+// a cube root, a square root and three divisions); the formula outside.
+static __device__ __forceinline__ void pz81(double n, double& exc, double& vxc) {
+  int i;
+  double t;
+  const double u = n * (4.0 * kPi / 3.0);
+  if (binade_cell(u, XC64_ELO, XC64_NINT, i, t)) {
+    binade_poly(xc64_tab[i], t, exc, vxc);
+    return;
+  }
+  const double third = 1.0 / 3.0;
+  const double cbn = cbrt(n);
   // r_s = (3 / (4 pi n))^(1/3)
-  const T rs = (T)0.62035049089940001666800681204778 / cbn;
-  const T ex = (T)-0.73855876638202240588423003268 * cbn;   // -(3/4)(3/pi)^(1/3) n^(1/3)
-  const T vx = (T)(4.0 / 3.0) * ex;
-  T ec, vc;
-  if (rs >= (T)1) {
-    const T g = (T)kPzG, b1 = (T)kPzB1, b2 = (T)kPzB2;
-    const T sq = sqrt(rs);
-    const T den = (T)1 + b1 * sq + b2 * rs;
-    ec = g / den;
-    vc = ec * ((T)1 + (T)(7.0 / 6.0) * b1 * sq + (T)(4.0 / 3.0) * b2 * rs) / den;
+  const double rs = 0.62035049089940001666800681204778 / cbn;
+  const double ex = -0.73855876638202240588423003268 * cbn;   // -(3/4)(3/pi)^(1/3) n^(1/3)
+  const double vx = (4.0 / 3.0) * ex;
+  double ec, vc;
+  if (rs >= 1.0) {
+    const double sq = sqrt(rs);
+    const double den = 1.0 + kPzB1 * sq + kPzB2 * rs;
+    ec = kPzG / den;
+    vc = ec * (1.0 + (7.0 / 6.0) * kPzB1 * sq + (4.0 / 3.0) * kPzB2 * rs) / den;
   } else {
-    const T A = (T)kPzA, B = (T)kPzB, C = (T)kPzC, D = (T)kPzD;
-    const T ln = log(rs);
-    ec = A * ln + B + C * rs * ln + D * rs;
-    vc = A * ln + (B - A * third) + (T)(2.0 / 3.0) * C * rs * ln + ((T)2 * D - C) * third * rs;
+    const double ln = log(rs);
+    ec = kPzA * ln + kPzB + kPzC * rs * ln + kPzD * rs;
+    vc = kPzA * ln + (kPzB - kPzA * third) + (2.0 / 3.0) * kPzC * rs * ln + (2.0 * kPzD - kPzC) * third * rs;
   }
   exc = ex + ec;
   vxc = vx + vc;
 }
 
-// FP32 plans: fast reciprocals (__fdividef, a few ulp: inside the float
-// rounding of the terms they feed)
-template <>
-__device__ __forceinline__ void pz81<float>(float n, float& exc, float& vxc) {
-  const float cbn = cbrtf(n);
-  const float rs = __fdividef(0.620350490899400017f, cbn);
-  const float ex = -0.738558766382022406f * cbn;
+// FP32: l2 = log2 n is given.  w = n^(-1/3) from 2^(-l2/3) and one Newton step
+// of w^-3 = n (to FP32 rounding), so no cube root, and ln r_s from l2; fast
+// reciprocals (a few ulp: inside the float rounding of the terms they feed).
+static __device__ __forceinline__ void pz81_l2(float n, float l2, float& exc, float& vxc) {
+  float w = exp2f(l2 * (-1.0f / 3.0f));
+  w = fmaf(w * (1.0f / 3.0f), fmaf(-(n * w), w * w, 1.0f), w);
+  const float rs = 0.620350490899400017f * w;
+  const float ex = -0.738558766382022406f * (n * w) * w;
   const float vx = (4.0f / 3.0f) * ex;
   float ec, vc;
   if (rs >= 1.0f) {
     const float g = (float)kPzG, b1 = (float)kPzB1, b2 = (float)kPzB2;
-    const float sq = sqrtf(rs);
+    const float sq = rs * rsqrtf(rs);
     const float inv = __fdividef(1.0f, 1.0f + b1 * sq + b2 * rs);
     ec = g * inv;
     vc = ec * (1.0f + (7.0f / 6.0f) * b1 * sq + (4.0f / 3.0f) * b2 * rs) * inv;
   } else {
     const float A = (float)kPzA, B = (float)kPzB, C = (float)kPzC, D = (float)kPzD;
-    const float ln = __logf(rs);
+    // ln r_s = ln 0.62035 - (ln 2 / 3) log2 n
+    const float ln = fmaf(l2, -0.231049060186648431f, -0.477470652767060400f);
     ec = A * ln + B + C * rs * ln + D * rs;
     vc = A * ln + (B - A * (1.0f / 3.0f)) + (2.0f / 3.0f) * C * rs * ln + (2.0f * D - C) * (1.0f / 3.0f) * rs;
   }
   exc = ex + ec;
   vxc = vx + vc;
 }
+static __device__ __forceinline__ void pz81(float n, float& exc, float& vxc) { pz81_l2(n, __log2f(n), exc, vxc); }
+
+static __device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
+static __device__ __forceinline__ double rsqrt_t(double x) { return rsqrt(x); }
 
 template <typename T> __device__ __forceinline__ T pow_t(T a, T b);
 template <> __device__ __forceinline__ double pow_t<double>(double a, double b) { return pow(a, b); }
@@ -595,6 +611,7 @@ template <typename T> struct EpiArgs {
   const double* dsc;     // when set, scale = dsc[0] and t = dsc[2] (a trial formed on the device)
   int fd64;              // FP32 plans: invert the Fermi-Dirac integral in FP64 (y = cy_d n in FP64)
   double cy_d;           // pi^2 / (sqrt2 T^(3/2)) in FP64, for fd64
+  T lcy;                 // ln cy (FP32 plans: ln y = ln 2 log2 n + ln cy)
 };
 
 // The pointwise functional at one grid point, shared by the z-pass epilogue
@@ -606,22 +623,27 @@ template <typename T> struct EpiArgs {
 // 5 int g' psi_t, 6 int n, 7 nonfinite count.
 template <typename T> struct EpiPoint {
   bool has_n, has_na, has_psi, merged;
-  T Te, cy, alpha, nmin, tstep, tscale, muref;
+  T Te, cy, lcy, alpha, nmin, tstep, tscale, muref;
   __device__ __forceinline__ EpiPoint(const Spectra<T>& sp, const EpiArgs<T>& a)
       : has_n(sp.s[0] != nullptr), has_na(sp.s[1] != nullptr), has_psi(sp.s[2] != nullptr),
-        merged(sp.merged != 0), Te(a.T_e), cy(a.cy), alpha(a.alpha), nmin((T)kNmin),
+        merged(sp.merged != 0), Te(a.T_e), cy(a.cy), lcy(a.lcy), alpha(a.alpha), nmin((T)kNmin),
         tstep(a.dsc ? (T)a.dsc[2] : a.t), tscale(a.dsc ? (T)a.dsc[0] : a.scale), muref(a.mu_ref) {}
   __device__ __forceinline__ void point(const EpiArgs<T>& a, T pv, T dq, T hv, T kv, T lv, size_t at,
                                         AccShort<T> (&acc)[8]) const {
-    T psit, nval;
+    T psit, nval, iphi = 0;              // iphi: 1 / max(psi, kPhiMin), mode 0 only
     if (a.mode == 0) {
+      // one reciprocal square root for psi and the division by it
       nval = pv;
-      psit = sqrt(fmax(nval, (T)0));
+      const T r = rsqrt_t(fmax(nval, (T)1e-30));
+      psit = fmax(nval, (T)0) * r;
+      iphi = fmin(r, (T)(1.0 / kPhiMin));
     } else {
       psit = pv + tstep * dq;
       nval = tscale * psit * psit;
     }
     const T nf = fmax(nval, nmin);
+    T l2 = 0;                            // FP32: one logarithm for TF and XC
+    if constexpr (sizeof(T) == 4) l2 = __log2f(nf);
     T vrest = 0;
     if (a.terms & 1) {              // TF
       if (sizeof(T) == 4 && a.fd64) {
@@ -633,21 +655,23 @@ template <typename T> struct EpiPoint {
         acc[0].add((T)((double)nf * te * (eta - p)));
       } else {
         T eta, p;
-        fd_eta_p(nf * cy, eta, p);
+        if constexpr (sizeof(T) == 4) fd_eta_p_s(nf * cy, fmaf(l2, 0.693147180559945309f, lcy), eta, p);
+        else fd_eta_p(nf * cy, eta, p);
         vrest += Te * eta;
         acc[0].add(nf * Te * (eta - p));
       }
     }
     if (a.terms & 8) {              // XC
       T exc, vxc;
-      pz81<T>(nf, exc, vxc);
+      if constexpr (sizeof(T) == 4) pz81_l2(nf, l2, exc, vxc);
+      else pz81(nf, exc, vxc);
       vrest += vxc;
       acc[1].add(nval * exc);
     }
-    finish(a, psit, nval, nf, dq, vrest, hv, kv, lv, at, acc);
+    finish(a, psit, nval, nf, iphi, dq, vrest, hv, kv, lv, at, acc);
   }
   // the nonlocal and G-space contributions, the output and the sums
-  __device__ __forceinline__ void finish(const EpiArgs<T>& a, T psit, T nval, T nf, T dq, T vrest, T hv, T kv,
+  __device__ __forceinline__ void finish(const EpiArgs<T>& a, T psit, T nval, T nf, T iphi, T dq, T vrest, T hv, T kv,
                                          T lv, size_t at, AccShort<T> (&acc)[8]) const {
     if (has_n) vrest += hv;
     if (has_na) vrest += (T)2 * alpha * pow_t<T>(nf, alpha - (T)1) * kv;
@@ -661,8 +685,7 @@ template <typename T> struct EpiPoint {
     const T gp = psit * (vrest - muref) + extra;
     T* __restrict__ gout = a.out;
     if (a.mode == 0) {
-      const T phi = fmax(psit, (T)kPhiMin);
-      const T v = vrest + extra / phi;
+      const T v = vrest + extra * iphi;
       if (gout) gout[at] = v;
       // residual pieces with psi = sqrt(rho), scale 1: g' = psi v_rest + lap/2
       if (!isfinite(v)) acc[7].add((T)1);

@@ -601,7 +601,7 @@ __global__ void __launch_bounds__(256) k_pressure_r(const T* __restrict__ rho, s
     }
     if (terms & 8) {
       T exc, vxc;
-      pz81<T>(nf, exc, vxc);
+      pz81(nf, exc, vxc);
       acc[1].add(nval * (vxc - exc));
     }
   }
