@@ -19,6 +19,8 @@ OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libofdft_gb300.so")
 SOURCES = ["api.cu", "engine_f32.cu", "engine_f64.cu", "plane_f32.cu", "plane_f64.cu", "plane2_f32.cu",
            "plane2_f64.cu", "noalloc.cu"]
+# sources compiled several times, each part with its own share of the kernels (-DCPASS_PART=i)
+PARTED = {"cpass_f32.cu": 4, "cpass_f64.cu": 4}
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -51,9 +53,14 @@ def build(force: bool = False, verbose: bool = False) -> str:
     flags = ARCH + ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
                     "-I", os.path.join(HERE, "..", "include")]
 
-    def compile_one(src):
-        obj = os.path.join(OUT, src.replace(".cu", ".o"))
-        cmd = [nvcc] + flags + ["-c", os.path.join(CSRC, src), "-o", obj]
+    jobs = [(src, part) for src, count in PARTED.items() for part in range(count)]
+    jobs += [(src, None) for src in SOURCES]
+
+    def compile_one(job):
+        src, part = job
+        obj = os.path.join(OUT, src.replace(".cu", ".o" if part is None else f"_{part}.o"))
+        define = [] if part is None else [f"-DCPASS_PART={part}"]
+        cmd = [nvcc] + flags + define + ["-c", os.path.join(CSRC, src), "-o", obj]
         if verbose:
             print(" ".join(cmd), file=sys.stderr)
         r = subprocess.run(cmd, capture_output=True, text=True)
@@ -61,8 +68,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
             raise RuntimeError(f"nvcc failed on {src}:\n{r.stderr[-4000:]}")
         return obj
 
-    with ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
-        objs = list(ex.map(compile_one, SOURCES))
+    with ThreadPoolExecutor(max_workers=len(jobs)) as ex:
+        objs = list(ex.map(compile_one, jobs))
     tmp = LIB + f".tmp{os.getpid()}"
     cmd = [nvcc] + ARCH + ["-shared", "-o", tmp] + objs + ["-lcudart"]
     r = subprocess.run(cmd, capture_output=True, text=True)

@@ -78,11 +78,11 @@ template <int N> struct CZ {
   static constexpr int L = ODD ? N : H;
   static constexpr int LINES = ODD ? R / 2 : R;         // transforms per block and field
   static constexpr CFac F = cfac(L, !ODD);
-  static constexpr int F0 = F.r[0], F1 = F.r[1], F2 = F.c == 3 ? F.r[2] : 1;
+  static constexpr int F0 = F.r[0], F1 = F.c >= 2 ? F.r[1] : 1, F2 = F.c == 3 ? F.r[2] : 1;
   static constexpr int NT = N <= 50 ? 128 : 256;
   // element e of a line sits at e + e / F0 (even F0: the first stage writes
   // with stride F0); odd pitch, so that lines differ in bank
-  static constexpr int pad(int e) { return (F0 & 1) ? e : e + e / F0; }
+  static __host__ __device__ constexpr int pad(int e) { return (F0 & 1) ? e : e + e / F0; }
   static constexpr int XP = (pad(L - 1) + 1) | 1;
   static constexpr int SP = (ODD ? (N + 1) / 2 : NH) | 1;   // spectrum row pitch (odd n: two rows hold a line of L <= 2 SP)
   static constexpr int BP = (ODD ? 2 : 1) * SP;             // the same region as lines: pitch
@@ -176,14 +176,16 @@ static __device__ void finalize_eval8(const FinArgs<T>& f, typename TreeVal<T>::
 
 // ---------------------------------------------------------------------------
 // The stages of a z pass after the first, in shared memory, all lines of the
-// block at once: data in xa (padded), the result as natural elements: get(line, e)
-// of the result's buffer is xa[line XP + pad(e)] for two stages and
+// block at once: data in xa (padded), the result as natural elements (cz_get):
+// element e of a line at xa[line XP + pad(e)] for one or two stages and at
 // xb[line BP + e] for three.  Ends with a barrier.
 template <typename T, int N, int DIR>
 __device__ __forceinline__ void cz_stages(cplx<T>* xa, cplx<T>* xb, int lines, const cplx<T>* __restrict__ tw) {
   using Z = CZ<N>;
   constexpr int L = Z::L, F0 = Z::F0, F1 = Z::F1, F2 = Z::F2;
-  if constexpr (Z::F.c == 2) {
+  if constexpr (Z::F.c == 1) {
+    return;
+  } else if constexpr (Z::F.c == 2) {
     for (int it = threadIdx.x; it < lines * F0; it += Z::NT) {
       const int ln = it / F0, j = it - ln * F0;
       cplx<T>* x = xa + ln * Z::XP;
@@ -244,9 +246,24 @@ __device__ __forceinline__ void cz_stages(cplx<T>* xa, cplx<T>* xb, int lines, c
 template <typename T, int N>
 __device__ __forceinline__ cplx<T> cz_get(const cplx<T>* xa, const cplx<T>* xb, int ln, int e) {
   using Z = CZ<N>;
-  if constexpr (Z::F.c == 2) return xa[ln * Z::XP + Z::pad(e)];
+  if constexpr (Z::F.c <= 2) return xa[ln * Z::XP + Z::pad(e)];
   else return xb[ln * Z::BP + e];
 }
+
+// The active fields' indices and spectra by selection: a parameter array indexed
+// at run time would be copied to local memory.
+template <typename T> struct CField {
+  int i0, i1, i2;
+  cplx<T>*s0, *s1, *s2;
+  __device__ __forceinline__ explicit CField(const Spectra<T>& sp) : i0(sp.idx[0]), i1(sp.idx[1]), i2(sp.idx[2]) {
+    s0 = pick(sp, i0); s1 = pick(sp, i1); s2 = pick(sp, i2);
+  }
+  static __device__ __forceinline__ cplx<T>* pick(const Spectra<T>& sp, int i) {
+    return i == 0 ? sp.s[0] : i == 1 ? sp.s[1] : sp.s[2];
+  }
+  __device__ __forceinline__ int id(int f) const { return f == 0 ? i0 : f == 1 ? i1 : i2; }
+  __device__ __forceinline__ cplx<T>* spec(int f) const { return f == 0 ? s0 : f == 1 ? s1 : s2; }
+};
 
 // shared memory: tw[L] | twn[NH] | xa[nf][LINES][XP] | xb[nf][LINES][BP] (three stages)
 template <typename T, int N> __host__ __device__ constexpr size_t czfwd_bytes(int nf) {
@@ -266,6 +283,7 @@ k_zfwd_c(ProArgs<T> a, Spectra<T> sp, const cplx<T>* __restrict__ tw_l, const cp
   C* twn = tw + L;
   C* xa = twn + NH;
   C* xb = xa + sp.nact * Z::LINES * Z::XP;
+  const CField<T> fl_(sp);
   const int row0 = blockIdx.x * R;
   const int rows = min(R, NN - row0);
   const int lines = Z::ODD ? (rows + 1) >> 1 : rows;
@@ -290,7 +308,7 @@ k_zfwd_c(ProArgs<T> a, Spectra<T> sp, const cplx<T>* __restrict__ tw_l, const cp
     const int fl = it / M0, j = it - fl * M0;
     const int f = fl / Z::LINES, ln = fl - f * Z::LINES;
     if (ln >= lines) continue;
-    const int fid = sp.idx[f];
+    const int fid = fl_.id(f);
     C v[F0];
     if constexpr (Z::ODD) {
       const bool two = 2 * ln + 1 < rows;
@@ -355,7 +373,7 @@ k_zfwd_c(ProArgs<T> a, Spectra<T> sp, const cplx<T>* __restrict__ tw_l, const cp
       const C wo = cmul(twn[k], csub(zk, zc));
       o = mk<T>((T)0.5 * (e.x + wo.y), (T)0.5 * (e.y - wo.x));
     }
-    sp.s[sp.idx[f]][(size_t)k * NN + row0 + r] = o;
+    fl_.spec(f)[(size_t)k * NN + row0 + r] = o;
   }
 }
 
@@ -380,13 +398,14 @@ k_zinv_c(Spectra<T> sp, EpiArgs<T> a, const cplx<T>* __restrict__ tw_l, const cp
   C* twn = tw + L;
   C* stg = twn + NH;
   C* xa = stg + sp.nact * R * Z::SP;
+  const CField<T> fl_(sp);
   const int row0 = blockIdx.x * R;
   const int rows = min(R, NN - row0);
   const size_t off = (size_t)row0 * N;
   for (int q = threadIdx.x; q < sp.nact * NH * R; q += Z::NT) {
     const int fk = q / R, r = q - fk * R;
     const int f = fk / NH, k = fk - f * NH;
-    if (r < rows) cp_async_c(stg + (f * R + r) * Z::SP + k, sp.s[sp.idx[f]] + (size_t)k * NN + row0 + r, true);
+    if (r < rows) cp_async_c(stg + (f * R + r) * Z::SP + k, fl_.spec(f) + (size_t)k * NN + row0 + r, true);
   }
   cp_async_commit();
   for (int q = threadIdx.x; q < L + NH; q += Z::NT) tw[q] = q < L ? tw_l[q] : tw_n[q - L];
@@ -453,8 +472,11 @@ k_zinv_c(Spectra<T> sp, EpiArgs<T> a, const cplx<T>* __restrict__ tw_l, const cp
     }
     return;
   }
-  int slot[3] = {-1, -1, -1};
-  for (int f = 0; f < sp.nact; ++f) slot[sp.idx[f]] = f;
+  // the slot of each field, -1: not active
+  int slot[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+    slot[i] = (sp.nact > 0 && fl_.i0 == i) ? 0 : (sp.nact > 1 && fl_.i1 == i) ? 1 : (sp.nact > 2 && fl_.i2 == i) ? 2 : -1;
   const EpiPoint<T> ep(sp, a);
   AccShort<T> acc[8];
   const T* src = (a.mode == 0 ? a.rho : a.psi) + off;
@@ -489,10 +511,11 @@ k_zinv_c(Spectra<T> sp, EpiArgs<T> a, const cplx<T>* __restrict__ tw_l, const cp
 template <typename T, int N, int CL> struct CP {
   static constexpr CFac F = cfac(N, false);
   static constexpr int NP = F.c, F0 = F.r[0], F1 = F.r[1], F2 = NP == 3 ? F.r[2] : 1;
-  static constexpr int ROWS = cdiv(N, CL), P = N + 1;
+  static constexpr int ROWS = cdiv(N, CL), P = N | 1;        // odd pitch: rows and columns free of bank conflicts
   static constexpr int CPT = CL == 1 ? P : (ROWS | 1);       // column buffer pitch
   static constexpr int NH = N / 2 + 1;
-  static constexpr int NT = fit_threads(ROWS * (N / F0), sizeof(T) == 4 ? 1024 : 512, 128);
+  // radix 16 takes more than the 64 registers of a 1024-thread block
+  static constexpr int NT = fit_threads(ROWS * (N / F0), sizeof(T) == 4 && F0 < 16 ? 1024 : 512, 128);
   static constexpr size_t BYTES = ((size_t)ROWS * P + (CL == 1 ? 0 : (size_t)N * CPT) + N) * sizeof(cplx<T>);
 };
 
@@ -571,8 +594,8 @@ k_plane_c(Spectra<T> sp, GArgs<T> g, const cplx<T>* __restrict__ tw_g) {
   const int kz = blockIdx.x / CL;
   const int row0 = c * Q::ROWS;                          // first row, and first column, of this block
   const int nr = min(Q::ROWS, N - row0);
-  const int fid = sp.idx[blockIdx.y];
-  C* gpl = sp.s[fid] + (size_t)kz * NN + (size_t)row0 * N;
+  const int fid = blockIdx.y == 0 ? sp.idx[0] : blockIdx.y == 1 ? sp.idx[1] : sp.idx[2];
+  C* gpl = CField<T>::pick(sp, fid) + (size_t)kz * NN + (size_t)row0 * N;
   for (int q = threadIdx.x; q < N; q += Q::NT) tw[q] = tw_g[q];
   __syncthreads();
   // along ky: stage 0 from memory
@@ -597,9 +620,6 @@ k_plane_c(Spectra<T> sp, GArgs<T> g, const cplx<T>* __restrict__ tw_g) {
   } else {
     cg::cluster_group cl = cg::this_cluster();
     cl.sync();
-    const C* part[CL];
-#pragma unroll
-    for (int o = 0; o < CL; ++o) part[o] = cl.map_shared_rank(a, o);
     for (int it = threadIdx.x; it < Q::ROWS * M0; it += Q::NT) {
       const int j = it / Q::ROWS, col = it - j * Q::ROWS;
       if (col >= nr) continue;
@@ -607,10 +627,7 @@ k_plane_c(Spectra<T> sp, GArgs<T> g, const cplx<T>* __restrict__ tw_g) {
 #pragma unroll
       for (int r = 0; r < F0; ++r) {
         const int row = j + r * M0, o = row / Q::ROWS;
-        const C* src = part[0];
-#pragma unroll
-        for (int u = 1; u < CL; ++u) if (o == u) src = part[u];
-        v[r] = src[(row - o * Q::ROWS) * P + row0 + col];
+        v[r] = cl.map_shared_rank(a, o)[(row - o * Q::ROWS) * P + row0 + col];
       }
       cp_bfly<T, N, F0, -1, N>(v, j, tw);
       C* y = bc + j * Q::CPT + col;
@@ -696,9 +713,6 @@ k_plane_c(Spectra<T> sp, GArgs<T> g, const cplx<T>* __restrict__ tw_g) {
     cp_cols<T, N, CL, F0, 1, N>(a, N, tw);
   } else {
     cg::cluster_group cl = cg::this_cluster();
-    C* part[CL];
-#pragma unroll
-    for (int o = 0; o < CL; ++o) part[o] = cl.map_shared_rank(a, o);
     for (int it = threadIdx.x; it < Q::ROWS * M0; it += Q::NT) {
       const int j = it / Q::ROWS, col = it - j * Q::ROWS;
       if (col >= nr) continue;
@@ -710,10 +724,7 @@ k_plane_c(Spectra<T> sp, GArgs<T> g, const cplx<T>* __restrict__ tw_g) {
 #pragma unroll
       for (int r = 0; r < F0; ++r) {
         const int row = j + r * M0, o = row / Q::ROWS;
-        C* dst = part[0];
-#pragma unroll
-        for (int u = 1; u < CL; ++u) if (o == u) dst = part[u];
-        dst[(row - o * Q::ROWS) * P + row0 + col] = v[r];
+        cl.map_shared_rank(a, o)[(row - o * Q::ROWS) * P + row0 + col] = v[r];
       }
     }
     cl.sync();                                           // (no remote access after this)
@@ -760,15 +771,23 @@ template <typename T> struct CPass {
   struct { PL kern; int cl, threads; size_t bytes; } pl[2];
 };
 
-// Cluster size for nf fields: the largest of 4, 2, 1 whose blocks fit about one
-// wave of the 152 SMs (more blocks than SMs would only queue behind a cluster
-// that is waiting), and whose two buffers fit a block.
+// Cluster size for nf fields.  FP32 (bound by latency and barriers): clusters
+// only where they fit about one wave of the 152 SMs (75^3, 76 planes: 17.9 ->
+// 13.8 us with 2; 108^3, 110 planes: 22.0 -> 30 us with 4, since the remote rows
+// cost more than the shorter stages save), or where single blocks need a second
+// wave (160^3, 162 planes: 93 -> 64 us with 5).  FP64 (bound by the FP64 pipe of
+// the busiest SM): the least rows there, ceil(nf nh CL / 152) blocks of ROWS
+// rows, the smaller cluster within 10% (96^3: 277 -> 224 us with 4; 45^3: 69 ->
+// 43 with 2), and what fits in shared memory.
+template <typename T, int N, int CL> constexpr int cp_load(int nf) {
+  return CP<T, N, CL>::BYTES > (size_t)225 * 1024 ? 1 << 20 : cdiv(nf * (N / 2 + 1) * CL, 152) * CP<T, N, CL>::ROWS;
+}
 template <typename T, int N> constexpr int cp_cluster(int nf) {
-  constexpr size_t lim = 225 * 1024;
-  const int nh = N / 2 + 1;
-  if (nf * nh * 4 <= 168 && CP<T, N, 4>::BYTES <= lim) return 4;
-  if (nf * nh * 2 <= 168 && CP<T, N, 2>::BYTES <= lim) return 2;
-  return CP<T, N, 1>::BYTES <= lim ? 1 : (CP<T, N, 4>::BYTES <= lim ? 4 : 0);
+  const int planes = nf * (N / 2 + 1);
+  if (sizeof(T) == 4) return planes * 4 <= 168 ? 4 : planes * 2 <= 168 ? 2 : planes <= 152 ? 1 : 5;
+  const int l1 = cp_load<T, N, 1>(nf), l2 = cp_load<T, N, 2>(nf), l4 = cp_load<T, N, 4>(nf);
+  const int best = l1 < l2 ? (l1 < l4 ? l1 : l4) : (l2 < l4 ? l2 : l4);
+  return 10 * l1 <= 11 * best ? 1 : 10 * l2 <= 11 * best ? 2 : 4;
 }
 
 template <typename T, int N> CPass<T> make_cpass() {

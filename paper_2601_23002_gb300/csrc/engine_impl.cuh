@@ -16,6 +16,7 @@
 #include "profiler.h"
 #include "fft.cuh"
 #include "passes.cuh"
+#include "cpass.cuh"
 #include "plane.cuh"
 #include "setup.cuh"
 #include "vecops.cuh"
@@ -115,6 +116,16 @@ class Engine : public IEngine {
   bool plane_allowed = true;
   bool planes = false;
   size_t smem_pl = 0;
+  // compile-time passes of this grid (cpass.cuh; OFDFT_CPASS=0: the generic
+  // ones), and whether the z passes' rows and radices are theirs
+  bool cpass_allowed = true;
+  const CPass<T>* cp = nullptr;
+  bool cpz() const {
+    if (!cp || zR != cp->rows || ph.npass != cp->fz.c) return false;
+    for (int i = 0; i < ph.npass; ++i) if (ph.radix[i] != cp->fz.r[i]) return false;
+    return true;
+  }
+  T* cou = nullptr;          // 4 pi / G^2 by m^2
   int* rev_d = nullptr;      // position -> frequency of the in-place transforms
   PlaneKernel<T> plane_kern = nullptr;   // k_plane compiled for this grid's radices
   // one-field preconditioning pass on two-block clusters (half a plane per
@@ -185,6 +196,8 @@ class Engine : public IEngine {
     tune.zR = env("OFDFT_ZR");
     const char* pe = std::getenv("OFDFT_PLANE");
     plane_allowed = !(pe && pe[0] == '0');
+    const char* c1 = std::getenv("OFDFT_CPASS");
+    cpass_allowed = !(c1 && c1[0] == '0');
     const char* z2 = std::getenv("OFDFT_Z256");
     z256_allowed = !(z2 && z2[0] == '0');
     const char* q2 = std::getenv("OFDFT_P256");
@@ -284,7 +297,9 @@ class Engine : public IEngine {
     L = cs.L; Omega = L * L * L; dV = Omega / (double)N;
     Ne = 0; for (double z : cs.Z) Ne += z;
     nbar = Ne / Omega; Te = cs.T;
+    cp = plane_allowed && cpass_allowed ? cpass_kernels<T>(n) : nullptr;
     zR = std::max(1, std::min(16, 1024 / h));     // 16 rows per block: best in a sweep at 128^3
+    if (cp) zR = cp->rows;
     zP = zpitch();
     yJ = sizeof(T) == 4 ? 16 : 8;
     xJ = yJ;
@@ -308,7 +323,7 @@ class Engine : public IEngine {
     grid_x = (int)(((size_t)n * nh + xJ - 1) / xJ);
     smem_pl = std::max(((size_t)n * (n + 1) + n) * sizeof(C) + (size_t)n * sizeof(int),
                        tree_scratch_bytes<T>(4, kPlaneThreads));
-    planes = plane_allowed && smem_pl <= (size_t)225 * 1024;
+    planes = cp || (plane_allowed && smem_pl <= (size_t)225 * 1024);
     // (rows per block even and dividing n^2: 8, 16 or 32)
     z256 = z256_allowed && sizeof(T) == 4 && n == 256 && !planes && (zR == 8 || zR == 16 || zR == 32);
     p256 = z256 && p256_possible();
@@ -320,7 +335,7 @@ class Engine : public IEngine {
     // 712 -> 669 snapshots/s with clusters)
     smem_pl2 = ((size_t)(n / 2) * (n + 1) + n) * sizeof(C) + (size_t)n * sizeof(int);
     // (even n only: the pair splits the plane's rows in two equal halves)
-    prec2 = plane_allowed && prec2_allowed && n >= 112 && n % 2 == 0 && smem_pl2 <= (size_t)225 * 1024;
+    prec2 = !cp && plane_allowed && prec2_allowed && n >= 112 && n % 2 == 0 && smem_pl2 <= (size_t)225 * 1024;
     // streaming vector kernels: a multiple of the SM count (4 resident blocks
     // per SM); the async-copy ring kernels hold 160 KB of shared memory, one
     // block per SM
@@ -364,6 +379,31 @@ class Engine : public IEngine {
       return OFDFT_ERR_INVALID;
     }
   }
+
+  // The compile-time passes.  Even grids read two reals at a time, so a
+  // density that is not aligned to them takes the generic forward pass.
+  bool czfwd_ok(const ProArgs<T>& pa) const {
+    return cpz() && ((n & 1) || pa.mode != 0 || reinterpret_cast<uintptr_t>(pa.rho) % sizeof(C) == 0);
+  }
+  int launch_zfwd(const ProArgs<T>& pa, const Spectra<T>& sp, double bytes, cudaStream_t st) {
+    if (z256) return launch_zfwd256(pa, sp, bytes, st);
+    if (czfwd_ok(pa)) OFDFT_RUN("k_zfwd_c", st, bytes, cp->zfwd<<<cp->zgrid, cp->zthreads, cp->zf_bytes[sp.nact], st>>>(pa, sp, tw_h, tw_n));
+    else OFDFT_RUN("k_zfwd", st, bytes, k_zfwd<T><<<grid_z, kThreads, smem_zf, st>>>(pa, sp, ph, tw_h, tw_n, n, zR, zP));
+    return OFDFT_OK;
+  }
+  int launch_zinv(const Spectra<T>& sp, const EpiArgs<T>& ea, double bytes, cudaStream_t st) {
+    if (z256) return launch_zinv256(sp, ea, bytes, st);
+    if (cpz()) OFDFT_RUN("k_zinv_c", st, bytes, cp->zinv<<<cp->zgrid, cp->zthreads, cp->zi_bytes[sp.nact], st>>>(sp, ea, tw_h, tw_n));
+    else OFDFT_RUN("k_zinv_epi", st, bytes, k_zinv_epi<T><<<grid_z, kThreads, smem_zi, st>>>(sp, ea, ph, tw_h, tw_n, n, zR, zP));
+    return OFDFT_OK;
+  }
+  int launch_cplane(const Spectra<T>& sp, const GArgs<T>& ga, double bytes, cudaStream_t st) {
+    const auto& pl = cp->pl[sp.nact > 1];
+    OFDFT_RUN("k_plane_c", st, bytes, pl.kern<<<dim3(pl.cl * nh, sp.nact), pl.threads, pl.bytes, st>>>(sp, ga, tw_n));
+    return OFDFT_OK;
+  }
+  // rows of G-space partials the epilogue's partials come after (3 fields)
+  size_t g_room() const { return (size_t)std::max(z256 ? kGridX256 : grid_x, 8 * nh) * 3; }
 
   size_t plan_bytes_estimate() {
     geometry();
@@ -411,7 +451,7 @@ class Engine : public IEngine {
       }
       if (prod == h) ph = q;
     }
-    if (planes) plane_kern = plane_kernel<T>(radix_mask(pn));
+    if (planes && !cp) plane_kern = plane_kernel<T>(radix_mask(pn));
     if (prec2) prec2_kern = plane_prec2_kernel<T>(radix_mask(pn));
     int rc;
     // twiddles
@@ -483,10 +523,20 @@ class Engine : public IEngine {
     const int nm2 = 3 * h * h + 1;
     if ((rc = alloc(&Kd, nm2))) return rc;
     if ((rc = alloc(&Kt, nm2))) return rc;
+    std::vector<T> couh;
+    if (cp) {
+      const double tp = 2.0 * kPi / L;
+      const T tp2 = (T)(tp * tp);
+      couh.resize(nm2);
+      couh[0] = 0;
+      for (int m2 = 1; m2 < nm2; ++m2) couh[m2] = (T)(4.0 * kPi) / (tp2 * (T)m2);
+      if ((rc = alloc(&cou, nm2))) return rc;
+      OFDFT_CK(cudaMemcpyAsync(cou, couh.data(), nm2 * sizeof(T), cudaMemcpyHostToDevice, st));
+    }
     // eval uses [0, 4 grid_x) for G-space partials and [4 grid_x, 4 grid_x + 8 grid_z) for the epilogue
     // (sized for the smallest tiles the autotuner may pick: 8 rows, 8 columns)
-    partials_cap = std::max<size_t>({(size_t)grid_x * 12 + (size_t)grid_z * 8,
-                                     ((size_t)n * nh + 7) / 8 * 12 + ((size_t)n * n + 7) / 8 * 8,
+    partials_cap = std::max<size_t>({g_room() * 4 + (size_t)grid_z * 8,
+                                     std::max((size_t)(n * nh + 7) / 8, (size_t)8 * nh) * 12 + ((size_t)n * n + 7) / 8 * 8,
                                      (size_t)grid_vec * kMaxV * kMaxW, (size_t)n * n, (size_t)4096});
     if ((rc = alloc(&partials, partials_cap))) return rc;
     if ((rc = alloc(&res_d, kResSlots))) return rc;
@@ -666,7 +716,13 @@ class Engine : public IEngine {
     if ((rc = raise((const void*)k_ypass<T, 1>, smem_y))) return rc;
     if ((rc = raise((const void*)k_xgspace<T>, smem_x))) return rc;
     if ((rc = raise((const void*)k_xpass<T, -1>, smem_xp))) return rc;
-    if (planes && (rc = raise((const void*)plane_kern, smem_pl))) return rc;
+    if (planes && !cp && (rc = raise((const void*)plane_kern, smem_pl))) return rc;
+    if (cp) {
+      if ((rc = raise((const void*)cp->zfwd, cp->zf_bytes[3]))) return rc;
+      if ((rc = raise((const void*)cp->zinv, cp->zi_bytes[3]))) return rc;
+      for (const auto& pl : cp->pl)
+        if ((rc = raise((const void*)pl.kern, pl.bytes))) return rc;
+    }
     if (prec2 && (rc = raise((const void*)prec2_kern, smem_pl2))) return rc;
     const size_t sring = StreamCfg<T>::ring_bytes(3, 17);   // largest ring any streaming launch uses
     if ((rc = raise((const void*)k_gram<T, 1, 3>, sring))) return rc;
@@ -830,14 +886,15 @@ class Engine : public IEngine {
     TV* pt = reinterpret_cast<TV*>(partials);
     GArgs<T> ga{(cs.terms & OFDFT_TERM_LOC) ? ((planes || p256) ? vloc_pl : vloc) : nullptr, Kt, (T)(tp * tp), (T)Omega,
                 (T)(0.5 * Omega), (T)(1.0 / (double)N), (T)g2cut_loc, (cs.terms & OFDFT_TERM_HARTREE) ? 1 : 0,
-                pt};
+                pt, nullptr, cou};
     int g_rows = 0;                       // rows of G-space partials [g_rows][4]
     if (sp.nact > 0) {
       const double zb = (double)(mode == 0 ? 1 : 2) * N * sizeof(T) + (double)sp.nact * NH * sizeof(C);
-      if (z256) {
-        if (int rc = launch_zfwd256(pa, sp, zb, st)) return rc;
-      } else OFDFT_RUN("k_zfwd", st, zb, k_zfwd<T><<<grid_z, kThreads, smem_zf, st>>>(pa, sp, ph, tw_h, tw_n, n, zR, zP));
-      if (planes) {
+      if (int rc = launch_zfwd(pa, sp, zb, st)) return rc;
+      if (cp) {
+        if (int rc = launch_cplane(sp, ga, 2.0 * sp.nact * NH * sizeof(C) + ((cs.terms & OFDFT_TERM_LOC) ? (double)n_vloc * sizeof(C) : 0.0), st)) return rc;
+        g_rows = cp->pl[sp.nact > 1].cl * nh * sp.nact;
+      } else if (planes) {
         OFDFT_RUN("k_plane", st, 2.0 * sp.nact * NH * sizeof(C) + ((cs.terms & OFDFT_TERM_LOC) ? (double)n_vloc * sizeof(C) : 0.0), plane_kern<<<dim3(nh, sp.nact), kPlaneThreads, smem_pl, st>>>(sp, ga, pn, rev_d, tw_n));
         g_rows = nh * sp.nact;
       } else if (p256) {
@@ -859,16 +916,14 @@ class Engine : public IEngine {
       }
     }
     // epilogue partials after room for 3 fields of G-space rows
-    TV* pe = pt + (size_t)std::max(z256 ? kGridX256 : grid_x, nh) * 3 * 4;
+    TV* pe = pt + g_room() * 4;
     if (mode == 0) mu_ref = 0.0;
     FinArgs<T> fa{pt, g_rows, pe, grid_z, res_d};
     const double cy = 9.8696044010893586188344909998762 / (1.4142135623730950488016887242097 * std::pow(Te, 1.5));
     EpiArgs<T> ea{mode, rho, ps, dd, (T)t, (T)scale, (T)cs.alpha, (T)Te, (T)cy, (T)mu_ref, cs.terms, out, pe, fa,
                   counters + 0, nullptr, nullptr, dsc, cs.fd64 ? 1 : 0, cy, (T)std::log(cy)};
     const double eb = (double)sp.nact * NH * sizeof(C) + (double)(mode == 0 ? 1 : 2) * N * sizeof(T) + (out ? (double)N * sizeof(T) : 0.0);
-    if (z256) {
-      if (int rc = launch_zinv256(sp, ea, eb, st)) return rc;
-    } else OFDFT_RUN("k_zinv_epi", st, eb, k_zinv_epi<T><<<grid_z, kThreads, smem_zi, st>>>(sp, ea, ph, tw_h, tw_n, n, zR, zP));
+    if (int rc = launch_zinv(sp, ea, eb, st)) return rc;
     if (sync) {
       OFDFT_CK(cudaMemcpyAsync(res_h, res_d, 12 * sizeof(double), cudaMemcpyDeviceToHost, st));
       OFDFT_CK(cudaStreamSynchronize(st));
@@ -887,12 +942,12 @@ class Engine : public IEngine {
     using TV = typename TreeVal<T>::type;
     TV* pt = reinterpret_cast<TV*>(partials);
     GArgs<T> ga{nullptr, Kt, (T)(tp * tp), (T)Omega, (T)(0.5 * Omega), (T)(1.0 / (double)N), (T)g2cut_loc, 0, pt,
-                precT};
+                precT, cou};
     const double fb = 2.0 * NH * sizeof(C);
-    if (z256) {
-      if (int rc = launch_zfwd256(pa, sp, (double)N * sizeof(T) + NH * sizeof(C), st)) return rc;
-    } else OFDFT_RUN("k_zfwd", st, (double)N * sizeof(T) + NH * sizeof(C), k_zfwd<T><<<grid_z, kThreads, smem_zf, st>>>(pa, sp, ph, tw_h, tw_n, n, zR, zP));
-    if (prec2) {
+    if (int rc = launch_zfwd(pa, sp, (double)N * sizeof(T) + NH * sizeof(C), st)) return rc;
+    if (cp) {
+      if (int rc = launch_cplane(sp, ga, fb, st)) return rc;
+    } else if (prec2) {
       // one field: two blocks (a cluster) per kz plane
       OFDFT_RUN("k_plane_prec2", st, fb, prec2_kern<<<dim3(2 * nh), kPlaneThreads, smem_pl2, st>>>(sp, ga, pn, rev_d, tw_n));
     } else if (planes) {
@@ -908,14 +963,12 @@ class Engine : public IEngine {
       OFDFT_RUN("k_xgspace", st, fb, k_xgspace<T><<<dim3(grid_x, 1), kThreads, smem_x, st>>>(sp, ga, pn, tw_n, n, xJ));
       OFDFT_RUN("k_ypass", st, fb, k_ypass<T, 1><<<dim3(grid_y1, 1), kThreads, smem_y, st>>>(sp, pn, tw_n, n, yJ));
     }
-    TV* pe = pt + (size_t)std::max(z256 ? kGridX256 : grid_x, nh) * 3 * 4;
+    TV* pe = pt + g_room() * 4;
     FinArgs<T> fa{pt, 0, pe, 0, res_d};
     EpiArgs<T> ea{3, nullptr, in, in, (T)0, (T)1, (T)cs.alpha, (T)Te, (T)1, (T)0, cs.terms, out, pe, fa,
                   counters + 0, pold, pyout};
     const double pb = (double)NH * sizeof(C) + (double)N * sizeof(T) * (pyout ? 3.0 : 1.0);
-    if (z256) {
-      if (int rc = launch_zinv256(sp, ea, pb, st)) return rc;
-    } else OFDFT_RUN("k_zinv_epi", st, pb, k_zinv_epi<T><<<grid_z, kThreads, smem_zi, st>>>(sp, ea, ph, tw_h, tw_n, n, zR, zP));
+    if (int rc = launch_zinv(sp, ea, pb, st)) return rc;
     return OFDFT_OK;
   }
 

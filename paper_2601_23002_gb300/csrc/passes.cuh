@@ -420,6 +420,7 @@ template <typename T> struct GArgs {
   // non-null: the psi field is the minimiser's preconditioning pass, and its
   // spectrum is multiplied by this table of p(m^2) instead (see minimize)
   const T* prec;
+  const T* cou;          // 4 pi / G^2 by m^2 (the compile-time plane pass)
 };
 
 // One block per (tile, field): blockIdx.y indexes the active fields.
