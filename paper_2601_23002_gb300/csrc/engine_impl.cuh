@@ -153,21 +153,27 @@ class Engine : public IEngine {
   unsigned int* counters = nullptr;   // last-block arrival counters (0 between launches)
   double* pos_d = nullptr;
   double* Z_d = nullptr;
-  double2* phases = nullptr;
+  C* phases = nullptr;       // exp(-2 pi i m R / L) per ion and axis (k_phases)
+  // row pairs (a, b) of the structure factor without the full S(G), and whether
+  // the entries outside their rows are zero
+  int2* sf_rows = nullptr;
+  int sf_nrows = 0, sf_m2 = 0;
+  bool sf_zeroed = false;
   double E_ion = 0;
   bool ions_set = false;
   double g2cut_loc = 0;
   // Ewald splitting of the last set_ions, reused by forces
   double ew_eta = 0, ew_rcut = 0;
   int ew_nimg = 0;
-  // forces: G list {kx, ky, kz, w} with 0 < |G|^2 <= g2cut_loc, its (vfac, efac),
-  // per-G weights qq, ion phases in T, device output; built on the first call
-  int4* f_gl = nullptr;
+  // forces: row pairs inside the cutoffs sorted by |m|^2, their tiles' kz
+  // offsets, (vfac, efac) by m^2, qq, partial sums, device output; built on the
+  // first call
+  int2* f_rows = nullptr;
+  int* f_tk = nullptr;
   double2* f_gf = nullptr;
-  C* f_qq = nullptr;
-  C* f_pt = nullptr;
-  double* f_out = nullptr;
-  int f_ng = -1;
+  Quad<T>* f_qq = nullptr;
+  double *f_part = nullptr, *f_out = nullptr;
+  int f_nrows = -1, f_ntile = 0, f_nk = 0, f_m2 = 0;
   // pressure: pnl(m^2) = (3 - 6a) K + dK/dlambda (FP64, built on the first call)
   double* p_tab = nullptr;
   bool p_ready = false;
@@ -629,6 +635,15 @@ class Engine : public IEngine {
       }
       if ((rc = alloc(&sf_tab, nm2))) return rc;
       OFDFT_CK(cudaMemcpyAsync(sf_tab, tab.data(), nm2 * sizeof(double2), cudaMemcpyHostToDevice, st));
+      // row pairs with a^2 + b^2 inside the local and Ewald range, and out to
+      // |m|^2 = 600 for the S_ei shells
+      sf_m2 = 0;
+      const double lim = std::max(ewald_g2max(), tp2d * 600.0);
+      while (sf_m2 < 2 * h * h && tp2d * (double)(sf_m2 + 1) <= lim) ++sf_m2;
+      const std::vector<int2> rows = row_pairs(sf_m2);
+      sf_nrows = (int)rows.size();
+      if ((rc = alloc(&sf_rows, rows.size()))) return rc;
+      OFDFT_CK(cudaMemcpyAsync(sf_rows, rows.data(), rows.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
       OFDFT_CK(cudaStreamSynchronize(st));
     }
     {
@@ -652,6 +667,15 @@ class Engine : public IEngine {
   }
 
   long long grid_points() const override { return (long long)N; }
+
+  // (a, b), 0 <= a, b <= n/2, with a^2 + b^2 <= m2, in the order of a^2 + b^2
+  std::vector<int2> row_pairs(int m2) const {
+    std::vector<int2> r;
+    for (int a = 0; a <= h; ++a)
+      for (int b = 0; b <= h && a * a + b * b <= m2; ++b) r.push_back(make_int2(a, b));
+    std::stable_sort(r.begin(), r.end(), [](const int2& p, const int2& q) { return p.x * p.x + p.y * p.y < q.x * q.x + q.y * q.y; });
+    return r;
+  }
 
   // |G|^2 range of the structure factor's rows and the Ewald reciprocal sum
   double ewald_g2max() const {
@@ -812,60 +836,77 @@ class Engine : public IEngine {
     return OFDFT_OK;
   }
 
+  // k_struct with the largest thread tile that still gives most SMs a block:
+  // FP32 2 x 4 (64 accumulators) or 2 x 2, FP64 2 x 2, small grids 1 x 1.
+  int launch_struct(const StructOut<T>& so, const double* zw, int full, int* nblk, cudaStream_t st) {
+    const int2* rows = full ? nullptr : sf_rows;
+    const int nrows = full ? nh * nh : sf_nrows;
+    bool done = false;
+    auto go = [&](auto TRc, auto TCc, auto NTc, bool last) -> int {
+      constexpr int TR = decltype(TRc)::value, TC = decltype(TCc)::value, NT = decltype(NTc)::value;
+      const int ctiles = (nh + TC * 64 - 1) / (TC * 64);        // at most 64 threads along kz
+      const int CT = (nh + TC * ctiles - 1) / (TC * ctiles);
+      const int RT = NT / CT * TR;
+      const int g = (nrows + RT - 1) / RT;
+      if (!last && g * ctiles < 120) return OFDFT_OK;
+      const size_t sm = struct_smem<T, TR, TC, NT>(CT);
+      OFDFT_RUN("k_struct", st, (double)nrows * 4 * nh * sizeof(C) * 3.0, k_struct<T, TR, TC, NT><<<dim3(g, ctiles), NT, sm, st>>>(phases, zw, (int)cs.Z.size(), n, rows, nrows, CT, so));
+      *nblk = g * ctiles;
+      done = true;
+      return OFDFT_OK;
+    };
+    using std::integral_constant;
+    int rc = OFDFT_OK;
+    if constexpr (sizeof(T) == 4) rc = go(integral_constant<int, 2>{}, integral_constant<int, 4>{}, integral_constant<int, 256>{}, false);
+    if (!rc && !done) rc = go(integral_constant<int, 2>{}, integral_constant<int, 2>{}, integral_constant<int, 256>{}, false);
+    if (!rc && !done) rc = go(integral_constant<int, 1>{}, integral_constant<int, 1>{}, integral_constant<int, 64>{}, true);
+    return rc;
+  }
+
   int set_ions(const double* pos, int on_device, void* S_out, void* stream_) override {
     cudaStream_t st = (cudaStream_t)stream_;
     const int nion = (int)cs.Z.size();
     OFDFT_CK(cudaMemcpyAsync(pos_d, pos, (size_t)nion * 3 * sizeof(double),
                              on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st));
-    const int tot = nion * 3 * n;
-    OFDFT_RUN("k_phases", st, (double)tot * 16, k_phases<<<std::min(4096, (tot + 255) / 256), 256, 0, st>>>(pos_d, nion, n, L, phases));
-    const double g2max = ewald_g2max();
+    const int tot = nion * 3 * nh;
+    OFDFT_RUN("k_phases", st, (double)nion * 3 * n * sizeof(C), k_phases<T><<<std::min(4096, (tot + 127) / 128), 128, 0, st>>>(pos_d, nion, n, L, phases));
     const double eta = ewald_eta();
     const int full = S_out != nullptr;
-    // rows are also kept out to |m|^2 = 600 for the S_ei shells
-    const double g2rows = std::max(g2max, (2.0 * kPi / L) * (2.0 * kPi / L) * 600.0);
-    // without the full S(G), only rows with |mx|, |my| <= mlim can reach g2rows:
-    // zero everything, then compute that square of rows
-    int mlim = (int)std::floor(std::sqrt(g2rows) / (2.0 * kPi / L));
-    if (full || mlim > (n - 1) / 2) mlim = -1;
-    const int nrows = mlim < 0 ? n * n : (2 * mlim + 1) * (2 * mlim + 1);
-    if (mlim >= 0) {
+    // without the full S(G) only the rows inside sf_m2 are formed, the others
+    // stay zero
+    if (full) sf_zeroed = false;
+    else if (!sf_zeroed) {
       OFDFT_CK(cudaMemsetAsync(Sg, 0, NH * sizeof(C), st));
       OFDFT_CK(cudaMemsetAsync(vloc, 0, NH * sizeof(C), st));
       OFDFT_CK(cudaMemsetAsync(SZg, 0, NH * sizeof(C), st));
+      sf_zeroed = true;
     }
-    // ions per shared-memory chunk: staged kz phases within 36 KB, so that
-    // with the row phases (8 x 64 complex), the charges and the kernel's own
-    // static scratch the block stays inside the default 48 KB (FP64, n = 80)
-    const int sch = std::max(1, std::min(64, (int)(36864 / ((size_t)nh * sizeof(C)))));
-    const size_t ssm = (size_t)sch * nh * sizeof(C) + (size_t)kStructRows * sch * sizeof(C) + (size_t)sch * sizeof(T);
-    const int sgrid = (nrows + kStructRows - 1) / kStructRows;
-    // one ion species (every workload here): S_Z = Z S, so the kernel sums S only
+    // one ion species (every workload here): S_Z = Z S, one sum over the ions
     bool uni = true;
     for (double z : cs.Z) uni = uni && z == cs.Z[0];
-    if (uni) OFDFT_RUN("k_struct", st, (double)NH * sizeof(C) * (full ? 2 : 1), k_struct<T, true><<<sgrid, 32 * kStructRows, ssm, st>>>(phases, Z_d, nion, n, L, sf_tab, g2rows, full, mlim, sch, Sg, vloc, SZg, partials));
-    else OFDFT_RUN("k_struct", st, (double)NH * sizeof(C) * (full ? 2 : 1), k_struct<T, false><<<sgrid, 32 * kStructRows, ssm, st>>>(phases, Z_d, nion, n, L, sf_tab, g2rows, full, mlim, sch, Sg, vloc, SZg, partials));
-    int rc;
-    if ((rc = sum_partials(sgrid, 1, 0, st))) return rc;
+    int nblk = 0;
+    StructOut<T> so{Sg, (C*)S_out, uni ? SZg : nullptr, vloc, cs.Z[0], sf_tab, (double)sf_m2, partials};
+    if (int rc = launch_struct(so, nullptr, full, &nblk, st)) return rc;
+    if (!uni) {
+      so.S = so.S2 = nullptr; so.SZ = SZg; so.zs = 1.0;
+      if (int rc = launch_struct(so, Z_d, full, &nblk, st)) return rc;
+    }
     const double rcut = 6.3 / eta;
-    // images per axis around minimum-image displacements
-    const int nimg_mi = (int)std::ceil(rcut / L + 0.5);
+    // images per axis around minimum-image displacements (see k_ewald_real)
+    const int nimg_mi = std::max(0, (int)std::ceil(rcut / L + 0.5) - 1);
     ew_eta = eta; ew_rcut = rcut; ew_nimg = nimg_mi;
-    const long ncomb = (long)nion * nion * (2 * nimg_mi + 1) * (2 * nimg_mi + 1) * (2 * nimg_mi + 1);
-    const int gb = (int)std::min<long>(std::min<long>(2048, 4L * nsm), (ncomb + 255) / 256);
-    OFDFT_RUN("k_ewald_real", st, (double)nion * 32, k_ewald_real<<<gb, 256, 0, st>>>(pos_d, Z_d, nion, L, eta, rcut, nimg_mi, partials));
-    if ((rc = sum_partials(gb, 1, 1, st))) return rc;
+    const long ncomb = (long)nion * (nion / 2 + 1) * (2 * nimg_mi + 1) * (2 * nimg_mi + 1) * (2 * nimg_mi + 1);
+    const int gb = (int)std::min<long>(4L * nsm, (ncomb + 255) / 256);
+    OFDFT_RUN("k_ewald_real", st, (double)nion * 32, k_ewald_real<<<gb, 256, 0, st>>>(pos_d, Z_d, nion, L, eta, rcut, nimg_mi, partials, nblk, partials + nblk, counters + 4, res_d));
+    if (planes)
+      OFDFT_RUN("k_vloc_planes", st, 2.0 * NH * sizeof(C), k_vloc_planes<T><<<4 * nsm, 256, 0, st>>>(vloc, vloc_pl, rev_d, n));
+    if (p256_possible())
+      OFDFT_RUN("k_vloc_planes256", st, 2.0 * NH * sizeof(C), k_vloc_planes256<T><<<4 * nsm, 256, 0, st>>>(vloc, vloc_pl));
     OFDFT_CK(cudaMemcpyAsync(res_h, res_d, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
     OFDFT_CK(cudaStreamSynchronize(st));
     double zz = 0;
     for (double z : cs.Z) zz += z * z;
     E_ion = res_h[0] + res_h[1] - eta / std::sqrt(kPi) * zz - kPi * Ne * Ne / (2.0 * Omega * eta * eta);
-    if (planes)
-      OFDFT_RUN("k_vloc_planes", st, 2.0 * NH * sizeof(C), k_vloc_planes<T><<<4 * nsm, 256, 0, st>>>(vloc, vloc_pl, rev_d, n));
-    if (p256_possible())
-      OFDFT_RUN("k_vloc_planes256", st, 2.0 * NH * sizeof(C), k_vloc_planes256<T><<<4 * nsm, 256, 0, st>>>(vloc, vloc_pl));
-    if (S_out) OFDFT_CK(cudaMemcpyAsync(S_out, Sg, NH * sizeof(C), cudaMemcpyDeviceToDevice, st));
-    OFDFT_CK(cudaStreamSynchronize(st));
     ions_set = true;
     return OFDFT_OK;
   }
@@ -1493,35 +1534,38 @@ int Engine<T>::forces(const void* rho, double* f_out_h, void* stream_) {
   const int nion = (int)cs.Z.size();
   const double tp = 2.0 * kPi / L;
   int rc;
-  if (f_ng < 0) {
-    // the G list of the local and reciprocal Ewald sums (independent of the ions)
-    std::vector<int4> gl;
-    std::vector<double2> gf;
-    const int r = (int)std::ceil(std::sqrt(g2cut_loc) / tp);
+  if (f_nrows < 0) {
+    // the G set of the local and reciprocal Ewald sums (independent of the ions)
+    f_m2 = 0;
+    while (f_m2 < 3 * h * h && tp * tp * (double)(f_m2 + 1) <= g2cut_loc) ++f_m2;
     const bool loc = (cs.terms & OFDFT_TERM_LOC) != 0;
-    for (int mx = std::max(-h, -r); mx <= std::min((n - 1) / 2, r); ++mx)
-      for (int my = std::max(-h, -r); my <= std::min((n - 1) / 2, r); ++my)
-        for (int kz = 0; kz <= std::min(h, r); ++kz) {
-          const int m2 = mx * mx + my * my + kz * kz;
-          const double G2 = tp * tp * (double)m2;
-          if (m2 == 0 || G2 > g2cut_loc) continue;
-          const int kx = mx < 0 ? mx + n : mx, ky = my < 0 ? my + n : my;
-          const int w = (kz == 0 || 2 * kz == n) ? 1 : 2;
-          gl.push_back(make_int4(kx, ky, kz, w));
-          const double vfac = loc ? -4.0 * kPi * std::exp(-G2 * cs.rc * cs.rc / 4.0) / G2 : 0.0;
-          const double efac = 4.0 * kPi / Omega * std::exp(-G2 / (4.0 * ew_eta * ew_eta)) / G2;
-          gf.push_back(make_double2(vfac, efac));
-        }
-    const size_t ng = std::max<size_t>(1, gl.size());
-    if ((rc = alloc(&f_gl, ng)) || (rc = alloc(&f_gf, ng)) || (rc = alloc(&f_qq, ng)) ||
-        (rc = alloc(&f_pt, (size_t)nion * 3 * n)) || (rc = alloc(&f_out, (size_t)nion * 3)))
-      return rc;
-    if (!gl.empty()) {
-      OFDFT_CK(cudaMemcpyAsync(f_gl, gl.data(), gl.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
-      OFDFT_CK(cudaMemcpyAsync(f_gf, gf.data(), gf.size() * sizeof(double2), cudaMemcpyHostToDevice, st));
+    const std::vector<int2> rows = row_pairs(f_m2);
+    std::vector<int> tk{0};
+    for (size_t t = 0; t < rows.size(); t += 32) {
+      const int left = f_m2 - rows[t].x * rows[t].x - rows[t].y * rows[t].y;
+      int kz = (int)std::sqrt((double)left);
+      while ((kz + 1) * (kz + 1) <= left) ++kz;
+      while (kz * kz > left) --kz;
+      tk.push_back(tk.back() + std::min(kz, h) + 1);
     }
+    std::vector<double2> gf(f_m2 + 1);
+    gf[0] = make_double2(0.0, 0.0);
+    for (int m2 = 1; m2 <= f_m2; ++m2) {
+      const double G2 = tp * tp * (double)m2;
+      gf[m2] = make_double2(loc ? -4.0 * kPi * std::exp(-G2 * cs.rc * cs.rc / 4.0) / G2 : 0.0,
+                            4.0 * kPi / Omega * std::exp(-G2 / (4.0 * ew_eta * ew_eta)) / G2);
+    }
+    f_ntile = (int)tk.size() - 1;
+    f_nk = tk.back();
+    if ((rc = alloc(&f_rows, rows.size())) || (rc = alloc(&f_tk, tk.size())) || (rc = alloc(&f_gf, gf.size())) ||
+        (rc = alloc(&f_qq, (size_t)f_nk * 64)) || (rc = alloc(&f_part, (size_t)f_ntile * nion * 3)) ||
+        (rc = alloc(&f_out, (size_t)nion * 3)))
+      return rc;
+    OFDFT_CK(cudaMemcpyAsync(f_rows, rows.data(), rows.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
+    OFDFT_CK(cudaMemcpyAsync(f_tk, tk.data(), tk.size() * sizeof(int), cudaMemcpyHostToDevice, st));
+    OFDFT_CK(cudaMemcpyAsync(f_gf, gf.data(), gf.size() * sizeof(double2), cudaMemcpyHostToDevice, st));
     OFDFT_CK(cudaStreamSynchronize(st));
-    f_ng = (int)gl.size();
+    f_nrows = (int)rows.size();
   }
   // n~ (unnormalised) into spec[0], tiled layout
   Spectra<T> sp{};
@@ -1530,21 +1574,15 @@ int Engine<T>::forces(const void* rho, double* f_out_h, void* stream_) {
   OFDFT_RUN("k_zfwd", st, (double)N * sizeof(T) + (double)NH * sizeof(C), k_zfwd<T><<<grid_z, kThreads, smem_zf, st>>>(pa, sp, ph, tw_h, tw_n, n, zR, zP));
   OFDFT_RUN("k_ypass", st, 2.0 * NH * sizeof(C), k_ypass<T, -1><<<dim3(grid_y1, 1), kThreads, smem_y, st>>>(sp, pn, tw_n, n, yJ));
   OFDFT_RUN("k_xpass", st, 2.0 * NH * sizeof(C), k_xpass<T, -1><<<dim3(grid_x, 1), kThreads, smem_xp, st>>>(sp, pn, tw_n, n, xJ));
-  const int tot = nion * 3 * n;
-  OFDFT_RUN("k_phases_t", st, (double)tot * (16 + sizeof(C)), k_phases_t<T><<<std::min(4096, (tot + 255) / 256), 256, 0, st>>>(phases, f_pt, tot));
-  if (f_ng > 0) {
-    const int gq = std::min(4 * nsm, (f_ng + 127) / 128);
-    OFDFT_RUN("k_forces_q", st, (double)f_ng * (3 * sizeof(C) + 32), k_forces_q<T><<<gq, 128, 0, st>>>(spec[0], f_gl, f_gf, f_ng, SZg, n, 1.0 / (double)N, f_qq));
-    OFDFT_RUN("k_forces_g", st, (double)nion * f_ng * (sizeof(C) + 16), k_forces_g<T><<<nion, 256, 0, st>>>(f_qq, f_gl, f_ng, f_pt, Z_d, n, tp, f_out));
-  } else {
-    OFDFT_CK(cudaMemsetAsync(f_out, 0, (size_t)nion * 3 * sizeof(double), st));
-  }
+  OFDFT_RUN("k_forces_q", st, (double)f_nk * 32 * (8 * sizeof(C) + 4 * sizeof(C)), k_forces_q<T><<<std::min(16 * nsm, (f_nk + 3) / 4), 128, 0, st>>>(spec[0], SZg, f_rows, f_nrows, f_tk, f_ntile, f_gf, f_m2, n, 1.0 / (double)N, f_qq));
+  constexpr int TI = sizeof(T) == 4 ? 4 : 2;
+  OFDFT_RUN("k_forces_g", st, (double)f_nk * 128 * sizeof(C), k_forces_g<T, TI><<<dim3(f_ntile, (nion + kForceWarps * TI - 1) / (kForceWarps * TI)), 32 * kForceWarps, 0, st>>>(f_qq, f_rows, f_nrows, f_tk, phases, nion, n, f_part));
   // several blocks per ion (about 4 per SM in all), shares added in a fixed order
   int nsplit = std::max(1, std::min(64, (4 * nsm + nion - 1) / nion));
   while (nsplit > 1 && (size_t)nion * nsplit * 3 > partials_cap) --nsplit;
   if ((size_t)nion * nsplit * 3 > partials_cap) { set_error("forces: too many ions for the scratch"); return OFDFT_ERR_INVALID; }
   OFDFT_RUN("k_ewald_force_real", st, (double)nion * nion * 32, k_ewald_force_real<<<nion * nsplit, 256, 0, st>>>(pos_d, Z_d, nion, L, ew_eta, ew_rcut, ew_nimg, nsplit, partials));
-  OFDFT_RUN("k_sum_force_parts", st, (double)nion * nsplit * 24, k_sum_force_parts<<<(3 * nion + 127) / 128, 128, 0, st>>>(partials, nion, nsplit, f_out));
+  OFDFT_RUN("k_sum_force_parts", st, (double)nion * nsplit * 24, k_sum_force_parts<<<(3 * nion + 3) / 4, 128, 0, st>>>(f_part, f_ntile, Z_d, tp, partials, nion, nsplit, f_out));
   OFDFT_CK(cudaMemcpyAsync(f_out_h, f_out, (size_t)nion * 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
   OFDFT_CK(cudaStreamSynchronize(st));
   return OFDFT_OK;

@@ -9,13 +9,14 @@ namespace ofdft {
 // ---------------------------------------------------------------------------
 // Structure factor on the half spectrum.  Phases factorise per axis:
 // exp(-i G.R) = e_x(m_x) e_y(m_y) e_z(m_z) with e_d(m) = exp(-2 pi i m R_d / L);
-// ph[(I*3 + d)*n + k] holds them (FP64, k in FFT order).
-static __global__ void k_phases(const double* __restrict__ pos, int n_ion, int n, double L,
-                         double2* __restrict__ ph) {
-  const int tot = n_ion * 3 * n;
+// ph[(I*3 + d)*n + k] holds them (k in FFT order), formed in FP64 and rounded to
+// the plan's type; one sine and cosine per |m|, the negative m by conjugation.
+template <typename T>
+__global__ void k_phases(const double* __restrict__ pos, int n_ion, int n, double L, cplx<T>* __restrict__ ph) {
+  const int h = n / 2 + 1;
+  const int tot = n_ion * 3 * h;
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < tot; q += gridDim.x * blockDim.x) {
-    const int k = q % n, d = (q / n) % 3, I = q / (3 * n);
-    const int m = k <= (n - 1) / 2 ? k : k - n;
+    const int m = q % h, d = (q / h) % 3, I = q / (3 * h);
     double f = pos[I * 3 + d] / L;
     f -= floor(f);                       // wrap into [0, 1)
     // angle = -2 pi m f; reduce m f modulo 1 before the trig call
@@ -23,160 +24,185 @@ static __global__ void k_phases(const double* __restrict__ pos, int n_ion, int n
     mf -= rint(mf);
     double s, c;
     sincospi(-2.0 * mf, &s, &c);
-    ph[q] = make_double2(c, s);
+    cplx<T>* o = ph + (size_t)(I * 3 + d) * n;
+    if (2 * m < n) o[m] = mk<T>((T)c, (T)s);
+    if (m > 0) o[n - m] = mk<T>((T)c, (T)-s);        // m = n/2 of even n is stored as -n/2
   }
 }
 
-// S(G) = sum_I exp(-i G.R_I) and S_Z(G) = sum_I Z_I exp(-i G.R_I) on the half
-// spectrum; V_loc(G) = (1/Omega) v~(G) S_Z(G) with the common smoothing radius
-// rc; the Ewald reciprocal sum (2 pi / Omega) sum_{G != 0} exp(-G^2/4eta^2)/G^2
-// |S_Z|^2 accumulated on the way.  A block takes kStructRows (kx, ky) rows, one
-// per warp, lanes over kz; the ions go in chunks of ch, whose kz phases are
-// staged in shared memory once for all rows of the block (with the rows' (kx,
-// ky) phase products).  Rows whose smallest |G|^2 exceeds g2max are written as
-// zero (their V_loc and Ewald weights are below double precision) unless
-// full != 0.
-//   sf_tab[m^2] = (v~(G)/Omega per unit charge, (2 pi/Omega) exp(-G^2/(4 eta^2))/G^2),
-// the second 0 at m^2 = 0: both depend on |G| only and are tabulated once per
-// plan in FP64, so no exponential is evaluated here.
-// S_Z itself is kept as well (SZ_out), for the forces.
-// Shared memory: ez[ch][nh] | xy[kStructRows][ch] (complex) | zz[ch] (T).
-constexpr int kStructRows = 8;
-constexpr int kStructMaxKJ = 9;     // kz per lane: nh <= 32 * 9
-
-// UNI: every ion has the charge Z[0]; S_Z is then Z[0] S and is not summed.
-template <typename T, bool UNI>
-__global__ void __launch_bounds__(32 * kStructRows) k_struct(const double2* __restrict__ ph,
-                                                             const double* __restrict__ Z, int n_ion, int n,
-                                                             double L, const double2* __restrict__ sf_tab,
-                                                             double g2max, int full, int mlim, int ch,
-                                                             cplx<T>* __restrict__ S_out,
-                                                             cplx<T>* __restrict__ vloc,
-                                                             cplx<T>* __restrict__ SZ_out,
-                                                             double* __restrict__ ew_partial) {
+// S(G) = sum_I w_I exp(-i G.R_I) as a real matrix product over the ions.  With
+// P = e_x(a) e_y(b) and M = e_x(a) e_y(b)*, a, b >= 0, and e_z = C + i D the four
+// rows (+-a, +-b) are
+//   P e_z, P* e_z:  (sum Pr C -+ sum Pi D) + i (sum Pr D +- sum Pi C)
+// and the same with M: eight real sums give four complex entries, two
+// multiply-adds per entry and ion.  (One product per entry and lane, with the
+// phase products re-read from shared memory for each, took 492 us for 300 ions
+// on the full 128^3 half spectrum; the FP32 pipe needs 17 us for these sums.)
+// A thread owns TR row pairs (a, b) and TC kz; the ions go in chunks of CH whose
+// row products and kz phases are staged in shared memory, so a chunk's step
+// reads TR + TC/2 16-byte groups for 8 TR TC multiply-adds.
+// rows: (a, b) list, or nullptr for all 0 <= a, b <= n/2.
+// zw: weights (nullptr: 1).  Outputs (any may be null): S, S2 (a second copy),
+// SZ = zs S, V_loc = f.x SZ, and per block the Ewald reciprocal sum
+// sum w f.y |SZ|^2 over the entries of rows with |G|^2 <= g2rows:
+//   sf_tab[m^2] = f = (v~(G)/Omega per unit charge, (2 pi/Omega) exp(-G^2/(4 eta^2))/G^2),
+// tabulated once per plan in FP64.
+// grid: (row tiles, kz tiles); CT threads along kz.
+template <typename T> struct StructOut {
+  cplx<T>*S, *S2, *SZ, *vloc;
+  double zs;
+  const double2* sf_tab;
+  double m2rows;              // vloc and the Ewald sum: rows with a^2 + b^2 <= m2rows
+  double* ew;
+};
+template <typename T> struct alignas(16) Quad { T a, b, c, d; };
+constexpr int kStructCH = 16;
+template <typename T, int TR, int TC, int NT>
+constexpr size_t struct_smem(int CT) {
+  return (size_t)kStructCH * ((size_t)CT * TC * sizeof(cplx<T>) + (size_t)(NT / CT) * TR * sizeof(Quad<T>));
+}
+template <typename T, int TR, int TC, int NT>
+__global__ void __launch_bounds__(NT) k_struct(const cplx<T>* __restrict__ ph, const double* __restrict__ zw, int n_ion,
+                                               int n, const int2* __restrict__ rows, int nrows, int CT, StructOut<T> o) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[32];
-  const int nh = n / 2 + 1;
-  cplx<T>* ez = reinterpret_cast<cplx<T>*>(smem_raw);
-  cplx<T>* sxy = ez + (size_t)ch * nh;
-  T* szz = reinterpret_cast<T*>(sxy + (size_t)kStructRows * ch);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // mlim < 0: every (kx, ky) row of the grid; mlim >= 0: the rows with |mx|,
-  // |my| <= mlim (the caller has zeroed the other rows)
-  const int side = 2 * mlim + 1;
-  const int nrows = mlim < 0 ? n * n : side * side;
-  auto row_of = [&](int rw, int& kx, int& ky, int& mx, int& my) {
-    if (mlim < 0) {
-      kx = rw / n; ky = rw % n;
-      mx = kx <= (n - 1) / 2 ? kx : kx - n;
-      my = ky <= (n - 1) / 2 ? ky : ky - n;
-    } else {
-      mx = rw / side - mlim; my = rw % side - mlim;
-      kx = mx < 0 ? mx + n : mx; ky = my < 0 ? my + n : my;
-    }
+  const int h = n / 2, nh = h + 1;
+  const int RB = NT / CT, RT = RB * TR, CC = CT * TC;    // row threads, rows and columns of the block
+  Quad<T>* sr = reinterpret_cast<Quad<T>*>(smem_raw);    // [CH][RT]
+  cplx<T>* se = reinterpret_cast<cplx<T>*>(sr + (size_t)kStructCH * RT);   // [CH][CC]
+  const int tid = threadIdx.x, ct = tid % CT, rt = tid / CT;
+  const bool act = rt < RB;
+  const int col0 = blockIdx.y * CC;
+  auto row_of = [&](int r, int& a, int& b) {
+    if (rows) { const int2 v = rows[r]; a = v.x; b = v.y; }
+    else { a = r / nh; b = r - a * nh; }
   };
-  const int row = blockIdx.x * kStructRows + warp;
-  int kx = 0, ky = 0, mx = 0, my = 0;
-  const bool valid = row < nrows;
-  if (valid) row_of(row, kx, ky, mx, my);
-  const double tp = 2.0 * kPi / L;
-  const bool skip = !full && tp * tp * (double)(mx * mx + my * my) > g2max;
-  T sr[kStructMaxKJ], si[kStructMaxKJ], zr[kStructMaxKJ], zi[kStructMaxKJ];
+  T acc[TR][TC][8];
 #pragma unroll
-  for (int j = 0; j < kStructMaxKJ; ++j) { sr[j] = 0; si[j] = 0; zr[j] = 0; zi[j] = 0; }
-  for (int I0 = 0; I0 < n_ion; I0 += ch) {
-    const int cnt = min(ch, n_ion - I0);
+  for (int i = 0; i < TR; ++i)
+#pragma unroll
+    for (int j = 0; j < TC; ++j)
+#pragma unroll
+      for (int k = 0; k < 8; ++k) acc[i][j][k] = 0;
+  for (int I0 = 0; I0 < n_ion; I0 += kStructCH) {
+    const int cnt = min(kStructCH, n_ion - I0);
     __syncthreads();
-    for (int q = threadIdx.x; q < cnt * nh; q += blockDim.x) {
-      const int c = q / nh, kz = q - c * nh;
-      const double2 e = ph[((size_t)(I0 + c) * 3 + 2) * n + kz];
-      ez[q] = mk<T>((T)e.x, (T)e.y);
-    }
-    for (int q = threadIdx.x; q < kStructRows * cnt; q += blockDim.x) {
-      const int r = q / cnt, c = q - r * cnt;
-      const int rw = blockIdx.x * kStructRows + r;
-      cplx<T> v = mk<T>((T)0, (T)0);
-      if (rw < nrows) {
-        int qx, qy, px, py;
-        row_of(rw, qx, qy, px, py);
-        const double2 ex = ph[((size_t)(I0 + c) * 3 + 0) * n + qx];
-        const double2 ey = ph[((size_t)(I0 + c) * 3 + 1) * n + qy];
-        v = mk<T>((T)(ex.x * ey.x - ex.y * ey.y), (T)(ex.x * ey.y + ex.y * ey.x));
+    for (int q = tid; q < cnt * CC; q += NT) {
+      const int c = q / CC, kz = col0 + q - c * CC;
+      cplx<T> e = mk<T>((T)0, (T)0);
+      if (kz < nh) {
+        e = ph[((size_t)(I0 + c) * 3 + 2) * n + kz];
       }
-      sxy[r * ch + c] = v;
+      se[q] = e;
     }
-    for (int c = threadIdx.x; c < cnt; c += blockDim.x) szz[c] = (T)Z[I0 + c];
+    for (int q = tid; q < cnt * RT; q += NT) {
+      const int c = q / RT, r = blockIdx.x * RT + q - c * RT;
+      Quad<T> v{0, 0, 0, 0};
+      if (r < nrows) {
+        int a, b;
+        row_of(r, a, b);
+        const cplx<T>* p = ph + (size_t)(I0 + c) * 3 * n;
+        cplx<T> ex = p[a], ey = p[n + b];
+        if (2 * a == n) ex.y = -ex.y;                    // index n/2 holds -n/2
+        if (2 * b == n) ey.y = -ey.y;
+        if (zw) { const T z = (T)zw[I0 + c]; ex.x *= z; ex.y *= z; }
+        v.a = ex.x * ey.x - ex.y * ey.y; v.b = ex.x * ey.y + ex.y * ey.x;
+        v.c = ex.x * ey.x + ex.y * ey.y; v.d = ex.y * ey.x - ex.x * ey.y;
+      }
+      sr[q] = v;
+    }
     __syncthreads();
-    if (valid && !skip) {
+    if (act) {
+#pragma unroll 2
       for (int c = 0; c < cnt; ++c) {
-        const cplx<T> xy = sxy[warp * ch + c];
-        const T zc = szz[c];
-        const cplx<T>* e = ez + (size_t)c * nh;
+        Quad<T> p[TR];
+        cplx<T> e[TC];
 #pragma unroll
-        for (int j = 0; j < kStructMaxKJ; ++j) {
-          const int kz = lane + 32 * j;
-          if (kz < nh) {
-            const cplx<T> w = e[kz];
-            const T pr = xy.x * w.x - xy.y * w.y, pi = xy.x * w.y + xy.y * w.x;
-            sr[j] += pr; si[j] += pi;
-            if constexpr (!UNI) { zr[j] += zc * pr; zi[j] += zc * pi; }
+        for (int i = 0; i < TR; ++i) p[i] = sr[c * RT + rt + RB * i];
+#pragma unroll
+        for (int j = 0; j < TC; ++j) e[j] = se[c * CC + ct + CT * j];
+#pragma unroll
+        for (int i = 0; i < TR; ++i)
+#pragma unroll
+          for (int j = 0; j < TC; ++j) {
+            T(&x)[8] = acc[i][j];
+            x[0] = fma(p[i].a, e[j].x, x[0]); x[1] = fma(p[i].b, e[j].y, x[1]);
+            x[2] = fma(p[i].a, e[j].y, x[2]); x[3] = fma(p[i].b, e[j].x, x[3]);
+            x[4] = fma(p[i].c, e[j].x, x[4]); x[5] = fma(p[i].d, e[j].y, x[5]);
+            x[6] = fma(p[i].c, e[j].y, x[6]); x[7] = fma(p[i].d, e[j].x, x[7]);
           }
-        }
       }
     }
-  }
-  if constexpr (UNI) {
-    const T z0 = (T)Z[0];
-#pragma unroll
-    for (int j = 0; j < kStructMaxKJ; ++j) { zr[j] = z0 * sr[j]; zi[j] = z0 * si[j]; }
   }
   double ew = 0;
-  if (valid) {
-    const size_t rowoff = ((size_t)kx * n + ky) * nh;
 #pragma unroll
-    for (int j = 0; j < kStructMaxKJ; ++j) {
-      const int kz = lane + 32 * j;
+  for (int i = 0; i < TR; ++i) {
+    const int r = blockIdx.x * RT + rt + RB * i;
+    if (!act || r >= nrows) continue;
+    int a, b;
+    row_of(r, a, b);
+    const bool pa = 2 * a < n, ma = a > 0, pb = 2 * b < n, mb = b > 0;
+    const bool inside = (double)(a * a + b * b) <= o.m2rows;
+#pragma unroll
+    for (int j = 0; j < TC; ++j) {
+      const int kz = col0 + ct + CT * j;
       if (kz >= nh) continue;
-      if (skip) {
-        if (S_out) S_out[rowoff + kz] = mk<T>(0, 0);
-        vloc[rowoff + kz] = mk<T>(0, 0);
-        SZ_out[rowoff + kz] = mk<T>(0, 0);
-        continue;
-      }
-      const int m2 = mx * mx + my * my + kz * kz;
-      if (S_out) S_out[rowoff + kz] = mk<T>(sr[j], si[j]);
-      SZ_out[rowoff + kz] = mk<T>(zr[j], zi[j]);
-      const double2 f = sf_tab[m2];
-      vloc[rowoff + kz] = mk<T>((T)(f.x * (double)zr[j]), (T)(f.x * (double)zi[j]));
+      const T(&x)[8] = acc[i][j];
+      const double2 f = inside ? o.sf_tab[a * a + b * b + kz * kz] : make_double2(0.0, 0.0);
       const double w = (kz == 0 || 2 * kz == n) ? 1.0 : 2.0;
-      ew += w * f.y * ((double)zr[j] * (double)zr[j] + (double)zi[j] * (double)zi[j]);
+      auto put = [&](int kx, int ky, T re, T im) {
+        const size_t at = ((size_t)kx * n + ky) * nh + kz;
+        const cplx<T> s = mk<T>(re, im);
+        if (o.S) o.S[at] = s;
+        if (o.S2) o.S2[at] = s;
+        if (o.SZ) {
+          const T z = (T)o.zs;
+          const cplx<T> sz = mk<T>(z * re, z * im);
+          o.SZ[at] = sz;
+          if (inside) {
+            o.vloc[at] = mk<T>((T)(f.x * (double)sz.x), (T)(f.x * (double)sz.y));
+            ew += w * f.y * ((double)sz.x * (double)sz.x + (double)sz.y * (double)sz.y);
+          } else {
+            o.vloc[at] = mk<T>((T)0, (T)0);
+          }
+        }
+      };
+      if (pa && pb) put(a, b, x[0] - x[1], x[2] + x[3]);
+      if (ma && mb) put(n - a, n - b, x[0] + x[1], x[2] - x[3]);
+      if (pa && mb) put(a, n - b, x[4] - x[5], x[6] + x[7]);
+      if (ma && pb) put(n - a, b, x[4] + x[5], x[6] - x[7]);
     }
   }
   double v[1] = {ew}, out[1];
   block_sum<1>(v, red, out);
-  if (threadIdx.x == 0) ew_partial[blockIdx.x] = out[0];
+  if (tid == 0) o.ew[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = out[0];
 }
 
 // ---------------------------------------------------------------------------
-// Ewald: real-space pair sum (all pairs I, J and lattice images within rcut).
-// Each pair's displacement is taken at minimum image (|d| <= L/2 per axis), so
-// images a with |a| <= nimg = ceil(rcut/L + 1/2) per axis cover every
-// distance below rcut.  A block walks its share of the (pair, image)
-// combinations 256 at a time, compacts the ones inside rcut into shared
-// memory (warp ballots and a block prefix, in combination order) and only
-// then evaluates erfc, on dense warps: the FP64 erfc is by far the costliest
-// step, and fewer than 1% of the combinations are inside.  Fixed order
-// throughout, so the sum is deterministic.
+// Ewald: real-space sum over ion pairs and lattice images within rcut.  Each
+// pair is taken once: ion I with I + d (mod n_ion), d = 0 .. n_ion/2 (d = 0, an
+// ion with its own images, and d = n_ion/2 of an even count, met from both ends,
+// count half).  Displacements are at minimum image (|x| <= L/2 per axis), so an
+// image shift by |a| cells lies at least (|a| - 1/2) L away and the images
+// |a| <= nimg = ceil(rcut/L + 1/2) - 1 per axis are all: none but the pair itself
+// once L >= 2 rcut.  (Shifts of +-1 were walked for every pair: 27 times the
+// distances, 152 us for 300 ions in a 28-bohr cell.)  A block walks its share of
+// the (pair, image) combinations 256 at a time, compacts the ones inside rcut
+// into shared memory (warp ballots and a block prefix, in combination order) and
+// only then evaluates erfc, on dense warps.  The last block adds the reciprocal
+// partials ew[0..new_) of k_struct (res[0]) and its own kind (res[1]).  Fixed
+// order throughout.
 static __global__ void __launch_bounds__(256) k_ewald_real(const double* __restrict__ pos,
                                                            const double* __restrict__ Z, int n_ion, double L,
-                                                           double eta, double rcut, int nimg,
-                                                           double* __restrict__ partial) {
+                                                           double eta, double rcut, int nimg, const double* ew, int new_,
+                                                           double* partial, unsigned int* counter, double* res) {
   __shared__ double red[32];
   __shared__ double sr[256], sz[256];
   __shared__ int wcount[8], wbase[8], total;
   const int side = 2 * nimg + 1;
-  const long nim3 = (long)side * side * side;
-  const long tot = (long)n_ion * n_ion * nim3;
+  const int nim3 = side * side * side;
+  const int nd = n_ion / 2 + 1;
+  const long tot = (long)n_ion * nd * nim3;
   const long per = (tot + gridDim.x - 1) / gridDim.x;
   const long q0 = (long)blockIdx.x * per, q1 = min(tot, q0 + per);
   const double rc2 = rcut * rcut;
@@ -189,7 +215,8 @@ static __global__ void __launch_bounds__(256) k_ewald_real(const double* __restr
     if (q < q1) {
       const long p = q / nim3;
       const int im = (int)(q - p * nim3);
-      const int I = (int)(p / n_ion), J = (int)(p % n_ion);
+      const int I = (int)(p / nd), d = (int)(p % nd);
+      const int J = I + d < n_ion ? I + d : I + d - n_ion;
       const int a = im / (side * side) - nimg, b = (im / side) % side - nimg, c = im % side - nimg;
       double x = pos[I * 3] - pos[J * 3], y = pos[I * 3 + 1] - pos[J * 3 + 1], z = pos[I * 3 + 2] - pos[J * 3 + 2];
       const double iL = 1.0 / L;     // uniform: folded to one reciprocal per thread
@@ -197,7 +224,7 @@ static __global__ void __launch_bounds__(256) k_ewald_real(const double* __restr
       x += a * L; y += b * L; z += c * L;
       const double r2 = x * x + y * y + z * z;
       inside = r2 > 1e-24 && r2 < rc2;
-      if (inside) { r = sqrt(r2); zz = Z[I] * Z[J]; }
+      if (inside) { r = sqrt(r2); zz = Z[I] * Z[J] * (d == 0 || 2 * d == n_ion ? 0.5 : 1.0); }
     }
     const unsigned bal = __ballot_sync(0xffffffffu, inside);
     if (lane == 0) wcount[wid] = __popc(bal);
@@ -213,12 +240,20 @@ static __global__ void __launch_bounds__(256) k_ewald_real(const double* __restr
       sr[slot] = r; sz[slot] = zz;
     }
     __syncthreads();
-    if ((int)threadIdx.x < total) acc += 0.5 * sz[threadIdx.x] * erfc(eta * sr[threadIdx.x]) / sr[threadIdx.x];
+    if ((int)threadIdx.x < total) acc += sz[threadIdx.x] * erfc(eta * sr[threadIdx.x]) / sr[threadIdx.x];
     __syncthreads();
   }
   double v[1] = {acc}, out[1];
   block_sum<1>(v, red, out);
   if (threadIdx.x == 0) partial[blockIdx.x] = out[0];
+  if (arrive_last(counter)) {
+    double s[2] = {0, 0}, t[2];
+    for (int i = threadIdx.x; i < new_; i += blockDim.x) s[0] += __ldcg(ew + i);
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) s[1] += __ldcg(partial + i);
+    __shared__ double red2[64];
+    block_sum<2>(s, red2, t);
+    if (threadIdx.x == 0) { res[0] = t[0]; res[1] = t[1]; *counter = 0u; }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -431,72 +466,140 @@ namespace ofdft {
 //   e_I(G) = exp(-i G.R_I),  qq(G) = w(G) conj(vfac(G) n~(G) + efac(G) A(G)),
 //   A(G) = sum_J Z_J exp(-i G.R_J),  vfac = -4 pi exp(-G^2 rc^2/4)/G^2 (per unit Z),
 //   efac = (4 pi / Omega) exp(-G^2/(4 eta^2))/G^2,
-// over the listed G (0 < |G|^2 within the local and Ewald cutoffs, half
-// spectrum with Hermitian weight w = 2, or 1 on the kz = 0 and n/2 planes).
-// The G list and the signed m of each index are those of k_struct, so the
-// forces are the exact derivative of the energy the evaluation computes.
+// over 0 < |G|^2 within the local and Ewald cutoffs (half spectrum with
+// Hermitian weight w = 2, or 1 on the kz = 0 and n/2 planes), the G set and
+// signed m of k_struct, so the forces are the exact derivative of the energy the
+// evaluation computes.
+//
+// The G are taken as row pairs (a, b), a, b >= 0, of four rows (+-a, +-b) each
+// (see k_struct), rows[] sorted by a^2 + b^2; a tile of 32 pairs shares its
+// largest kz.  qq in the order [tile][kz][half][lane] of float4 / 2 double2
+// (half 0: rows (+a,+b), (-a,-b); half 1: (+a,-b), (-a,+b)), zero where a row or
+// kz is outside; tile t starts at kz offset tk[t] and has tk[t + 1] - tk[t] kz.
 
-// one thread per listed G: qq(G) = w conj(vfac n~ + efac S_Z), with S_Z(G) as
-// k_struct formed it (plan precision)
+// one thread per (tile, kz, lane): the four rows' qq
 template <typename T>
-__global__ void k_forces_q(const cplx<T>* __restrict__ nt, const int4* __restrict__ gl,
-                           const double2* __restrict__ gf, int ng, const cplx<T>* __restrict__ SZ, int n,
-                           double invN, cplx<T>* __restrict__ qq) {
+__global__ void k_forces_q(const cplx<T>* __restrict__ nt, const cplx<T>* __restrict__ SZ,
+                           const int2* __restrict__ rows, int nrows, const int* __restrict__ tk, int ntile,
+                           const double2* __restrict__ gf, int m2max, int n, double invN, Quad<T>* __restrict__ qq) {
   const int nh = n / 2 + 1;
-  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < ng; g += gridDim.x * blockDim.x) {
-    const int4 e = gl[g];
-    const size_t q = ((size_t)e.x * n + e.y) * nh + e.z;
-    const cplx<T> v = nt[q], A = SZ[q];
-    const double2 f = gf[g];                        // (vfac, efac)
-    const double w = (double)e.w;
-    const double qr = f.x * (double)v.x * invN + f.y * (double)A.x;
-    const double qi = f.x * (double)v.y * invN + f.y * (double)A.y;
-    qq[g] = mk<T>((T)(w * qr), (T)(-w * qi));       // w conj(Q)
+  const int lane = threadIdx.x & 31;
+  const int tot = tk[ntile];
+  for (int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < tot; g += (gridDim.x * blockDim.x) >> 5) {
+    // the tile of this kz slot (uniform per warp)
+    int lo = 0, hi = ntile;
+    while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (tk[mid] <= g) lo = mid; else hi = mid; }
+    const int kz = g - tk[lo], r = lo * 32 + lane;
+    Quad<T> q0{0, 0, 0, 0}, q1{0, 0, 0, 0};
+    if (r < nrows) {
+      const int2 ab = rows[r];
+      const int a = ab.x, b = ab.y, m2 = a * a + b * b + kz * kz;
+      if (m2 > 0 && m2 <= m2max) {
+        const double2 f = gf[m2];                        // (vfac, efac)
+        const double w = (kz == 0 || 2 * kz == n) ? 1.0 : 2.0;
+        auto one = [&](int kx, int ky, T& re, T& im) {
+          const size_t q = ((size_t)kx * n + ky) * nh + kz;
+          const cplx<T> v = nt[q], A = SZ[q];
+          re = (T)(w * (f.x * (double)v.x * invN + f.y * (double)A.x));
+          im = (T)(-w * (f.x * (double)v.y * invN + f.y * (double)A.y));   // w conj(Q)
+        };
+        const bool pa = 2 * a < n, ma = a > 0, pb = 2 * b < n, mb = b > 0;
+        if (pa && pb) one(a, b, q0.a, q0.b);
+        if (ma && mb) one(n - a, n - b, q0.c, q0.d);
+        if (pa && mb) one(a, n - b, q1.a, q1.b);
+        if (ma && pb) one(n - a, b, q1.c, q1.d);
+      }
+    }
+    qq[((size_t)g * 2) * 32 + lane] = q0;
+    qq[((size_t)g * 2 + 1) * 32 + lane] = q1;
   }
 }
 
-// e_I phases in the plan's precision: pt[(I*3 + d)*n + k] = ph[...]
-template <typename T>
-__global__ void k_phases_t(const double2* __restrict__ ph, cplx<T>* __restrict__ pt, int tot) {
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < tot; q += gridDim.x * blockDim.x)
-    pt[q] = mk<T>((T)ph[q].x, (T)ph[q].y);
-}
-
-// one block per ion: F_I(G part) = -Z_I tp sum_G Im[qq e_I] m(G) -> out[I*3 .. I*3+2]
-template <typename T>
-__global__ void __launch_bounds__(256) k_forces_g(const cplx<T>* __restrict__ qq, const int4* __restrict__ gl,
-                                                  int ng, const cplx<T>* __restrict__ pt,
-                                                  const double* __restrict__ Z, int n, double tp,
-                                                  double* __restrict__ out) {
-  __shared__ typename TreeVal<T>::type scr[3 * 257];
-  const int I = blockIdx.x;
-  const cplx<T>* px = pt + (size_t)I * 3 * n;
-  const cplx<T>* py = px + n;
-  const cplx<T>* pz = py + n;
-  Acc<T> acc[3];
-  for (int g = threadIdx.x; g < ng; g += blockDim.x) {
-    const int4 e = gl[g];
-    const cplx<T> a = px[e.x], b = py[e.y], c = pz[e.z];
-    const cplx<T> ab = cmul(a, b);
-    const cplx<T> eI = cmul(ab, c);
-    const cplx<T> q = qq[g];
-    const T im = q.x * eI.y + q.y * eI.x;          // Im[q e_I]
-    const int mx = e.x <= (n - 1) / 2 ? e.x : e.x - n;
-    const int my = e.y <= (n - 1) / 2 ? e.y : e.y - n;
-    const int mz = e.z <= (n - 1) / 2 ? e.z : e.z - n;   // the phase tables' convention
-    acc[0].add(im * (T)mx); acc[1].add(im * (T)my); acc[2].add(im * (T)mz);
+// Block: one tile of 32 row pairs (a lane each) and NW TI ions (TI per warp).
+// Along kz (from the tile's largest down) a lane sums U = sum qq e_z and
+// V = sum kz qq e_z for its four rows (V by adding the running U after every
+// step kz >= 1), six operations per G and ion, against the tile's qq (registers,
+// read once per TI ions) and the ions' e_z (broadcast from shared memory); then
+// Im[P U] etc. times (a, b) and Im[P V], summed over the lanes.  (A gather of
+// three phases and two complex products per G and ion took 186 us for 128 ions
+// at 108^3.)  part[tile][ion][3], FP64, without the factor -Z_I 2 pi / L.
+constexpr int kForceWarps = 4;
+template <typename T, int TI>
+__global__ void __launch_bounds__(32 * kForceWarps) k_forces_g(const Quad<T>* __restrict__ qq, const int2* __restrict__ rows,
+                                                               int nrows, const int* __restrict__ tk,
+                                                               const cplx<T>* __restrict__ ph, int n_ion, int n,
+                                                               double* __restrict__ part) {
+  constexpr int NI = kForceWarps * TI, KC = 32;
+  __shared__ cplx<T> se[KC][NI];
+  const int tile = blockIdx.x, I0 = blockIdx.y * NI;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int k0 = tk[tile], nk = tk[tile + 1] - k0;
+  cplx<T> U[TI][4], V[TI][4];
+#pragma unroll
+  for (int i = 0; i < TI; ++i)
+#pragma unroll
+    for (int s = 0; s < 4; ++s) { U[i][s] = mk<T>((T)0, (T)0); V[i][s] = mk<T>((T)0, (T)0); }
+  for (int kt = nk; kt > 0; kt -= KC) {                  // chunks [kb, kt), top first
+    const int kb = max(0, kt - KC);
+    __syncthreads();
+    for (int q = threadIdx.x; q < (kt - kb) * NI; q += 32 * kForceWarps) {
+      const int i = q / (kt - kb), k = q - i * (kt - kb);
+      se[k][i] = I0 + i < n_ion ? ph[((size_t)(I0 + i) * 3 + 2) * n + kb + k] : mk<T>((T)0, (T)0);
+    }
+    __syncthreads();
+    for (int k = kt - 1; k >= kb; --k) {
+      const Quad<T> q0 = qq[((size_t)(k0 + k) * 2) * 32 + lane], q1 = qq[((size_t)(k0 + k) * 2 + 1) * 32 + lane];
+#pragma unroll
+      for (int i = 0; i < TI; ++i) {
+        const cplx<T> e = se[k - kb][warp * TI + i];
+        U[i][0].x = fma(q0.a, e.x, fma(-q0.b, e.y, U[i][0].x)); U[i][0].y = fma(q0.a, e.y, fma(q0.b, e.x, U[i][0].y));
+        U[i][1].x = fma(q0.c, e.x, fma(-q0.d, e.y, U[i][1].x)); U[i][1].y = fma(q0.c, e.y, fma(q0.d, e.x, U[i][1].y));
+        U[i][2].x = fma(q1.a, e.x, fma(-q1.b, e.y, U[i][2].x)); U[i][2].y = fma(q1.a, e.y, fma(q1.b, e.x, U[i][2].y));
+        U[i][3].x = fma(q1.c, e.x, fma(-q1.d, e.y, U[i][3].x)); U[i][3].y = fma(q1.c, e.y, fma(q1.d, e.x, U[i][3].y));
+        if (2 * k == n) {                                // kz = n/2 is -n/2: n/2 steps follow
+#pragma unroll
+          for (int s = 0; s < 4; ++s) { V[i][s].x = (T)-n * U[i][s].x; V[i][s].y = (T)-n * U[i][s].y; }
+        }
+        if (k > 0) {
+#pragma unroll
+          for (int s = 0; s < 4; ++s) { V[i][s].x += U[i][s].x; V[i][s].y += U[i][s].y; }
+        }
+      }
+    }
   }
-  double s[3];
-  block_sum_tree<3, T>(acc, 3, s, scr);
-  if (threadIdx.x < 3) out[(size_t)I * 3 + threadIdx.x] = -Z[I] * tp * s[threadIdx.x];
+  const int r = tile * 32 + lane;
+  const int2 ab = rows[min(r, nrows - 1)];               // (lanes past the end hold zeros)
+  const int a = ab.x, b = ab.y;
+#pragma unroll
+  for (int i = 0; i < TI; ++i) {
+    const int I = I0 + warp * TI + i;
+    if (I >= n_ion) break;                               // the whole warp
+    const cplx<T>* p = ph + (size_t)I * 3 * n;
+    cplx<T> ex = p[a], ey = p[n + b];
+    if (2 * a == n) ex.y = -ex.y;
+    if (2 * b == n) ey.y = -ey.y;
+    const T Pr = ex.x * ey.x - ex.y * ey.y, Pi = ex.x * ey.y + ex.y * ey.x;
+    const T Mr = ex.x * ey.x + ex.y * ey.y, Mi = ex.y * ey.x - ex.x * ey.y;
+    // Im[P u], Im[P* u]
+    const T u0 = Pr * U[i][0].y + Pi * U[i][0].x, u1 = Pr * U[i][1].y - Pi * U[i][1].x;
+    const T u2 = Mr * U[i][2].y + Mi * U[i][2].x, u3 = Mr * U[i][3].y - Mi * U[i][3].x;
+    const T z0 = Pr * V[i][0].y + Pi * V[i][0].x, z1 = Pr * V[i][1].y - Pi * V[i][1].x;
+    const T z2 = Mr * V[i][2].y + Mi * V[i][2].x, z3 = Mr * V[i][3].y - Mi * V[i][3].x;
+    double f[3] = {(double)a * ((double)u0 - (double)u1 + (double)u2 - (double)u3),
+                   (double)b * ((double)u0 - (double)u1 - (double)u2 + (double)u3),
+                   (double)z0 + (double)z1 + (double)z2 + (double)z3};
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const double s = warp_sum(f[d]);
+      if (lane == 0) part[((size_t)tile * n_ion + I) * 3 + d] = s;
+    }
+  }
 }
 
 // Ewald real-space force on ion I = blockIdx.x / nsplit from the share
 // blockIdx.x % nsplit of its (J, image) terms, FP64, into part[blockIdx.x * 3
-// ..] (k_sum_force_parts adds the shares to the forces in a fixed order).  As
-// in k_ewald_real, displacements are taken at minimum image (|a| <= nimg
-// images per axis then cover every distance below rcut) and the in-range terms
-// are compacted before their erfc and exp are evaluated.
+// ..] (k_sum_force_parts adds the shares in a fixed order).  Images and
+// compaction of the in-range terms as in k_ewald_real.
 static __global__ void __launch_bounds__(256) k_ewald_force_real(const double* __restrict__ pos,
                                                                  const double* __restrict__ Z, int n_ion, double L,
                                                                  double eta, double rcut, int nimg, int nsplit,
@@ -559,15 +662,21 @@ static __global__ void __launch_bounds__(256) k_ewald_force_real(const double* _
   }
 }
 
-// out[I * 3 + d] += sum_s part[(I nsplit + s) * 3 + d], s in order; one thread per (I, d)
-static __global__ void k_sum_force_parts(const double* __restrict__ part, int n_ion, int nsplit,
+// The force component t = 3 I + d: -Z_I tp times the G-space sums gpart[tile][I][d]
+// of the ntile tiles, plus the real-space shares part[(I nsplit + s) 3 + d].  One
+// warp per component: lanes take the tiles and shares in turn, the lane sums are
+// added by a fixed tree.
+static __global__ void k_sum_force_parts(const double* __restrict__ gpart, int ntile, const double* __restrict__ Z,
+                                         double tp, const double* __restrict__ part, int n_ion, int nsplit,
                                          double* __restrict__ out) {
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n_ion * 3; t += gridDim.x * blockDim.x) {
-    const int I = t / 3, d = t - I * 3;
-    double s = 0;
-    for (int k = 0; k < nsplit; ++k) s += part[((size_t)I * nsplit + k) * 3 + d];
-    out[t] += s;
-  }
+  const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (t >= n_ion * 3) return;
+  const int I = t / 3, d = t - I * 3;
+  double g = 0, s = 0;
+  for (int k = lane; k < ntile; k += 32) g += gpart[(size_t)k * n_ion * 3 + t];
+  for (int k = lane; k < nsplit; k += 32) s += part[((size_t)I * nsplit + k) * 3 + d];
+  s = warp_sum(s - Z[I] * tp * g);
+  if (lane == 0) out[t] = s;
 }
 
 }  // namespace ofdft
