@@ -305,15 +305,16 @@ __host__ __device__ constexpr size_t tree_scratch_bytes(int nq, int nt) {
 // (after its thread 0 has written the block's partial results); the last one
 // then reads all partials (use __ldcg) and resets the counter for the next
 // launch in the stream.
-__device__ __forceinline__ bool arrive_last(unsigned int* counter) {
+__device__ __forceinline__ bool arrive_last(unsigned int* counter, unsigned int blocks) {
   __shared__ bool s_last;
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(counter, 1u) == gridDim.x - 1;
+  if (threadIdx.x == 0) s_last = atomicAdd(counter, 1u) == blocks - 1;
   __syncthreads();
   if (s_last) __threadfence();
   return s_last;
 }
+__device__ __forceinline__ bool arrive_last(unsigned int* counter) { return arrive_last(counter, gridDim.x); }
 
 // One block: out[c] = sum_r partial[r * cols + c], fixed order, FP64.  Thread
 // t sums column t % cols over rows t / cols, t / cols + k, ... (k = blockDim /

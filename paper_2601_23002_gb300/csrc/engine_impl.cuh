@@ -149,7 +149,9 @@ class Engine : public IEngine {
   size_t partials_cap = 0;
   double* res_d = nullptr;
   TwoLoopState* tl_state = nullptr;   // L-BFGS history scalars on the device
-  double* res_h = nullptr;     // pinned
+  // pinned: the kernels whose results the host waits for write them here
+  // themselves (a copy per result took 2-3 us of the stream and of the host)
+  double* res_h = nullptr;
   unsigned int* counters = nullptr;   // last-block arrival counters (0 between launches)
   double* pos_d = nullptr;
   double* Z_d = nullptr;
@@ -829,37 +831,38 @@ class Engine : public IEngine {
     return OFDFT_OK;
   }
 
-  // Sum columns of partials[rows][cols] into res_d[off ...] (fixed order).
+  // Sum columns of partials[rows][cols] into res_h[off ...] (fixed order).
   int sum_partials(int rows, int cols, int off, cudaStream_t st) {
     if (cols > 256) { set_error("sum_partials: too many columns"); return OFDFT_ERR_INVALID; }
-    OFDFT_RUN("k_sum_columns", st, (double)rows * cols * 8, k_sum_columns<<<1, 256, 0, st>>>(partials, rows, cols, res_d + off));
+    OFDFT_RUN("k_sum_columns", st, (double)rows * cols * 8, k_sum_columns<<<1, 256, 0, st>>>(partials, rows, cols, res_h + off));
     return OFDFT_OK;
   }
 
-  // k_struct with the largest thread tile that still gives most SMs a block:
-  // FP32 2 x 4 (64 accumulators) or 2 x 2, FP64 2 x 2, small grids 1 x 1.
-  int launch_struct(const StructOut<T>& so, const double* zw, int full, int* nblk, cudaStream_t st) {
+  // k_struct with the largest thread tile that still gives every SM two blocks
+  // (a block waits for its staged ions at two barriers per chunk; the other one
+  // works meanwhile): FP32 2 x 4 (64 accumulators), 2 x 2, 1 x 2; small grids 1 x 1.
+  int launch_struct(const StructOut<T>& so, const double* zw, int full, cudaStream_t st) {
     const int2* rows = full ? nullptr : sf_rows;
     const int nrows = full ? nh * nh : sf_nrows;
     bool done = false;
-    auto go = [&](auto TRc, auto TCc, auto NTc, bool last) -> int {
+    auto go = [&](auto TRc, auto TCc, auto NTc, int least) -> int {
       constexpr int TR = decltype(TRc)::value, TC = decltype(TCc)::value, NT = decltype(NTc)::value;
       const int ctiles = (nh + TC * 64 - 1) / (TC * 64);        // at most 64 threads along kz
       const int CT = (nh + TC * ctiles - 1) / (TC * ctiles);
       const int RT = NT / CT * TR;
       const int g = (nrows + RT - 1) / RT;
-      if (!last && g * ctiles < 120) return OFDFT_OK;
+      if (g * ctiles < least) return OFDFT_OK;
       const size_t sm = struct_smem<T, TR, TC, NT>(CT);
       OFDFT_RUN("k_struct", st, (double)nrows * 4 * nh * sizeof(C) * 3.0, k_struct<T, TR, TC, NT><<<dim3(g, ctiles), NT, sm, st>>>(phases, zw, (int)cs.Z.size(), n, rows, nrows, CT, so));
-      *nblk = g * ctiles;
       done = true;
       return OFDFT_OK;
     };
     using std::integral_constant;
     int rc = OFDFT_OK;
-    if constexpr (sizeof(T) == 4) rc = go(integral_constant<int, 2>{}, integral_constant<int, 4>{}, integral_constant<int, 256>{}, false);
-    if (!rc && !done) rc = go(integral_constant<int, 2>{}, integral_constant<int, 2>{}, integral_constant<int, 256>{}, false);
-    if (!rc && !done) rc = go(integral_constant<int, 1>{}, integral_constant<int, 1>{}, integral_constant<int, 64>{}, true);
+    if constexpr (sizeof(T) == 4) rc = go(integral_constant<int, 2>{}, integral_constant<int, 4>{}, integral_constant<int, 256>{}, 2 * nsm - 8);
+    if (!rc && !done) rc = go(integral_constant<int, 2>{}, integral_constant<int, 2>{}, integral_constant<int, 256>{}, 2 * nsm - 8);
+    if (!rc && !done) rc = go(integral_constant<int, 1>{}, integral_constant<int, 2>{}, integral_constant<int, 128>{}, nsm);
+    if (!rc && !done) rc = go(integral_constant<int, 1>{}, integral_constant<int, 1>{}, integral_constant<int, 64>{}, 0);
     return rc;
   }
 
@@ -868,9 +871,16 @@ class Engine : public IEngine {
     const int nion = (int)cs.Z.size();
     OFDFT_CK(cudaMemcpyAsync(pos_d, pos, (size_t)nion * 3 * sizeof(double),
                              on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st));
-    const int tot = nion * 3 * nh;
-    OFDFT_RUN("k_phases", st, (double)nion * 3 * n * sizeof(C), k_phases<T><<<std::min(4096, (tot + 127) / 128), 128, 0, st>>>(pos_d, nion, n, L, phases));
     const double eta = ewald_eta();
+    const double rcut = 6.3 / eta;
+    // images per axis around minimum-image displacements (see ewald_real_part)
+    const int nimg_mi = std::max(0, (int)std::ceil(rcut / L + 0.5) - 1);
+    ew_eta = eta; ew_rcut = rcut; ew_nimg = nimg_mi;
+    const long ncomb = (long)nion * (nion / 2 + 1) * (2 * nimg_mi + 1) * (2 * nimg_mi + 1) * (2 * nimg_mi + 1);
+    const int gb = (int)std::min<long>(2L * nsm, (ncomb + 255) / 256);
+    const int gp = std::min(2 * nsm, (nion * 3 * nh + 255) / 256);
+    double* real = partials + partials_cap - gb;         // behind k_struct's partials
+    OFDFT_RUN("k_ions", st, (double)nion * 3 * n * sizeof(C), k_ions<T><<<gb + gp, 256, 0, st>>>(pos_d, Z_d, nion, n, L, phases, eta, rcut, nimg_mi, gb, real));
     const int full = S_out != nullptr;
     // without the full S(G) only the rows inside sf_m2 are formed, the others
     // stay zero
@@ -884,25 +894,18 @@ class Engine : public IEngine {
     // one ion species (every workload here): S_Z = Z S, one sum over the ions
     bool uni = true;
     for (double z : cs.Z) uni = uni && z == cs.Z[0];
-    int nblk = 0;
-    StructOut<T> so{Sg, (C*)S_out, uni ? SZg : nullptr, vloc, cs.Z[0], sf_tab, (double)sf_m2, partials};
-    if (int rc = launch_struct(so, nullptr, full, &nblk, st)) return rc;
+    StructOut<T> so{Sg, (C*)S_out, uni ? SZg : nullptr, vloc, cs.Z[0], sf_tab, (double)sf_m2, partials, uni ? res_h : nullptr, real, gb, counters + 4};
+    if (int rc = launch_struct(so, nullptr, full, st)) return rc;
     if (!uni) {
-      so.S = so.S2 = nullptr; so.SZ = SZg; so.zs = 1.0;
-      if (int rc = launch_struct(so, Z_d, full, &nblk, st)) return rc;
+      so.S = so.S2 = nullptr; so.SZ = SZg; so.zs = 1.0; so.res = res_h;
+      if (int rc = launch_struct(so, Z_d, full, st)) return rc;
     }
-    const double rcut = 6.3 / eta;
-    // images per axis around minimum-image displacements (see k_ewald_real)
-    const int nimg_mi = std::max(0, (int)std::ceil(rcut / L + 0.5) - 1);
-    ew_eta = eta; ew_rcut = rcut; ew_nimg = nimg_mi;
-    const long ncomb = (long)nion * (nion / 2 + 1) * (2 * nimg_mi + 1) * (2 * nimg_mi + 1) * (2 * nimg_mi + 1);
-    const int gb = (int)std::min<long>(4L * nsm, (ncomb + 255) / 256);
-    OFDFT_RUN("k_ewald_real", st, (double)nion * 32, k_ewald_real<<<gb, 256, 0, st>>>(pos_d, Z_d, nion, L, eta, rcut, nimg_mi, partials, nblk, partials + nblk, counters + 4, res_d));
-    if (planes)
-      OFDFT_RUN("k_vloc_planes", st, 2.0 * NH * sizeof(C), k_vloc_planes<T><<<4 * nsm, 256, 0, st>>>(vloc, vloc_pl, rev_d, n));
-    if (p256_possible())
-      OFDFT_RUN("k_vloc_planes256", st, 2.0 * NH * sizeof(C), k_vloc_planes256<T><<<4 * nsm, 256, 0, st>>>(vloc, vloc_pl));
-    OFDFT_CK(cudaMemcpyAsync(res_h, res_d, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
+    if (vloc_pl) {
+      // (a little past the cutoff: the passes test it in the plan's precision)
+      const double tp = 2.0 * kPi / L;
+      const int m2max = (int)std::min(3.0 * h * h, std::floor(g2cut_loc / (tp * tp) * (1.0 + 1e-5)) + 1.0);
+      OFDFT_RUN("k_vloc_planes", st, 2.0 * n_vloc * sizeof(C), k_vloc_planes<T><<<dim3((n + 31) / 32, n), 256, 0, st>>>(vloc, vloc_pl, planes ? rev_d : nullptr, n, m2max));
+    }
     OFDFT_CK(cudaStreamSynchronize(st));
     double zz = 0;
     for (double z : cs.Z) zz += z * z;
@@ -912,12 +915,14 @@ class Engine : public IEngine {
   }
 
   // One evaluation.  mode 0: density rho; mode 1: psi + t d with scale.
-  // Leaves results in res_d[0..13]; copies them to res_h when sync != 0.
+  // Leaves the raw sums in res_d[0..11], or in res_h when the host will read
+  // them (sync: here; to_host: after its own synchronisation).
   // dsc (device, optional): the trial's scale and psi shift as formed by
   // k_lincomb (TrialScale); the host values scale, Q, psid are then only used
   // when sync is set, and the caller finishes with finish_eval instead.
   int eval(int mode, const T* rho, const T* ps, const T* dd, double t, double scale, double Q, double psid,
-           T* out, cudaStream_t st, bool sync, double mu_ref = 0.0, const double* dsc = nullptr) {
+           T* out, cudaStream_t st, bool sync, double mu_ref = 0.0, const double* dsc = nullptr,
+           bool to_host = false) {
     Spectra<T> sp = spectra();
     // psi of the uniform density: sqrt(nbar) for a given rho, sqrt(nbar / scale) for psi + t d
     const double psi_bar = std::sqrt(nbar / (mode == 0 ? 1.0 : scale));
@@ -959,14 +964,13 @@ class Engine : public IEngine {
     // epilogue partials after room for 3 fields of G-space rows
     TV* pe = pt + g_room() * 4;
     if (mode == 0) mu_ref = 0.0;
-    FinArgs<T> fa{pt, g_rows, pe, grid_z, res_d};
+    FinArgs<T> fa{pt, g_rows, pe, grid_z, sync || to_host ? res_h : res_d};
     const double cy = 9.8696044010893586188344909998762 / (1.4142135623730950488016887242097 * std::pow(Te, 1.5));
     EpiArgs<T> ea{mode, rho, ps, dd, (T)t, (T)scale, (T)cs.alpha, (T)Te, (T)cy, (T)mu_ref, cs.terms, out, pe, fa,
                   counters + 0, nullptr, nullptr, dsc, cs.fd64 ? 1 : 0, cy, (T)std::log(cy)};
     const double eb = (double)sp.nact * NH * sizeof(C) + (double)(mode == 0 ? 1 : 2) * N * sizeof(T) + (out ? (double)N * sizeof(T) : 0.0);
     if (int rc = launch_zinv(sp, ea, eb, st)) return rc;
     if (sync) {
-      OFDFT_CK(cudaMemcpyAsync(res_h, res_d, 12 * sizeof(double), cudaMemcpyDeviceToHost, st));
       OFDFT_CK(cudaStreamSynchronize(st));
       finish_eval(mode, scale, Q, psid, mu_ref, sp.merged != 0);
     }
@@ -1072,13 +1076,14 @@ class Engine : public IEngine {
     if ((size_t)nv * nw > 104 || nw > kMaxW) { set_error("gram: too many vectors"); return OFDFT_ERR_INVALID; }
     out.assign((size_t)nv * nw, 0.0);
     // every chunk's last block writes its columns to res_d[16 + c0 * nw ...]
+    // (readback: res_h)
     const int chunk = std::min(kMaxV, kMaxLin - nw);      // a launch streams cn + nw <= kMaxLin vectors
     for (int c0 = 0; c0 < nv; c0 += chunk) {
       const int cn = std::min(chunk, nv - c0);
       VecList<T> xl{}; xl.nv = cn + nw;
       for (int i = 0; i < cn; ++i) xl.v[i] = V[c0 + i];
       for (int j = 0; j < nw; ++j) xl.v[cn + j] = W[j];
-      double* o = res_d + 16 + (size_t)c0 * nw;
+      double* o = (readback ? res_h : res_d) + 16 + (size_t)c0 * nw;
       const int S = cn + nw <= 17 ? 3 : 2;   // k_gram is built for 2 or 3 ring stages
       const size_t sm = std::max(StreamCfg<T>::ring_bytes(S, cn + nw), tree_scratch_bytes<T>(cn * nw, kStreamThreads));
       prof.begin("k_gram", st, (double)(cn + nw) * N * sizeof(T));
@@ -1100,8 +1105,7 @@ class Engine : public IEngine {
       OFDFT_LAUNCH_CK();
     }
     if (!readback) return OFDFT_OK;
-    int rc;
-    if ((rc = read_results(st))) return rc;
+    OFDFT_CK(cudaStreamSynchronize(st));
     for (int i = 0; i < nv; ++i)
       for (int j = 0; j < nw; ++j) out[(size_t)i * nw + j] = res_h[16 + i * nw + j] * dV;
     return OFDFT_OK;
@@ -1117,18 +1121,10 @@ class Engine : public IEngine {
     xl.nv = nv + 2;
     OFDFT_RUN("k_lincomb", st, (double)(nv + 3) * N * sizeof(T),
               k_lincomb<T><<<grid_stream, kStreamThreads, StreamCfg<T>::ring_bytes(stream_stages(kMaxLin - 1), nv + 2), st>>>(
-                  xl, nv, out, Nv, partials, counters + 2, res_d + 16, ts, dcoef));
+                  xl, nv, out, Nv, partials, counters + 2, res_d + 16, res_h + 16, ts, dcoef));
     if (!dd) return OFDFT_OK;
-    int rc;
-    if ((rc = read_results(st))) return rc;
-    *dd = res_h[16] * dV; *dg = res_h[17] * dV; *dpsi = res_h[18] * dV;
-    return OFDFT_OK;
-  }
-
-  // copy the reduction results res_d[16, 120) to the host
-  int read_results(cudaStream_t st) {
-    OFDFT_CK(cudaMemcpyAsync(res_h + 16, res_d + 16, (120 - 16) * sizeof(double), cudaMemcpyDeviceToHost, st));
     OFDFT_CK(cudaStreamSynchronize(st));
+    *dd = res_h[16] * dV; *dg = res_h[17] * dV; *dpsi = res_h[18] * dV;
     return OFDFT_OK;
   }
 
@@ -1297,7 +1293,7 @@ int Engine<T>::minimize(void* rho_io, int start_uniform, const ofdft_min_opts& o
       if ((rc = gram(V, {g, pgv[pcur], Yh[new_slot], PYh[new_slot]}, cross, st, false))) return rc;
       // two-loop recursion on the device (k_twoloop), then the direction
       // d = coef[0] P g + sum (coef[1+2j] P y_j + coef[2+2j] s_j)
-      OFDFT_RUN("k_twoloop", st, 0.0, k_twoloop<<<1, 32, 0, st>>>(ta, res_d + 16, res_d + 120, tl_state, res_d + 129));
+      OFDFT_RUN("k_twoloop", st, 0.0, k_twoloop<<<1, 32, 0, st>>>(ta, res_d + 16, res_d + 120, tl_state, res_h + 129));
       VecList<T> vl{};
       vl.nv = 0;
       vl.v[vl.nv++] = pgv[pcur];
@@ -1305,15 +1301,12 @@ int Engine<T>::minimize(void* rho_io, int start_uniform, const ofdft_min_opts& o
         vl.v[vl.nv++] = PYh[ring.slot(j)];
         vl.v[vl.nv++] = Sh[ring.slot(j)];
       }
-      TrialScale ts{0.0, 1.0, Ne, dV, nbar, res_d + 126, &tl_state->Q, &tl_state->kk};
+      TrialScale ts{0.0, 1.0, Ne, dV, nbar, res_d + 126, res_h + 126, &tl_state->Q, &tl_state->kk};
       if ((rc = lincomb(vl, d, nullptr, nullptr, nullptr, st, ts, tl_state->coef))) return rc;
-      if ((rc = eval(1, nullptr, psi, d, 1.0, 1.0, 0.0, 0.0, gp, st, false, mu_ref, res_d + 126))) return rc;
+      if ((rc = eval(1, nullptr, psi, d, 1.0, 1.0, 0.0, 0.0, gp, st, false, mu_ref, res_d + 126, true))) return rc;
       ++evals;
-      OFDFT_CK(cudaMemcpyAsync(res_h, res_d, 12 * sizeof(double), cudaMemcpyDeviceToHost, st));
-      OFDFT_CK(cudaMemcpyAsync(res_h + 16, res_d + 16, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
-      OFDFT_CK(cudaMemcpyAsync(res_h + 126, res_d + 126, 5 * sizeof(double), cudaMemcpyDeviceToHost, st));
       OFDFT_CK(cudaStreamSynchronize(st));
-      // k_accept's dots (copied after the accept) are on the host now
+      // k_accept's dots are on the host now
       Qcur = res_h[122] * dV;
       gg = res_h[123] * dV;
       gamma = res_h[129];
@@ -1391,8 +1384,7 @@ int Engine<T>::minimize(void* rho_io, int start_uniform, const ofdft_min_opts& o
     OFDFT_RUN("k_accept", st, 8.0 * N * sizeof(T),
               k_accept<T><<<grid_stream, kStreamThreads, StreamCfg<T>::ring_bytes(stream_stages(4), 4), st>>>(
                   xa, (T)acc.t, (T)(2.0 * lastScale), (T)(lastMu - mu_ref), psi, g, Sh[slot], Yh[slot], Nv,
-                  partials, counters + 3, res_d + 120));
-    OFDFT_CK(cudaMemcpyAsync(res_h + 120, res_d + 120, 6 * sizeof(double), cudaMemcpyDeviceToHost, st));
+                  partials, counters + 3, res_d + 120, res_h + 120));
     new_slot = slot;
     mu_ref = lastMu;
     const double dF = std::fabs(acc.f - F) / n_ion;
@@ -1575,13 +1567,14 @@ int Engine<T>::forces(const void* rho, double* f_out_h, void* stream_) {
   OFDFT_RUN("k_ypass", st, 2.0 * NH * sizeof(C), k_ypass<T, -1><<<dim3(grid_y1, 1), kThreads, smem_y, st>>>(sp, pn, tw_n, n, yJ));
   OFDFT_RUN("k_xpass", st, 2.0 * NH * sizeof(C), k_xpass<T, -1><<<dim3(grid_x, 1), kThreads, smem_xp, st>>>(sp, pn, tw_n, n, xJ));
   OFDFT_RUN("k_forces_q", st, (double)f_nk * 32 * (8 * sizeof(C) + 4 * sizeof(C)), k_forces_q<T><<<std::min(16 * nsm, (f_nk + 3) / 4), 128, 0, st>>>(spec[0], SZg, f_rows, f_nrows, f_tk, f_ntile, f_gf, f_m2, n, 1.0 / (double)N, f_qq));
-  constexpr int TI = sizeof(T) == 4 ? 4 : 2;
-  OFDFT_RUN("k_forces_g", st, (double)f_nk * 128 * sizeof(C), k_forces_g<T, TI><<<dim3(f_ntile, (nion + kForceWarps * TI - 1) / (kForceWarps * TI)), 32 * kForceWarps, 0, st>>>(f_qq, f_rows, f_nrows, f_tk, phases, nion, n, f_part));
   // several blocks per ion (about 4 per SM in all), shares added in a fixed order
   int nsplit = std::max(1, std::min(64, (4 * nsm + nion - 1) / nion));
   while (nsplit > 1 && (size_t)nion * nsplit * 3 > partials_cap) --nsplit;
   if ((size_t)nion * nsplit * 3 > partials_cap) { set_error("forces: too many ions for the scratch"); return OFDFT_ERR_INVALID; }
-  OFDFT_RUN("k_ewald_force_real", st, (double)nion * nion * 32, k_ewald_force_real<<<nion * nsplit, 256, 0, st>>>(pos_d, Z_d, nion, L, ew_eta, ew_rcut, ew_nimg, nsplit, partials));
+  constexpr int TI = sizeof(T) == 4 ? 4 : 2;
+  const int ny = (nion + kForceWarps * TI - 1) / (kForceWarps * TI);
+  const EwaldForceArgs wa{pos_d, Z_d, L, ew_eta, ew_rcut, ew_nimg, nsplit, partials};
+  OFDFT_RUN("k_forces_g", st, (double)f_nk * 128 * sizeof(C), k_forces_g<T, TI><<<f_ntile * ny + nion * nsplit, 32 * kForceWarps, 0, st>>>(f_qq, f_rows, f_nrows, f_tk, phases, nion, n, f_part, f_ntile, ny, wa));
   OFDFT_RUN("k_sum_force_parts", st, (double)nion * nsplit * 24, k_sum_force_parts<<<(3 * nion + 3) / 4, 128, 0, st>>>(f_part, f_ntile, Z_d, tp, partials, nion, nsplit, f_out));
   OFDFT_CK(cudaMemcpyAsync(f_out_h, f_out, (size_t)nion * 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
   OFDFT_CK(cudaStreamSynchronize(st));
@@ -1655,7 +1648,6 @@ int Engine<T>::pressure(const void* rho, double* p_out_h, void* stream_) {
   const double* pn_d = nl ? p_tab + (size_t)4 * (3 * h * h + 1) : nullptr;
   OFDFT_RUN("k_pressure_g", st, 3.0 * NH * sizeof(C), k_pressure_g<T><<<gb, 256, 0, st>>>(spec[0], spec[1], vl, pn_d, n, tp * tp, g2cut_loc, cs.rc * cs.rc, 1.0 / (double)N, partials));
   if ((rc = sum_partials(gb, 2, 2, st))) return rc;
-  OFDFT_CK(cudaMemcpyAsync(res_h, res_d, 4 * sizeof(double), cudaMemcpyDeviceToHost, st));
   OFDFT_CK(cudaStreamSynchronize(st));
   double* P = p_out_h;
   P[0] = res_h[0] / (double)N;              // (1/Omega) dV sum n T p

@@ -379,18 +379,37 @@ using PlaneKernel = void (*)(Spectra<T>, GArgs<T>, FftPlan1, const int*, const c
 template <typename T> PlaneKernel<T> plane_kernel(unsigned mask);
 template <typename T> PlaneKernel<T> plane_prec2_kernel(unsigned mask);
 
-// One-time reorder of V_loc from the tiled layout [kx][ky][kz] into plane
-// layout and position order: dst[(kz n + px) n + py] = src[(rev[px] n + rev[py]) nh + kz].
+// Reorder of V_loc from the tiled layout [kx][ky][kz] into plane layout, once per
+// structure factor: dst[(kz n + px) n + py] = src[(kx n + ky) nh + kz] with kx, ky
+// the frequencies at positions px, py (rev; nullptr: the positions themselves).
+// Only the entries with |m|^2 <= m2max are copied (the others are never read),
+// through 32 x 32 tiles of (py, kz), so both sides move whole rows.
+// grid: (ceil(n / 32), n).
 template <typename T>
-__global__ void k_vloc_planes(const cplx<T>* __restrict__ src, cplx<T>* __restrict__ dst,
-                              const int* __restrict__ rev, int n) {
-  const int nh = n / 2 + 1;
-  const size_t tot = (size_t)nh * n * n;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < tot; i += (size_t)gridDim.x * blockDim.x) {
-    const int py = (int)(i % n);
-    const int px = (int)((i / n) % n);
-    const int kz = (int)(i / ((size_t)n * n));
-    dst[i] = src[((size_t)rev[px] * n + rev[py]) * nh + kz];
+__global__ void __launch_bounds__(256) k_vloc_planes(const cplx<T>* __restrict__ src, cplx<T>* __restrict__ dst,
+                                                     const int* __restrict__ rev, int n, int m2max) {
+  __shared__ cplx<T> tile[32][33];
+  const int nh = n / 2 + 1, px = blockIdx.y, py0 = blockIdx.x * 32;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  auto sq = [&](int p) {
+    const int k = rev ? rev[p] : p, m = k <= (n - 1) / 2 ? k : k - n;
+    return m * m;
+  };
+  const int kx = rev ? rev[px] : px, mx2 = sq(px);
+  if (mx2 > m2max) return;
+  const int my2 = py0 + lane < n ? sq(py0 + lane) : m2max + 1;
+  for (int k0 = 0; k0 < nh && mx2 + k0 * k0 <= m2max; k0 += 32) {
+    for (int i = w; i < 32; i += 8) {
+      const int py = py0 + i, kz = k0 + lane;
+      if (py < n && kz < nh && mx2 + sq(py) + kz * kz <= m2max)
+        tile[i][lane] = src[((size_t)kx * n + (rev ? rev[py] : py)) * nh + kz];
+    }
+    __syncthreads();
+    for (int i = w; i < 32; i += 8) {
+      const int kz = k0 + i;
+      if (kz < nh && mx2 + my2 + kz * kz <= m2max) dst[((size_t)kz * n + px) * n + py0 + lane] = tile[lane][i];
+    }
+    __syncthreads();
   }
 }
 

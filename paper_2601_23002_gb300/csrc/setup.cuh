@@ -12,10 +12,11 @@ namespace ofdft {
 // ph[(I*3 + d)*n + k] holds them (k in FFT order), formed in FP64 and rounded to
 // the plan's type; one sine and cosine per |m|, the negative m by conjugation.
 template <typename T>
-__global__ void k_phases(const double* __restrict__ pos, int n_ion, int n, double L, cplx<T>* __restrict__ ph) {
+__device__ __forceinline__ void phases_part(const double* __restrict__ pos, int n_ion, int n, double L,
+                                            cplx<T>* __restrict__ ph, int block, int blocks) {
   const int h = n / 2 + 1;
   const int tot = n_ion * 3 * h;
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < tot; q += gridDim.x * blockDim.x) {
+  for (int q = block * blockDim.x + threadIdx.x; q < tot; q += blocks * blockDim.x) {
     const int m = q % h, d = (q / h) % 3, I = q / (3 * h);
     double f = pos[I * 3 + d] / L;
     f -= floor(f);                       // wrap into [0, 1)
@@ -54,6 +55,11 @@ template <typename T> struct StructOut {
   const double2* sf_tab;
   double m2rows;              // vloc and the Ewald sum: rows with a^2 + b^2 <= m2rows
   double* ew;
+  // when set, the last block writes res[0] = sum of ew, res[1] = sum of the
+  // nreal real-space partials
+  double* res;
+  const double* real; int nreal;
+  unsigned int* counter;
 };
 template <typename T> struct alignas(16) Quad { T a, b, c, d; };
 constexpr int kStructCH = 16;
@@ -176,6 +182,15 @@ __global__ void __launch_bounds__(NT) k_struct(const cplx<T>* __restrict__ ph, c
   double v[1] = {ew}, out[1];
   block_sum<1>(v, red, out);
   if (tid == 0) o.ew[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = out[0];
+  const int nb = gridDim.x * gridDim.y;
+  if (o.res && arrive_last(o.counter, nb)) {
+    double t2[2] = {0, 0}, t[2];
+    for (int i = tid; i < nb; i += NT) t2[0] += __ldcg(o.ew + i);
+    for (int i = tid; i < o.nreal; i += NT) t2[1] += o.real[i];
+    __shared__ double red2[64];
+    block_sum<2>(t2, red2, t);
+    if (tid == 0) { o.res[0] = t[0]; o.res[1] = t[1]; *o.counter = 0u; }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -189,13 +204,10 @@ __global__ void __launch_bounds__(NT) k_struct(const cplx<T>* __restrict__ ph, c
 // distances, 152 us for 300 ions in a 28-bohr cell.)  A block walks its share of
 // the (pair, image) combinations 256 at a time, compacts the ones inside rcut
 // into shared memory (warp ballots and a block prefix, in combination order) and
-// only then evaluates erfc, on dense warps.  The last block adds the reciprocal
-// partials ew[0..new_) of k_struct (res[0]) and its own kind (res[1]).  Fixed
-// order throughout.
-static __global__ void __launch_bounds__(256) k_ewald_real(const double* __restrict__ pos,
-                                                           const double* __restrict__ Z, int n_ion, double L,
-                                                           double eta, double rcut, int nimg, const double* ew, int new_,
-                                                           double* partial, unsigned int* counter, double* res) {
+// only then evaluates erfc, on dense warps (partial[block]; fixed order).
+static __device__ __forceinline__ void ewald_real_part(const double* __restrict__ pos, const double* __restrict__ Z,
+                                                       int n_ion, double L, double eta, double rcut, int nimg,
+                                                       double* __restrict__ partial, int block, int blocks) {
   __shared__ double red[32];
   __shared__ double sr[256], sz[256];
   __shared__ int wcount[8], wbase[8], total;
@@ -203,8 +215,8 @@ static __global__ void __launch_bounds__(256) k_ewald_real(const double* __restr
   const int nim3 = side * side * side;
   const int nd = n_ion / 2 + 1;
   const long tot = (long)n_ion * nd * nim3;
-  const long per = (tot + gridDim.x - 1) / gridDim.x;
-  const long q0 = (long)blockIdx.x * per, q1 = min(tot, q0 + per);
+  const long per = (tot + blocks - 1) / blocks;
+  const long q0 = (long)block * per, q1 = min(tot, q0 + per);
   const double rc2 = rcut * rcut;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   double acc = 0;
@@ -245,15 +257,18 @@ static __global__ void __launch_bounds__(256) k_ewald_real(const double* __restr
   }
   double v[1] = {acc}, out[1];
   block_sum<1>(v, red, out);
-  if (threadIdx.x == 0) partial[blockIdx.x] = out[0];
-  if (arrive_last(counter)) {
-    double s[2] = {0, 0}, t[2];
-    for (int i = threadIdx.x; i < new_; i += blockDim.x) s[0] += __ldcg(ew + i);
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) s[1] += __ldcg(partial + i);
-    __shared__ double red2[64];
-    block_sum<2>(s, red2, t);
-    if (threadIdx.x == 0) { res[0] = t[0]; res[1] = t[1]; *counter = 0u; }
-  }
+  if (threadIdx.x == 0) partial[block] = out[0];
+}
+
+// What depends on the positions alone, in one launch: blocks 0 .. ne - 1 the
+// Ewald real-space sum, the others the phases (independent chains of FP64
+// latency that overlap).
+template <typename T>
+__global__ void __launch_bounds__(256) k_ions(const double* __restrict__ pos, const double* __restrict__ Z, int n_ion,
+                                              int n, double L, cplx<T>* __restrict__ ph, double eta, double rcut,
+                                              int nimg, int ne, double* __restrict__ partial) {
+  if ((int)blockIdx.x < ne) ewald_real_part(pos, Z, n_ion, L, eta, rcut, nimg, partial, blockIdx.x, ne);
+  else phases_part<T>(pos, n_ion, n, L, ph, blockIdx.x - ne, gridDim.x - ne);
 }
 
 // ---------------------------------------------------------------------------
@@ -515,6 +530,79 @@ __global__ void k_forces_q(const cplx<T>* __restrict__ nt, const cplx<T>* __rest
   }
 }
 
+// Ewald real-space force on ion I = block / nsplit from the share
+// block % nsplit of its (J, image) terms, FP64, into part[block * 3
+// ..] (k_sum_force_parts adds the shares in a fixed order).  Images and
+// compaction of the in-range terms as in k_ewald_real.
+struct EwaldForceArgs {
+  const double *pos, *Z;
+  double L, eta, rcut;
+  int nimg, nsplit;
+  double* part;
+};
+static __device__ __forceinline__ void ewald_force_part(const EwaldForceArgs& w, int n_ion, int block) {
+  const double *pos = w.pos, *Z = w.Z;
+  const double L = w.L, eta = w.eta, rcut = w.rcut;
+  const int nimg = w.nimg, nsplit = w.nsplit;
+  double* part = w.part;
+  __shared__ double red[3 * 32];
+  __shared__ double sx[128], sy[128], sz[128], sq[128];
+  __shared__ int wcount[8], wbase[8], total;
+  const int I = block / nsplit, sh = block % nsplit;
+  const int side = 2 * nimg + 1;
+  const int nim3 = side * side * side;
+  const long tot = (long)n_ion * nim3;
+  const long per = (tot + nsplit - 1) / nsplit;
+  const long q0 = (long)sh * per, q1 = min(tot, q0 + per);
+  const double rc2 = rcut * rcut;
+  const double c2 = 2.0 * eta / 1.7724538509055160273;   // 2 eta / sqrt(pi)
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const double iL = 1.0 / L;
+  double f[3] = {0, 0, 0};
+  for (long base = q0; base < q1; base += blockDim.x) {
+    const long q = base + threadIdx.x;
+    bool inside = false;
+    double x = 0, y = 0, z = 0, r2 = 0;
+    if (q < q1) {
+      const int J = (int)(q / nim3), im = (int)(q % nim3);
+      const int a = im / (side * side) - nimg, b = (im / side) % side - nimg, c = im % side - nimg;
+      x = pos[I * 3] - pos[J * 3]; y = pos[I * 3 + 1] - pos[J * 3 + 1]; z = pos[I * 3 + 2] - pos[J * 3 + 2];
+      x -= L * rint(x * iL); y -= L * rint(y * iL); z -= L * rint(z * iL);
+      x += a * L; y += b * L; z += c * L;
+      r2 = x * x + y * y + z * z;
+      inside = r2 > 1e-24 && r2 < rc2;
+      if (inside) r2 = Z[I] * Z[J];     // reused below as the charge product
+    }
+    const unsigned bal = __ballot_sync(0xffffffffu, inside);
+    if (lane == 0) wcount[wid] = __popc(bal);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      int s = 0;
+      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { wbase[w] = s; s += wcount[w]; }
+      total = s;
+    }
+    __syncthreads();
+    if (inside) {
+      const int slot = wbase[wid] + __popc(bal & ((1u << lane) - 1u));
+      sx[slot] = x; sy[slot] = y; sz[slot] = z; sq[slot] = r2;
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < total) {
+      const double dx = sx[threadIdx.x], dy = sy[threadIdx.x], dz = sz[threadIdx.x];
+      const double rr = dx * dx + dy * dy + dz * dz, r = sqrt(rr);
+      const double s = sq[threadIdx.x] * (erfc(eta * r) / rr + c2 * exp(-eta * eta * rr) / r) / r;
+      f[0] += s * dx; f[1] += s * dy; f[2] += s * dz;
+    }
+    __syncthreads();
+  }
+  double o[3];
+  block_sum<3>(f, red, o);
+  if (threadIdx.x == 0) {
+    part[(size_t)block * 3 + 0] = o[0]; part[(size_t)block * 3 + 1] = o[1];
+    part[(size_t)block * 3 + 2] = o[2];
+  }
+}
+
 // Block: one tile of 32 row pairs (a lane each) and NW TI ions (TI per warp).
 // Along kz (from the tile's largest down) a lane sums U = sum qq e_z and
 // V = sum kz qq e_z for its four rows (V by adding the running U after every
@@ -523,15 +611,22 @@ __global__ void k_forces_q(const cplx<T>* __restrict__ nt, const cplx<T>* __rest
 // Im[P U] etc. times (a, b) and Im[P V], summed over the lanes.  (A gather of
 // three phases and two complex products per G and ion took 186 us for 128 ions
 // at 108^3.)  part[tile][ion][3], FP64, without the factor -Z_I 2 pi / L.
+// grid.x: ntile tiles times ny ion groups, then n_ion nsplit blocks of the
+// Ewald real-space part, which overlap with them.
 constexpr int kForceWarps = 4;
 template <typename T, int TI>
 __global__ void __launch_bounds__(32 * kForceWarps) k_forces_g(const Quad<T>* __restrict__ qq, const int2* __restrict__ rows,
                                                                int nrows, const int* __restrict__ tk,
                                                                const cplx<T>* __restrict__ ph, int n_ion, int n,
-                                                               double* __restrict__ part) {
+                                                               double* __restrict__ part, int ntile, int ny,
+                                                               EwaldForceArgs ewald) {
   constexpr int NI = kForceWarps * TI, KC = 32;
   __shared__ cplx<T> se[KC][NI];
-  const int tile = blockIdx.x, I0 = blockIdx.y * NI;
+  if ((int)blockIdx.x >= ntile * ny) {
+    ewald_force_part(ewald, n_ion, blockIdx.x - ntile * ny);
+    return;
+  }
+  const int tile = blockIdx.x % ntile, I0 = blockIdx.x / ntile * NI;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int k0 = tk[tile], nk = tk[tile + 1] - k0;
   cplx<T> U[TI][4], V[TI][4];
@@ -593,72 +688,6 @@ __global__ void __launch_bounds__(32 * kForceWarps) k_forces_g(const Quad<T>* __
       const double s = warp_sum(f[d]);
       if (lane == 0) part[((size_t)tile * n_ion + I) * 3 + d] = s;
     }
-  }
-}
-
-// Ewald real-space force on ion I = blockIdx.x / nsplit from the share
-// blockIdx.x % nsplit of its (J, image) terms, FP64, into part[blockIdx.x * 3
-// ..] (k_sum_force_parts adds the shares in a fixed order).  Images and
-// compaction of the in-range terms as in k_ewald_real.
-static __global__ void __launch_bounds__(256) k_ewald_force_real(const double* __restrict__ pos,
-                                                                 const double* __restrict__ Z, int n_ion, double L,
-                                                                 double eta, double rcut, int nimg, int nsplit,
-                                                                 double* __restrict__ part) {
-  __shared__ double red[3 * 32];
-  __shared__ double sx[256], sy[256], sz[256], sq[256];
-  __shared__ int wcount[8], wbase[8], total;
-  const int I = blockIdx.x / nsplit, sh = blockIdx.x % nsplit;
-  const int side = 2 * nimg + 1;
-  const int nim3 = side * side * side;
-  const long tot = (long)n_ion * nim3;
-  const long per = (tot + nsplit - 1) / nsplit;
-  const long q0 = (long)sh * per, q1 = min(tot, q0 + per);
-  const double rc2 = rcut * rcut;
-  const double c2 = 2.0 * eta / 1.7724538509055160273;   // 2 eta / sqrt(pi)
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const double iL = 1.0 / L;
-  double f[3] = {0, 0, 0};
-  for (long base = q0; base < q1; base += blockDim.x) {
-    const long q = base + threadIdx.x;
-    bool inside = false;
-    double x = 0, y = 0, z = 0, r2 = 0;
-    if (q < q1) {
-      const int J = (int)(q / nim3), im = (int)(q % nim3);
-      const int a = im / (side * side) - nimg, b = (im / side) % side - nimg, c = im % side - nimg;
-      x = pos[I * 3] - pos[J * 3]; y = pos[I * 3 + 1] - pos[J * 3 + 1]; z = pos[I * 3 + 2] - pos[J * 3 + 2];
-      x -= L * rint(x * iL); y -= L * rint(y * iL); z -= L * rint(z * iL);
-      x += a * L; y += b * L; z += c * L;
-      r2 = x * x + y * y + z * z;
-      inside = r2 > 1e-24 && r2 < rc2;
-      if (inside) r2 = Z[I] * Z[J];     // reused below as the charge product
-    }
-    const unsigned bal = __ballot_sync(0xffffffffu, inside);
-    if (lane == 0) wcount[wid] = __popc(bal);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int s = 0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { wbase[w] = s; s += wcount[w]; }
-      total = s;
-    }
-    __syncthreads();
-    if (inside) {
-      const int slot = wbase[wid] + __popc(bal & ((1u << lane) - 1u));
-      sx[slot] = x; sy[slot] = y; sz[slot] = z; sq[slot] = r2;
-    }
-    __syncthreads();
-    if ((int)threadIdx.x < total) {
-      const double dx = sx[threadIdx.x], dy = sy[threadIdx.x], dz = sz[threadIdx.x];
-      const double rr = dx * dx + dy * dy + dz * dz, r = sqrt(rr);
-      const double s = sq[threadIdx.x] * (erfc(eta * r) / rr + c2 * exp(-eta * eta * rr) / r) / r;
-      f[0] += s * dx; f[1] += s * dy; f[2] += s * dz;
-    }
-    __syncthreads();
-  }
-  double o[3];
-  block_sum<3>(f, red, o);
-  if (threadIdx.x == 0) {
-    part[(size_t)blockIdx.x * 3 + 0] = o[0]; part[(size_t)blockIdx.x * 3 + 1] = o[1];
-    part[(size_t)blockIdx.x * 3 + 2] = o[2];
   }
 }
 

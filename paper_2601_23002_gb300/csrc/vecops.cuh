@@ -172,6 +172,7 @@ k_gram(VecList<T> X, int nv, size_t N, double* __restrict__ partial, unsigned in
 struct TrialScale {
   double q, t, ne, dv, nbar;
   double* out;       // out[0] = scale, out[1] = sqrt(nbar / scale), out[2] = t
+  double* hout;      // the same three for the host (pinned memory)
   // when set: q = *qdev, and t = 1 if *kkdev > 0 (a quasi-Newton step), else
   // the first step 0.1 sqrt(q / <d,d>) (10% of |psi| along -P g)
   const double* qdev;
@@ -298,12 +299,12 @@ static __global__ void __launch_bounds__(32) k_twoloop(TwoLoopArgs a, const doub
 }
 
 // out = sum_{i < nv} c_i X_i, with X_nv = A and X_{nv+1} = B; the last block
-// writes res[0..2] = <out,out>, <out,A>, <out,B> (raw sums, without dV) and,
-// with B = psi, the trial scale of ts
+// writes res[0..2] = <out,out>, <out,A>, <out,B> (raw sums, without dV; hres:
+// the same in pinned host memory) and, with B = psi, the trial scale of ts
 template <typename T>
 __global__ void __launch_bounds__(kStreamThreads, 1)
 k_lincomb(VecList<T> X, int nv, T* __restrict__ out, size_t N, double* __restrict__ partial,
-          unsigned int* __restrict__ counter, double* __restrict__ res, TrialScale ts,
+          unsigned int* __restrict__ counter, double* __restrict__ res, double* __restrict__ hres, TrialScale ts,
           const double* __restrict__ dcoef) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ double red[32];
@@ -341,6 +342,7 @@ k_lincomb(VecList<T> X, int nv, T* __restrict__ out, size_t N, double* __restric
   if (arrive_last(counter)) {
     block_sum_columns(partial, gridDim.x, 3, res, red);
     if (threadIdx.x == 0) *counter = 0u;
+    if (threadIdx.x < 3) hres[threadIdx.x] = res[threadIdx.x];
     if (ts.out) {
       __syncthreads();                   // res[] written by this block's threads
       if (threadIdx.x == 0) {
@@ -352,6 +354,7 @@ k_lincomb(VecList<T> X, int nv, T* __restrict__ out, size_t N, double* __restric
         ts.out[0] = sc;
         ts.out[1] = sqrt(ts.nbar / sc);
         ts.out[2] = t;
+        ts.hout[0] = sc; ts.hout[1] = ts.out[1]; ts.hout[2] = t;
       }
     }
   }
@@ -362,13 +365,14 @@ k_lincomb(VecList<T> X, int nv, T* __restrict__ out, size_t N, double* __restric
 //   s = psi_t - psi (= t d); y = g_t - g; psi <- psi_t; g <- g_t;
 // and, on the way, the dot products of the new pair with itself, the new
 // gradient and the new psi; the last block writes res[0..5] =
-//   <s,y>, <y,y>, <psi,psi>, <g,g>, <s,g>, <y,g>   (new psi, new g).
+//   <s,y>, <y,y>, <psi,psi>, <g,g>, <s,g>, <y,g>   (new psi, new g)
+// (hres: the same in pinned host memory).
 // A thread rewrites psi and g only at the groups it has already copied in.
 template <typename T>
 __global__ void __launch_bounds__(kStreamThreads, 1)
 k_accept(VecList<T> X, T tt, T a, T m, T* __restrict__ psi, T* __restrict__ g, T* __restrict__ s,
          T* __restrict__ y, size_t N, double* __restrict__ partial, unsigned int* __restrict__ counter,
-         double* __restrict__ res) {
+         double* __restrict__ res, double* __restrict__ hres) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ double red[32];
   // tt = step, a = 2 scale_t, m = mu_t - mu_ref (converted on the host)
@@ -398,6 +402,7 @@ k_accept(VecList<T> X, T tt, T a, T m, T* __restrict__ psi, T* __restrict__ g, T
   block_sum_tree<6, T>(acc, 6, partial + (size_t)blockIdx.x * 6, reinterpret_cast<typename TreeVal<T>::type*>(smem));
   if (arrive_last(counter)) {
     block_sum_columns(partial, gridDim.x, 6, res, red);
+    if (threadIdx.x < 6) hres[threadIdx.x] = res[threadIdx.x];
     if (threadIdx.x == 0) *counter = 0u;
   }
 }

@@ -679,18 +679,4 @@ k_plane256cl(Spectra<T> sp, GArgs<T> g, const cplx<T>* __restrict__ tw_n) {
   block_sum_tree_raw<4, T>(acc, g.partials + bi * 4, reinterpret_cast<typename TreeVal<T>::type*>(smem_raw));
 }
 
-// One-time reorder of V_loc from the tiled layout [kx][ky][kz] into plane
-// layout, natural order: dst[(kz 256 + kx) 256 + ky] = src[(kx 256 + ky) 129 + kz].
-template <typename T>
-__global__ void k_vloc_planes256(const cplx<T>* __restrict__ src, cplx<T>* __restrict__ dst) {
-  constexpr int N = 256, NH = 129;
-  const size_t tot = (size_t)NH * N * N;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < tot; i += (size_t)gridDim.x * blockDim.x) {
-    const int ky = (int)(i % N);
-    const int kx = (int)((i / N) % N);
-    const int kz = (int)(i / ((size_t)N * N));
-    dst[i] = src[((size_t)kx * N + ky) * NH + kz];
-  }
-}
-
 }  // namespace ofdft
