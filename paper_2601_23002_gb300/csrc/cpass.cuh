@@ -351,7 +351,7 @@ k_zfwd_c(ProArgs<T> a, Spectra<T> sp, const cplx<T>* __restrict__ tw_l, const cp
   for (int q = threadIdx.x; q < sp.nact * NH * R; q += Z::NT) {
     const int fk = q / R, r = q - fk * R;
     const int f = fk / NH, k = fk - f * NH;
-    if (r >= rows) continue;
+    if (r >= rows || k >= a.nkz) continue;
     C o;
     if constexpr (Z::ODD) {
       // X_a[k] = (Z[k] + Z*[n-k]) / 2, X_b[k] = -i (Z[k] - Z*[n-k]) / 2
@@ -659,6 +659,13 @@ k_plane_c(Spectra<T> sp, GArgs<T> g, const cplx<T>* __restrict__ tw_g) {
 #pragma unroll
     for (int r = 0; r < RL; ++r) v[r] = x[r * Q::CPT];
     Codelet<C, RL, -1>::run(v);
+    if (g.forward) {
+      // (every block of the cluster has read its rows: they can be overwritten)
+      C* y = CField<T>::pick(sp, fid) + (size_t)kz * NN + b * RL * N + row0 + col;
+#pragma unroll
+      for (int r = 0; r < RL; ++r) y[r * N] = v[r];
+      continue;
+    }
     const int py = row0 + col, my = sgn(freq(py));
     const int mk2 = my * my + kz * kz;
     const int kx0 = freq(b * RL);
@@ -705,6 +712,10 @@ k_plane_c(Spectra<T> sp, GArgs<T> g, const cplx<T>* __restrict__ tw_g) {
     Codelet<C, RL, +1>::run(v);
 #pragma unroll
     for (int r = 0; r < RL; ++r) x[r * Q::CPT] = v[r];
+  }
+  if (g.forward) {
+    if constexpr (CL > 1) cg::this_cluster().sync();     // other blocks may still read this one's rows
+    return;
   }
   __syncthreads();
   // inverse along kx

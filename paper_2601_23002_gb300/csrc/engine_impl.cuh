@@ -126,6 +126,7 @@ class Engine : public IEngine {
     return true;
   }
   T* cou = nullptr;          // 4 pi / G^2 by m^2
+  int* pos_of = nullptr;     // frequency -> position (compile-time plane pass)
   int* rev_d = nullptr;      // position -> frequency of the in-place transforms
   PlaneKernel<T> plane_kern = nullptr;   // k_plane compiled for this grid's radices
   // one-field preconditioning pass on two-block clusters (half a plane per
@@ -176,8 +177,10 @@ class Engine : public IEngine {
   Quad<T>* f_qq = nullptr;
   double *f_part = nullptr, *f_out = nullptr;
   int f_nrows = -1, f_ntile = 0, f_nk = 0, f_m2 = 0;
-  // pressure: pnl(m^2) = (3 - 6a) K + dK/dlambda (FP64, built on the first call)
+  // pressure: kernel tables on dilated cells and pnl(m^2) = (3 - 6a) K +
+  // dK/dlambda, built on the first call
   double* p_tab = nullptr;
+  T* p_pnl = nullptr;
   bool p_ready = false;
   // |q| shells of the structure factors: CSR lists of half-spectrum entries
   // with Hermitian weights, kept for the last n_shells asked for
@@ -185,13 +188,15 @@ class Engine : public IEngine {
   long long sh_entries = 0;
   std::vector<int> sh_m2;
   int* sh_ptr = nullptr;
-  long long* sh_idx = nullptr;
+  int* sh_idx = nullptr;
   float* sh_w = nullptr;
-  double* sh_out = nullptr;
+  double* sh_out = nullptr;   // pinned
+  int sh_kz = 0;              // largest kz of the lists
   size_t sh_bytes[4] = {0, 0, 0, 0};
   void free_shells() {
-    void* p[4] = {sh_ptr, sh_idx, sh_w, sh_out};
-    for (int i = 0; i < 4; ++i) cached_dev_release(p[i], sh_bytes[i]);
+    void* p[3] = {sh_ptr, sh_idx, sh_w};
+    for (int i = 0; i < 3; ++i) cached_dev_release(p[i], sh_bytes[i]);
+    if (sh_out) cached_host_release(sh_out, sh_bytes[3]);
     sh_ptr = nullptr; sh_idx = nullptr; sh_w = nullptr; sh_out = nullptr; sh_ns = 0;
   }
   size_t n_vloc = 0;         // half-spectrum entries with |G|^2 <= g2cut_loc
@@ -377,10 +382,10 @@ class Engine : public IEngine {
 
   bool p256_possible() const { return z256_allowed && p256_allowed && sizeof(T) == 4 && n == 256 && !planes; }
 
-  // the cluster plane pass over nf fields
-  int launch_p256(const Spectra<T>& sp, const GArgs<T>& ga, int nf, double bytes, cudaStream_t st) {
+  // the cluster plane pass over the first nkz planes of nf fields
+  int launch_p256(const Spectra<T>& sp, const GArgs<T>& ga, int nf, double bytes, cudaStream_t st, int nkz = 129) {
     if constexpr (sizeof(T) == 4) {
-      OFDFT_RUN("k_plane256cl", st, bytes, k_plane256cl<T><<<dim3(P256::CL * nh, nf), P256::THREADS, p256_bytes<T>(), st>>>(sp, ga, tw_n));
+      OFDFT_RUN("k_plane256cl", st, bytes, k_plane256cl<T><<<dim3(P256::CL * nkz, nf), P256::THREADS, p256_bytes<T>(), st>>>(sp, ga, tw_n));
       return OFDFT_OK;
     } else {
       set_error("the cluster plane pass is FP32 only");
@@ -501,6 +506,13 @@ class Engine : public IEngine {
       if ((rc = alloc(&rev_d, n))) return rc;
       OFDFT_CK(cudaMemcpyAsync(rev_d, rev.data(), n * sizeof(int), cudaMemcpyHostToDevice, st));
       if (planes && (rc = alloc(&vloc_pl, NH))) return rc;
+      if (cp) {
+        std::vector<int> inv(n);
+        for (int q = 0; q < n; ++q) inv[rev[q]] = q;
+        if ((rc = alloc(&pos_of, n))) return rc;
+        OFDFT_CK(cudaMemcpyAsync(pos_of, inv.data(), n * sizeof(int), cudaMemcpyHostToDevice, st));
+        OFDFT_CK(cudaStreamSynchronize(st));
+      }
     }
     if (p256_possible() && (rc = alloc(&vloc_pl, NH))) return rc;
     {
@@ -532,7 +544,7 @@ class Engine : public IEngine {
     if ((rc = alloc(&Kd, nm2))) return rc;
     if ((rc = alloc(&Kt, nm2))) return rc;
     std::vector<T> couh;
-    if (cp) {
+    {
       const double tp = 2.0 * kPi / L;
       const T tp2 = (T)(tp * tp);
       couh.resize(nm2);
@@ -831,13 +843,6 @@ class Engine : public IEngine {
     return OFDFT_OK;
   }
 
-  // Sum columns of partials[rows][cols] into res_h[off ...] (fixed order).
-  int sum_partials(int rows, int cols, int off, cudaStream_t st) {
-    if (cols > 256) { set_error("sum_partials: too many columns"); return OFDFT_ERR_INVALID; }
-    OFDFT_RUN("k_sum_columns", st, (double)rows * cols * 8, k_sum_columns<<<1, 256, 0, st>>>(partials, rows, cols, res_h + off));
-    return OFDFT_OK;
-  }
-
   // k_struct with the largest thread tile that still gives every SM two blocks
   // (a block waits for its staged ions at two barriers per chunk; the other one
   // works meanwhile): FP32 2 x 4 (64 accumulators), 2 x 2, 1 x 2; small grids 1 x 1.
@@ -973,6 +978,39 @@ class Engine : public IEngine {
     if (sync) {
       OFDFT_CK(cudaStreamSynchronize(st));
       finish_eval(mode, scale, Q, psid, mu_ref, sp.merged != 0);
+    }
+    return OFDFT_OK;
+  }
+
+  // Unnormalised forward transforms of a density's fields fld[0..nf) (0 n, 1 n^a,
+  // 2 sqrt n less its mean) into spec[], for the analysis kernels, with every kz
+  // <= kzmax (where the plane passes allow it no other).
+  int forward(const T* rho, const int* fld, int nf, int kzmax, SpecView& view, cudaStream_t st) {
+    Spectra<T> sp{};
+    sp.nact = nf;
+    for (int i = 0; i < nf; ++i) { sp.idx[i] = fld[i]; sp.s[fld[i]] = spec[fld[i]]; }
+    // (the 256^3 pass reads two reals at a time)
+    const bool pl256 = p256 && reinterpret_cast<uintptr_t>(rho) % sizeof(C) == 0;
+    sp.planes = (cp || pl256) ? 1 : 0;
+    ProArgs<T> pa{0, rho, nullptr, nullptr, (T)0, (T)1, (T)cs.alpha, (T)std::sqrt(nbar), nullptr, kzmax + 1};
+    const int nk = std::min(nh, kzmax + 1);
+    const double zb = (double)N * sizeof(T) + (double)nf * n * n * nk * sizeof(C);
+    const double yb = 2.0 * nf * n * n * nk * sizeof(C);
+    view = SpecView{sp.planes, n, nullptr, nullptr};
+    GArgs<T> ga{};
+    ga.forward = 1;
+    if (cp) {
+      view.pos = pos_of; view.rev = rev_d;
+      if (int rc = launch_zfwd(pa, sp, zb, st)) return rc;
+      const auto& pl = cp->pl[nf > 1];
+      OFDFT_RUN("k_plane_c", st, yb, pl.kern<<<dim3(pl.cl * nk, nf), pl.threads, pl.bytes, st>>>(sp, ga, tw_n));
+    } else if (pl256) {
+      if (int rc = launch_zfwd(pa, sp, zb, st)) return rc;
+      if (int rc = launch_p256(sp, ga, nf, yb, st, nk)) return rc;
+    } else {
+      OFDFT_RUN("k_zfwd", st, (double)N * sizeof(T) + (double)nf * NH * sizeof(C), k_zfwd<T><<<grid_z, kThreads, smem_zf, st>>>(pa, sp, ph, tw_h, tw_n, n, zR, zP));
+      OFDFT_RUN("k_ypass", st, 2.0 * nf * NH * sizeof(C), k_ypass<T, -1><<<dim3(grid_y1, nf), kThreads, smem_y, st>>>(sp, pn, tw_n, n, yJ));
+      OFDFT_RUN("k_xpass", st, 2.0 * nf * NH * sizeof(C), k_xpass<T, -1><<<dim3(grid_x, nf), kThreads, smem_xp, st>>>(sp, pn, tw_n, n, xJ));
     }
     return OFDFT_OK;
   }
@@ -1440,7 +1478,7 @@ int Engine<T>::build_shells(int n_shells, cudaStream_t st) {
   }
   std::vector<int> shell_of(m2max + 1, -1);
   for (int i = 0; i < ns; ++i) shell_of[shell_m2[i]] = i;
-  std::vector<std::vector<long long>> lists(ns);
+  std::vector<std::vector<int>> lists(ns);
   std::vector<std::vector<float>> wl(ns);
   const int r = (int)std::ceil(std::sqrt((double)m2max));
   for (int mx = -std::min(r, lim); mx <= std::min(r, mhi); ++mx)
@@ -1449,12 +1487,11 @@ int Engine<T>::build_shells(int n_shells, cudaStream_t st) {
         const int m2 = mx * mx + my * my + mz * mz;
         if (m2 == 0 || m2 > m2max || shell_of[m2] < 0) continue;
         const int kx = mx < 0 ? mx + n : mx, ky = my < 0 ? my + n : my;
-        const long long q = ((long long)kx * n + ky) * nh + mz;
-        lists[shell_of[m2]].push_back(q);
+        lists[shell_of[m2]].push_back(kx | ky << 10 | mz << 20);
         wl[shell_of[m2]].push_back((mz == 0 || 2 * mz == n) ? 1.0f : 2.0f);
       }
   std::vector<int> ptr(ns + 1, 0);
-  std::vector<long long> idx;
+  std::vector<int> idx;
   std::vector<float> wts;
   for (int i = 0; i < ns; ++i) {
     ptr[i + 1] = ptr[i] + (int)lists[i].size();
@@ -1464,18 +1501,19 @@ int Engine<T>::build_shells(int n_shells, cudaStream_t st) {
   OFDFT_CK(cudaStreamSynchronize(st));
   free_shells();
   sh_bytes[0] = ptr.size() * sizeof(int);
-  sh_bytes[1] = std::max<size_t>(1, idx.size()) * sizeof(long long);
+  sh_bytes[1] = std::max<size_t>(1, idx.size()) * sizeof(int);
   sh_bytes[2] = std::max<size_t>(1, wts.size()) * sizeof(float);
   sh_bytes[3] = 3 * (size_t)ns * sizeof(double);
   OFDFT_CK(cached_dev_alloc((void**)&sh_ptr, sh_bytes[0]));
   OFDFT_CK(cached_dev_alloc((void**)&sh_idx, sh_bytes[1]));
   OFDFT_CK(cached_dev_alloc((void**)&sh_w, sh_bytes[2]));
-  OFDFT_CK(cached_dev_alloc((void**)&sh_out, sh_bytes[3]));
+  OFDFT_CK(cached_host_alloc((void**)&sh_out, sh_bytes[3]));
   OFDFT_CK(cudaMemcpyAsync(sh_ptr, ptr.data(), ptr.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-  OFDFT_CK(cudaMemcpyAsync(sh_idx, idx.data(), idx.size() * sizeof(long long), cudaMemcpyHostToDevice, st));
+  OFDFT_CK(cudaMemcpyAsync(sh_idx, idx.data(), idx.size() * sizeof(int), cudaMemcpyHostToDevice, st));
   OFDFT_CK(cudaMemcpyAsync(sh_w, wts.data(), wts.size() * sizeof(float), cudaMemcpyHostToDevice, st));
   OFDFT_CK(cudaStreamSynchronize(st));
   sh_m2 = shell_m2;
+  sh_kz = std::min(lim, (int)std::sqrt((double)m2max));
   sh_ns = ns;
   sh_entries = (long long)idx.size();
   return OFDFT_OK;
@@ -1485,19 +1523,14 @@ int Engine<T>::build_shells(int n_shells, cudaStream_t st) {
 // (sum w Re[n_e S*] / sqrt(N_e N_i), sum w |S|^2, sum w).
 template <typename T>
 int Engine<T>::shell_sums(const void* rho, cudaStream_t st, std::vector<double>& hout) {
-  // forward transform of rho into spec[0]
-  Spectra<T> sp{};
-  sp.s[0] = spec[0]; sp.nact = 1; sp.idx[0] = 0;
-  ProArgs<T> pa{0, (const T*)rho, nullptr, nullptr, (T)0, (T)1, (T)cs.alpha};
-  OFDFT_RUN("k_zfwd", st, (double)N * sizeof(T) + (double)NH * sizeof(C), k_zfwd<T><<<grid_z, kThreads, smem_zf, st>>>(pa, sp, ph, tw_h, tw_n, n, zR, zP));
-  OFDFT_RUN("k_ypass", st, 2.0 * NH * sizeof(C), k_ypass<T, -1><<<dim3(grid_y1, 1), kThreads, smem_y, st>>>(sp, pn, tw_n, n, yJ));
-  OFDFT_RUN("k_xpass", st, 2.0 * NH * sizeof(C), k_xpass<T, -1><<<dim3(grid_x, 1), kThreads, smem_xp, st>>>(sp, pn, tw_n, n, xJ));
+  SpecView view;
+  const int fld[1] = {0};
+  if (int rc = forward((const T*)rho, fld, 1, sh_kz, view, st)) return rc;
   const double nion = (double)cs.Z.size();
   const double scale = Omega / (double)N / std::sqrt(Ne * nion);
-  OFDFT_RUN("k_sei_shells", st, (double)sh_entries * (2 * sizeof(C) + 12), k_sei_shells<T><<<sh_ns, 256, 0, st>>>(spec[0], Sg, sh_ptr, sh_idx, sh_w, scale, sh_out));
-  hout.resize(3 * (size_t)sh_ns);
-  OFDFT_CK(cudaMemcpyAsync(hout.data(), sh_out, hout.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
+  OFDFT_RUN("k_sei_shells", st, (double)sh_entries * (2 * sizeof(C) + 8), k_sei_shells<T><<<sh_ns, 256, 0, st>>>(spec[0], view, Sg, sh_ptr, sh_idx, sh_w, scale, sh_out));
   OFDFT_CK(cudaStreamSynchronize(st));
+  hout.assign(sh_out, sh_out + 3 * (size_t)sh_ns);
   return OFDFT_OK;
 }
 
@@ -1559,14 +1592,11 @@ int Engine<T>::forces(const void* rho, double* f_out_h, void* stream_) {
     OFDFT_CK(cudaStreamSynchronize(st));
     f_nrows = (int)rows.size();
   }
-  // n~ (unnormalised) into spec[0], tiled layout
-  Spectra<T> sp{};
-  sp.s[0] = spec[0]; sp.nact = 1; sp.idx[0] = 0;
-  ProArgs<T> pa{0, (const T*)rho, nullptr, nullptr, (T)0, (T)1, (T)cs.alpha};
-  OFDFT_RUN("k_zfwd", st, (double)N * sizeof(T) + (double)NH * sizeof(C), k_zfwd<T><<<grid_z, kThreads, smem_zf, st>>>(pa, sp, ph, tw_h, tw_n, n, zR, zP));
-  OFDFT_RUN("k_ypass", st, 2.0 * NH * sizeof(C), k_ypass<T, -1><<<dim3(grid_y1, 1), kThreads, smem_y, st>>>(sp, pn, tw_n, n, yJ));
-  OFDFT_RUN("k_xpass", st, 2.0 * NH * sizeof(C), k_xpass<T, -1><<<dim3(grid_x, 1), kThreads, smem_xp, st>>>(sp, pn, tw_n, n, xJ));
-  OFDFT_RUN("k_forces_q", st, (double)f_nk * 32 * (8 * sizeof(C) + 4 * sizeof(C)), k_forces_q<T><<<std::min(16 * nsm, (f_nk + 3) / 4), 128, 0, st>>>(spec[0], SZg, f_rows, f_nrows, f_tk, f_ntile, f_gf, f_m2, n, 1.0 / (double)N, f_qq));
+  // n~ (unnormalised) into spec[0]
+  SpecView view;
+  const int fld[1] = {0};
+  if ((rc = forward((const T*)rho, fld, 1, std::min(h, (int)std::sqrt((double)f_m2)), view, st))) return rc;
+  OFDFT_RUN("k_forces_q", st, (double)f_nk * 32 * (8 * sizeof(C) + 4 * sizeof(C)), k_forces_q<T><<<std::min(16 * nsm, (f_nk + 3) / 4), 128, 0, st>>>(spec[0], view, SZg, f_rows, f_nrows, f_tk, f_ntile, f_gf, f_m2, n, 1.0 / (double)N, f_qq));
   // several blocks per ion (about 4 per SM in all), shares added in a fixed order
   int nsplit = std::max(1, std::min(64, (4 * nsm + nion - 1) / nion));
   while (nsplit > 1 && (size_t)nion * nsplit * 3 > partials_cap) --nsplit;
@@ -1589,9 +1619,9 @@ template <typename T>
 int Engine<T>::build_pressure_table(cudaStream_t st) {
   const int nm2 = 3 * h * h + 1;
   int rc;
-  if (!p_tab && (rc = alloc(&p_tab, (size_t)5 * nm2 + 16))) return rc;
+  if (!p_tab && ((rc = alloc(&p_tab, (size_t)4 * nm2 + 16)) || (rc = alloc(&p_pnl, nm2)))) return rc;
   const double lam[4] = {1.002, 0.998, 1.001, 0.999};
-  double* mp = p_tab + (size_t)5 * nm2;
+  double* mp = p_tab + (size_t)4 * nm2;
   for (int i = 0; i < 4; ++i) {
     const double nb = nbar / (lam[i] * lam[i] * lam[i]);
     const double y = 9.8696044010893586188 * nb / (1.4142135623730950488 * std::pow(Te, 1.5));
@@ -1613,7 +1643,8 @@ int Engine<T>::build_pressure_table(cudaStream_t st) {
     const double c2 = (tabs[(size_t)2 * nm2 + m] - tabs[(size_t)3 * nm2 + m]) / (2.0 * 1e-3);
     pnl[m] = (3.0 - 6.0 * cs.alpha) * K0[m] + (4.0 * c2 - c1) / 3.0;
   }
-  OFDFT_CK(cudaMemcpyAsync(p_tab + (size_t)4 * nm2, pnl.data(), nm2 * sizeof(double), cudaMemcpyHostToDevice, st));
+  const std::vector<T> pt(pnl.begin(), pnl.end());
+  OFDFT_CK(cudaMemcpyAsync(p_pnl, pt.data(), nm2 * sizeof(T), cudaMemcpyHostToDevice, st));
   OFDFT_CK(cudaStreamSynchronize(st));
   p_ready = true;
   return OFDFT_OK;
@@ -1627,36 +1658,38 @@ int Engine<T>::pressure(const void* rho, double* p_out_h, void* stream_) {
   if (!ions_set) { set_error("ofdft_structure_factor must be called before ofdft_pressure"); return OFDFT_ERR_INVALID; }
   cudaStream_t st = (cudaStream_t)stream_;
   int rc;
-  // energies of the degree -2 / -1 terms from one evaluation
-  if ((rc = eval(0, (const T*)rho, nullptr, nullptr, 0.0, 1.0, 0.0, 0.0, nullptr, st, true))) return rc;
-  const double E_vW = res_h[1], E_H = res_h[3], Eion = res_h[6];
-  const bool nl = use_na();
+  const bool nl = use_na(), vw = use_psi();
   if (nl && !p_ready && (rc = build_pressure_table(st))) return rc;
-  // n~ into spec[0], (n^a)~ into spec[1], tiled layout
-  Spectra<T> sp{};
-  sp.s[0] = spec[0]; sp.s[1] = spec[1]; sp.nact = 2; sp.idx[0] = 0; sp.idx[1] = 1;
-  ProArgs<T> pa{0, (const T*)rho, nullptr, nullptr, (T)0, (T)1, (T)cs.alpha};
-  OFDFT_RUN("k_zfwd", st, (double)N * sizeof(T) + 2.0 * NH * sizeof(C), k_zfwd<T><<<grid_z, kThreads, smem_zf, st>>>(pa, sp, ph, tw_h, tw_n, n, zR, zP));
-  OFDFT_RUN("k_ypass", st, 4.0 * NH * sizeof(C), k_ypass<T, -1><<<dim3(grid_y1, 2), kThreads, smem_y, st>>>(sp, pn, tw_n, n, yJ));
-  OFDFT_RUN("k_xpass", st, 4.0 * NH * sizeof(C), k_xpass<T, -1><<<dim3(grid_x, 2), kThreads, smem_xp, st>>>(sp, pn, tw_n, n, xJ));
+  // n~, (n^a)~ and (sqrt n)~ as needed; a = 1/2: one transform for the last two
+  // (its mean is left out, and both terms' factors vanish at G = 0)
+  const bool half = cs.alpha == 0.5;
+  int fld[3], nf = 0;
+  if (use_n()) fld[nf++] = 0;
+  if (nl && !half) fld[nf++] = 1;
+  if (vw || (nl && half)) fld[nf++] = 2;
+  SpecView view{};
+  if (nf && (rc = forward((const T*)rho, fld, nf, h, view, st))) return rc;
   const int gb = 4 * nsm;
   const double cy = 9.8696044010893586188344909998762 / (1.4142135623730950488016887242097 * std::pow(Te, 1.5));
-  OFDFT_RUN("k_pressure_r", st, (double)N * sizeof(T), k_pressure_r<T><<<gb, 256, 0, st>>>((const T*)rho, N, (T)cy, (T)Te, cs.terms, partials, cs.fd64 ? 1 : 0, cy));
-  if ((rc = sum_partials(gb, 2, 0, st))) return rc;
-  const double tp = 2.0 * kPi / L;
-  const C* vl = (cs.terms & OFDFT_TERM_LOC) ? vloc : nullptr;
-  const double* pn_d = nl ? p_tab + (size_t)4 * (3 * h * h + 1) : nullptr;
-  OFDFT_RUN("k_pressure_g", st, 3.0 * NH * sizeof(C), k_pressure_g<T><<<gb, 256, 0, st>>>(spec[0], spec[1], vl, pn_d, n, tp * tp, g2cut_loc, cs.rc * cs.rc, 1.0 / (double)N, partials));
-  if ((rc = sum_partials(gb, 2, 2, st))) return rc;
+  OFDFT_RUN("k_pressure_r", st, (double)N * sizeof(T), k_pressure_r<T><<<gb, 256, 0, st>>>((const T*)rho, N, (T)cy, (T)Te, cs.terms, partials, cs.fd64 ? 1 : 0, cy, counters + 5, res_h));
+  if (nf) {
+    const double tp = 2.0 * kPi / L;
+    const C* vl = (cs.terms & OFDFT_TERM_LOC) ? (view.planes ? vloc_pl : vloc) : nullptr;
+    OFDFT_RUN("k_pressure_g", st, (double)(nf + (vl != nullptr)) * NH * sizeof(C), k_pressure_g<T><<<gb, 256, 0, st>>>(use_n() ? spec[0] : nullptr, nl ? (half ? spec[2] : spec[1]) : nullptr, vw ? spec[2] : nullptr, view, vl, cou, p_pnl, (T)(tp * tp), (T)g2cut_loc, (T)(cs.rc * cs.rc), (T)(1.0 / (double)N), partials, counters + 5, res_h + 2));
+  } else {
+    std::memset(res_h + 2, 0, 4 * sizeof(double));
+  }
   OFDFT_CK(cudaStreamSynchronize(st));
   double* P = p_out_h;
+  const double E_vW = 0.5 * Omega * res_h[5];
+  const double E_H = (cs.terms & OFDFT_TERM_HARTREE) ? 0.5 * Omega * res_h[4] : 0.0;
   P[0] = res_h[0] / (double)N;              // (1/Omega) dV sum n T p
   P[1] = 2.0 * E_vW / (3.0 * Omega);
   P[2] = -res_h[3] / 3.0;
   P[3] = E_H / (3.0 * Omega);
   P[4] = res_h[2] / 3.0;
   P[5] = res_h[1] / (double)N;
-  P[6] = Eion / (3.0 * Omega);
+  P[6] = E_ion / (3.0 * Omega);
   P[7] = P[0] + P[1] + P[2] + P[3] + P[4] + P[5] + P[6];
   return OFDFT_OK;
 }

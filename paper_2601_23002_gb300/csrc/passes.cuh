@@ -215,6 +215,22 @@ template <typename T> struct ProArgs {
   // when set, scale = dsc[0], psi_shift = dsc[1] and t = dsc[2] (a trial
   // formed on the device, see TrialScale)
   const double* dsc;
+  // kz planes to store (analysis transforms that read low |m| only; plane
+  // layout, compile-time and 256^3 passes)
+  int nkz = 1 << 30;
+};
+
+// A forward transform as the analysis kernels read it: entry (kx, ky, kz) of the
+// tiled layout [kx][ky][kz], or of the plane layout [kz][px][py] at the positions
+// px = pos[kx], py = pos[ky] (pos == nullptr: kx, ky themselves).
+struct SpecView {
+  int planes, n;
+  const int* pos;         // frequency -> position
+  const int* rev;         // position -> frequency
+  __device__ __forceinline__ size_t at(int kx, int ky, int kz) const {
+    if (!planes) return ((size_t)kx * n + ky) * (n / 2 + 1) + kz;
+    return ((size_t)kz * n + (pos ? pos[kx] : kx)) * n + (pos ? pos[ky] : ky);
+  }
 };
 
 // Rows of one z-pass FFT buffer: even n transforms each real row as a
@@ -421,6 +437,7 @@ template <typename T> struct GArgs {
   // spectrum is multiplied by this table of p(m^2) instead (see minimize)
   const T* prec;
   const T* cou;          // 4 pi / G^2 by m^2 (the compile-time plane pass)
+  int forward = 0;       // 1: stop after the forward transform, stored at its positions
 };
 
 // One block per (tile, field): blockIdx.y indexes the active fields.

@@ -441,20 +441,20 @@ static __global__ void __launch_bounds__(kMeanThreads) k_mean_density(double y, 
 
 // ---------------------------------------------------------------------------
 // Structure-factor shells: block s sums over the half-spectrum entries of
-// shell s (CSR lists built on the host; w = Hermitian weight), FP64, fixed
-// order.  out[3 s] = sum w Re[n~ S*] scale, out[3 s + 1] = sum w |S|^2,
-// out[3 s + 2] = sum w.
+// shell s (CSR lists built on the host; entry kx | ky << 10 | kz << 20, w =
+// Hermitian weight), FP64, fixed order.  out[3 s] = sum w Re[n~ S*] scale,
+// out[3 s + 1] = sum w |S|^2, out[3 s + 2] = sum w (pinned host memory).
 template <typename T>
-__global__ void __launch_bounds__(256) k_sei_shells(const cplx<T>* __restrict__ nt, const cplx<T>* __restrict__ S,
-                                                    const int* __restrict__ ptr, const long long* __restrict__ idx,
-                                                    const float* __restrict__ wgt, double scale,
-                                                    double* __restrict__ out) {
+__global__ void __launch_bounds__(256) k_sei_shells(const cplx<T>* __restrict__ nt, SpecView view,
+                                                    const cplx<T>* __restrict__ S, const int* __restrict__ ptr,
+                                                    const int* __restrict__ idx, const float* __restrict__ wgt,
+                                                    double scale, double* __restrict__ out) {
   __shared__ double red[3 * 32];
-  const int s = blockIdx.x;
+  const int s = blockIdx.x, n = view.n, nh = n / 2 + 1;
   double acc[3] = {0, 0, 0};
   for (int e = ptr[s] + threadIdx.x; e < ptr[s + 1]; e += blockDim.x) {
-    const long long q = idx[e];
-    const cplx<T> a = nt[q], b = S[q];
+    const int q = idx[e], kx = q & 1023, ky = (q >> 10) & 1023, kz = q >> 20;
+    const cplx<T> a = nt[view.at(kx, ky, kz)], b = S[((size_t)kx * n + ky) * nh + kz];
     const double w = (double)wgt[e];
     acc[0] += w * ((double)a.x * (double)b.x + (double)a.y * (double)b.y) * scale;
     acc[1] += w * ((double)b.x * (double)b.x + (double)b.y * (double)b.y);
@@ -463,11 +463,6 @@ __global__ void __launch_bounds__(256) k_sei_shells(const cplx<T>* __restrict__ 
   double o[3];
   block_sum<3>(acc, red, o);
   if (threadIdx.x == 0) { out[3 * s] = o[0]; out[3 * s + 1] = o[1]; out[3 * s + 2] = o[2]; }
-}
-
-// out[c] = sum_r partial[r * cols + c] in a fixed order; one block, cols <= blockDim.x
-static __global__ void k_sum_columns(const double* __restrict__ partial, int rows, int cols, double* __restrict__ out) {
-  block_sum_columns(partial, rows, cols, out, nullptr);
 }
 
 }  // namespace ofdft
@@ -494,7 +489,7 @@ namespace ofdft {
 
 // one thread per (tile, kz, lane): the four rows' qq
 template <typename T>
-__global__ void k_forces_q(const cplx<T>* __restrict__ nt, const cplx<T>* __restrict__ SZ,
+__global__ void k_forces_q(const cplx<T>* __restrict__ nt, SpecView view, const cplx<T>* __restrict__ SZ,
                            const int2* __restrict__ rows, int nrows, const int* __restrict__ tk, int ntile,
                            const double2* __restrict__ gf, int m2max, int n, double invN, Quad<T>* __restrict__ qq) {
   const int nh = n / 2 + 1;
@@ -513,8 +508,7 @@ __global__ void k_forces_q(const cplx<T>* __restrict__ nt, const cplx<T>* __rest
         const double2 f = gf[m2];                        // (vfac, efac)
         const double w = (kz == 0 || 2 * kz == n) ? 1.0 : 2.0;
         auto one = [&](int kx, int ky, T& re, T& im) {
-          const size_t q = ((size_t)kx * n + ky) * nh + kz;
-          const cplx<T> v = nt[q], A = SZ[q];
+          const cplx<T> v = nt[view.at(kx, ky, kz)], A = SZ[((size_t)kx * n + ky) * nh + kz];
           re = (T)(w * (f.x * (double)v.x * invN + f.y * (double)A.x));
           im = (T)(-w * (f.x * (double)v.y * invN + f.y * (double)A.y));   // w conj(Q)
         };
@@ -716,10 +710,12 @@ namespace ofdft {
 // Pressure P = -dF/dOmega under a homogeneous dilation (L, R_I -> lambda L,
 // lambda R_I; n -> n / lambda^3; fixed T).  The local functionals contribute
 // (1/Omega) int (n v - f): for TF that is n T p(y), for LDA xc n (v_xc - e_xc).
-// partial[block][2] = (sum n T p, sum n (v_xc - e_xc)) over the grid.
+// partial[block][2] = (sum n T p, sum n (v_xc - e_xc)) over the grid; the last
+// block adds them into out[0..1].
 template <typename T>
 __global__ void __launch_bounds__(256) k_pressure_r(const T* __restrict__ rho, size_t N, T cy, T Te, int terms,
-                                                    double* __restrict__ partial, int fd64, double cy_d) {
+                                                    double* __restrict__ partial, int fd64, double cy_d,
+                                                    unsigned int* counter, double* out) {
   __shared__ typename TreeVal<T>::type scr[2 * 257];
   Acc<T> acc[2];
   const T nmin = (T)kNmin;
@@ -744,45 +740,69 @@ __global__ void __launch_bounds__(256) k_pressure_r(const T* __restrict__ rho, s
     }
   }
   block_sum_tree<2, T>(acc, 2, partial + (size_t)blockIdx.x * 2, scr);
+  if (arrive_last(counter)) {
+    block_sum_columns(partial, gridDim.x, 2, out, nullptr);
+    if (threadIdx.x == 0) *counter = 0u;
+  }
 }
 
-// G-space parts over the half spectrum (tiled layout, Hermitian weight w):
-//   partial[block][0] = sum w Re[n~* V_loc] c(G),  c = 3 at G = 0, 1 - G^2 rc^2/2 else
-//                       (entries with |G|^2 <= g2cut, as in the energy),
-//   partial[block][1] = sum w |(n^a)~|^2 pnl(m^2),  pnl = (3 - 6a) K + dK/dlambda.
-// nt, wt are unnormalised transforms (times invN).  FP64 sums.
+// G-space sums over the half spectrum (Hermitian weight w) of the unnormalised
+// transforms nt (n), wt (n^a) and pt (sqrt n), any of them null; V_loc and the
+// transforms in the view's layout:
+//   0: sum w Re[n~* V_loc] c(G),  c = 3 at G = 0, 1 - G^2 rc^2/2 else (entries with
+//      |G|^2 <= g2cut, as in the energy)
+//   1: sum w |(n^a)~|^2 pnl(m^2),  pnl = (3 - 6a) K + dK/dlambda
+//   2: sum w 4 pi |n~|^2 / G^2      3: sum w G^2 |(sqrt n)~|^2
+// A warp takes a row of the layout at a time.  Products in the plan's precision,
+// compensated sums; the last block adds the blocks' partial[block][4] into out[].
 template <typename T>
 __global__ void __launch_bounds__(256) k_pressure_g(const cplx<T>* __restrict__ nt, const cplx<T>* __restrict__ wt,
-                                                    const cplx<T>* __restrict__ vloc, const double* __restrict__ pnl,
-                                                    int n, double tp2, double g2cut, double rc2, double invN,
-                                                    double* __restrict__ partial) {
-  __shared__ double red[2 * 32];
-  const int nh = n / 2 + 1;
-  const size_t NH = (size_t)n * n * nh;
-  double acc[2] = {0, 0};
-  for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < NH; q += (size_t)gridDim.x * blockDim.x) {
-    const int kz = (int)(q % nh);
-    const size_t row = q / nh;
-    const int kx = (int)(row / n), ky = (int)(row % n);
-    const int mx = kx <= (n - 1) / 2 ? kx : kx - n, my = ky <= (n - 1) / 2 ? ky : ky - n;
-    const int m2 = mx * mx + my * my + kz * kz;
-    const double w = (kz == 0 || 2 * kz == n) ? 1.0 : 2.0;
-    if (vloc) {
-      const double G2 = tp2 * (double)m2;
-      if (G2 <= g2cut) {
-        const cplx<T> a = nt[q], v = vloc[q];
-        const double c = m2 == 0 ? 3.0 : 1.0 - 0.5 * G2 * rc2;
-        acc[0] += w * c * invN * ((double)a.x * (double)v.x + (double)a.y * (double)v.y);
+                                                    const cplx<T>* __restrict__ pt, SpecView view,
+                                                    const cplx<T>* __restrict__ vloc, const T* __restrict__ cou,
+                                                    const T* __restrict__ pnl, T tp2, T g2cut, T rc2, T invN,
+                                                    double* __restrict__ partial, unsigned int* counter,
+                                                    double* __restrict__ out) {
+  __shared__ typename TreeVal<T>::type scr[4 * 257];
+  const int n = view.n, nh = n / 2 + 1;
+  const int len = view.planes ? n : nh, rows = view.planes ? nh * n : n * n;
+  const int lane = threadIdx.x & 31;
+  auto sgn = [&](int k) { return k <= (n - 1) / 2 ? k : k - n; };
+  Acc<T> acc[4];
+  for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < rows; r += (gridDim.x * blockDim.x) >> 5) {
+    const int a = r / n, b = r - a * n;
+    // plane layout: row (kz = a, px = b) over py; tiled: row (kx = a, ky = b) over kz
+    const int m0 = view.planes ? sgn(view.rev ? view.rev[b] : b) : sgn(a);
+    const int m1 = view.planes ? 0 : sgn(b);
+    for (int c = lane; c < len; c += 32) {
+      const int kz = view.planes ? a : c;
+      const int my = view.planes ? sgn(view.rev ? view.rev[c] : c) : m1;
+      const int m2 = m0 * m0 + my * my + kz * kz;
+      const T w = (kz == 0 || 2 * kz == n) ? (T)1 : (T)2;
+      const size_t q = (size_t)r * len + c;
+      const T G2 = tp2 * (T)m2;
+      if (nt) {
+        const T x = nt[q].x * invN, y = nt[q].y * invN;
+        acc[2].add(w * cou[m2] * (x * x + y * y));
+        if (vloc && G2 <= g2cut) {
+          const cplx<T> v = vloc[q];
+          acc[0].add(w * (m2 == 0 ? (T)3 : (T)1 - (T)0.5 * G2 * rc2) * (x * v.x + y * v.y));
+        }
+      }
+      if (wt) {
+        const T x = wt[q].x * invN, y = wt[q].y * invN;
+        acc[1].add(w * (x * x + y * y) * pnl[m2]);
+      }
+      if (pt) {
+        const T x = pt[q].x * invN, y = pt[q].y * invN;
+        acc[3].add(w * G2 * (x * x + y * y));
       }
     }
-    if (pnl) {
-      const cplx<T> b = wt[q];
-      acc[1] += w * invN * invN * ((double)b.x * (double)b.x + (double)b.y * (double)b.y) * pnl[m2];
-    }
   }
-  double o[2];
-  block_sum<2>(acc, red, o);
-  if (threadIdx.x == 0) { partial[(size_t)blockIdx.x * 2] = o[0]; partial[(size_t)blockIdx.x * 2 + 1] = o[1]; }
+  block_sum_tree<4, T>(acc, 4, partial + (size_t)blockIdx.x * 4, scr);
+  if (arrive_last(counter)) {
+    block_sum_columns(partial, gridDim.x, 4, out, nullptr);
+    if (threadIdx.x == 0) *counter = 0u;
+  }
 }
 
 }  // namespace ofdft

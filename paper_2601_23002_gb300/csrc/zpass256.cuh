@@ -166,6 +166,7 @@ __global__ void __launch_bounds__(256, 4) k_zfwd256(ProArgs<T> a, Spectra<T> sp,
       for (int s = 0; s <= A; ++s) {
         const int k = j + B * s;
         if (s == A && j != 0) break;                   // k = H: thread 0 only
+        if (k >= a.nkz) break;
         const cplx<T> zk = xb[Z256::xpos(k == H ? 0 : k)];
         const cplx<T> zc = cconj(xb[Z256::xpos(k == 0 ? 0 : H - k)]);
         const cplx<T> e = cadd(zk, zc);
@@ -643,6 +644,12 @@ k_plane256cl(Spectra<T> sp, GArgs<T> g, const cplx<T>* __restrict__ tw_n) {
 #pragma unroll
     for (int o = 0; o < CL; ++o) z[o] = part[o][k2 * P + t];
     Codelet<cplx<T>, 8, -1>::run(z);                   // z[k1] = F(kx = k2 + 32 k1)
+    if (g.forward) {                                   // (all blocks of the cluster have read their rows)
+      cplx<T>* y = sp.s[fid] + (size_t)kz * N * N + (size_t)k2 * N + t;
+#pragma unroll
+      for (int k1 = 0; k1 < CL; ++k1) y[(size_t)k1 * 32 * N] = z[k1];
+      continue;
+    }
     // V_loc in plane layout [kz][kx][ky]
     const cplx<T>* vl = with_loc ? g.vloc + (size_t)kz * N * N + t : nullptr;
 #pragma unroll
@@ -657,6 +664,7 @@ k_plane256cl(Spectra<T> sp, GArgs<T> g, const cplx<T>* __restrict__ tw_n) {
     for (int o = 0; o < CL; ++o) part[o][k2 * P + t] = z[o];
   }
   cl.sync();                                           // (no remote access after this)
+  if (g.forward) return;
   // 4. column ky = t: twiddles W_256^(-c k2), inverse 32-point transforms
   {
     cplx<T> v[32];
