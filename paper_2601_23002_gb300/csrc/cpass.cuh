@@ -385,9 +385,9 @@ template <typename T, int N> __host__ __device__ constexpr size_t czinv_bytes(in
   return b > s ? b : s;
 }
 // Inverse z pass: complex-to-real transform of R rows of every active field
-// (plane layout) and the pointwise functional, or (mode 3) the
-// preconditioning pass's output.
-template <typename T, int N>
+// (plane layout) and the pointwise functional (KIND 0, 1, 2: see EpiPoint), or
+// the preconditioning pass's output (KIND 3: mode 3).
+template <typename T, int N, int KIND>
 __global__ void __launch_bounds__(CZ<N>::NT, (sizeof(T) == 4 ? 1024 : 512) / CZ<N>::NT)
 k_zinv_c(Spectra<T> sp, EpiArgs<T> a, const cplx<T>* __restrict__ tw_l, const cplx<T>* __restrict__ tw_n) {
   using Z = CZ<N>;
@@ -452,41 +452,47 @@ k_zinv_c(Spectra<T> sp, EpiArgs<T> a, const cplx<T>* __restrict__ tw_l, const cp
   }
   __syncthreads();                                       // (the staged spectra are free)
   cz_stages<T, N, +1>(xa, stg, sp.nact * Z::LINES, tw);
-  // real value i of row r, field f: element i / 2 (even n; pairs of reals) or
-  // the row's component of element i (odd n)
+  // real value i of row r, field slot f: component i % 2 of element i / 2 (even
+  // n) or the row's component of element i (odd n)
+  const T* xr = reinterpret_cast<const T*>(Z::F.c <= 2 ? xa : stg);
   auto real_at = [&](int f, int r, int i) -> T {
-    if constexpr (Z::ODD) {
-      const C z = cz_get<T, N>(xa, stg, f * Z::LINES + (r >> 1), i);
-      return (r & 1) ? z.y : z.x;
-    } else {
-      const C z = cz_get<T, N>(xa, stg, f * Z::LINES + r, i >> 1);
-      return (i & 1) ? z.y : z.x;
-    }
+    constexpr int PT = Z::F.c <= 2 ? Z::XP : Z::BP;
+    const int ln = f * Z::LINES + (Z::ODD ? r >> 1 : r), e = Z::ODD ? i : i >> 1, c = (Z::ODD ? r : i) & 1;
+    return xr[2 * (ln * PT + (Z::F.c <= 2 ? Z::pad(e) : e)) + c];
   };
-  if (a.mode == 3) {
-    for (int q = threadIdx.x; q < rows * N; q += Z::NT) {
-      const int r = q / N, i = q - r * N;
+  // (r, i) of the thread's points tid, tid + NT, ...
+  int r = threadIdx.x / N, i = threadIdx.x - r * N;
+  auto step = [&]() {
+    i += Z::NT % N; r += Z::NT / N;
+    if (Z::NT % N != 0 && i >= N) { i -= N; ++r; }
+  };
+  if constexpr (KIND == 3) {
+#pragma unroll 2
+    for (int q = threadIdx.x; q < rows * N; q += Z::NT, step()) {
       const T v = real_at(0, r, i);
       a.out[off + q] = v;
       if (a.pyout) a.pyout[off + q] = v - __ldg(a.pold + off + q);
     }
     return;
-  }
+  } else {
   // the slot of each field, -1: not active
   int slot[3];
 #pragma unroll
-  for (int i = 0; i < 3; ++i)
-    slot[i] = (sp.nact > 0 && fl_.i0 == i) ? 0 : (sp.nact > 1 && fl_.i1 == i) ? 1 : (sp.nact > 2 && fl_.i2 == i) ? 2 : -1;
-  const EpiPoint<T> ep(sp, a);
+  for (int k = 0; k < 3; ++k)
+    slot[k] = (sp.nact > 0 && fl_.i0 == k) ? 0 : (sp.nact > 1 && fl_.i1 == k) ? 1 : (sp.nact > 2 && fl_.i2 == k) ? 2 : -1;
+  const EpiPoint<T, KIND> ep(sp, a);
   AccShort<T> acc[8];
-  const T* src = (a.mode == 0 ? a.rho : a.psi) + off;
-  const T* dsrc = a.mode == 1 ? a.d + off : nullptr;
+  const bool with_d = KIND == 1 || (KIND == 0 && a.mode == 1);
+  const T* src = (EpiPoint<T, KIND>::mode(a) == 0 ? a.rho : a.psi) + off;
+  const T* dsrc = with_d ? a.d + off : src;
 #pragma unroll 2
-  for (int q = threadIdx.x; q < rows * N; q += Z::NT) {
-    const int r = q / N, i = q - r * N;
-    const T x = __ldg(src + q), d = dsrc ? __ldg(dsrc + q) : (T)0;
-    ep.point(a, x, d, slot[0] >= 0 ? real_at(slot[0], r, i) : (T)0, slot[1] >= 0 ? real_at(slot[1], r, i) : (T)0,
-             slot[2] >= 0 ? real_at(slot[2], r, i) : (T)0, off + q, acc);
+  for (int q = threadIdx.x; q < rows * N; q += Z::NT, step()) {
+    const T x = __ldg(src + q), d = with_d ? __ldg(dsrc + q) : (T)0;
+    if constexpr (KIND != 0)                             // slots 0 (n) and 1 (psi)
+      ep.point(a, x, d, real_at(0, r, i), (T)0, real_at(1, r, i), off + q, acc);
+    else
+      ep.point(a, x, d, slot[0] >= 0 ? real_at(slot[0], r, i) : (T)0, slot[1] >= 0 ? real_at(slot[1], r, i) : (T)0,
+               slot[2] >= 0 ? real_at(slot[2], r, i) : (T)0, off + q, acc);
   }
   using V = typename TreeVal<T>::type;
   V v[8];
@@ -497,6 +503,7 @@ k_zinv_c(Spectra<T> sp, EpiArgs<T> a, const cplx<T>* __restrict__ tw_l, const cp
   if (arrive_last(a.counter)) {
     finalize_eval8<T>(a.fin, scr);
     if (threadIdx.x == 0) *a.counter = 0u;
+  }
   }
 }
 
@@ -776,7 +783,7 @@ template <typename T> struct CPass {
   using PL = void (*)(Spectra<T>, GArgs<T>, const cplx<T>*);
   int n, rows, zthreads, zgrid;
   CFac fz, fp;
-  ZF zfwd; ZI zinv;
+  ZF zfwd; ZI zinv[4];                  // zinv by KIND
   size_t zf_bytes[4], zi_bytes[4];      // by number of fields
   // the plane pass with one field, and with more
   struct { PL kern; int cl, threads; size_t bytes; } pl[2];
@@ -807,7 +814,8 @@ template <typename T, int N> CPass<T> make_cpass() {
   p.n = N; p.rows = Z::R; p.zthreads = Z::NT; p.zgrid = Z::GRID;
   p.fz = Z::F; p.fp = cfac(N, false);
   p.zfwd = k_zfwd_c<T, N>;
-  p.zinv = k_zinv_c<T, N>;
+  p.zinv[0] = k_zinv_c<T, N, 0>; p.zinv[1] = k_zinv_c<T, N, 1>;
+  p.zinv[2] = k_zinv_c<T, N, 2>; p.zinv[3] = k_zinv_c<T, N, 3>;
   for (int f = 0; f < 4; ++f) { p.zf_bytes[f] = czfwd_bytes<T, N>(f); p.zi_bytes[f] = czinv_bytes<T, N>(f); }
   constexpr int c1 = cp_cluster<T, N>(1), c2 = cp_cluster<T, N>(2);
   if constexpr (c1 > 0) { p.pl[0].kern = k_plane_c<T, N, c1>; p.pl[0].cl = c1; p.pl[0].threads = CP<T, N, c1>::NT; p.pl[0].bytes = CP<T, N, c1>::BYTES; }

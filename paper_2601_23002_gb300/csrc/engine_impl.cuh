@@ -313,6 +313,8 @@ class Engine : public IEngine {
     cp = plane_allowed && cpass_allowed ? cpass_kernels<T>(n) : nullptr;
     zR = std::max(1, std::min(16, 1024 / h));     // 16 rows per block: best in a sweep at 128^3
     if (cp) zR = cp->rows;
+    // 256^3: 16 rows (8: k_zinv256 252 us instead of 226, k_zfwd256 103 instead of 84)
+    if (sizeof(T) == 4 && n == 256 && z256_allowed) zR = 16;
     zP = zpitch();
     yJ = sizeof(T) == 4 ? 16 : 8;
     xJ = yJ;
@@ -358,6 +360,12 @@ class Engine : public IEngine {
 
   // the cluster plane pass at 256^3 for some row count (V_loc in its order is
   // then kept whatever the tiles)
+  // the epilogue's KIND (see EpiPoint; 3: the preconditioning pass's output)
+  int epi_kind(const Spectra<T>& sp, const EpiArgs<T>& ea) const {
+    if (ea.mode == 3) return 3;
+    const bool full = sp.merged && sp.nact == 2 && sp.s[0] && (ea.terms & 9) == 9 && !(sizeof(T) == 4 && ea.fd64);
+    return !full || (ea.mode == 1 && !ea.out) ? 0 : ea.mode == 1 ? 1 : 2;
+  }
   // the z passes at 256^3 for the plan's rows per block (FP32 plans)
   int launch_zfwd256(const ProArgs<T>& pa, const Spectra<T>& sp, double bytes, cudaStream_t st) {
     if constexpr (sizeof(T) == 4) {
@@ -371,7 +379,10 @@ class Engine : public IEngine {
   }
   int launch_zinv256(const Spectra<T>& sp, const EpiArgs<T>& ea, double bytes, cudaStream_t st) {
     if constexpr (sizeof(T) == 4) {
-      auto k = zR == 8 ? k_zinv256<T, 8> : (zR == 16 ? k_zinv256<T, 16> : k_zinv256<T, 32>);
+      // (16 rows, the default, with the specialised epilogues)
+      const int kd = epi_kind(sp, ea);
+      auto k = zR == 8 ? k_zinv256<T, 8, 0> : zR == 32 ? k_zinv256<T, 32, 0> : kd == 1 ? k_zinv256<T, 16, 1>
+               : kd == 2 ? k_zinv256<T, 16, 2> : kd == 3 ? k_zinv256<T, 16, 3> : k_zinv256<T, 16, 0>;
       OFDFT_RUN("k_zinv256", st, bytes, k<<<grid_z, kThreads, smem_zi256, st>>>(sp, ea, tw_h, tw_n));
       return OFDFT_OK;
     } else {
@@ -406,7 +417,7 @@ class Engine : public IEngine {
   }
   int launch_zinv(const Spectra<T>& sp, const EpiArgs<T>& ea, double bytes, cudaStream_t st) {
     if (z256) return launch_zinv256(sp, ea, bytes, st);
-    if (cpz()) OFDFT_RUN("k_zinv_c", st, bytes, cp->zinv<<<cp->zgrid, cp->zthreads, cp->zi_bytes[sp.nact], st>>>(sp, ea, tw_h, tw_n));
+    if (cpz()) OFDFT_RUN("k_zinv_c", st, bytes, cp->zinv[epi_kind(sp, ea)]<<<cp->zgrid, cp->zthreads, cp->zi_bytes[sp.nact], st>>>(sp, ea, tw_h, tw_n));
     else OFDFT_RUN("k_zinv_epi", st, bytes, k_zinv_epi<T><<<grid_z, kThreads, smem_zi, st>>>(sp, ea, ph, tw_h, tw_n, n, zR, zP));
     return OFDFT_OK;
   }
@@ -741,9 +752,10 @@ class Engine : public IEngine {
       if (z256 && (rc = raise((const void*)k_zfwd256<T, 8>, z256_fwd_bytes<T>(8)))) return rc;
       if (z256 && (rc = raise((const void*)k_zfwd256<T, 16>, z256_fwd_bytes<T>(16)))) return rc;
       if (z256 && (rc = raise((const void*)k_zfwd256<T, 32>, z256_fwd_bytes<T>(32)))) return rc;
-      if (z256 && (rc = raise((const void*)k_zinv256<T, 8>, smem_zi256))) return rc;
-      if (z256 && (rc = raise((const void*)k_zinv256<T, 16>, smem_zi256))) return rc;
-      if (z256 && (rc = raise((const void*)k_zinv256<T, 32>, smem_zi256))) return rc;
+      const void* zi[] = {(const void*)k_zinv256<T, 8, 0>, (const void*)k_zinv256<T, 32, 0>, (const void*)k_zinv256<T, 16, 0>,
+                          (const void*)k_zinv256<T, 16, 1>, (const void*)k_zinv256<T, 16, 2>, (const void*)k_zinv256<T, 16, 3>};
+      for (const void* f : zi)
+        if (z256 && (rc = raise(f, smem_zi256))) return rc;
     }
     if (z256 && (rc = raise((const void*)k_ypass256<T, -1>, y256_bytes<T>()))) return rc;
     if (z256 && (rc = raise((const void*)k_ypass256<T, 1>, y256_bytes<T>()))) return rc;
@@ -757,7 +769,8 @@ class Engine : public IEngine {
     if (planes && !cp && (rc = raise((const void*)plane_kern, smem_pl))) return rc;
     if (cp) {
       if ((rc = raise((const void*)cp->zfwd, cp->zf_bytes[3]))) return rc;
-      if ((rc = raise((const void*)cp->zinv, cp->zi_bytes[3]))) return rc;
+      for (auto f : cp->zinv)
+        if ((rc = raise((const void*)f, cp->zi_bytes[3]))) return rc;
       for (const auto& pl : cp->pl)
         if ((rc = raise((const void*)pl.kern, pl.bytes))) return rc;
     }

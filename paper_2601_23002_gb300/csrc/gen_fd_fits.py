@@ -203,7 +203,7 @@ def main():
     a, b = series_coefficients()
     lines = [
         "/* Generated by gen_fd_fits.py -- do not edit.",
-        " * fd32_eta, fd32_p: power series in x in [-1, 1] on intervals of s = ln y for",
+        " * fd32_tab: power series in x in [-1, 1] (eta's, then p's) on intervals of s = ln y for",
         " * eta(s) = I_{1/2}^{-1}(e^s) and p(s) = (2/3) I_{3/2}(eta(s)) / e^s on [FD_S_LO, FD_S_HI):",
         f" * {n32} intervals of width {W32}, degree {D32}; max rel err eta {worst[0][0]:.2e}, p {worst[0][1]:.2e}.",
         f" * fd64_tab: (eta, p) of y on {SUB} intervals per binade of [2^{FD_ELO}, 2^{FD_EHI}), degree {D64}, coefficient pairs;",
@@ -237,8 +237,7 @@ def main():
     pairs = lambda rr: [[v for q in zip(r[0], r[1]) for v in q] for r in rr]
     arr("fd64_tab", pairs(rfd), False, "double")
     arr("xc64_tab", pairs(rxc), False, "double")
-    arr("fd32_eta", [r[0] for r in r32], True, "float")
-    arr("fd32_p", [r[1] for r in r32], True, "float")
+    arr("fd32_tab", [r[0] + r[1] for r in r32], True, "float")
     with open(out, "w") as f:
         f.write("\n".join(lines) + "\n")
     sys.stderr.write(f"worst errors {worst}\n")

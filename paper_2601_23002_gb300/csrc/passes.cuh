@@ -106,11 +106,10 @@ static __device__ __forceinline__ void fd_eta_p_s(float y, float s, float& eta, 
     int i = (int)r;
     i = i < 0 ? 0 : (i >= FD32_NINT ? FD32_NINT - 1 : i);
     const float x = 2.0f * (r - (float)i) - 1.0f;
-    // each interval's 8 coefficients as two 16-byte loads per table
-    static_assert(FD32_NC == 8, "two float4 per interval");
-    const float4* e4 = reinterpret_cast<const float4*>(fd32_eta[i]);
-    const float4* p4 = reinterpret_cast<const float4*>(fd32_p[i]);
-    const float4 ea = __ldg(e4), eb = __ldg(e4 + 1), pa = __ldg(p4), pb = __ldg(p4 + 1);
+    // an interval's 8 + 8 coefficients as four 16-byte loads of one 64-byte row
+    static_assert(FD32_NC == 8, "four float4 per interval");
+    const float4* e4 = reinterpret_cast<const float4*>(fd32_tab[i]);
+    const float4 ea = __ldg(e4), eb = __ldg(e4 + 1), pa = __ldg(e4 + 2), pb = __ldg(e4 + 3);
     eta = fmaf(fmaf(fmaf(eb.w, x, eb.z), x, eb.y), x, eb.x);
     eta = fmaf(fmaf(fmaf(fmaf(eta, x, ea.w), x, ea.z), x, ea.y), x, ea.x);
     p = fmaf(fmaf(fmaf(pb.w, x, pb.z), x, pb.y), x, pb.x);
@@ -639,17 +638,22 @@ template <typename T> struct EpiArgs {
 // potential (mode 0) or g' (mode 1) written to out[at], and the block's
 // partial sums acc: 0 F_TF, 1 E_xc, 2 int v_rest n, 3 int g' d, 4 int g'^2,
 // 5 int g' psi_t, 6 int n, 7 nonfinite count.
-template <typename T> struct EpiPoint {
+// KIND: 0 any call; 1 and 2 the full functional with a = 1/2 (fields n and psi,
+// merged) without fd64, mode 1 and mode 0: every choice but the radius of the
+// XC branches is then made at compile time (about 25 of 200 instructions per
+// point and a tenth of the registers).
+template <typename T, int KIND> struct EpiPoint {
   bool has_n, has_na, has_psi, merged;
   T Te, cy, lcy, alpha, nmin, tstep, tscale, muref;
   __device__ __forceinline__ EpiPoint(const Spectra<T>& sp, const EpiArgs<T>& a)
-      : has_n(sp.s[0] != nullptr), has_na(sp.s[1] != nullptr), has_psi(sp.s[2] != nullptr),
-        merged(sp.merged != 0), Te(a.T_e), cy(a.cy), lcy(a.lcy), alpha(a.alpha), nmin((T)kNmin),
+      : has_n(KIND || sp.s[0] != nullptr), has_na(!KIND && sp.s[1] != nullptr), has_psi(KIND || sp.s[2] != nullptr),
+        merged(KIND || sp.merged != 0), Te(a.T_e), cy(a.cy), lcy(a.lcy), alpha(a.alpha), nmin((T)kNmin),
         tstep(a.dsc ? (T)a.dsc[2] : a.t), tscale(a.dsc ? (T)a.dsc[0] : a.scale), muref(a.mu_ref) {}
+  static __device__ __forceinline__ int mode(const EpiArgs<T>& a) { return KIND == 1 ? 1 : KIND == 2 ? 0 : a.mode; }
   __device__ __forceinline__ void point(const EpiArgs<T>& a, T pv, T dq, T hv, T kv, T lv, size_t at,
                                         AccShort<T> (&acc)[8]) const {
     T psit, nval, iphi = 0;              // iphi: 1 / max(psi, kPhiMin), mode 0 only
-    if (a.mode == 0) {
+    if (mode(a) == 0) {
       // one reciprocal square root for psi and the division by it
       nval = pv;
       const T r = rsqrt_t(fmax(nval, (T)1e-30));
@@ -663,8 +667,8 @@ template <typename T> struct EpiPoint {
     T l2 = 0;                            // FP32: one logarithm for TF and XC
     if constexpr (sizeof(T) == 4) l2 = __log2f(nf);
     T vrest = 0;
-    if (a.terms & 1) {              // TF
-      if (sizeof(T) == 4 && a.fd64) {
+    if (KIND || (a.terms & 1)) {              // TF
+      if (!KIND && sizeof(T) == 4 && a.fd64) {
         // FP64 inversion from the stored density value; f_TF formed in FP64
         double eta, p;
         fd_eta_p((double)nf * a.cy_d, eta, p);
@@ -679,7 +683,7 @@ template <typename T> struct EpiPoint {
         acc[0].add(nf * Te * (eta - p));
       }
     }
-    if (a.terms & 8) {              // XC
+    if (KIND || (a.terms & 8)) {              // XC
       T exc, vxc;
       if constexpr (sizeof(T) == 4) pz81_l2(nf, l2, exc, vxc);
       else pz81(nf, exc, vxc);
@@ -701,14 +705,14 @@ template <typename T> struct EpiPoint {
     // g' = psi (v_rest - mu_ref) + lap/2: near convergence mu_ref is close to
     // mu, so the projection g = 2 scale (g' - (mu - mu_ref) psi) cancels little
     const T gp = psit * (vrest - muref) + extra;
-    T* __restrict__ gout = a.out;
-    if (a.mode == 0) {
+    T* __restrict__ gout = a.out;        // (null: no output wanted, mode 0 only)
+    if (mode(a) == 0) {
       const T v = vrest + extra * iphi;
       if (gout) gout[at] = v;
       // residual pieces with psi = sqrt(rho), scale 1: g' = psi v_rest + lap/2
       if (!isfinite(v)) acc[7].add((T)1);
     } else {
-      if (gout) gout[at] = gp;
+      if (KIND || gout) gout[at] = gp;
       acc[3].add(gp * dq);
       if (!isfinite(gp)) acc[7].add((T)1);
     }
@@ -846,7 +850,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_zinv_epi(Spectr
   const T* fH = realf[0];
   const T* fK = realf[1];
   const T* fL = realf[2];
-  const EpiPoint<T> ep(sp, a);
+  const EpiPoint<T, 0> ep(sp, a);
   AccShort<T> acc[8];
   const T* pd = pin + (size_t)Rfull * n;
   for (int q = threadIdx.x; q < tot; q += blockDim.x)

@@ -186,7 +186,8 @@ __global__ void __launch_bounds__(256, 4) k_zfwd256(ProArgs<T> a, Spectra<T> sp,
 // straight from memory in the pointwise loop, one row ahead, rather than
 // staged: 33 KB less shared memory per block at 16 rows, three blocks per SM
 // instead of two.
-template <typename T, int R>
+// KIND: see EpiPoint (3: mode 3).
+template <typename T, int R, int KIND>
 __global__ void __launch_bounds__(256, 3) k_zinv256(Spectra<T> sp, EpiArgs<T> a, const cplx<T>* __restrict__ tw_h,
                                                    const cplx<T>* __restrict__ tw_n) {
   constexpr int N = Z256::N, H = Z256::H, NH = Z256::NH, A = Z256::A, B = Z256::B;
@@ -256,7 +257,7 @@ __global__ void __launch_bounds__(256, 3) k_zinv256(Spectra<T> sp, EpiArgs<T> a,
   T* realf[3] = {nullptr, nullptr, nullptr};
   for (int f = 0; f < sp.nact; ++f) realf[sp.idx[f]] = reinterpret_cast<T*>(stg + (size_t)f * R * NH);
   const int jt = threadIdx.x;                          // one grid point of each row (blockDim = N)
-  if (a.mode == 3) {
+  if (KIND == 3 || (KIND == 0 && a.mode == 3)) {
     const T* fP = realf[2];
     T po[R];                                           // P g_old, loaded ahead of the stores
     if (a.pyout) {
@@ -271,24 +272,29 @@ __global__ void __launch_bounds__(256, 3) k_zinv256(Spectra<T> sp, EpiArgs<T> a,
     }
     return;
   }
-  const EpiPoint<T> ep(sp, a);
+  if constexpr (KIND != 3) {
+  const EpiPoint<T, KIND> ep(sp, a);
   AccShort<T> acc[8];
   // (the loads of the next row are issued before this row's stores of g')
-  const T* src0 = (a.mode == 0 ? a.rho : a.psi) + off + jt;
-  const T* dsrc = a.mode == 1 ? a.d + off + jt : nullptr;
-  T xn = __ldg(src0), dn = dsrc ? __ldg(dsrc) : (T)0;
+  const bool with_d = KIND == 1 || (KIND == 0 && a.mode == 1);
+  const T* src0 = (EpiPoint<T, KIND>::mode(a) == 0 ? a.rho : a.psi) + off + jt;
+  const T* dsrc = with_d ? a.d + off + jt : src0;
+  T xn = __ldg(src0), dn = with_d ? __ldg(dsrc) : (T)0;
+  const T* f0 = realf[0];
+  const T* f2 = KIND ? reinterpret_cast<const T*>(stg + (size_t)R * NH) : realf[2];
   for (int r = 0; r < R; ++r) {
     const int qs = r * rp + jt, q = r * N + jt;
     const T x = xn, dd = dn;
-    if (r + 1 < R) { xn = __ldg(src0 + (r + 1) * N); if (dsrc) dn = __ldg(dsrc + (r + 1) * N); }
-    ep.point(a, x, dd, realf[0] ? realf[0][qs] : (T)0,
-             realf[1] ? realf[1][qs] : (T)0, realf[2] ? realf[2][qs] : (T)0, off + q, acc);
+    if (r + 1 < R) { xn = __ldg(src0 + (r + 1) * N); if (with_d) dn = __ldg(dsrc + (r + 1) * N); }
+    if constexpr (KIND != 0) ep.point(a, x, dd, reinterpret_cast<const T*>(stg)[qs], (T)0, f2[qs], off + q, acc);
+    else ep.point(a, x, dd, f0 ? f0[qs] : (T)0, realf[1] ? realf[1][qs] : (T)0, f2 ? f2[qs] : (T)0, off + q, acc);
   }
   typename TreeVal<T>::type* scr = reinterpret_cast<typename TreeVal<T>::type*>(smem_raw);
   block_sum_tree_raw<8, T>(acc, a.partials + (size_t)blockIdx.x * 8, scr);
   if (arrive_last(a.counter)) {
     finalize_eval<T>(a.fin, scr);
     if (threadIdx.x == 0) *a.counter = 0u;
+  }
   }
 }
 
