@@ -288,6 +288,7 @@ k_zfwd_c(ProArgs<T> a, Spectra<T> sp, const cplx<T>* __restrict__ tw_l, const cp
   const int rows = min(R, NN - row0);
   const int lines = Z::ODD ? (rows + 1) >> 1 : rows;
   for (int q = threadIdx.x; q < L + NH; q += Z::NT) tw[q] = q < L ? tw_l[q] : tw_n[q - L];
+  dependency_wait();
   const T* src = (a.mode == 0 ? a.rho : a.psi) + (size_t)row0 * N;
   const bool has_d = a.mode != 0 && a.d != nullptr;
   const T* dsrc = has_d ? a.d + (size_t)row0 * N : src;
@@ -315,12 +316,12 @@ k_zfwd_c(ProArgs<T> a, Spectra<T> sp, const cplx<T>* __restrict__ tw_l, const cp
       const T* p0 = src + 2 * ln * N + j;
       const T* d0 = dsrc + 2 * ln * N + j;
 #pragma unroll
-      for (int s = 0; s < F0; ++s) v[s] = mk<T>(__ldg(p0 + s * M0), two ? __ldg(p0 + N + s * M0) : (T)0);
+      for (int s = 0; s < F0; ++s) v[s] = mk<T>(p0[s * M0], two ? p0[N + s * M0] : (T)0);
       if (has_d) {
 #pragma unroll
         for (int s = 0; s < F0; ++s) {
-          v[s].x = v[s].x + tstep * __ldg(d0 + s * M0);
-          if (two) v[s].y = v[s].y + tstep * __ldg(d0 + N + s * M0);
+          v[s].x = v[s].x + tstep * d0[s * M0];
+          if (two) v[s].y = v[s].y + tstep * d0[N + s * M0];
         }
       }
 #pragma unroll
@@ -329,11 +330,11 @@ k_zfwd_c(ProArgs<T> a, Spectra<T> sp, const cplx<T>* __restrict__ tw_l, const cp
       const C* p0 = reinterpret_cast<const C*>(src + ln * N) + j;
       const C* d0 = reinterpret_cast<const C*>(dsrc + ln * N) + j;
 #pragma unroll
-      for (int s = 0; s < F0; ++s) v[s] = __ldg(p0 + s * M0);
+      for (int s = 0; s < F0; ++s) v[s] = p0[s * M0];
       if (has_d) {
 #pragma unroll
         for (int s = 0; s < F0; ++s) {
-          const C d = __ldg(d0 + s * M0);
+          const C d = d0[s * M0];
           v[s].x = v[s].x + tstep * d.x; v[s].y = v[s].y + tstep * d.y;
         }
       }
@@ -402,13 +403,14 @@ k_zinv_c(Spectra<T> sp, EpiArgs<T> a, const cplx<T>* __restrict__ tw_l, const cp
   const int row0 = blockIdx.x * R;
   const int rows = min(R, NN - row0);
   const size_t off = (size_t)row0 * N;
+  for (int q = threadIdx.x; q < L + NH; q += Z::NT) tw[q] = q < L ? tw_l[q] : tw_n[q - L];
+  dependency_wait();
   for (int q = threadIdx.x; q < sp.nact * NH * R; q += Z::NT) {
     const int fk = q / R, r = q - fk * R;
     const int f = fk / NH, k = fk - f * NH;
     if (r < rows) cp_async_c(stg + (f * R + r) * Z::SP + k, fl_.spec(f) + (size_t)k * NN + row0 + r, true);
   }
   cp_async_commit();
-  for (int q = threadIdx.x; q < L + NH; q += Z::NT) tw[q] = q < L ? tw_l[q] : tw_n[q - L];
   cp_async_wait<0>();
   __syncthreads();
   // stage 0: Z at j + s M0 from the staged spectra, radix F0
@@ -471,7 +473,7 @@ k_zinv_c(Spectra<T> sp, EpiArgs<T> a, const cplx<T>* __restrict__ tw_l, const cp
     for (int q = threadIdx.x; q < rows * N; q += Z::NT, step()) {
       const T v = real_at(0, r, i);
       a.out[off + q] = v;
-      if (a.pyout) a.pyout[off + q] = v - __ldg(a.pold + off + q);
+      if (a.pyout) a.pyout[off + q] = v - a.pold[off + q];
     }
     return;
   } else {
@@ -487,7 +489,7 @@ k_zinv_c(Spectra<T> sp, EpiArgs<T> a, const cplx<T>* __restrict__ tw_l, const cp
   const T* dsrc = with_d ? a.d + off : src;
 #pragma unroll 2
   for (int q = threadIdx.x; q < rows * N; q += Z::NT, step()) {
-    const T x = __ldg(src + q), d = with_d ? __ldg(dsrc + q) : (T)0;
+    const T x = src[q], d = with_d ? dsrc[q] : (T)0;
     if constexpr (KIND != 0)                             // slots 0 (n) and 1 (psi)
       ep.point(a, x, d, real_at(0, r, i), (T)0, real_at(1, r, i), off + q, acc);
     else
@@ -605,6 +607,7 @@ k_plane_c(Spectra<T> sp, GArgs<T> g, const cplx<T>* __restrict__ tw_g) {
   C* gpl = CField<T>::pick(sp, fid) + (size_t)kz * NN + (size_t)row0 * N;
   for (int q = threadIdx.x; q < N; q += Q::NT) tw[q] = tw_g[q];
   __syncthreads();
+  dependency_wait();
   // along ky: stage 0 from memory
   for (int it = threadIdx.x; it < Q::ROWS * M0; it += Q::NT) {
     const int ln = it / M0, j = it - ln * M0;

@@ -52,6 +52,24 @@ namespace ofdft {
 
 constexpr int kThreads = 256;
 
+// Launch with programmatic stream serialisation (see dependency_wait): the chain
+// of an evaluation or an L-BFGS iteration is ten kernels of a few microseconds on
+// small grids, and the gap between two dependent launches was 1-2 us.
+template <typename... KA, typename... A>
+inline void launch_pdl(void (*kern)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kern, static_cast<KA>(args)...);
+}
+
 template <typename T>
 __global__ void k_convert_table(const double* __restrict__ a, T* __restrict__ b, int cnt) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -370,7 +388,7 @@ class Engine : public IEngine {
   int launch_zfwd256(const ProArgs<T>& pa, const Spectra<T>& sp, double bytes, cudaStream_t st) {
     if constexpr (sizeof(T) == 4) {
       auto k = zR == 8 ? k_zfwd256<T, 8> : (zR == 16 ? k_zfwd256<T, 16> : k_zfwd256<T, 32>);
-      OFDFT_RUN("k_zfwd256", st, bytes, k<<<grid_z, kThreads, smem_zf256, st>>>(pa, sp, tw_h, tw_n));
+      OFDFT_RUN("k_zfwd256", st, bytes, launch_pdl(k, grid_z, kThreads, smem_zf256, st, pa, sp, tw_h, tw_n));
       return OFDFT_OK;
     } else {
       set_error("the 256^3 register z passes are FP32 only");
@@ -383,7 +401,7 @@ class Engine : public IEngine {
       const int kd = epi_kind(sp, ea);
       auto k = zR == 8 ? k_zinv256<T, 8, 0> : zR == 32 ? k_zinv256<T, 32, 0> : kd == 1 ? k_zinv256<T, 16, 1>
                : kd == 2 ? k_zinv256<T, 16, 2> : kd == 3 ? k_zinv256<T, 16, 3> : k_zinv256<T, 16, 0>;
-      OFDFT_RUN("k_zinv256", st, bytes, k<<<grid_z, kThreads, smem_zi256, st>>>(sp, ea, tw_h, tw_n));
+      OFDFT_RUN("k_zinv256", st, bytes, launch_pdl(k, grid_z, kThreads, smem_zi256, st, sp, ea, tw_h, tw_n));
       return OFDFT_OK;
     } else {
       set_error("the 256^3 register z passes are FP32 only");
@@ -396,7 +414,7 @@ class Engine : public IEngine {
   // the cluster plane pass over the first nkz planes of nf fields
   int launch_p256(const Spectra<T>& sp, const GArgs<T>& ga, int nf, double bytes, cudaStream_t st, int nkz = 129) {
     if constexpr (sizeof(T) == 4) {
-      OFDFT_RUN("k_plane256cl", st, bytes, k_plane256cl<T><<<dim3(P256::CL * nkz, nf), P256::THREADS, p256_bytes<T>(), st>>>(sp, ga, tw_n));
+      OFDFT_RUN("k_plane256cl", st, bytes, launch_pdl(k_plane256cl<T>, dim3(P256::CL * nkz, nf), P256::THREADS, p256_bytes<T>(), st, sp, ga, tw_n));
       return OFDFT_OK;
     } else {
       set_error("the cluster plane pass is FP32 only");
@@ -411,19 +429,19 @@ class Engine : public IEngine {
   }
   int launch_zfwd(const ProArgs<T>& pa, const Spectra<T>& sp, double bytes, cudaStream_t st) {
     if (z256) return launch_zfwd256(pa, sp, bytes, st);
-    if (czfwd_ok(pa)) OFDFT_RUN("k_zfwd_c", st, bytes, cp->zfwd<<<cp->zgrid, cp->zthreads, cp->zf_bytes[sp.nact], st>>>(pa, sp, tw_h, tw_n));
+    if (czfwd_ok(pa)) OFDFT_RUN("k_zfwd_c", st, bytes, launch_pdl(cp->zfwd, cp->zgrid, cp->zthreads, cp->zf_bytes[sp.nact], st, pa, sp, tw_h, tw_n));
     else OFDFT_RUN("k_zfwd", st, bytes, k_zfwd<T><<<grid_z, kThreads, smem_zf, st>>>(pa, sp, ph, tw_h, tw_n, n, zR, zP));
     return OFDFT_OK;
   }
   int launch_zinv(const Spectra<T>& sp, const EpiArgs<T>& ea, double bytes, cudaStream_t st) {
     if (z256) return launch_zinv256(sp, ea, bytes, st);
-    if (cpz()) OFDFT_RUN("k_zinv_c", st, bytes, cp->zinv[epi_kind(sp, ea)]<<<cp->zgrid, cp->zthreads, cp->zi_bytes[sp.nact], st>>>(sp, ea, tw_h, tw_n));
+    if (cpz()) OFDFT_RUN("k_zinv_c", st, bytes, launch_pdl(cp->zinv[epi_kind(sp, ea)], cp->zgrid, cp->zthreads, cp->zi_bytes[sp.nact], st, sp, ea, tw_h, tw_n));
     else OFDFT_RUN("k_zinv_epi", st, bytes, k_zinv_epi<T><<<grid_z, kThreads, smem_zi, st>>>(sp, ea, ph, tw_h, tw_n, n, zR, zP));
     return OFDFT_OK;
   }
   int launch_cplane(const Spectra<T>& sp, const GArgs<T>& ga, double bytes, cudaStream_t st) {
     const auto& pl = cp->pl[sp.nact > 1];
-    OFDFT_RUN("k_plane_c", st, bytes, pl.kern<<<dim3(pl.cl * nh, sp.nact), pl.threads, pl.bytes, st>>>(sp, ga, tw_n));
+    OFDFT_RUN("k_plane_c", st, bytes, launch_pdl(pl.kern, dim3(pl.cl * nh, sp.nact), pl.threads, pl.bytes, st, sp, ga, tw_n));
     return OFDFT_OK;
   }
   // rows of G-space partials the epilogue's partials come after (3 fields)
@@ -1016,7 +1034,7 @@ class Engine : public IEngine {
       view.pos = pos_of; view.rev = rev_d;
       if (int rc = launch_zfwd(pa, sp, zb, st)) return rc;
       const auto& pl = cp->pl[nf > 1];
-      OFDFT_RUN("k_plane_c", st, yb, pl.kern<<<dim3(pl.cl * nk, nf), pl.threads, pl.bytes, st>>>(sp, ga, tw_n));
+      OFDFT_RUN("k_plane_c", st, yb, launch_pdl(pl.kern, dim3(pl.cl * nk, nf), pl.threads, pl.bytes, st, sp, ga, tw_n));
     } else if (pl256) {
       if (int rc = launch_zfwd(pa, sp, zb, st)) return rc;
       if (int rc = launch_p256(sp, ga, nf, yb, st, nk)) return rc;
@@ -1138,7 +1156,7 @@ class Engine : public IEngine {
       const int S = cn + nw <= 17 ? 3 : 2;   // k_gram is built for 2 or 3 ring stages
       const size_t sm = std::max(StreamCfg<T>::ring_bytes(S, cn + nw), tree_scratch_bytes<T>(cn * nw, kStreamThreads));
       prof.begin("k_gram", st, (double)(cn + nw) * N * sizeof(T));
-      auto launch = [&](auto kern) { kern<<<grid_stream, kStreamThreads, sm, st>>>(xl, cn, Nv, partials, counters + 1, o); };
+      auto launch = [&](auto kern) { launch_pdl(kern, grid_stream, kStreamThreads, sm, st, xl, cn, Nv, partials, counters + 1, o); };
       switch (nw * 8 + S) {
         case 1 * 8 + 3: launch(k_gram<T, 1, 3>); break;
         case 2 * 8 + 3: launch(k_gram<T, 2, 3>); break;
@@ -1171,7 +1189,7 @@ class Engine : public IEngine {
     xl.v[nv] = g; xl.v[nv + 1] = psi;
     xl.nv = nv + 2;
     OFDFT_RUN("k_lincomb", st, (double)(nv + 3) * N * sizeof(T),
-              k_lincomb<T><<<grid_stream, kStreamThreads, StreamCfg<T>::ring_bytes(stream_stages(kMaxLin - 1), nv + 2), st>>>(
+              launch_pdl(k_lincomb<T>, grid_stream, kStreamThreads, StreamCfg<T>::ring_bytes(stream_stages(kMaxLin - 1), nv + 2), st, 
                   xl, nv, out, Nv, partials, counters + 2, res_d + 16, res_h + 16, ts, dcoef));
     if (!dd) return OFDFT_OK;
     OFDFT_CK(cudaStreamSynchronize(st));
@@ -1344,7 +1362,7 @@ int Engine<T>::minimize(void* rho_io, int start_uniform, const ofdft_min_opts& o
       if ((rc = gram(V, {g, pgv[pcur], Yh[new_slot], PYh[new_slot]}, cross, st, false))) return rc;
       // two-loop recursion on the device (k_twoloop), then the direction
       // d = coef[0] P g + sum (coef[1+2j] P y_j + coef[2+2j] s_j)
-      OFDFT_RUN("k_twoloop", st, 0.0, k_twoloop<<<1, 32, 0, st>>>(ta, res_d + 16, res_d + 120, tl_state, res_h + 129));
+      OFDFT_RUN("k_twoloop", st, 0.0, launch_pdl(k_twoloop, 1, 32, 0, st, ta, res_d + 16, res_d + 120, tl_state, res_h + 129));
       VecList<T> vl{};
       vl.nv = 0;
       vl.v[vl.nv++] = pgv[pcur];
@@ -1433,7 +1451,7 @@ int Engine<T>::minimize(void* rho_io, int start_uniform, const ofdft_min_opts& o
     VecList<T> xa{};
     xa.nv = 4; xa.v[0] = psi; xa.v[1] = d; xa.v[2] = gp; xa.v[3] = g;
     OFDFT_RUN("k_accept", st, 8.0 * N * sizeof(T),
-              k_accept<T><<<grid_stream, kStreamThreads, StreamCfg<T>::ring_bytes(stream_stages(4), 4), st>>>(
+              launch_pdl(k_accept<T>, grid_stream, kStreamThreads, StreamCfg<T>::ring_bytes(stream_stages(4), 4), st, 
                   xa, (T)acc.t, (T)(2.0 * lastScale), (T)(lastMu - mu_ref), psi, g, Sh[slot], Yh[slot], Nv,
                   partials, counters + 3, res_d + 120, res_h + 120));
     new_slot = slot;

@@ -136,6 +136,7 @@ k_gram(VecList<T> X, int nv, size_t N, double* __restrict__ partial, unsigned in
   using V = typename V16<T>::type;
   constexpr int K = V16<T>::K;
   Acc<T> acc[kMaxV][NW];
+  dependency_wait();
   cpa_stream<T, S>(X, nv + NW, N, smem, [&](const V* mine, size_t) {
     T w[NW][K];
 #pragma unroll
@@ -221,12 +222,13 @@ static __global__ void __launch_bounds__(32) k_twoloop(TwoLoopArgs a, const doub
   __shared__ double sgam;
   __shared__ int skk;
   const int lane = threadIdx.x;
+  dependency_wait();
   const int no = a.no, ns = a.new_slot;
   const double dv = a.dv;
   for (int q = lane; q < M2; q += 32) { sSY[q] = st->SY[q]; sYY[q] = st->YY[q]; sYPY[q] = st->YPY[q]; }
   if (lane < kTLMax) { sSg[lane] = st->Sg[lane]; sYg[lane] = st->Yg[lane]; sYPg[lane] = st->YPg[lane]; }
-  for (int q = lane; q < (2 * no + 1) * 4; q += 32) sX[q] = cross[q] * dv;
-  if (lane < 6) sA[lane] = acc[lane] * dv;
+  for (int q = lane; q < (2 * no + 1) * 4; q += 32) sX[q] = __ldcg(cross + q) * dv;
+  if (lane < 6) sA[lane] = __ldcg(acc + lane) * dv;
   __syncwarp();
   // the new pair's rows and columns (lane i < no: older pair i; lane 31: own dots)
   if (lane < no) {
@@ -311,9 +313,10 @@ k_lincomb(VecList<T> X, int nv, T* __restrict__ out, size_t N, double* __restric
   using V = typename V16<T>::type;
   constexpr int K = V16<T>::K;
   Acc<T> acc[3];
+  dependency_wait();
   T c[kMaxLin - 2];
 #pragma unroll
-  for (int i = 0; i < kMaxLin - 2; ++i) c[i] = i < nv ? (T)(dcoef ? dcoef[i] : X.c[i]) : (T)0;
+  for (int i = 0; i < kMaxLin - 2; ++i) c[i] = i < nv ? (T)(dcoef ? __ldcg(dcoef + i) : X.c[i]) : (T)0;
   cpa_stream<T, stream_stages(kMaxLin - 1)>(X, nv + 2, N, smem, [&](const V* mine, size_t p) {
     T s[K];
 #pragma unroll
@@ -379,6 +382,7 @@ k_accept(VecList<T> X, T tt, T a, T m, T* __restrict__ psi, T* __restrict__ g, T
   using V = typename V16<T>::type;
   constexpr int K = V16<T>::K;
   Acc<T> acc[6];
+  dependency_wait();
   cpa_stream<T, stream_stages(4)>(X, 4, N, smem, [&](const V* mine, size_t p) {
     T p0[K], dd[K], gpi[K], g0[K], pt[K], gt[K], si[K], yi[K];
     lds16<T>(mine, p0);

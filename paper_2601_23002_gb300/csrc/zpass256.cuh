@@ -100,6 +100,7 @@ __global__ void __launch_bounds__(256, 4) k_zfwd256(ProArgs<T> a, Spectra<T> sp,
   const bool has_d = a.mode != 0 && a.d != nullptr;
   for (int q = threadIdx.x; q < NH + H; q += blockDim.x) twN[q] = q < NH ? tw_n[q] : tw_h[q - NH];
   __syncthreads();
+  dependency_wait();
   const T tstep = a.dsc ? (T)a.dsc[2] : a.t;
   const T scale = a.dsc ? (T)a.dsc[0] : a.scale, alpha = a.alpha, nmin = (T)kNmin;
   const T psi_shift = a.dsc ? (T)a.dsc[1] : a.psi_shift;
@@ -119,11 +120,11 @@ __global__ void __launch_bounds__(256, 4) k_zfwd256(ProArgs<T> a, Spectra<T> sp,
       const float2* dr = has_d ? reinterpret_cast<const float2*>(a.d + off + (size_t)r * N) : nullptr;
       float2 w[A];
 #pragma unroll
-      for (int s = 0; s < A; ++s) w[s] = __ldg(pr + j + B * s);
+      for (int s = 0; s < A; ++s) w[s] = pr[j + B * s];
       if (has_d) {
 #pragma unroll
         for (int s = 0; s < A; ++s) {
-          const float2 dd = __ldg(dr + j + B * s);
+          const float2 dd = dr[j + B * s];
           w[s].x = w[s].x + tstep * dd.x; w[s].y = w[s].y + tstep * dd.y;
         }
       }
@@ -198,6 +199,8 @@ __global__ void __launch_bounds__(256, 3) k_zinv256(Spectra<T> sp, EpiArgs<T> a,
   cplx<T>* stg = xbuf + (size_t)Z256::TEAMS * Z256::XP;
   const size_t row0 = (size_t)blockIdx.x * R;
   const size_t off = row0 * N;
+  for (int q = threadIdx.x; q < NH + H; q += blockDim.x) twN[q] = q < NH ? tw_n[q] : tw_h[q - NH];
+  dependency_wait();
   // spectra rows: tiled layout, contiguous per field (R NH complex, 16-byte
   // aligned since R is even); plane layout, runs of R rows per kz
   for (int f = 0; f < sp.nact; ++f) {
@@ -212,7 +215,6 @@ __global__ void __launch_bounds__(256, 3) k_zinv256(Spectra<T> sp, EpiArgs<T> a,
       cp_async_block16(stg + (size_t)f * R * NH, sp.s[sp.idx[f]] + row0 * NH, (size_t)R * NH * sizeof(cplx<T>));
     }
   }
-  for (int q = threadIdx.x; q < NH + H; q += blockDim.x) twN[q] = q < NH ? tw_n[q] : tw_h[q - NH];
   cp_async_commit();
   cp_async_wait<0>();
   __syncthreads();
@@ -262,7 +264,7 @@ __global__ void __launch_bounds__(256, 3) k_zinv256(Spectra<T> sp, EpiArgs<T> a,
     T po[R];                                           // P g_old, loaded ahead of the stores
     if (a.pyout) {
 #pragma unroll
-      for (int r = 0; r < R; ++r) po[r] = __ldg(a.pold + off + r * N + jt);
+      for (int r = 0; r < R; ++r) po[r] = a.pold[off + r * N + jt];
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) {
@@ -279,13 +281,13 @@ __global__ void __launch_bounds__(256, 3) k_zinv256(Spectra<T> sp, EpiArgs<T> a,
   const bool with_d = KIND == 1 || (KIND == 0 && a.mode == 1);
   const T* src0 = (EpiPoint<T, KIND>::mode(a) == 0 ? a.rho : a.psi) + off + jt;
   const T* dsrc = with_d ? a.d + off + jt : src0;
-  T xn = __ldg(src0), dn = with_d ? __ldg(dsrc) : (T)0;
+  T xn = src0[0], dn = with_d ? dsrc[0] : (T)0;
   const T* f0 = realf[0];
   const T* f2 = KIND ? reinterpret_cast<const T*>(stg + (size_t)R * NH) : realf[2];
   for (int r = 0; r < R; ++r) {
     const int qs = r * rp + jt, q = r * N + jt;
     const T x = xn, dd = dn;
-    if (r + 1 < R) { xn = __ldg(src0 + (r + 1) * N); if (with_d) dn = __ldg(dsrc + (r + 1) * N); }
+    if (r + 1 < R) { xn = src0[(r + 1) * N]; if (with_d) dn = dsrc[(r + 1) * N]; }
     if constexpr (KIND != 0) ep.point(a, x, dd, reinterpret_cast<const T*>(stg)[qs], (T)0, f2[qs], off + q, acc);
     else ep.point(a, x, dd, f0 ? f0[qs] : (T)0, realf[1] ? realf[1][qs] : (T)0, f2 ? f2[qs] : (T)0, off + q, acc);
   }
@@ -612,12 +614,13 @@ k_plane256cl(Spectra<T> sp, GArgs<T> g, const cplx<T>* __restrict__ tw_n) {
   const int kz = blockIdx.x / CL;
   const int fid = sp.idx[blockIdx.y];
   cplx<T>* gpl = sp.s[fid] + (size_t)kz * N * N + (size_t)c * N;   // row x = 8 b + c at gpl + 8 b N
+  tw[threadIdx.x] = tw_n[threadIdx.x];
+  dependency_wait();
   for (int q = threadIdx.x; q < ROWS * N / 2; q += blockDim.x) {   // 16-byte pieces
     const int b = q >> 7, y = (q & 127) * 2;
     cp_async<16>(slice + b * P + y, gpl + (size_t)b * CL * N + y, true);
   }
   cp_async_commit();
-  tw[threadIdx.x] = tw_n[threadIdx.x];
   cp_async_wait<0>();
   __syncthreads();
   const int team = threadIdx.x >> 4, j = threadIdx.x & 15, t = threadIdx.x;
