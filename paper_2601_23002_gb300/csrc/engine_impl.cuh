@@ -124,7 +124,7 @@ class Engine : public IEngine {
   size_t nbytes = 0;
   C *tw_n = nullptr, *tw_h = nullptr;
   double* Kd = nullptr;
-  double2* sf_tab = nullptr;   // per m^2: (v~/Omega per unit charge, Ewald reciprocal weight)
+  SfEntry<T>* sf_tab = nullptr;   // per m^2: v~/Omega per unit charge, Ewald reciprocal weight
   T* Kt = nullptr;
   C* vloc = nullptr;
   C* Sg = nullptr;
@@ -669,15 +669,15 @@ class Engine : public IEngine {
       // weight (2 pi/Omega) exp(-G^2/(4 eta^2))/G^2
       const double tp2d = (2.0 * kPi / L) * (2.0 * kPi / L);
       const double eta = ewald_eta();
-      std::vector<double2> tab(nm2);
+      std::vector<SfEntry<T>> tab(nm2);
       for (int m2 = 0; m2 < nm2; ++m2) {
         const double G2 = tp2d * m2;
-        if (m2 == 0) { tab[m2] = make_double2(kPi * cs.rc * cs.rc / Omega, 0.0); continue; }
-        tab[m2] = make_double2(-4.0 * kPi * std::exp(-G2 * cs.rc * cs.rc / 4.0) / G2 / Omega,
+        if (m2 == 0) { tab[m2] = SfEntry<T>::make(kPi * cs.rc * cs.rc / Omega, 0.0); continue; }
+        tab[m2] = SfEntry<T>::make(-4.0 * kPi * std::exp(-G2 * cs.rc * cs.rc / 4.0) / G2 / Omega,
                                2.0 * kPi / Omega * std::exp(-G2 / (4.0 * eta * eta)) / G2);
       }
       if ((rc = alloc(&sf_tab, nm2))) return rc;
-      OFDFT_CK(cudaMemcpyAsync(sf_tab, tab.data(), nm2 * sizeof(double2), cudaMemcpyHostToDevice, st));
+      OFDFT_CK(cudaMemcpyAsync(sf_tab, tab.data(), nm2 * sizeof(SfEntry<T>), cudaMemcpyHostToDevice, st));
       // row pairs with a^2 + b^2 inside the local and Ewald range, and out to
       // |m|^2 = 600 for the S_ei shells
       sf_m2 = 0;
@@ -874,9 +874,8 @@ class Engine : public IEngine {
     return OFDFT_OK;
   }
 
-  // k_struct with the largest thread tile that still gives every SM two blocks
-  // (a block waits for its staged ions at two barriers per chunk; the other one
-  // works meanwhile): FP32 2 x 4 (64 accumulators), 2 x 2, 1 x 2; small grids 1 x 1.
+  // k_struct with the largest thread tile that still gives most SMs a block:
+  // FP32 2 x 4 (64 accumulators), 2 x 2, 1 x 2; small grids 1 x 1.
   int launch_struct(const StructOut<T>& so, const double* zw, int full, cudaStream_t st) {
     const int2* rows = full ? nullptr : sf_rows;
     const int nrows = full ? nh * nh : sf_nrows;
@@ -886,6 +885,7 @@ class Engine : public IEngine {
       const int ctiles = (nh + TC * 64 - 1) / (TC * 64);        // at most 64 threads along kz
       const int CT = (nh + TC * ctiles - 1) / (TC * ctiles);
       const int RT = NT / CT * TR;
+      if (RT > 32 * struct_nr(TR, TC)) return OFDFT_OK;
       const int g = (nrows + RT - 1) / RT;
       if (g * ctiles < least) return OFDFT_OK;
       const size_t sm = struct_smem<T, TR, TC, NT>(CT);
@@ -895,8 +895,8 @@ class Engine : public IEngine {
     };
     using std::integral_constant;
     int rc = OFDFT_OK;
-    if constexpr (sizeof(T) == 4) rc = go(integral_constant<int, 2>{}, integral_constant<int, 4>{}, integral_constant<int, 256>{}, 2 * nsm - 8);
-    if (!rc && !done) rc = go(integral_constant<int, 2>{}, integral_constant<int, 2>{}, integral_constant<int, 256>{}, 2 * nsm - 8);
+    if constexpr (sizeof(T) == 4) rc = go(integral_constant<int, 2>{}, integral_constant<int, 4>{}, integral_constant<int, 256>{}, (nsm * 4) / 5);
+    if (!rc && !done) rc = go(integral_constant<int, 2>{}, integral_constant<int, 2>{}, integral_constant<int, 256>{}, (nsm * 4) / 5);
     if (!rc && !done) rc = go(integral_constant<int, 1>{}, integral_constant<int, 2>{}, integral_constant<int, 128>{}, nsm);
     if (!rc && !done) rc = go(integral_constant<int, 1>{}, integral_constant<int, 1>{}, integral_constant<int, 64>{}, 0);
     return rc;
@@ -914,7 +914,7 @@ class Engine : public IEngine {
     ew_eta = eta; ew_rcut = rcut; ew_nimg = nimg_mi;
     const long ncomb = (long)nion * (nion / 2 + 1) * (2 * nimg_mi + 1) * (2 * nimg_mi + 1) * (2 * nimg_mi + 1);
     const int gb = (int)std::min<long>(2L * nsm, (ncomb + 255) / 256);
-    const int gp = std::min(2 * nsm, (nion * 3 * nh + 255) / 256);
+    const int gp = std::min(4 * nsm, (nion * 3 + 7) / 8);
     double* real = partials + partials_cap - gb;         // behind k_struct's partials
     OFDFT_RUN("k_ions", st, (double)nion * 3 * n * sizeof(C), k_ions<T><<<gb + gp, 256, 0, st>>>(pos_d, Z_d, nion, n, L, phases, eta, rcut, nimg_mi, gb, real));
     const int full = S_out != nullptr;
@@ -1628,8 +1628,10 @@ int Engine<T>::forces(const void* rho, double* f_out_h, void* stream_) {
   const int fld[1] = {0};
   if ((rc = forward((const T*)rho, fld, 1, std::min(h, (int)std::sqrt((double)f_m2)), view, st))) return rc;
   OFDFT_RUN("k_forces_q", st, (double)f_nk * 32 * (8 * sizeof(C) + 4 * sizeof(C)), k_forces_q<T><<<std::min(16 * nsm, (f_nk + 3) / 4), 128, 0, st>>>(spec[0], view, SZg, f_rows, f_nrows, f_tk, f_ntile, f_gf, f_m2, n, 1.0 / (double)N, f_qq));
-  // several blocks per ion (about 4 per SM in all), shares added in a fixed order
-  int nsplit = std::max(1, std::min(64, (4 * nsm + nion - 1) / nion));
+  // blocks per ion: about 4 per SM in all, but at least 256 (J, image) each, so
+  // that the few in range fill a warp; shares added in a fixed order
+  const long comb = (long)nion * (2 * ew_nimg + 1) * (2 * ew_nimg + 1) * (2 * ew_nimg + 1);
+  int nsplit = (int)std::max<long>(1, std::min<long>({64, (4 * nsm + nion - 1) / nion, comb / 256}));
   while (nsplit > 1 && (size_t)nion * nsplit * 3 > partials_cap) --nsplit;
   if ((size_t)nion * nsplit * 3 > partials_cap) { set_error("forces: too many ions for the scratch"); return OFDFT_ERR_INVALID; }
   constexpr int TI = sizeof(T) == 4 ? 4 : 2;

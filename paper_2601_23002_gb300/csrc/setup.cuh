@@ -11,23 +11,36 @@ namespace ofdft {
 // exp(-i G.R) = e_x(m_x) e_y(m_y) e_z(m_z) with e_d(m) = exp(-2 pi i m R_d / L);
 // ph[(I*3 + d)*n + k] holds them (k in FFT order), formed in FP64 and rounded to
 // the plan's type; one sine and cosine per |m|, the negative m by conjugation.
+// One warp per (ion, axis): its lanes evaluate e(0..15) and e(16 k), k = 0..15
+// (one FP64 sine and cosine each; 65 of them per axis at 128^3 kept the FP64 pipe
+// busy for 13 us with 300 ions), and e(16 k + l) = e(16 k) e(l).
 template <typename T>
 __device__ __forceinline__ void phases_part(const double* __restrict__ pos, int n_ion, int n, double L,
                                             cplx<T>* __restrict__ ph, int block, int blocks) {
-  const int h = n / 2 + 1;
-  const int tot = n_ion * 3 * h;
-  for (int q = block * blockDim.x + threadIdx.x; q < tot; q += blocks * blockDim.x) {
-    const int m = q % h, d = (q / h) % 3, I = q / (3 * h);
-    double f = pos[I * 3 + d] / L;
+  const int h = n / 2 + 1, lane = threadIdx.x & 31;
+  const int per = blockDim.x >> 5;
+  for (int q = block * per + (threadIdx.x >> 5); q < n_ion * 3; q += blocks * per) {
+    double f = pos[q] / L;
     f -= floor(f);                       // wrap into [0, 1)
     // angle = -2 pi m f; reduce m f modulo 1 before the trig call
-    double mf = (double)m * f;
+    const int m0 = lane < 16 ? lane : (lane - 16) * 16;
+    double mf = (double)m0 * f;
     mf -= rint(mf);
-    double s, c;
-    sincospi(-2.0 * mf, &s, &c);
-    cplx<T>* o = ph + (size_t)(I * 3 + d) * n;
-    if (2 * m < n) o[m] = mk<T>((T)c, (T)s);
-    if (m > 0) o[n - m] = mk<T>((T)c, (T)-s);        // m = n/2 of even n is stored as -n/2
+    double s0, c0;
+    sincospi(-2.0 * mf, &s0, &c0);
+    cplx<T>* o = ph + (size_t)q * n;
+    for (int mb = 0; mb < h; mb += 32) {
+      const int m = mb + lane;
+      const int k = min(m >> 4, 15), l = m - 16 * k;     // m <= 256: l = 16 only with k = 15
+      const int ll = l < 16 ? l : 17;
+      const double ck = __shfl_sync(0xffffffffu, c0, 16 + k), sk = __shfl_sync(0xffffffffu, s0, 16 + k);
+      const double cl = __shfl_sync(0xffffffffu, c0, ll & 31), sl = __shfl_sync(0xffffffffu, s0, ll & 31);
+      double c = cl, s = sl;
+      if (k > 0) { c = ck * cl - sk * sl; s = ck * sl + sk * cl; }
+      if (m >= h) continue;
+      if (2 * m < n) o[m] = mk<T>((T)c, (T)s);
+      if (m > 0) o[n - m] = mk<T>((T)c, (T)-s);          // m = n/2 of even n is stored as -n/2
+    }
   }
 }
 
@@ -41,18 +54,34 @@ __device__ __forceinline__ void phases_part(const double* __restrict__ pos, int 
 // on the full 128^3 half spectrum; the FP32 pipe needs 17 us for these sums.)
 // A thread owns TR row pairs (a, b) and TC kz; the ions go in chunks of CH whose
 // row products and kz phases are staged in shared memory, so a chunk's step
-// reads TR + TC/2 16-byte groups for 8 TR TC multiply-adds.
+// reads TR + TC/2 16-byte groups for 8 TR TC multiply-adds.  Two stages: the next
+// chunk's kz phases are copied asynchronously and its row phases loaded before
+// the current chunk's sums, one barrier per chunk.
 // rows: (a, b) list, or nullptr for all 0 <= a, b <= n/2.
 // zw: weights (nullptr: 1).  Outputs (any may be null): S, S2 (a second copy),
 // SZ = zs S, V_loc = f.x SZ, and per block the Ewald reciprocal sum
 // sum w f.y |SZ|^2 over the entries of rows with |G|^2 <= g2rows:
-//   sf_tab[m^2] = f = (v~(G)/Omega per unit charge, (2 pi/Omega) exp(-G^2/(4 eta^2))/G^2),
-// tabulated once per plan in FP64.
+//   f = (v~(G)/Omega per unit charge, (2 pi/Omega) exp(-G^2/(4 eta^2))/G^2) by m^2,
+// tabulated once per plan.  FP32 plans hold the first as two floats, so that V_loc
+// is the FP32 rounding of the exact product as before without FP64 conversions and
+// products (a third of the kernel's time on the FP64 pipe), and sum the second in
+// compensated FP32: |SZ|^2 carries 3e-7 already.
 // grid: (row tiles, kz tiles); CT threads along kz.
+template <typename T> struct SfEntry;
+template <> struct alignas(16) SfEntry<float> {
+  float v, vlo, e, pad;
+  static SfEntry make(double a, double b) { return {(float)a, (float)(a - (double)(float)a), (float)b, 0.f}; }
+  __device__ __forceinline__ float vloc(float z) const { return fmaf(v, z, vlo * z); }
+};
+template <> struct alignas(16) SfEntry<double> {
+  double v, e;
+  static SfEntry make(double a, double b) { return {a, b}; }
+  __device__ __forceinline__ double vloc(double z) const { return v * z; }
+};
 template <typename T> struct StructOut {
   cplx<T>*S, *S2, *SZ, *vloc;
   double zs;
-  const double2* sf_tab;
+  const SfEntry<T>* sf_tab;
   double m2rows;              // vloc and the Ewald sum: rows with a^2 + b^2 <= m2rows
   double* ew;
   // when set, the last block writes res[0] = sum of ew, res[1] = sum of the
@@ -62,20 +91,23 @@ template <typename T> struct StructOut {
   unsigned int* counter;
 };
 template <typename T> struct alignas(16) Quad { T a, b, c, d; };
-constexpr int kStructCH = 16;
+template <typename T> struct StructCH { static constexpr int v = sizeof(T) == 4 ? 16 : 8; };   // ions per chunk
+// rows a lane of the staging holds: a block has at most 32 of these rows
+__host__ __device__ constexpr int struct_nr(int TR, int TC) { return TR * TC == 4 ? 2 : 1; }
 template <typename T, int TR, int TC, int NT>
 constexpr size_t struct_smem(int CT) {
-  return (size_t)kStructCH * ((size_t)CT * TC * sizeof(cplx<T>) + (size_t)(NT / CT) * TR * sizeof(Quad<T>));
+  return 2 * (size_t)StructCH<T>::v * ((size_t)CT * TC * sizeof(cplx<T>) + (size_t)(NT / CT) * TR * sizeof(Quad<T>));
 }
 template <typename T, int TR, int TC, int NT>
 __global__ void __launch_bounds__(NT) k_struct(const cplx<T>* __restrict__ ph, const double* __restrict__ zw, int n_ion,
                                                int n, const int2* __restrict__ rows, int nrows, int CT, StructOut<T> o) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[32];
+  constexpr int CH = StructCH<T>::v;
   const int h = n / 2, nh = h + 1;
   const int RB = NT / CT, RT = RB * TR, CC = CT * TC;    // row threads, rows and columns of the block
-  Quad<T>* sr = reinterpret_cast<Quad<T>*>(smem_raw);    // [CH][RT]
-  cplx<T>* se = reinterpret_cast<cplx<T>*>(sr + (size_t)kStructCH * RT);   // [CH][CC]
+  Quad<T>* sr = reinterpret_cast<Quad<T>*>(smem_raw);    // [2][CH][RT]
+  cplx<T>* se = reinterpret_cast<cplx<T>*>(sr + (size_t)2 * CH * RT);   // [2][CH][CC]
   const int tid = threadIdx.x, ct = tid % CT, rt = tid / CT;
   const bool act = rt < RB;
   const int col0 = blockIdx.y * CC;
@@ -90,43 +122,80 @@ __global__ void __launch_bounds__(NT) k_struct(const cplx<T>* __restrict__ ph, c
     for (int j = 0; j < TC; ++j)
 #pragma unroll
       for (int k = 0; k < 8; ++k) acc[i][j][k] = 0;
-  for (int I0 = 0; I0 < n_ion; I0 += kStructCH) {
-    const int cnt = min(kStructCH, n_ion - I0);
-    __syncthreads();
-    for (int q = tid; q < cnt * CC; q += NT) {
-      const int c = q / CC, kz = col0 + q - c * CC;
-      cplx<T> e = mk<T>((T)0, (T)0);
-      if (kz < nh) {
-        e = ph[((size_t)(I0 + c) * 3 + 2) * n + kz];
-      }
-      se[q] = e;
+  // Staging.  kz phases: the block's columns of an ion's z row by its warps in
+  // turn (columns past nh stay zero).  Row products: a warp per ion as well, its
+  // lanes over the block's rows; lane l holds row l of the block (l < RT <= 32 NR).
+  constexpr int NW = NT / 32, NR = struct_nr(TR, TC);
+  const int lane = tid & 31, wid = tid >> 5;
+  int ra[NR], rb[NR];                                    // this lane's rows (a < 0: none)
+#pragma unroll
+  for (int u = 0; u < NR; ++u) {
+    const int l = lane + 32 * u, r = blockIdx.x * RT + l;
+    ra[u] = -1; rb[u] = 0;
+    if (l < RT && r < nrows) row_of(r, ra[u], rb[u]);
+  }
+  for (int q = tid; q < 2 * CH * CC; q += NT) se[q] = mk<T>((T)0, (T)0);
+  __syncthreads();
+  const int ncol = min(CC, nh - col0);
+  auto stage_z = [&](int I0, int buf) {
+    for (int c = wid; c < CH && I0 + c < n_ion; c += NW) {
+      const cplx<T>* p = ph + ((size_t)(I0 + c) * 3 + 2) * n + col0;
+      cplx<T>* d = se + ((size_t)buf * CH + c) * CC;
+      for (int k = lane; k < ncol; k += 32) cp_async_c(d + k, p + k, true);
     }
-    for (int q = tid; q < cnt * RT; q += NT) {
-      const int c = q / RT, r = blockIdx.x * RT + q - c * RT;
-      Quad<T> v{0, 0, 0, 0};
-      if (r < nrows) {
-        int a, b;
-        row_of(r, a, b);
-        const cplx<T>* p = ph + (size_t)(I0 + c) * 3 * n;
-        cplx<T> ex = p[a], ey = p[n + b];
-        if (2 * a == n) ex.y = -ex.y;                    // index n/2 holds -n/2
-        if (2 * b == n) ey.y = -ey.y;
-        if (zw) { const T z = (T)zw[I0 + c]; ex.x *= z; ex.y *= z; }
-        v.a = ex.x * ey.x - ex.y * ey.y; v.b = ex.x * ey.y + ex.y * ey.x;
-        v.c = ex.x * ey.x + ex.y * ey.y; v.d = ex.y * ey.x - ex.x * ey.y;
-      }
-      sr[q] = v;
+    cp_async_commit();
+  };
+  constexpr int CW = (CH + NW - 1) / NW;                 // ions per warp and chunk
+  cplx<T> vx[CW][NR], vy[CW][NR];
+  auto load_rows = [&](int I0) {
+#pragma unroll
+    for (int w = 0; w < CW; ++w) {
+      const int I = I0 + wid + NW * w;
+      if (wid + NW * w >= CH || I >= n_ion) continue;
+      const cplx<T>* p = ph + (size_t)I * 3 * n;
+#pragma unroll
+      for (int u = 0; u < NR; ++u)
+        if (ra[u] >= 0) { vx[w][u] = p[ra[u]]; vy[w][u] = p[n + rb[u]]; }
     }
-    __syncthreads();
+  };
+  auto store_rows = [&](int I0, int buf) {
+#pragma unroll
+    for (int w = 0; w < CW; ++w) {
+      const int c = wid + NW * w, I = I0 + c;
+      if (c >= CH || I >= n_ion) continue;
+      const T z = zw ? (T)zw[I] : (T)1;
+#pragma unroll
+      for (int u = 0; u < NR; ++u) {
+        if (ra[u] < 0) continue;
+        cplx<T> ex = vx[w][u], ey = vy[w][u];
+        if (2 * ra[u] == n) ex.y = -ex.y;                // index n/2 holds -n/2
+        if (2 * rb[u] == n) ey.y = -ey.y;
+        ex.x *= z; ex.y *= z;
+        sr[((size_t)buf * CH + c) * RT + lane + 32 * u] =
+            Quad<T>{ex.x * ey.x - ex.y * ey.y, ex.x * ey.y + ex.y * ey.x, ex.x * ey.x + ex.y * ey.y, ex.y * ey.x - ex.x * ey.y};
+      }
+    }
+  };
+  stage_z(0, 0);
+  load_rows(0);
+  store_rows(0, 0);
+  cp_async_wait<0>();
+  __syncthreads();
+  for (int I0 = 0, buf = 0; I0 < n_ion; I0 += CH, buf ^= 1) {
+    const int cnt = min(CH, n_ion - I0);
+    const bool more = I0 + CH < n_ion;
+    if (more) { stage_z(I0 + CH, buf ^ 1); load_rows(I0 + CH); }
     if (act) {
+      const Quad<T>* pr = sr + (size_t)buf * CH * RT + rt;
+      const cplx<T>* pe = se + (size_t)buf * CH * CC + ct;
 #pragma unroll 2
       for (int c = 0; c < cnt; ++c) {
         Quad<T> p[TR];
         cplx<T> e[TC];
 #pragma unroll
-        for (int i = 0; i < TR; ++i) p[i] = sr[c * RT + rt + RB * i];
+        for (int i = 0; i < TR; ++i) p[i] = pr[c * RT + RB * i];
 #pragma unroll
-        for (int j = 0; j < TC; ++j) e[j] = se[c * CC + ct + CT * j];
+        for (int j = 0; j < TC; ++j) e[j] = pe[c * CC + CT * j];
 #pragma unroll
         for (int i = 0; i < TR; ++i)
 #pragma unroll
@@ -139,8 +208,10 @@ __global__ void __launch_bounds__(NT) k_struct(const cplx<T>* __restrict__ ph, c
           }
       }
     }
+    if (more) { store_rows(I0 + CH, buf ^ 1); cp_async_wait<0>(); }
+    __syncthreads();
   }
-  double ew = 0;
+  Acc<T> ewa;
 #pragma unroll
   for (int i = 0; i < TR; ++i) {
     const int r = blockIdx.x * RT + rt + RB * i;
@@ -154,8 +225,9 @@ __global__ void __launch_bounds__(NT) k_struct(const cplx<T>* __restrict__ ph, c
       const int kz = col0 + ct + CT * j;
       if (kz >= nh) continue;
       const T(&x)[8] = acc[i][j];
-      const double2 f = inside ? o.sf_tab[a * a + b * b + kz * kz] : make_double2(0.0, 0.0);
-      const double w = (kz == 0 || 2 * kz == n) ? 1.0 : 2.0;
+      SfEntry<T> f{};
+      if (inside) f = o.sf_tab[a * a + b * b + kz * kz];
+      const T w = (kz == 0 || 2 * kz == n) ? (T)1 : (T)2;
       auto put = [&](int kx, int ky, T re, T im) {
         const size_t at = ((size_t)kx * n + ky) * nh + kz;
         const cplx<T> s = mk<T>(re, im);
@@ -166,8 +238,8 @@ __global__ void __launch_bounds__(NT) k_struct(const cplx<T>* __restrict__ ph, c
           const cplx<T> sz = mk<T>(z * re, z * im);
           o.SZ[at] = sz;
           if (inside) {
-            o.vloc[at] = mk<T>((T)(f.x * (double)sz.x), (T)(f.x * (double)sz.y));
-            ew += w * f.y * ((double)sz.x * (double)sz.x + (double)sz.y * (double)sz.y);
+            o.vloc[at] = mk<T>(f.vloc(sz.x), f.vloc(sz.y));
+            ewa.add(w * f.e * (sz.x * sz.x + sz.y * sz.y));
           } else {
             o.vloc[at] = mk<T>((T)0, (T)0);
           }
@@ -179,7 +251,7 @@ __global__ void __launch_bounds__(NT) k_struct(const cplx<T>* __restrict__ ph, c
       if (ma && pb) put(n - a, b, x[4] + x[5], x[6] - x[7]);
     }
   }
-  double v[1] = {ew}, out[1];
+  double v[1] = {ewa.get()}, out[1];
   block_sum<1>(v, red, out);
   if (tid == 0) o.ew[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = out[0];
   const int nb = gridDim.x * gridDim.y;
@@ -202,15 +274,58 @@ __global__ void __launch_bounds__(NT) k_struct(const cplx<T>* __restrict__ ph, c
 // |a| <= nimg = ceil(rcut/L + 1/2) - 1 per axis are all: none but the pair itself
 // once L >= 2 rcut.  (Shifts of +-1 were walked for every pair: 27 times the
 // distances, 152 us for 300 ions in a 28-bohr cell.)  A block walks its share of
-// the (pair, image) combinations 256 at a time, compacts the ones inside rcut
-// into shared memory (warp ballots and a block prefix, in combination order) and
-// only then evaluates erfc, on dense warps (partial[block]; fixed order).
+// the (pair, image) combinations blockDim at a time, screens them in FP32 with a
+// margin, compacts the ones that may be inside rcut into shared memory (warp
+// ballots and a block prefix, in combination order), and only these, on dense
+// warps, are measured and evaluated in FP64 (partial[block]; fixed order).
+
+// Cells to shift a separation x by: nearest integer to x / L in FP32 where x is
+// good to 3e-4 bohr there (|x| < 4e3), else in FP64.  Screening and evaluation use
+// the same shift, so a pair at half a cell has one and the same image a = 0.
+static __device__ __forceinline__ float cell_shift(double x, double L, float iL) {
+  const float xf = (float)x;
+  return fabsf(xf) < 4e3f ? rintf(xf * iL) : (float)rint(x / L);
+}
+// The squared distance in FP32 at image (a, b, c), each axis good to 1e-3 bohr.
+static __device__ __forceinline__ bool maybe_inside(const double* p, const double* q, double L, float Lf, float iL,
+                                                    int a, int b, int c, float rc2m) {
+  const int im[3] = {a, b, c};
+  float r2 = 0;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const double x = p[d] - q[d];
+    const float k = cell_shift(x, L, iL), xf = (float)x;
+    const float v = fabsf(xf) < 4e3f ? fmaf(-Lf, k, xf) : (float)(x - L * (double)k);
+    const float u = v + (float)im[d] * Lf;
+    r2 += u * u;
+  }
+  return r2 < rc2m;
+}
+// the displacement at that image in FP64
+static __device__ __forceinline__ double3 displacement(const double* p, const double* q, double L, float iL, int a,
+                                                       int b, int c) {
+  const double x = p[0] - q[0], y = p[1] - q[1], z = p[2] - q[2];
+  return make_double3(x + L * (double)(a - cell_shift(x, L, iL)), y + L * (double)(b - cell_shift(y, L, iL)),
+                      z + L * (double)(c - cell_shift(z, L, iL)));
+}
+// Slots, in thread order, of the threads with `in` among blockDim <= 256; the
+// count in total.  Between two block barriers.
+static __device__ __forceinline__ int compact_slot(bool in, int* wcount, int* total) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const unsigned bal = __ballot_sync(0xffffffffu, in);
+  if (lane == 0) wcount[wid] = __popc(bal);
+  __syncthreads();
+  int base = 0, tot = 0;
+  for (int w = 0; w < nw; ++w) { if (w == wid) base = tot; tot += wcount[w]; }
+  *total = tot;
+  return base + __popc(bal & ((1u << lane) - 1u));
+}
+
 static __device__ __forceinline__ void ewald_real_part(const double* __restrict__ pos, const double* __restrict__ Z,
                                                        int n_ion, double L, double eta, double rcut, int nimg,
                                                        double* __restrict__ partial, int block, int blocks) {
   __shared__ double red[32];
-  __shared__ double sr[256], sz[256];
-  __shared__ int wcount[8], wbase[8], total;
+  __shared__ int list[256], wcount[8];
   const int side = 2 * nimg + 1;
   const int nim3 = side * side * side;
   const int nd = n_ion / 2 + 1;
@@ -218,41 +333,36 @@ static __device__ __forceinline__ void ewald_real_part(const double* __restrict_
   const long per = (tot + blocks - 1) / blocks;
   const long q0 = (long)block * per, q1 = min(tot, q0 + per);
   const double rc2 = rcut * rcut;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const float rc2m = (float)((rcut + 4e-3) * (rcut + 4e-3)), Lf = (float)L, iLf = 1.0f / Lf;
+  auto decode = [&](long q, int& I, int& J, int& d, int& a, int& b, int& c) {
+    const long p = q / nim3;
+    const int im = (int)(q - p * nim3);
+    I = (int)(p / nd); d = (int)(p - (long)I * nd);
+    J = I + d < n_ion ? I + d : I + d - n_ion;
+    a = im / (side * side) - nimg; b = (im / side) % side - nimg; c = im % side - nimg;
+  };
   double acc = 0;
+  int I, J, d, a, b, c;
   for (long base = q0; base < q1; base += blockDim.x) {
     const long q = base + threadIdx.x;
-    bool inside = false;
-    double r = 0, zz = 0;
+    bool in = false;
     if (q < q1) {
-      const long p = q / nim3;
-      const int im = (int)(q - p * nim3);
-      const int I = (int)(p / nd), d = (int)(p % nd);
-      const int J = I + d < n_ion ? I + d : I + d - n_ion;
-      const int a = im / (side * side) - nimg, b = (im / side) % side - nimg, c = im % side - nimg;
-      double x = pos[I * 3] - pos[J * 3], y = pos[I * 3 + 1] - pos[J * 3 + 1], z = pos[I * 3 + 2] - pos[J * 3 + 2];
-      const double iL = 1.0 / L;     // uniform: folded to one reciprocal per thread
-      x -= L * rint(x * iL); y -= L * rint(y * iL); z -= L * rint(z * iL);
-      x += a * L; y += b * L; z += c * L;
-      const double r2 = x * x + y * y + z * z;
-      inside = r2 > 1e-24 && r2 < rc2;
-      if (inside) { r = sqrt(r2); zz = Z[I] * Z[J] * (d == 0 || 2 * d == n_ion ? 0.5 : 1.0); }
+      decode(q, I, J, d, a, b, c);
+      in = maybe_inside(pos + I * 3, pos + J * 3, L, Lf, iLf, a, b, c, rc2m);
     }
-    const unsigned bal = __ballot_sync(0xffffffffu, inside);
-    if (lane == 0) wcount[wid] = __popc(bal);
+    int total;
+    const int slot = compact_slot(in, wcount, &total);
+    if (in) list[slot] = threadIdx.x;
     __syncthreads();
-    if (threadIdx.x == 0) {
-      int s = 0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { wbase[w] = s; s += wcount[w]; }
-      total = s;
+    if ((int)threadIdx.x < total) {
+      decode(base + list[threadIdx.x], I, J, d, a, b, c);
+      const double3 x = displacement(pos + I * 3, pos + J * 3, L, iLf, a, b, c);
+      const double r2 = x.x * x.x + x.y * x.y + x.z * x.z;
+      if (r2 > 1e-24 && r2 < rc2) {
+        const double r = sqrt(r2);
+        acc += Z[I] * Z[J] * (d == 0 || 2 * d == n_ion ? 0.5 : 1.0) * erfc(eta * r) / r;
+      }
     }
-    __syncthreads();
-    if (inside) {
-      const int slot = wbase[wid] + __popc(bal & ((1u << lane) - 1u));
-      sr[slot] = r; sz[slot] = zz;
-    }
-    __syncthreads();
-    if ((int)threadIdx.x < total) acc += sz[threadIdx.x] * erfc(eta * sr[threadIdx.x]) / sr[threadIdx.x];
     __syncthreads();
   }
   double v[1] = {acc}, out[1];
@@ -535,65 +645,53 @@ struct EwaldForceArgs {
   double* part;
 };
 static __device__ __forceinline__ void ewald_force_part(const EwaldForceArgs& w, int n_ion, int block) {
-  const double *pos = w.pos, *Z = w.Z;
-  const double L = w.L, eta = w.eta, rcut = w.rcut;
-  const int nimg = w.nimg, nsplit = w.nsplit;
-  double* part = w.part;
   __shared__ double red[3 * 32];
-  __shared__ double sx[128], sy[128], sz[128], sq[128];
-  __shared__ int wcount[8], wbase[8], total;
-  const int I = block / nsplit, sh = block % nsplit;
-  const int side = 2 * nimg + 1;
+  __shared__ int list[256], wcount[8];
+  const int I = block / w.nsplit, sh = block % w.nsplit;
+  const int side = 2 * w.nimg + 1;
   const int nim3 = side * side * side;
   const long tot = (long)n_ion * nim3;
-  const long per = (tot + nsplit - 1) / nsplit;
+  const long per = (tot + w.nsplit - 1) / w.nsplit;
   const long q0 = (long)sh * per, q1 = min(tot, q0 + per);
-  const double rc2 = rcut * rcut;
-  const double c2 = 2.0 * eta / 1.7724538509055160273;   // 2 eta / sqrt(pi)
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const double iL = 1.0 / L;
+  const double rc2 = w.rcut * w.rcut;
+  const double c2 = 2.0 * w.eta / 1.7724538509055160273;   // 2 eta / sqrt(pi)
+  const float rc2m = (float)((w.rcut + 4e-3) * (w.rcut + 4e-3)), Lf = (float)w.L, iLf = 1.0f / Lf;
+  auto decode = [&](long q, int& J, int& a, int& b, int& c) {
+    J = (int)(q / nim3);
+    const int im = (int)(q - (long)J * nim3);
+    a = im / (side * side) - w.nimg; b = (im / side) % side - w.nimg; c = im % side - w.nimg;
+  };
+  const double* pI = w.pos + I * 3;
   double f[3] = {0, 0, 0};
+  int J, a, b, c;
   for (long base = q0; base < q1; base += blockDim.x) {
     const long q = base + threadIdx.x;
-    bool inside = false;
-    double x = 0, y = 0, z = 0, r2 = 0;
+    bool in = false;
     if (q < q1) {
-      const int J = (int)(q / nim3), im = (int)(q % nim3);
-      const int a = im / (side * side) - nimg, b = (im / side) % side - nimg, c = im % side - nimg;
-      x = pos[I * 3] - pos[J * 3]; y = pos[I * 3 + 1] - pos[J * 3 + 1]; z = pos[I * 3 + 2] - pos[J * 3 + 2];
-      x -= L * rint(x * iL); y -= L * rint(y * iL); z -= L * rint(z * iL);
-      x += a * L; y += b * L; z += c * L;
-      r2 = x * x + y * y + z * z;
-      inside = r2 > 1e-24 && r2 < rc2;
-      if (inside) r2 = Z[I] * Z[J];     // reused below as the charge product
+      decode(q, J, a, b, c);
+      in = maybe_inside(pI, w.pos + J * 3, w.L, Lf, iLf, a, b, c, rc2m);
     }
-    const unsigned bal = __ballot_sync(0xffffffffu, inside);
-    if (lane == 0) wcount[wid] = __popc(bal);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int s = 0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { wbase[w] = s; s += wcount[w]; }
-      total = s;
-    }
-    __syncthreads();
-    if (inside) {
-      const int slot = wbase[wid] + __popc(bal & ((1u << lane) - 1u));
-      sx[slot] = x; sy[slot] = y; sz[slot] = z; sq[slot] = r2;
-    }
+    int total;
+    const int slot = compact_slot(in, wcount, &total);
+    if (in) list[slot] = threadIdx.x;
     __syncthreads();
     if ((int)threadIdx.x < total) {
-      const double dx = sx[threadIdx.x], dy = sy[threadIdx.x], dz = sz[threadIdx.x];
-      const double rr = dx * dx + dy * dy + dz * dz, r = sqrt(rr);
-      const double s = sq[threadIdx.x] * (erfc(eta * r) / rr + c2 * exp(-eta * eta * rr) / r) / r;
-      f[0] += s * dx; f[1] += s * dy; f[2] += s * dz;
+      decode(base + list[threadIdx.x], J, a, b, c);
+      const double3 x = displacement(pI, w.pos + J * 3, w.L, iLf, a, b, c);
+      const double rr = x.x * x.x + x.y * x.y + x.z * x.z;
+      if (rr > 1e-24 && rr < rc2) {
+        const double r = sqrt(rr);
+        const double s = w.Z[I] * w.Z[J] * (erfc(w.eta * r) / rr + c2 * exp(-w.eta * w.eta * rr) / r) / r;
+        f[0] += s * x.x; f[1] += s * x.y; f[2] += s * x.z;
+      }
     }
     __syncthreads();
   }
   double o[3];
   block_sum<3>(f, red, o);
   if (threadIdx.x == 0) {
-    part[(size_t)block * 3 + 0] = o[0]; part[(size_t)block * 3 + 1] = o[1];
-    part[(size_t)block * 3 + 2] = o[2];
+    double* part = w.part + (size_t)block * 3;
+    part[0] = o[0]; part[1] = o[1]; part[2] = o[2];
   }
 }
 

@@ -69,3 +69,26 @@ def test_ewald_and_forces(n, L, n_ion, two):
     if math.pi * n / L > 12.6:
         fo = oracle_forces(cell, rho)
         assert np.max(np.abs(f - fo)) <= 1e-10 * max(1.0, np.max(np.abs(fo)))
+
+
+# Positions outside [0, L) are wrapped: the same energy and forces (rounding of
+# x + k L: 1e-16 |k| L in the positions times forces of a few hartree/bohr).
+@pytest.mark.gpu
+@pytest.mark.parametrize("shift", [3, -700, 90000])
+def test_unwrapped_positions(shift):
+    L, n = 9.0, 36
+    Z, pos = ions(6, L, True)
+    pos[1] = pos[0] + [L / 2, 0.0, 0.0]              # a pair at half a cell
+    rho = torch.full((n ** 3,), float(np.sum(Z)) / L ** 3, dtype=torch.float64, device="cuda")
+    got = []
+    for s in (0, shift):
+        p = pos.copy()
+        p[::2, 0] += s * L
+        p[1::3, 2] -= s * L
+        plan = Plan(L, n, Z, 0.4, precision="fp64")
+        plan.structure_factor(p)
+        got.append((plan.energy_potential(rho)["E_ion"], plan.forces(rho)))
+        plan.close()
+    tol = 1e-11 + 1e-14 * abs(shift) * L
+    assert abs(got[0][0] - got[1][0]) <= tol * 100
+    assert np.max(np.abs(got[0][1] - got[1][1])) <= tol * 100
