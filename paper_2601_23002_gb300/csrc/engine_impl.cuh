@@ -6,8 +6,8 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <map>
 #include <mutex>
-#include <set>
 #include <string>
 #include <utility>
 #include <vector>
@@ -751,16 +751,18 @@ class Engine : public IEngine {
     // memory; set once per (device, kernel) for the process (plan creation
     // stays cheap for the serving loop), after checking this plan's need
     static std::mutex mu;
-    static std::set<std::pair<int, const void*>> done;
+    static std::map<std::pair<int, const void*>, int> done;      // its dynamic limit
     auto raise = [&](const void* f, size_t need) -> int {
       std::lock_guard<std::mutex> lock(mu);
-      cudaFuncAttributes fa;
-      OFDFT_CK(cudaFuncGetAttributes(&fa, f));
-      const int dyn = lim - (int)fa.sharedSizeBytes;
-      if (dyn < (int)need) { set_error("grid too large for shared memory"); return OFDFT_ERR_INVALID; }
-      if (done.count({dev, f})) return OFDFT_OK;
-      OFDFT_CK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-      done.insert({dev, f});
+      auto it = done.find({dev, f});
+      if (it == done.end()) {
+        cudaFuncAttributes fa;
+        OFDFT_CK(cudaFuncGetAttributes(&fa, f));
+        const int dyn = lim - (int)fa.sharedSizeBytes;
+        OFDFT_CK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
+        it = done.emplace(std::make_pair(dev, f), dyn).first;
+      }
+      if (it->second < (int)need) { set_error("grid too large for shared memory"); return OFDFT_ERR_INVALID; }
       return OFDFT_OK;
     };
     int rc;

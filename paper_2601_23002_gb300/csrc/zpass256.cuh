@@ -22,7 +22,7 @@
 // rounding; the parity tests run both against the oracle.
 #pragma once
 #include <cooperative_groups.h>
-#include "passes.cuh"
+#include "cpass.cuh"
 
 namespace ofdft {
 
@@ -31,7 +31,7 @@ struct Z256 {
   static constexpr int A = 16, B = 8;                  // H = A * B
   static constexpr int TEAM = B;                       // threads per row transform
   static constexpr int TEAMS = 256 / TEAM;             // per 256-thread block
-  static constexpr int XP = H + H / A;                 // exchange buffer per team (padded)
+  static constexpr int XP = H + H / A + 1;             // exchange buffer per team (padded; odd)
   static __host__ __device__ constexpr int xpos(int e) { return e + e / A; }
 };
 
@@ -107,11 +107,12 @@ __global__ void __launch_bounds__(256, 4) k_zfwd256(ProArgs<T> a, Spectra<T> sp,
   const int team = threadIdx.x / B, j = threadIdx.x % B;
   cplx<T>* xb = xbuf + (size_t)team * Z256::XP;
   const int ntr = R * sp.nact;
+  const CField<T> fl(sp);
   for (int t0 = 0; t0 < ntr; t0 += Z256::TEAMS) {
     const int t = t0 + team;
     const bool act = t < ntr;                          // the whole team alike
     const int f = act ? t / R : 0, r = act ? t - f * R : 0;
-    const int fid = sp.idx[f];
+    const int fid = fl.id(f);
     cplx<T> u[2][B];
     if (act) {
       // pass 1: z_m = (x_2m, x_2m+1) at m = j + 8 s, radix 16
@@ -156,26 +157,26 @@ __global__ void __launch_bounds__(256, 4) k_zfwd256(ProArgs<T> a, Spectra<T> sp,
 #pragma unroll
         for (int rr = 0; rr < B; ++rr) xb[j + B * it + (A + 1) * rr] = u[it][rr];
     }
-    __syncwarp();
-    if (act) {
-      // X[k] = (Z[k] + Z*[H-k])/2 - (i/2) W_N^k (Z[k] - Z*[H-k]), k = 0..H (Z[H] = Z[0]);
-      // plane layout: entry (k, row) at k N^2 + row (the four teams of a
-      // warp, consecutive rows, fill whole 32-byte sectors)
-      cplx<T>* out = sp.planes ? sp.s[fid] + row0 + r : sp.s[fid] + (row0 + r) * NH;
-      const size_t kstride = sp.planes ? (size_t)N * N : 1;
-#pragma unroll
-      for (int s = 0; s <= A; ++s) {
-        const int k = j + B * s;
-        if (s == A && j != 0) break;                   // k = H: thread 0 only
-        if (k >= a.nkz) break;
-        const cplx<T> zk = xb[Z256::xpos(k == H ? 0 : k)];
-        const cplx<T> zc = cconj(xb[Z256::xpos(k == 0 ? 0 : H - k)]);
-        const cplx<T> e = cadd(zk, zc);
-        const cplx<T> wo = cmul(twN[k], csub(zk, zc));
-        out[k * kstride] = mk<T>((T)0.5 * (e.x + wo.y), (T)0.5 * (e.y - wo.x));
-      }
+    __syncthreads();
+    // X[k] = (Z[k] + Z*[H-k])/2 - (i/2) W_N^k (Z[k] - Z*[H-k]), k = 0..H (Z[H] = Z[0]),
+    // of the round's transforms; consecutive lanes take consecutive rows of one k, so
+    // that plane layout's entries (k, row) at k N^2 + row fill whole lines (a team
+    // storing its own row moved 32 bytes per line: the load-store unit 65% busy)
+    const int units = min(Z256::TEAMS, ntr - t0), lg = units > 16 ? 5 : units > 8 ? 4 : 3;
+    const int nk = min(NH, a.nkz);
+    for (int q = threadIdx.x; q < (nk << lg); q += 256) {
+      const int un = q & ((1 << lg) - 1), k = q >> lg;
+      if (un >= units) continue;
+      const int tt = t0 + un, row = tt % R;
+      const cplx<T>* zb = xbuf + (size_t)un * Z256::XP;
+      const cplx<T> zk = zb[Z256::xpos(k == H ? 0 : k)];
+      const cplx<T> zc = cconj(zb[Z256::xpos(k == 0 ? 0 : H - k)]);
+      const cplx<T> e = cadd(zk, zc);
+      const cplx<T> wo = cmul(twN[k], csub(zk, zc));
+      const size_t at = sp.planes ? (size_t)k * N * N + row0 + row : (row0 + row) * NH + k;
+      fl.spec(tt / R)[at] = mk<T>((T)0.5 * (e.x + wo.y), (T)0.5 * (e.y - wo.x));
     }
-    __syncwarp();                                      // xb is rewritten by the next round
+    __syncthreads();                                   // xb is rewritten by the next round
   }
 }
 
@@ -205,14 +206,14 @@ __global__ void __launch_bounds__(256, 3) k_zinv256(Spectra<T> sp, EpiArgs<T> a,
   // aligned since R is even); plane layout, runs of R rows per kz
   for (int f = 0; f < sp.nact; ++f) {
     if (sp.planes) {
-      const cplx<T>* src = sp.s[sp.idx[f]] + row0;
+      const cplx<T>* src = CField<T>(sp).spec(f) + row0;
       cplx<T>* dst = stg + (size_t)f * R * NH;
       for (int q = threadIdx.x; q < R * NH; q += blockDim.x) {
         const int k = q / R, r = q % R;
         cp_async_c(dst + r * NH + k, src + (size_t)k * N * N + r, true);
       }
     } else {
-      cp_async_block16(stg + (size_t)f * R * NH, sp.s[sp.idx[f]] + row0 * NH, (size_t)R * NH * sizeof(cplx<T>));
+      cp_async_block16(stg + (size_t)f * R * NH, CField<T>(sp).spec(f) + row0 * NH, (size_t)R * NH * sizeof(cplx<T>));
     }
   }
   cp_async_commit();
@@ -257,10 +258,11 @@ __global__ void __launch_bounds__(256, 3) k_zinv256(Spectra<T> sp, EpiArgs<T> a,
   __syncthreads();
   const int rp = 2 * NH;                               // real row pitch in the staging slots
   T* realf[3] = {nullptr, nullptr, nullptr};
-  for (int f = 0; f < sp.nact; ++f) realf[sp.idx[f]] = reinterpret_cast<T*>(stg + (size_t)f * R * NH);
+  if constexpr (KIND == 0)
+    for (int f = 0; f < sp.nact; ++f) realf[sp.idx[f]] = reinterpret_cast<T*>(stg + (size_t)f * R * NH);
   const int jt = threadIdx.x;                          // one grid point of each row (blockDim = N)
   if (KIND == 3 || (KIND == 0 && a.mode == 3)) {
-    const T* fP = realf[2];
+    const T* fP = KIND == 3 ? reinterpret_cast<const T*>(stg) : realf[2];
     T po[R];                                           // P g_old, loaded ahead of the stores
     if (a.pyout) {
 #pragma unroll
@@ -291,10 +293,14 @@ __global__ void __launch_bounds__(256, 3) k_zinv256(Spectra<T> sp, EpiArgs<T> a,
     if constexpr (KIND != 0) ep.point(a, x, dd, reinterpret_cast<const T*>(stg)[qs], (T)0, f2[qs], off + q, acc);
     else ep.point(a, x, dd, f0 ? f0[qs] : (T)0, realf[1] ? realf[1][qs] : (T)0, f2 ? f2[qs] : (T)0, off + q, acc);
   }
-  typename TreeVal<T>::type* scr = reinterpret_cast<typename TreeVal<T>::type*>(smem_raw);
-  block_sum_tree_raw<8, T>(acc, a.partials + (size_t)blockIdx.x * 8, scr);
+  using V = typename TreeVal<T>::type;
+  V* scr = reinterpret_cast<V*>(smem_raw);
+  V v8[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) v8[q] = short_val<T>(acc[q]);
+  block_sum8(v8, scr, a.partials + (size_t)blockIdx.x * 8, 8);
   if (arrive_last(a.counter)) {
-    finalize_eval<T>(a.fin, scr);
+    finalize_eval8<T>(a.fin, scr);
     if (threadIdx.x == 0) *a.counter = 0u;
   }
   }
@@ -549,18 +555,16 @@ __host__ __device__ constexpr size_t p256_bytes() {
 }
 
 // A half-warp team's length-256 transform of one row (256 = 16 x 16, the
-// butterflies of t256_stage2), in place: the exchange between the two
-// stages goes through the row itself, element e at
-// 16 (e / 16) + (e + e / 16) % 16 (the 16 lanes hit 16 different bank pairs
-// in both exchange patterns).
-template <typename T, int DIR>
-__device__ __forceinline__ void p256_row(cplx<T>* row, const cplx<T>* __restrict__ tw, int j) {
+// butterflies of t256_stage2): v[s] = element j + 16 s on entry, v[r] = the
+// result's element j + 16 r on return.  The exchange between the two stages goes
+// through `row` (256 slots; DIRTY: the team may still be reading it), element e
+// at 16 (e / 16) + (e + e / 16) % 16 (the 16 lanes hit 16 different bank pairs in
+// both exchange patterns).
+template <typename T, int DIR, bool DIRTY>
+__device__ __forceinline__ void p256_row(cplx<T> (&v)[16], cplx<T>* row, const cplx<T>* __restrict__ tw, int j) {
   const unsigned mask = half_warp_mask();
-  cplx<T> v[16];
-#pragma unroll
-  for (int s = 0; s < 16; ++s) v[s] = row[j + 16 * s];
   Codelet<cplx<T>, 16, DIR>::run(v);
-  __syncwarp(mask);                                    // the team has read the row
+  if (DIRTY) __syncwarp(mask);                         // the team has read the row
 #pragma unroll
   for (int s = 0; s < 16; ++s) row[16 * j + ((s + j) & 15)] = v[s];   // y[16 j + s]
   __syncwarp(mask);
@@ -573,9 +577,6 @@ __device__ __forceinline__ void p256_row(cplx<T>* row, const cplx<T>* __restrict
     v[r] = cmul(v[r], w);
   }
   Codelet<cplx<T>, 16, DIR>::run(v);
-  __syncwarp(mask);                                    // the team has read the exchange
-#pragma unroll
-  for (int r = 0; r < 16; ++r) row[j + 16 * r] = v[r];
 }
 
 // Length-32 transform of v in registers, natural order in and out: one
@@ -612,20 +613,27 @@ k_plane256cl(Spectra<T> sp, GArgs<T> g, const cplx<T>* __restrict__ tw_n) {
   cplx<T>* tw = slice + ROWS * P;
   const int c = (int)cl.block_rank();
   const int kz = blockIdx.x / CL;
-  const int fid = sp.idx[blockIdx.y];
-  cplx<T>* gpl = sp.s[fid] + (size_t)kz * N * N + (size_t)c * N;   // row x = 8 b + c at gpl + 8 b N
+  const int fid = blockIdx.y == 0 ? sp.idx[0] : blockIdx.y == 1 ? sp.idx[1] : sp.idx[2];
+  cplx<T>* const spec = CField<T>::pick(sp, fid) + (size_t)kz * N * N;
+  cplx<T>* gpl = spec + (size_t)c * N;   // row x = 8 b + c at gpl + 8 b N
   tw[threadIdx.x] = tw_n[threadIdx.x];
   dependency_wait();
-  for (int q = threadIdx.x; q < ROWS * N / 2; q += blockDim.x) {   // 16-byte pieces
-    const int b = q >> 7, y = (q & 127) * 2;
-    cp_async<16>(slice + b * P + y, gpl + (size_t)b * CL * N + y, true);
-  }
-  cp_async_commit();
-  cp_async_wait<0>();
-  __syncthreads();
+  __syncthreads();                                     // (the twiddles)
   const int team = threadIdx.x >> 4, j = threadIdx.x & 15, t = threadIdx.x;
-  // 1. along y
-  for (int b0 = 0; b0 < ROWS; b0 += 16) p256_row<T, -1>(slice + (b0 + team) * P, tw, j);
+  // 1. along y, the rows read straight from memory (128 bytes per half warp and
+  // element)
+#pragma unroll 1
+  for (int b = team; b < ROWS; b += 16) {
+    const cplx<T>* src = gpl + (size_t)b * CL * N + j;
+    cplx<T>* row = slice + b * P;
+    cplx<T> v[16];
+#pragma unroll
+    for (int s = 0; s < 16; ++s) v[s] = __ldcg(src + 16 * s);
+    p256_row<T, -1, false>(v, row, tw, j);
+    __syncwarp(half_warp_mask());                      // the team has read the exchange
+#pragma unroll
+    for (int r = 0; r < 16; ++r) row[j + 16 * r] = v[r];
+  }
   __syncthreads();
   // 2. column ky = t: 32-point transforms along b, twiddles W_256^(c k2)
   {
@@ -643,34 +651,82 @@ k_plane256cl(Spectra<T> sp, GArgs<T> g, const cplx<T>* __restrict__ tw_n) {
   cplx<T>* part[CL];
 #pragma unroll
   for (int o = 0; o < CL; ++o) part[o] = cl.map_shared_rank(slice, o);
+  // A thread takes the columns ky = u and -u (u = 0: ky = 0 and -128), which share
+  // their |m|^2 and with it the factors (a table gather or a division each).
   const bool with_loc = fid == 0 && g.vloc != nullptr;
   const T w = (kz == 0 || kz == N / 2) ? (T)1 : (T)2;
-  const int my = t <= 127 ? t : t - N;
-  AccShort<T> acc[4];
-  for (int i = 0; i < 4; ++i) {
-    const int k2 = 4 * c + i;
-    cplx<T> z[CL];
+  const int u = t & 127, kya = u, kyb = u ? N - u : N / 2;
+  const cplx<T>* vl = with_loc ? g.vloc + (size_t)kz * N * N : nullptr;   // plane layout [kz][kx][ky]
+  AccShort<T> e0, e1;                                  // (E_H, E_loc) or (E_NL, E_vW), before the factors
+  for (int i = 0; i < 2; ++i) {
+    const int k2 = 4 * c + 2 * (t >> 7) + i;
+    cplx<T> za[CL], zb[CL];
 #pragma unroll
-    for (int o = 0; o < CL; ++o) z[o] = part[o][k2 * P + t];
-    Codelet<cplx<T>, 8, -1>::run(z);                   // z[k1] = F(kx = k2 + 32 k1)
+    for (int o = 0; o < CL; ++o) { za[o] = part[o][k2 * P + kya]; zb[o] = part[o][k2 * P + kyb]; }
+    Codelet<cplx<T>, 8, -1>::run(za);                  // za[k1] = F(kx = k2 + 32 k1)
+    Codelet<cplx<T>, 8, -1>::run(zb);
     if (g.forward) {                                   // (all blocks of the cluster have read their rows)
-      cplx<T>* y = sp.s[fid] + (size_t)kz * N * N + (size_t)k2 * N + t;
+      cplx<T>* y = spec + (size_t)k2 * N;
 #pragma unroll
-      for (int k1 = 0; k1 < CL; ++k1) y[(size_t)k1 * 32 * N] = z[k1];
+      for (int k1 = 0; k1 < CL; ++k1) { y[(size_t)k1 * 32 * N + kya] = za[k1]; y[(size_t)k1 * 32 * N + kyb] = zb[k1]; }
       continue;
     }
-    // V_loc in plane layout [kz][kx][ky]
-    const cplx<T>* vl = with_loc ? g.vloc + (size_t)kz * N * N + t : nullptr;
 #pragma unroll
     for (int k1 = 0; k1 < CL; ++k1) {
       const int kx = k2 + 32 * k1;
       const int mx = kx <= 127 ? kx : kx - N;
-      const int m2 = mx * mx + my * my + kz * kz;
-      z[k1] = gspace_point<T>(fid, g, sp.merged, with_loc, m2, w, z[k1], [&]() { return vl[(size_t)kx * N]; }, acc);
+      const int mxz = mx * mx + kz * kz, m2a = mxz + u * u, m2b = u ? m2a : mxz + 128 * 128;
+      const T Ga = g.tp2 * (T)m2a, Gb = g.tp2 * (T)m2b;
+      const T ar = za[k1].x * g.invN, ai = za[k1].y * g.invN, br = zb[k1].x * g.invN, bi = zb[k1].y * g.invN;
+      const T a2 = ar * ar + ai * ai, b2 = br * br + bi * bi;
+      if (fid == 0) {
+        T ca = 0, cb = 0;
+        if (g.hartree) {
+          ca = m2a > 0 ? (T)(4.0 * kPi) / Ga : (T)0;
+          cb = u ? ca : (T)(4.0 * kPi) / Gb;
+          e0.add(ca * a2 + cb * b2);
+        }
+        cplx<T> oa = mk<T>(ca * ar, ca * ai), ob = mk<T>(cb * br, cb * bi);
+        if (with_loc && Ga <= g.g2cut_loc) {
+          const cplx<T> v = vl[kx * N + kya];
+          e1.add(ar * v.x + ai * v.y);
+          oa.x += v.x; oa.y += v.y;
+        }
+        if (with_loc && Gb <= g.g2cut_loc) {
+          const cplx<T> v = vl[kx * N + kyb];
+          e1.add(br * v.x + bi * v.y);
+          ob.x += v.x; ob.y += v.y;
+        }
+        za[k1] = oa; zb[k1] = ob;
+      } else {
+        T ca, cb;
+        if (fid == 1 || g.prec != nullptr || sp.merged) {
+          const T* tab = fid != 1 && g.prec != nullptr ? g.prec : g.K;
+          ca = __ldg(tab + m2a);
+          cb = u ? ca : __ldg(tab + m2b);
+        } else {
+          ca = 0; cb = 0;
+        }
+        if (fid == 1) {
+          e0.add(ca * a2 + cb * b2);
+        } else if (g.prec == nullptr) {
+          e1.add(Ga * a2 + Gb * b2);
+          if (sp.merged) {
+            e0.add(ca * a2 + cb * b2);
+            ca = ca + (T)0.5 * Ga;
+            cb = cb + (T)0.5 * Gb;
+          } else {
+            ca = Ga; cb = Gb;
+          }
+        }
+        za[k1] = mk<T>(ca * ar, ca * ai);
+        zb[k1] = mk<T>(cb * br, cb * bi);
+      }
     }
-    Codelet<cplx<T>, 8, +1>::run(z);
+    Codelet<cplx<T>, 8, +1>::run(za);
+    Codelet<cplx<T>, 8, +1>::run(zb);
 #pragma unroll
-    for (int o = 0; o < CL; ++o) part[o][k2 * P + t] = z[o];
+    for (int o = 0; o < CL; ++o) { part[o][k2 * P + kya] = za[o]; part[o][k2 * P + kyb] = zb[o]; }
   }
   cl.sync();                                           // (no remote access after this)
   if (g.forward) return;
@@ -686,14 +742,30 @@ k_plane256cl(Spectra<T> sp, GArgs<T> g, const cplx<T>* __restrict__ tw_n) {
     for (int b = 0; b < 32; ++b) slice[b * P + t] = v[b];
   }
   __syncthreads();
-  for (int b0 = 0; b0 < ROWS; b0 += 16) p256_row<T, 1>(slice + (b0 + team) * P, tw, j);
-  __syncthreads();
-  for (int q = threadIdx.x; q < ROWS * N / 2; q += blockDim.x) {
-    const int b = q >> 7, y = (q & 127) * 2;
-    *reinterpret_cast<float4*>(gpl + (size_t)b * CL * N + y) = *reinterpret_cast<const float4*>(slice + b * P + y);
+  // the rows, straight to memory
+#pragma unroll 1
+  for (int b = team; b < ROWS; b += 16) {
+    cplx<T>* row = slice + b * P;
+    cplx<T> v[16];
+#pragma unroll
+    for (int s = 0; s < 16; ++s) v[s] = row[j + 16 * s];
+    p256_row<T, 1, true>(v, row, tw, j);
+    cplx<T>* dst = gpl + (size_t)b * CL * N + j;
+#pragma unroll
+    for (int r = 0; r < 16; ++r) dst[16 * r] = v[r];
   }
+  if (g.prec != nullptr) return;                       // (no sums)
+  using V = typename TreeVal<T>::type;
+  V v8[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) v8[q] = V{};
+  AccShort<T> sa, sb;
+  sa.s = (fid == 0 ? g.halfOm : g.Om) * w * e0.s;      // E_H or E_NL
+  sb.s = (fid == 0 ? g.Om : g.halfOm) * w * e1.s;      // E_loc or E_vW (raw)
+  if (fid == 0) { v8[0] = short_val<T>(sa); v8[1] = short_val<T>(sb); }
+  else { v8[2] = short_val<T>(sa); v8[3] = short_val<T>(sb); }
   const size_t bi = (size_t)blockIdx.y * gridDim.x + blockIdx.x;
-  block_sum_tree_raw<4, T>(acc, g.partials + bi * 4, reinterpret_cast<typename TreeVal<T>::type*>(smem_raw));
+  block_sum8(v8, reinterpret_cast<V*>(smem_raw), g.partials + bi * 4, 4);
 }
 
 }  // namespace ofdft
