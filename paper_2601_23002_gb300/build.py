@@ -20,7 +20,7 @@ LIB = os.path.join(OUT, "libofdft_gb300.so")
 SOURCES = ["api.cu", "engine_f32.cu", "engine_f64.cu", "plane_f32.cu", "plane_f64.cu", "plane2_f32.cu",
            "plane2_f64.cu", "noalloc.cu"]
 # sources compiled several times, each part with its own share of the kernels (-DCPASS_PART=i)
-PARTED = {"cpass_f32.cu": 4, "cpass_f64.cu": 4}
+PARTED = {"cpass_f32.cu": 6, "cpass_f64.cu": 4}
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -1,6 +1,6 @@
 // The passes of the plane path with the grid size known at compile time
-// (2,3,5-smooth n from 24 to 160): the z passes and the plane pass of one
-// evaluation, or of one preconditioning pass.
+// (2,3,5-smooth n from 24 to 160, FP32 to 250): the z passes and the plane pass of
+// one evaluation, or of one preconditioning pass.
 //
 // What bounds the generic passes (k_zfwd, k_plane, k_zinv_epi) on these grids is
 // neither memory (the spectra stay in L2) nor arithmetic but instructions and
@@ -796,7 +796,9 @@ template <typename T> struct CPass {
 // only where they fit about one wave of the 152 SMs (75^3, 76 planes: 17.9 ->
 // 13.8 us with 2; 108^3, 110 planes: 22.0 -> 30 us with 4, since the remote rows
 // cost more than the shorter stages save), or where single blocks need a second
-// wave (160^3, 162 planes: 93 -> 64 us with 5).  FP64 (bound by the FP64 pipe of
+// wave (160^3, 162 planes: 93 -> 64 us with 5).  Above 160 a plane takes several
+// blocks: 4 up to 200 (200^3: 147 us, 165 with 5), then 5 (216^3: 207, 213 with 4;
+// 240^3: 296, 379 with 8); the tiled chain took 264 us at 200^3, 332 at 216^3.  FP64 (bound by the FP64 pipe of
 // the busiest SM): the least rows there, ceil(nf nh CL / 152) blocks of ROWS
 // rows, the smaller cluster within 10% (96^3: 277 -> 224 us with 4; 45^3: 69 ->
 // 43 with 2), and what fits in shared memory.
@@ -805,7 +807,8 @@ template <typename T, int N, int CL> constexpr int cp_load(int nf) {
 }
 template <typename T, int N> constexpr int cp_cluster(int nf) {
   const int planes = nf * (N / 2 + 1);
-  if (sizeof(T) == 4) return planes * 4 <= 168 ? 4 : planes * 2 <= 168 ? 2 : planes <= 152 ? 1 : 5;
+  if (sizeof(T) == 4)
+    return planes * 4 <= 168 ? 4 : planes * 2 <= 168 ? 2 : planes <= 152 && N <= 160 ? 1 : N > 160 && N <= 200 ? 4 : 5;
   const int l1 = cp_load<T, N, 1>(nf), l2 = cp_load<T, N, 2>(nf), l4 = cp_load<T, N, 4>(nf);
   const int best = l1 < l2 ? (l1 < l4 ? l1 : l4) : (l2 < l4 ? l2 : l4);
   return 10 * l1 <= 11 * best ? 1 : 10 * l2 <= 11 * best ? 2 : 4;

@@ -66,6 +66,33 @@ def test_evaluation_matches_the_generic_passes(monkeypatch, n, alpha, precision,
         assert abs(e1[k] - e0[k]) <= tol_e * max(scale, abs(e0[k])), k
 
 
+# FP32 above 160: planes over clusters, where the generic passes are the tiled ones
+# with another order of the stages along x and y.  Both round the psi transform,
+# amplified by G^2; against the FP64 plan the error must not be larger (a factor
+# 1.5 for two independent roundings).
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [162, 180, 192, 200, 216, 225, 240, 243, 250])
+def test_large_grids_are_as_exact_as_the_tiled_passes(monkeypatch, n):
+    cell = random_cell(7, 8, 1.0, 2.0, 0.8, n)
+    cell.L *= 2.5
+    cell.pos *= 2.5
+    rho = density(cell, torch.float32)
+
+    def go(plan):
+        r = rho.to(plan.dtype)
+        v = torch.empty_like(r)
+        e = plan.energy_potential(r, v)
+        return v.double(), e
+
+    v64, e64 = both(monkeypatch, cell, "fp64", go)[1]
+    (v1, e1), (v0, e0) = both(monkeypatch, cell, "fp32", go)
+    err = [float((v - v64).norm() / v64.norm()) for v in (v1, v0)]
+    assert err[0] <= 1.5 * err[1]
+    size = max(abs(x) for x in e64.values())
+    for k in e64:
+        assert abs(e1[k] - e64[k]) <= max(1.5 * abs(e0[k] - e64[k]), 1e-6 * size), k
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("precision,tol", [("fp32", 2e-6), ("fp64", 1e-12)])
 @pytest.mark.parametrize("n", [24, 45, 64, 75, 128])
