@@ -19,6 +19,7 @@
 // has the same bits: the rounding of the psi transform, amplified by G^2, is
 // the largest error of an FP32 potential.
 #pragma once
+#include <initializer_list>
 #include <cooperative_groups.h>
 #include "passes.cuh"
 
@@ -62,6 +63,50 @@ constexpr CFac cfac(int n, bool bal) {
   return best;
 }
 constexpr int cdiv(int a, int b) { return (a + b - 1) / b; }
+
+// FP64 plans choose their radices by time instead: one FP64 instruction of a warp
+// takes its SM quarter's pipe 64 cycles whatever the number of active lanes, so a
+// stage of `items` butterflies of radix R costs ceil(warps / 4) times the
+// butterfly's instructions.  Large radices leave that pipe to one warp on small
+// grids (30^3: radix 10 on 24 lanes, 140 instructions = 4.3 us per stage).
+// Evaluation, all passes: 24^3 84 -> 53 us, 30^3 73 -> 60, 32^3 101 -> 55, 45^3 105 ->
+// 94, 96^3 480 -> 449, 120^3 1018 -> 987, 128^3 unchanged (the same radices win).
+constexpr int dcost(int r) {      // FP64 instructions of a butterfly and its twiddles
+  return r == 2 ? 8 : r == 3 ? 22 : r == 4 ? 28 : r == 5 ? 50 : r == 6 ? 64 : r == 8 ? 84 : r == 9 ? 130
+         : r == 10 ? 140 : r == 12 ? 155 : 230;
+}
+// `points` of the block in lines of `len`, nb blocks sharing an SM; per stage 24
+// more for its barriers and latency and the round trip through shared memory (8
+// cycles for 32 points): 128^3 keeps 8 x 16 (465 us; 4 x 4 x 8: 473)
+constexpr long dstage(int points, int r, int nb) {
+  return (long)cdiv(nb * cdiv(points / r, 32), 4) * dcost(r) + 24 + nb * points / 256;
+}
+constexpr long dtime(const CFac& f, int points, int nb) {
+  long t = 0;
+  for (int i = 0; i < f.c; ++i) t += dstage(points, f.r[i], nb);
+  return t;
+}
+constexpr CFac dfac(int n, int points, int nb) {
+  CFac best{0, {0, 0, 0, 0}};
+  long tb = 1L << 60;
+  auto look = [&](const CFac& f) {
+    const long t = dtime(f, points, nb);
+    if (t < tb) { tb = t; best = f; }
+  };
+  if (is_cand(n)) look(CFac{1, {n, 0, 0, 0}});
+  for (int i = 9; i >= 0; --i) {
+    const int a = kCand[i];
+    if (n % a) continue;
+    if (is_cand(n / a)) look(CFac{2, {a, n / a, 0, 0}});
+    for (int j = i; j >= 0; --j) {
+      const int b = kCand[j];
+      if ((n / a) % b || !is_cand(n / a / b) || n / a / b < b) continue;
+      look(CFac{3, {a, b, n / a / b, 0}});
+    }
+  }
+  return best;
+}
+constexpr int least(int a, int b) { return a < b ? a : b; }
 // threads for `items` items, at most `most`, in as few and as full rounds as possible
 constexpr int fit_threads(int items, int most, int least) {
   const int rounds = cdiv(items, most);
@@ -71,13 +116,15 @@ constexpr int fit_threads(int items, int most, int least) {
 
 // z passes: rows per block, transform length (half for even n, full for odd n:
 // two rows per transform), radices, threads, pitches.
-template <int N> struct CZ {
+// D: FP64.
+template <int N, bool D> struct CZ {
   static constexpr bool ODD = N & 1;
   static constexpr int H = N / 2, NH = H + 1;
   static constexpr int R = N <= 50 ? 8 : 16;            // at least 152 blocks from n = 36 up
   static constexpr int L = ODD ? N : H;
   static constexpr int LINES = ODD ? R / 2 : R;         // transforms per block and field
-  static constexpr CFac F = cfac(L, !ODD);
+  static constexpr int GRID = cdiv(N * N, R);
+  static constexpr CFac F = D ? dfac(L, 2 * LINES * L, cdiv(GRID, 152) < 2 ? 1 : 2) : cfac(L, !ODD);
   static constexpr int F0 = F.r[0], F1 = F.c >= 2 ? F.r[1] : 1, F2 = F.c == 3 ? F.r[2] : 1;
   static constexpr int NT = N <= 50 ? 128 : 256;
   // element e of a line sits at e + e / F0 (even F0: the first stage writes
@@ -86,7 +133,6 @@ template <int N> struct CZ {
   static constexpr int XP = (pad(L - 1) + 1) | 1;
   static constexpr int SP = (ODD ? (N + 1) / 2 : NH) | 1;   // spectrum row pitch (odd n: two rows hold a line of L <= 2 SP)
   static constexpr int BP = (ODD ? 2 : 1) * SP;             // the same region as lines: pitch
-  static constexpr int GRID = cdiv(N * N, R);
 };
 
 // ---------------------------------------------------------------------------
@@ -181,7 +227,7 @@ static __device__ void finalize_eval8(const FinArgs<T>& f, typename TreeVal<T>::
 // xb[line BP + e] for three.  Ends with a barrier.
 template <typename T, int N, int DIR>
 __device__ __forceinline__ void cz_stages(cplx<T>* xa, cplx<T>* xb, int lines, const cplx<T>* __restrict__ tw) {
-  using Z = CZ<N>;
+  using Z = CZ<N, sizeof(T) == 8>;
   constexpr int L = Z::L, F0 = Z::F0, F1 = Z::F1, F2 = Z::F2;
   if constexpr (Z::F.c == 1) {
     return;
@@ -245,7 +291,7 @@ __device__ __forceinline__ void cz_stages(cplx<T>* xa, cplx<T>* xb, int lines, c
 }
 template <typename T, int N>
 __device__ __forceinline__ cplx<T> cz_get(const cplx<T>* xa, const cplx<T>* xb, int ln, int e) {
-  using Z = CZ<N>;
+  using Z = CZ<N, sizeof(T) == 8>;
   if constexpr (Z::F.c <= 2) return xa[ln * Z::XP + Z::pad(e)];
   else return xb[ln * Z::BP + e];
 }
@@ -265,17 +311,19 @@ template <typename T> struct CField {
   __device__ __forceinline__ cplx<T>* spec(int f) const { return f == 0 ? s0 : f == 1 ? s1 : s2; }
 };
 
-// shared memory: tw[L] | twn[NH] | xa[nf][LINES][XP] | xb[nf][LINES][BP] (three stages)
+// shared memory: tw[L] | twn[NH] | xa[nf][LINES][XP] | xb[nf][LINES][BP] (three
+// stages) | FP64: sq[R][N] reals
 template <typename T, int N> __host__ __device__ constexpr size_t czfwd_bytes(int nf) {
-  using Z = CZ<N>;
-  return ((size_t)Z::L + Z::NH + (size_t)nf * Z::LINES * (Z::XP + (Z::F.c == 3 ? Z::BP : 0))) * sizeof(cplx<T>);
+  using Z = CZ<N, sizeof(T) == 8>;
+  return ((size_t)Z::L + Z::NH + (size_t)nf * Z::LINES * (Z::XP + (Z::F.c == 3 ? Z::BP : 0))) * sizeof(cplx<T>) +
+         (sizeof(T) == 8 ? (size_t)Z::R * N * sizeof(T) : 0);
 }
 // Forward z pass: prologue (n, n^a, psi from rho or from psi + t d) and the
 // real-to-complex transform of R rows of every active field, plane layout.
 template <typename T, int N>
-__global__ void __launch_bounds__(CZ<N>::NT, (sizeof(T) == 4 ? 1024 : 512) / CZ<N>::NT)
+__global__ void __launch_bounds__(CZ<N, sizeof(T) == 8>::NT, (sizeof(T) == 4 ? 1024 : 512) / CZ<N, sizeof(T) == 8>::NT)
 k_zfwd_c(ProArgs<T> a, Spectra<T> sp, const cplx<T>* __restrict__ tw_l, const cplx<T>* __restrict__ tw_n) {
-  using Z = CZ<N>;
+  using Z = CZ<N, sizeof(T) == 8>;
   using C = cplx<T>;
   constexpr int R = Z::R, L = Z::L, H = Z::H, NH = Z::NH, F0 = Z::F0, M0 = L / F0, NN = N * N;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -304,6 +352,15 @@ k_zfwd_c(ProArgs<T> a, Spectra<T> sp, const cplx<T>* __restrict__ tw_l, const cp
     const T nv = a.mode == 0 ? x : scale * x * x;
     return fid == 0 ? nv : pow_t<T>(fmax(nv, nmin), alpha);
   };
+  // FP64 and a given density: psi = sqrt(rho) by all threads first (about 20 FP64
+  // instructions a point; in stage 0 the threads of the psi field alone would take
+  // 2 F0 each; 45^3: 23.4 -> 16.8 us with the radices)
+  T* sq = reinterpret_cast<T*>(xb + (Z::F.c == 3 ? sp.nact * Z::LINES * Z::BP : 0));
+  const bool pre = sizeof(T) == 8 && a.mode == 0 && (fl_.id(sp.nact - 1) == 2);
+  if (pre) {
+    for (int q = threadIdx.x; q < rows * N; q += Z::NT) sq[q] = val(2, src[q]);
+    __syncthreads();
+  }
   // stage 0: the line's elements j + s M0 from memory, radix F0
   for (int it = threadIdx.x; it < sp.nact * Z::LINES * M0; it += Z::NT) {
     const int fl = it / M0, j = it - fl * M0;
@@ -313,7 +370,8 @@ k_zfwd_c(ProArgs<T> a, Spectra<T> sp, const cplx<T>* __restrict__ tw_l, const cp
     C v[F0];
     if constexpr (Z::ODD) {
       const bool two = 2 * ln + 1 < rows;
-      const T* p0 = src + 2 * ln * N + j;
+      const bool ready = pre && fid == 2;
+      const T* p0 = (ready ? sq : src) + 2 * ln * N + j;
       const T* d0 = dsrc + 2 * ln * N + j;
 #pragma unroll
       for (int s = 0; s < F0; ++s) v[s] = mk<T>(p0[s * M0], two ? p0[N + s * M0] : (T)0);
@@ -324,10 +382,13 @@ k_zfwd_c(ProArgs<T> a, Spectra<T> sp, const cplx<T>* __restrict__ tw_l, const cp
           if (two) v[s].y = v[s].y + tstep * d0[N + s * M0];
         }
       }
+      if (!ready) {
 #pragma unroll
-      for (int s = 0; s < F0; ++s) v[s] = mk<T>(val(fid, v[s].x), two ? val(fid, v[s].y) : (T)0);
+        for (int s = 0; s < F0; ++s) v[s] = mk<T>(val(fid, v[s].x), two ? val(fid, v[s].y) : (T)0);
+      }
     } else {
-      const C* p0 = reinterpret_cast<const C*>(src + ln * N) + j;
+      const bool ready = pre && fid == 2;
+      const C* p0 = reinterpret_cast<const C*>((ready ? sq : src) + ln * N) + j;
       const C* d0 = reinterpret_cast<const C*>(dsrc + ln * N) + j;
 #pragma unroll
       for (int s = 0; s < F0; ++s) v[s] = p0[s * M0];
@@ -338,8 +399,10 @@ k_zfwd_c(ProArgs<T> a, Spectra<T> sp, const cplx<T>* __restrict__ tw_l, const cp
           v[s].x = v[s].x + tstep * d.x; v[s].y = v[s].y + tstep * d.y;
         }
       }
+      if (!ready) {
 #pragma unroll
-      for (int s = 0; s < F0; ++s) v[s] = mk<T>(val(fid, v[s].x), val(fid, v[s].y));
+        for (int s = 0; s < F0; ++s) v[s] = mk<T>(val(fid, v[s].x), val(fid, v[s].y));
+      }
     }
     Codelet<C, F0, -1>::run(v);
     C* x = xa + fl * Z::XP + Z::pad(j * F0);
@@ -380,7 +443,7 @@ k_zfwd_c(ProArgs<T> a, Spectra<T> sp, const cplx<T>* __restrict__ tw_l, const cp
 
 // shared memory: tw[L] | twn[NH] | stg[nf][R][SP] | xa[nf][LINES][XP]
 template <typename T, int N> __host__ __device__ constexpr size_t czinv_bytes(int nf) {
-  using Z = CZ<N>;
+  using Z = CZ<N, sizeof(T) == 8>;
   const size_t b = ((size_t)Z::L + Z::NH + (size_t)nf * (Z::R * Z::SP + Z::LINES * Z::XP)) * sizeof(cplx<T>);
   const size_t s = (size_t)(Z::NT / 32) * 8 * 8;
   return b > s ? b : s;
@@ -389,9 +452,9 @@ template <typename T, int N> __host__ __device__ constexpr size_t czinv_bytes(in
 // (plane layout) and the pointwise functional (KIND 0, 1, 2: see EpiPoint), or
 // the preconditioning pass's output (KIND 3: mode 3).
 template <typename T, int N, int KIND>
-__global__ void __launch_bounds__(CZ<N>::NT, (sizeof(T) == 4 ? 1024 : 512) / CZ<N>::NT)
+__global__ void __launch_bounds__(CZ<N, sizeof(T) == 8>::NT, (sizeof(T) == 4 ? 1024 : 512) / CZ<N, sizeof(T) == 8>::NT)
 k_zinv_c(Spectra<T> sp, EpiArgs<T> a, const cplx<T>* __restrict__ tw_l, const cplx<T>* __restrict__ tw_n) {
-  using Z = CZ<N>;
+  using Z = CZ<N, sizeof(T) == 8>;
   using C = cplx<T>;
   constexpr int R = Z::R, L = Z::L, H = Z::H, NH = Z::NH, F0 = Z::F0, M0 = L / F0, NN = N * N;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -517,15 +580,44 @@ k_zinv_c(Spectra<T> sp, EpiArgs<T> a, const cplx<T>* __restrict__ tw_l, const cp
 // the first stage along x reads its rows from the cluster's blocks through
 // distributed shared memory into a column buffer of its own, the last inverse
 // stage writes the rows back; two cluster barriers in all.
+
+// Shared memory of a plane pass (bytes) and, in FP64, the cluster size and radices
+// by dtime: CL of 1, 2, 4 for nf fields, ROWS lines a block, cdiv(planes CL, 152)
+// blocks on an SM (32^3: 16 x 2 -> 2 x 4 x 4, 38 -> 18 us a pass;
+// 96^3: 16 x 6 -> 8 x 12, 225 -> 194).
+constexpr size_t cp_bytes(int n, int cl, int csize) {
+  const int rows = cdiv(n, cl);
+  return ((size_t)rows * (n | 1) + (cl == 1 ? 0 : (size_t)n * (rows | 1)) + n) * csize;
+}
+constexpr long cp_time64(int n, int cl, int nf, const CFac& f) {
+  if (cp_bytes(n, cl, 16) > (size_t)225 * 1024) return 1L << 60;
+  return dtime(f, cdiv(n, cl) * n, cdiv(nf * (n / 2 + 1) * cl, 152));
+}
+constexpr CFac cp_fac64(int n) {
+  CFac best{0, {0, 0, 0, 0}};
+  long tb = 1L << 61;
+  for (int cl : {1, 2, 4}) {
+    const CFac f = dfac(n, cdiv(n, cl) * n, cdiv(2 * (n / 2 + 1) * cl, 152));
+    const long t = cp_time64(n, cl, 2, f);
+    if (f.c >= 2 && t < tb) { tb = t; best = f; }
+  }
+  return best;
+}
+template <typename T, int N> constexpr CFac cp_fac() { return sizeof(T) == 4 ? cfac(N, false) : cp_fac64(N); }
 template <typename T, int N, int CL> struct CP {
-  static constexpr CFac F = cfac(N, false);
+  static constexpr CFac F = cp_fac<T, N>();
   static constexpr int NP = F.c, F0 = F.r[0], F1 = F.r[1], F2 = NP == 3 ? F.r[2] : 1;
   static constexpr int ROWS = cdiv(N, CL), P = N | 1;        // odd pitch: rows and columns free of bank conflicts
   static constexpr int CPT = CL == 1 ? P : (ROWS | 1);       // column buffer pitch
   static constexpr int NH = N / 2 + 1;
-  // radix 16 takes more than the 64 registers of a 1024-thread block
-  static constexpr int NT = fit_threads(ROWS * (N / F0), sizeof(T) == 4 && F0 < 16 ? 1024 : 512, 128);
-  static constexpr size_t BYTES = ((size_t)ROWS * P + (CL == 1 ? 0 : (size_t)N * CPT) + N) * sizeof(cplx<T>);
+  static constexpr size_t BYTES = cp_bytes(N, CL, sizeof(cplx<T>));
+  // FP64: blocks of a plane that share an SM (two fields, and what its memory takes)
+  static constexpr int SHARE = sizeof(T) == 4 ? 1 : least(cdiv(2 * NH * CL, 152), (int)((size_t)227 * 1024 / (BYTES + 1024)));
+  // radix 16 takes more than the 64 registers of a 1024-thread block; blocks that
+  // share an SM in FP64 take at most 288 threads, so that their registers do not keep
+  // them apart (108^3: 279 us with 256, 382 with 512)
+  static constexpr int NT = fit_threads(ROWS * (N / F0), sizeof(T) == 4 && F0 < 16 ? 1024 : SHARE > 1 ? 288 : 512, 128);
+  static constexpr int MIN_BLOCKS = SHARE > 1 ? least(SHARE, 512 / NT) : 1;
 };
 
 // One in-place butterfly with its twiddles (ip_stage's arithmetic).
@@ -589,7 +681,7 @@ __device__ __forceinline__ void cp_cols(cplx<T>* b0, int nc, const cplx<T>* __re
 }
 
 template <typename T, int N, int CL>
-__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(CP<T, N, CL>::NT, 1)
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(CP<T, N, CL>::NT, CP<T, N, CL>::MIN_BLOCKS)
 k_plane_c(Spectra<T> sp, GArgs<T> g, const cplx<T>* __restrict__ tw_g) {
   namespace cg = cooperative_groups;
   using Q = CP<T, N, CL>;
@@ -798,27 +890,24 @@ template <typename T> struct CPass {
 // cost more than the shorter stages save), or where single blocks need a second
 // wave (160^3, 162 planes: 93 -> 64 us with 5).  Above 160 a plane takes several
 // blocks: 4 up to 200 (200^3: 147 us, 165 with 5), then 5 (216^3: 207, 213 with 4;
-// 240^3: 296, 379 with 8); the tiled chain took 264 us at 200^3, 332 at 216^3.  FP64 (bound by the FP64 pipe of
-// the busiest SM): the least rows there, ceil(nf nh CL / 152) blocks of ROWS
-// rows, the smaller cluster within 10% (96^3: 277 -> 224 us with 4; 45^3: 69 ->
-// 43 with 2), and what fits in shared memory.
-template <typename T, int N, int CL> constexpr int cp_load(int nf) {
-  return CP<T, N, CL>::BYTES > (size_t)225 * 1024 ? 1 << 20 : cdiv(nf * (N / 2 + 1) * CL, 152) * CP<T, N, CL>::ROWS;
-}
+// 240^3: 296, 379 with 8); the tiled chain took 264 us at 200^3, 332 at 216^3.  FP64: the
+// least dtime (two fields, before the radices were chosen with it: 96^3 277 us with
+// 1, 224 with 4; 45^3 69 with 1, 43 with 2).
 template <typename T, int N> constexpr int cp_cluster(int nf) {
   const int planes = nf * (N / 2 + 1);
   if (sizeof(T) == 4)
     return planes * 4 <= 168 ? 4 : planes * 2 <= 168 ? 2 : planes <= 152 && N <= 160 ? 1 : N > 160 && N <= 200 ? 4 : 5;
-  const int l1 = cp_load<T, N, 1>(nf), l2 = cp_load<T, N, 2>(nf), l4 = cp_load<T, N, 4>(nf);
-  const int best = l1 < l2 ? (l1 < l4 ? l1 : l4) : (l2 < l4 ? l2 : l4);
-  return 10 * l1 <= 11 * best ? 1 : 10 * l2 <= 11 * best ? 2 : 4;
+  int best = 1;
+  for (int cl : {2, 4})
+    if (cp_time64(N, cl, nf, cp_fac64(N)) < cp_time64(N, best, nf, cp_fac64(N))) best = cl;
+  return cp_bytes(N, best, 16) <= (size_t)225 * 1024 ? best : 0;
 }
 
 template <typename T, int N> CPass<T> make_cpass() {
-  using Z = CZ<N>;
+  using Z = CZ<N, sizeof(T) == 8>;
   CPass<T> p{};
   p.n = N; p.rows = Z::R; p.zthreads = Z::NT; p.zgrid = Z::GRID;
-  p.fz = Z::F; p.fp = cfac(N, false);
+  p.fz = Z::F; p.fp = cp_fac<T, N>();
   p.zfwd = k_zfwd_c<T, N>;
   p.zinv[0] = k_zinv_c<T, N, 0>; p.zinv[1] = k_zinv_c<T, N, 1>;
   p.zinv[2] = k_zinv_c<T, N, 2>; p.zinv[3] = k_zinv_c<T, N, 3>;

@@ -493,6 +493,12 @@ class Engine : public IEngine {
       }
       if (prod == h) ph = q;
     }
+    if (cp && sizeof(T) == 8) {
+      // FP64 plans: the radices of the compile-time passes (chosen for the FP64 pipe)
+      auto take = [](FftPlan1& p, const CFac& f) { p.npass = f.c; for (int i = 0; i < f.c; ++i) p.radix[i] = f.r[i]; };
+      take(pn, cp->fp);
+      if (!std::getenv("OFDFT_ZRADIX")) take(ph, cp->fz);
+    }
     if (planes && !cp) plane_kern = plane_kernel<T>(radix_mask(pn));
     if (prec2) prec2_kern = plane_prec2_kernel<T>(radix_mask(pn));
     int rc;
