@@ -114,19 +114,42 @@ constexpr int fit_threads(int items, int most, int least) {
   return nt < least ? least : nt;
 }
 
+// Rows per block of the z passes: 8 up to 50^3 and 16 above.  In FP64 another count
+// (even: whole sectors of a spectrum's run) where it leaves the busiest SM 5% less to
+// do: the blocks run in about one wave, ceil(blocks / 152) on an SM, and the pass takes
+// as long as the warps' worth of points on a quarter's FP64 pipe (plus a quarter of one
+// a block).  Both z passes: 54^3 87 -> 65 us with 20 rows, 72^3 151 -> 126 with 18,
+// 100^3 349 -> 292 with 22.  The same count in FP32 changed nothing beyond 2% either
+// way up to 90^3 (latency, not work, fills those passes).
+constexpr long z_load(int n, int r) {
+  const int nb = cdiv(cdiv(n * n, r), 152);
+  return 4L * cdiv(nb * cdiv(r * n, 32), 4) + nb;
+}
+constexpr int z_rows(int n, bool d) {
+  int best = n <= 50 ? 8 : 16;
+  if (!d) return best;
+  long tb = z_load(n, best) * 95 / 100;
+  // at least a tile schedule's 8; above 108 points more than 16 leave one block an SM
+  for (int r = 8; r <= (n <= 108 ? 24 : 16); r += 2) {
+    const long t = z_load(n, r);
+    if (t <= tb) { tb = t; best = r; }
+  }
+  return best;
+}
+
 // z passes: rows per block, transform length (half for even n, full for odd n:
 // two rows per transform), radices, threads, pitches.
 // D: FP64.
 template <int N, bool D> struct CZ {
   static constexpr bool ODD = N & 1;
   static constexpr int H = N / 2, NH = H + 1;
-  static constexpr int R = N <= 50 ? 8 : 16;            // at least 152 blocks from n = 36 up
+  static constexpr int R = z_rows(N, D);
   static constexpr int L = ODD ? N : H;
   static constexpr int LINES = ODD ? R / 2 : R;         // transforms per block and field
   static constexpr int GRID = cdiv(N * N, R);
   static constexpr CFac F = D ? dfac(L, 2 * LINES * L, cdiv(GRID, 152) < 2 ? 1 : 2) : cfac(L, !ODD);
   static constexpr int F0 = F.r[0], F1 = F.c >= 2 ? F.r[1] : 1, F2 = F.c == 3 ? F.r[2] : 1;
-  static constexpr int NT = N <= 50 ? 128 : 256;
+  static constexpr int NT = N <= 50 && R * N <= 400 ? 128 : 256;
   // element e of a line sits at e + e / F0 (even F0: the first stage writes
   // with stride F0); odd pitch, so that lines differ in bank
   static __host__ __device__ constexpr int pad(int e) { return (F0 & 1) ? e : e + e / F0; }

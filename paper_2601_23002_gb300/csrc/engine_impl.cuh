@@ -839,6 +839,7 @@ class Engine : public IEngine {
     OFDFT_RUN("k_fill", st, (double)N * sizeof(T), k_fill<T><<<grid_vec, kThreads, 0, st>>>(psi, (T)std::sqrt(nbar), N));
     const double Q = Ne / nbar;
     std::vector<int> rows{8, 16, 32}, cols{8, 16, 32};
+    if (cp && std::find(rows.begin(), rows.end(), cp->rows) == rows.end()) rows.push_back(cp->rows);
     if (planes) cols = {16};           // the plane pass has no column tiles
     const Tune saved = tune;
     double best = 1e300;

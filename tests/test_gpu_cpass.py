@@ -122,3 +122,31 @@ def test_density_aligned_to_single_values(n):
     plan.energy_potential(off, b)
     plan.close()
     assert float((a - b).abs().max()) <= 1e-12 * float(a.abs().max())
+
+
+# FP64 passes whose rows per block are none of a tile schedule's usual counts: the
+# plan's own schedule, one it does not have a compile-time pass for, and the
+# autotuner's choice give the same potential (bound as above).
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [45, 54, 100])
+def test_tile_schedules_beside_the_compile_time_rows(n):
+    cell = random_cell(11, 8, 1.0, 2.0, 0.8, n)
+    rho = density(cell, torch.float64)
+    plan = plan_for_cell(cell, "fp64")
+
+    def go():
+        v = torch.empty_like(rho)
+        plan.profile_enable(False)
+        plan.energy_potential(rho, v)
+        return v, set(plan.profile_read())
+
+    v0, k0 = go()
+    plan.set_tiles((16, 16, 16))
+    v1, k1 = go()
+    tiles, _ = plan.autotune()
+    v2, _ = go()
+    plan.close()
+    assert "k_zinv_c" in k0 and "k_zinv_epi" in k1
+    assert all(8 <= t <= 64 for t in tiles)
+    for v in (v1, v2):
+        assert float((v - v0).abs().max()) <= 1e-12 * float(v0.abs().max())
