@@ -12,12 +12,15 @@
 // G-space terms sit between the last forward and the first inverse stage in
 // registers, the last inverse stage stores to memory; all fields of a z pass go
 // through each stage together (three barriers instead of a dozen); and the plane
-// of a small grid is spread over a cluster of up to four blocks.
+// of a small grid, or one too large for a block, is spread over a cluster of up to
+// five blocks.  One evaluation with its call, before and now: FP32 75^3 92 -> 48 us,
+// 128^3 143 -> 87; FP64 45^3 193 -> 96.
 //
-// The transforms keep the generic passes' radices (the same search, evaluated
-// at compile time), twiddles and operation order, so a spectrum or a potential
-// has the same bits: the rounding of the psi transform, amplified by G^2, is
-// the largest error of an FP32 potential.
+// The FP32 transforms up to 160 keep the generic passes' radices (the same search,
+// evaluated at compile time), twiddles and operation order, so a spectrum or a
+// potential has the same bits: the rounding of the psi transform, amplified by G^2,
+// is the largest error of an FP32 potential.  FP64 takes the radices that suit its
+// pipe (dfac).
 #pragma once
 #include <initializer_list>
 #include <cooperative_groups.h>

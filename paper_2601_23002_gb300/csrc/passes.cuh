@@ -1,6 +1,9 @@
-// The per-evaluation kernels of the functional (templated on the real type T).
+// The per-evaluation kernels of the functional (templated on the real type T), in
+// their general form: grids without a plane pass (plane.cuh), compile-time passes
+// (cpass.cuh) or those of 256^3 (zpass256.cuh), which share the pointwise
+// functional below.
 //
-// One evaluation of F[n] and its potential is five launches over the grid:
+// One evaluation of F[n] and its potential is then five launches over the grid:
 //   1. k_zfwd      prologue (n, n^a, psi from rho or from psi + t d) fused with
 //                  the real-to-complex FFT along z (a half-length complex FFT
 //                  per row for even n, one length-n complex FFT per two rows
@@ -13,7 +16,7 @@
 //   5. k_zinv_epi  complex-to-real FFT along z fused with the pointwise
 //                  functional (finite-T TF through the inverse Fermi-Dirac
 //                  integral, PZ LDA XC, v_NL) and the potential / gradient.
-// plus k_finalize, a one-block FP64 reduction of the per-block partial sums.
+// The last block of 5 adds the per-block partial sums.
 //
 // Layouts: real fields [n][n][n] (z fastest); half spectra [n][n][n/2+1].
 #pragma once

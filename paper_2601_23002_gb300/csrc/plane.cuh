@@ -1,9 +1,10 @@
 // Fused x-y transform and G-space pass over whole kz planes (plane layout).
 //
 // With the half spectrum stored plane by plane, [kz][kx][ky], one kz plane of
-// one field (n x n complex) fits in shared memory for the grids most cells
-// use (FP32 n <= 160, FP64 n <= 112).  One block then does, on data that stays
-// on chip:
+// one field (n x n complex) fits in shared memory for FP32 n <= 160 and FP64
+// n <= 112.  This is the form with run-time sizes, for the grids of 8 to 20 points
+// (those from 24 up have compile-time passes, cpass.cuh; OFDFT_CPASS=0 takes them
+// here).  One block does, on data that stays on chip:
 //   forward FFT along y, forward FFT along x, the G-space terms, inverse FFT
 //   along x, inverse FFT along y
 // -- the work of the y-pass / x-G-space / y-pass chain, with one read and one
@@ -305,7 +306,8 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) k_plane(Spectra<T> sp, GArgs
 // columns between the pair and reach the partner's rows through distributed
 // shared memory, with a cluster barrier after every stage.  With one field the
 // plain plane pass occupies only n/2 + 1 SMs; this uses twice as many, each
-// with half the work.  grid.x = 2 (n/2 + 1).
+// with half the work.  grid.x = 2 (n/2 + 1).  For the grids without compile-time
+// passes: 162^3 in FP64.
 template <typename T, unsigned MASK>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPlaneThreads, 1)
 k_plane_prec2(Spectra<T> sp, GArgs<T> g, FftPlan1 pn, const int* __restrict__ rev_g,

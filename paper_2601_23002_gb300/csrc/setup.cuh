@@ -637,7 +637,7 @@ __global__ void k_forces_q(const cplx<T>* __restrict__ nt, SpecView view, const 
 // Ewald real-space force on ion I = block / nsplit from the share
 // block % nsplit of its (J, image) terms, FP64, into part[block * 3
 // ..] (k_sum_force_parts adds the shares in a fixed order).  Images and
-// compaction of the in-range terms as in k_ewald_real.
+// compaction of the in-range terms as in ewald_real_part.
 struct EwaldForceArgs {
   const double *pos, *Z;
   double L, eta, rcut;

@@ -85,7 +85,9 @@ __device__ __forceinline__ void z256_pass2(const cplx<T>* __restrict__ xb, const
 // parameter, so the row arithmetic is shifts and masks).  Each team reads its
 // row's pairs (x_2m, x_2m+1) straight from memory (rho, or psi and d) and
 // forms the field's input in registers.  smem: twN[NH] | twH[H] | xbuf[TEAMS][XP]
-// (37 KB: four blocks per SM).
+// (37 KB: four blocks per SM).  Bound by instruction issue and its scattered stores:
+// 16 rows fill a 128-byte line of a spectrum (two fields 103 us with 8 rows, 84 with
+// 16); lines stored whole instead of by halves, one field 69 -> 54 us, two 83 -> 88.
 template <typename T, int R>
 __global__ void __launch_bounds__(256, 4) k_zfwd256(ProArgs<T> a, Spectra<T> sp, const cplx<T>* __restrict__ tw_h,
                                                    const cplx<T>* __restrict__ tw_n) {
@@ -188,7 +190,9 @@ __global__ void __launch_bounds__(256, 4) k_zfwd256(ProArgs<T> a, Spectra<T> sp,
 // straight from memory in the pointwise loop, one row ahead, rather than
 // staged: 33 KB less shared memory per block at 16 rows, three blocks per SM
 // instead of two.
-// KIND: see EpiPoint (3: mode 3).
+// KIND: see EpiPoint (3: mode 3).  Bound by instruction issue, half of it the
+// functional: 270 us (8 rows), 226 (16 rows), 197 (the functional specialised by
+// KIND, binade polynomials), 186 (block sums by warp halving).
 template <typename T, int R, int KIND>
 __global__ void __launch_bounds__(256, 3) k_zinv256(Spectra<T> sp, EpiArgs<T> a, const cplx<T>* __restrict__ tw_h,
                                                    const cplx<T>* __restrict__ tw_n) {
@@ -543,8 +547,11 @@ __global__ void __launch_bounds__(256, 3) k_xgspace256(Spectra<T> sp, GArgs<T> g
 // in the row); the x transforms group the same sums differently (32 x 8 in
 // place of 16 x 16), so results agree with the other passes to FP32 rounding.
 // grid = (8 * 129 kz, active field), 256 threads, 66 KB of shared memory
-// (slice[32][256] | tw[256]): up to three blocks per SM.  FP32 only (the
-// row copies move two complex values per 16 bytes).
+// (slice[32][256] | tw[256]): up to three blocks per SM.  FP32 only.
+//
+// Bound by instruction issue and its cluster barriers: rows go from and to memory in
+// registers, without a staging copy, and a thread takes the columns +-ky, which share
+// the factors of two points: two fields 209 -> 189 us, one field 120 -> 103.
 struct P256 {
   static constexpr int N = 256, NH = 129, CL = 8, ROWS = N / CL, P = N, THREADS = 256;
 };
