@@ -1012,7 +1012,8 @@ class Engine : public IEngine {
     FinArgs<T> fa{pt, g_rows, pe, grid_z, sync || to_host ? res_h : res_d};
     const double cy = 9.8696044010893586188344909998762 / (1.4142135623730950488016887242097 * std::pow(Te, 1.5));
     EpiArgs<T> ea{mode, rho, ps, dd, (T)t, (T)scale, (T)cs.alpha, (T)Te, (T)cy, (T)mu_ref, cs.terms, out, pe, fa,
-                  counters + 0, nullptr, nullptr, dsc, cs.fd64 ? 1 : 0, cy, (T)std::log(cy)};
+                  counters + 0, nullptr, nullptr, dsc, cs.fd64 ? 1 : 0, cy, (T)(std::log2(cy) / 3.0),
+                  (T)(std::log(cy) / 3.0 + std::log(0.62035049089940001666800681204778))};
     const double eb = (double)sp.nact * NH * sizeof(C) + (double)(mode == 0 ? 1 : 2) * N * sizeof(T) + (out ? (double)N * sizeof(T) : 0.0);
     if (int rc = launch_zinv(sp, ea, eb, st)) return rc;
     if (sync) {

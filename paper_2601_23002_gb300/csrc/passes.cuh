@@ -164,11 +164,14 @@ static __device__ __forceinline__ void pz81(double n, double& exc, double& vxc) 
   vxc = vx + vc;
 }
 
-// FP32: l2 = log2 n is given.  w = n^(-1/3) from 2^(-l2/3) and one Newton step
-// of w^-3 = n (to FP32 rounding), so no cube root, and ln r_s from l2; fast
-// reciprocals (a few ulp: inside the float rounding of the terms they feed).
-static __device__ __forceinline__ void pz81_l2(float n, float l2, float& exc, float& vxc) {
-  float w = exp2f(l2 * (-1.0f / 3.0f));
+// FP32: l2 = log2(n c) is given, with c3 = log2(c) / 3 and lr = ln(c) / 3 +
+// ln 0.62035.  w = n^(-1/3) from 2^(-log2(n) / 3) and one Newton step of w^-3 = n
+// (to FP32 rounding), so no cube root, and ln r_s from l2; the square root with a
+// Newton step of its own; fast reciprocals (a few ulp: inside the float rounding of
+// the terms they feed).
+constexpr float kLnRs1 = -0.477470652767060400f;       // ln 0.62035049
+static __device__ __forceinline__ void pz81_l2(float n, float l2, float c3, float lr, float& exc, float& vxc) {
+  float w = exp2f(fmaf(l2, -1.0f / 3.0f, c3));
   w = fmaf(w * (1.0f / 3.0f), fmaf(-(n * w), w * w, 1.0f), w);
   const float rs = 0.620350490899400017f * w;
   const float ex = -0.738558766382022406f * (n * w) * w;
@@ -176,21 +179,22 @@ static __device__ __forceinline__ void pz81_l2(float n, float l2, float& exc, fl
   float ec, vc;
   if (rs >= 1.0f) {
     const float g = (float)kPzG, b1 = (float)kPzB1, b2 = (float)kPzB2;
-    const float sq = rs * rsqrtf(rs);
+    const float q = rsqrtf(rs), s0 = rs * q;
+    const float sq = fmaf(fmaf(-s0, s0, rs), 0.5f * q, s0);
     const float inv = __fdividef(1.0f, 1.0f + b1 * sq + b2 * rs);
     ec = g * inv;
     vc = ec * (1.0f + (7.0f / 6.0f) * b1 * sq + (4.0f / 3.0f) * b2 * rs) * inv;
   } else {
     const float A = (float)kPzA, B = (float)kPzB, C = (float)kPzC, D = (float)kPzD;
     // ln r_s = ln 0.62035 - (ln 2 / 3) log2 n
-    const float ln = fmaf(l2, -0.231049060186648431f, -0.477470652767060400f);
+    const float ln = fmaf(l2, -0.231049060186648431f, lr);
     ec = A * ln + B + C * rs * ln + D * rs;
     vc = A * ln + (B - A * (1.0f / 3.0f)) + (2.0f / 3.0f) * C * rs * ln + (2.0f * D - C) * (1.0f / 3.0f) * rs;
   }
   exc = ex + ec;
   vxc = vx + vc;
 }
-static __device__ __forceinline__ void pz81(float n, float& exc, float& vxc) { pz81_l2(n, __log2f(n), exc, vxc); }
+static __device__ __forceinline__ void pz81(float n, float& exc, float& vxc) { pz81_l2(n, __log2f(n), 0.0f, kLnRs1, exc, vxc); }
 
 static __device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
 static __device__ __forceinline__ double rsqrt_t(double x) { return rsqrt(x); }
@@ -631,7 +635,7 @@ template <typename T> struct EpiArgs {
   const double* dsc;     // when set, scale = dsc[0] and t = dsc[2] (a trial formed on the device)
   int fd64;              // FP32 plans: invert the Fermi-Dirac integral in FP64 (y = cy_d n in FP64)
   double cy_d;           // pi^2 / (sqrt2 T^(3/2)) in FP64, for fd64
-  T lcy;                 // ln cy (FP32 plans: ln y = ln 2 log2 n + ln cy)
+  T c3, lr;              // log2(cy) / 3, ln(cy) / 3 + ln 0.62035 (FP32 plans: XC from log2 y, pz81_l2)
 };
 
 // The pointwise functional at one grid point, shared by the z-pass epilogue
@@ -647,10 +651,10 @@ template <typename T> struct EpiArgs {
 // point and a tenth of the registers).
 template <typename T, int KIND> struct EpiPoint {
   bool has_n, has_na, has_psi, merged;
-  T Te, cy, lcy, alpha, nmin, tstep, tscale, muref;
+  T Te, cy, c3, lr, alpha, nmin, tstep, tscale, muref;
   __device__ __forceinline__ EpiPoint(const Spectra<T>& sp, const EpiArgs<T>& a)
       : has_n(KIND || sp.s[0] != nullptr), has_na(!KIND && sp.s[1] != nullptr), has_psi(KIND || sp.s[2] != nullptr),
-        merged(KIND || sp.merged != 0), Te(a.T_e), cy(a.cy), lcy(a.lcy), alpha(a.alpha), nmin((T)kNmin),
+        merged(KIND || sp.merged != 0), Te(a.T_e), cy(a.cy), c3(a.c3), lr(a.lr), alpha(a.alpha), nmin((T)kNmin),
         tstep(a.dsc ? (T)a.dsc[2] : a.t), tscale(a.dsc ? (T)a.dsc[0] : a.scale), muref(a.mu_ref) {}
   static __device__ __forceinline__ int mode(const EpiArgs<T>& a) { return KIND == 1 ? 1 : KIND == 2 ? 0 : a.mode; }
   __device__ __forceinline__ void point(const EpiArgs<T>& a, T pv, T dq, T hv, T kv, T lv, size_t at,
@@ -667,8 +671,11 @@ template <typename T, int KIND> struct EpiPoint {
       nval = tscale * psit * psit;
     }
     const T nf = fmax(nval, nmin);
-    T l2 = 0;                            // FP32: one logarithm for TF and XC
-    if constexpr (sizeof(T) == 4) l2 = __log2f(nf);
+    // FP32: one logarithm for TF and XC, of y = n cy itself: ln n + ln cy, with a
+    // rounded constant, moved eta by the same 1e-7 at every point (F_TF off by 6e-8
+    // Ha/ion at 128^3, 1.6e-8 so)
+    T l2 = 0;
+    if constexpr (sizeof(T) == 4) l2 = __log2f(nf * cy);
     T vrest = 0;
     if (KIND || (a.terms & 1)) {              // TF
       if (!KIND && sizeof(T) == 4 && a.fd64) {
@@ -680,7 +687,7 @@ template <typename T, int KIND> struct EpiPoint {
         acc[0].add((T)((double)nf * te * (eta - p)));
       } else {
         T eta, p;
-        if constexpr (sizeof(T) == 4) fd_eta_p_s(nf * cy, fmaf(l2, 0.693147180559945309f, lcy), eta, p);
+        if constexpr (sizeof(T) == 4) fd_eta_p_s(nf * cy, l2 * 0.693147180559945309f, eta, p);
         else fd_eta_p(nf * cy, eta, p);
         vrest += Te * eta;
         acc[0].add(nf * Te * (eta - p));
@@ -688,7 +695,7 @@ template <typename T, int KIND> struct EpiPoint {
     }
     if (KIND || (a.terms & 8)) {              // XC
       T exc, vxc;
-      if constexpr (sizeof(T) == 4) pz81_l2(nf, l2, exc, vxc);
+      if constexpr (sizeof(T) == 4) pz81_l2(nf, l2, c3, lr, exc, vxc);
       else pz81(nf, exc, vxc);
       vrest += vxc;
       acc[1].add(nval * exc);
