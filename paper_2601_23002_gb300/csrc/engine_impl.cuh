@@ -801,6 +801,13 @@ class Engine : public IEngine {
         if ((rc = raise((const void*)pl.kern, pl.bytes))) return rc;
     }
     if (prec2 && (rc = raise((const void*)prec2_kern, smem_pl2))) return rc;
+    // (the 2 x 4 tile of FP32 plans takes 52 to 69 KB where its threads along kz
+    // are more than 42: 360 to 500 points)
+    if constexpr (sizeof(T) == 4)
+      if ((rc = raise((const void*)k_struct<T, 2, 4, 256>, struct_smem<T, 2, 4, 256>(struct_ct(nh, 4))))) return rc;
+    if ((rc = raise((const void*)k_struct<T, 2, 2, 256>, struct_smem<T, 2, 2, 256>(struct_ct(nh, 2))))) return rc;
+    if ((rc = raise((const void*)k_struct<T, 1, 2, 128>, struct_smem<T, 1, 2, 128>(struct_ct(nh, 2))))) return rc;
+    if ((rc = raise((const void*)k_struct<T, 1, 1, 64>, struct_smem<T, 1, 1, 64>(struct_ct(nh, 1))))) return rc;
     const size_t sring = StreamCfg<T>::ring_bytes(3, 17);   // largest ring any streaming launch uses
     if ((rc = raise((const void*)k_gram<T, 1, 3>, sring))) return rc;
     if ((rc = raise((const void*)k_gram<T, 2, 3>, sring))) return rc;
@@ -891,8 +898,7 @@ class Engine : public IEngine {
     bool done = false;
     auto go = [&](auto TRc, auto TCc, auto NTc, int least) -> int {
       constexpr int TR = decltype(TRc)::value, TC = decltype(TCc)::value, NT = decltype(NTc)::value;
-      const int ctiles = (nh + TC * 64 - 1) / (TC * 64);        // at most 64 threads along kz
-      const int CT = (nh + TC * ctiles - 1) / (TC * ctiles);
+      const int ctiles = struct_ctiles(nh, TC), CT = struct_ct(nh, TC);
       const int RT = NT / CT * TR;
       if (RT > 32 * struct_nr(TR, TC)) return OFDFT_OK;
       const int g = (nrows + RT - 1) / RT;

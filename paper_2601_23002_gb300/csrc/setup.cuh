@@ -94,6 +94,9 @@ template <typename T> struct alignas(16) Quad { T a, b, c, d; };
 template <typename T> struct StructCH { static constexpr int v = sizeof(T) == 4 ? 16 : 8; };   // ions per chunk
 // rows a lane of the staging holds: a block has at most 32 of these rows
 __host__ __device__ constexpr int struct_nr(int TR, int TC) { return TR * TC == 4 ? 2 : 1; }
+// kz tiles and threads along kz (at most 64) for nh columns, TC to a thread
+constexpr int struct_ctiles(int nh, int TC) { return (nh + TC * 64 - 1) / (TC * 64); }
+constexpr int struct_ct(int nh, int TC) { return (nh + TC * struct_ctiles(nh, TC) - 1) / (TC * struct_ctiles(nh, TC)); }
 template <typename T, int TR, int TC, int NT>
 constexpr size_t struct_smem(int CT) {
   return 2 * (size_t)StructCH<T>::v * ((size_t)CT * TC * sizeof(cplx<T>) + (size_t)(NT / CT) * TR * sizeof(Quad<T>));
