@@ -945,7 +945,10 @@ class Engine : public IEngine {
     // one ion species (every workload here): S_Z = Z S, one sum over the ions
     bool uni = true;
     for (double z : cs.Z) uni = uni && z == cs.Z[0];
-    StructOut<T> so{Sg, (C*)S_out, uni ? SZg : nullptr, vloc, cs.Z[0], sf_tab, (double)sf_m2, partials, uni ? res_h : nullptr, real, gb, counters + 4};
+    // S_out may be aligned to single values (C's double complex is): k_struct, which
+    // stores whole complex values, then leaves the second copy to a copy at the end
+    const bool direct = S_out && reinterpret_cast<uintptr_t>(S_out) % sizeof(C) == 0;
+    StructOut<T> so{Sg, direct ? (C*)S_out : nullptr, uni ? SZg : nullptr, vloc, cs.Z[0], sf_tab, (double)sf_m2, partials, uni ? res_h : nullptr, real, gb, counters + 4};
     if (int rc = launch_struct(so, nullptr, full, st)) return rc;
     if (!uni) {
       so.S = so.S2 = nullptr; so.SZ = SZg; so.zs = 1.0; so.res = res_h;
@@ -957,6 +960,7 @@ class Engine : public IEngine {
       const int m2max = (int)std::min(3.0 * h * h, std::floor(g2cut_loc / (tp * tp) * (1.0 + 1e-5)) + 1.0);
       OFDFT_RUN("k_vloc_planes", st, 2.0 * n_vloc * sizeof(C), k_vloc_planes<T><<<dim3((n + 31) / 32, n), 256, 0, st>>>(vloc, vloc_pl, planes ? rev_d : nullptr, n, m2max));
     }
+    if (S_out && !direct) OFDFT_CK(cudaMemcpyAsync(S_out, Sg, NH * sizeof(C), cudaMemcpyDeviceToDevice, st));
     OFDFT_CK(cudaStreamSynchronize(st));
     double zz = 0;
     for (double z : cs.Z) zz += z * z;
