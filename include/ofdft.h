@@ -28,6 +28,7 @@
  *   f~(G) = (1/N) sum_r f(r) exp(-i G.r), N = n^3.
  * Element type: double for OFDFT_FP64 plans, float for OFDFT_FP32 plans
  * (FP32 bulk arithmetic with FP64 reductions, FP64 line search).
+ * Alignment: device arrays need that of their single values (4 or 8 bytes).
  *
  * Errors: every call returns an ofdft_status; 0 is success.  On failure the
  * outputs are left unspecified unless the call says otherwise, and

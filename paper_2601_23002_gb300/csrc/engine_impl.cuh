@@ -422,14 +422,12 @@ class Engine : public IEngine {
     }
   }
 
-  // The compile-time passes.  Even grids read two reals at a time, so a
-  // density that is not aligned to them takes the generic forward pass.
-  bool czfwd_ok(const ProArgs<T>& pa) const {
-    return cpz() && ((n & 1) || pa.mode != 0 || reinterpret_cast<uintptr_t>(pa.rho) % sizeof(C) == 0);
-  }
+  // The compile-time passes of even grids and the 256^3 pass read two reals at a
+  // time: a density that is not aligned to them takes the generic forward pass.
+  static bool pairs_ok(const ProArgs<T>& pa) { return pa.mode != 0 || reinterpret_cast<uintptr_t>(pa.rho) % sizeof(C) == 0; }
   int launch_zfwd(const ProArgs<T>& pa, const Spectra<T>& sp, double bytes, cudaStream_t st) {
-    if (z256) return launch_zfwd256(pa, sp, bytes, st);
-    if (czfwd_ok(pa)) OFDFT_RUN("k_zfwd_c", st, bytes, launch_pdl(cp->zfwd, cp->zgrid, cp->zthreads, cp->zf_bytes[sp.nact], st, pa, sp, tw_h, tw_n));
+    if (z256 && pairs_ok(pa)) return launch_zfwd256(pa, sp, bytes, st);
+    if (cpz() && ((n & 1) || pairs_ok(pa))) OFDFT_RUN("k_zfwd_c", st, bytes, launch_pdl(cp->zfwd, cp->zgrid, cp->zthreads, cp->zf_bytes[sp.nact], st, pa, sp, tw_h, tw_n));
     else OFDFT_RUN("k_zfwd", st, bytes, k_zfwd<T><<<grid_z, kThreads, smem_zf, st>>>(pa, sp, ph, tw_h, tw_n, n, zR, zP));
     return OFDFT_OK;
   }
@@ -1040,10 +1038,9 @@ class Engine : public IEngine {
     Spectra<T> sp{};
     sp.nact = nf;
     for (int i = 0; i < nf; ++i) { sp.idx[i] = fld[i]; sp.s[fld[i]] = spec[fld[i]]; }
-    // (the 256^3 pass reads two reals at a time)
-    const bool pl256 = p256 && reinterpret_cast<uintptr_t>(rho) % sizeof(C) == 0;
-    sp.planes = (cp || pl256) ? 1 : 0;
     ProArgs<T> pa{0, rho, nullptr, nullptr, (T)0, (T)1, (T)cs.alpha, (T)std::sqrt(nbar), nullptr, kzmax + 1};
+    const bool pl256 = p256 && pairs_ok(pa);
+    sp.planes = (cp || pl256) ? 1 : 0;
     const int nk = std::min(nh, kzmax + 1);
     const double zb = (double)N * sizeof(T) + (double)nf * n * n * nk * sizeof(C);
     const double yb = 2.0 * nf * n * n * nk * sizeof(C);

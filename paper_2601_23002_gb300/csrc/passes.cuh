@@ -772,16 +772,20 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_zinv_epi(Spectr
     // starts on an 8-byte boundary (n even, or an even number of rows per
     // block); an odd element count leaves one element for a 4-byte copy
     constexpr int E = 8 / sizeof(T);
-    const int pieces = tot / E;
     // (mode 3: the previous output pold, when P y = out - pold is wanted)
     const T* src0 = a.mode == 0 ? a.rho : (a.mode == 3 ? a.pold : a.psi);
     const bool want = a.mode != 3 || a.pyout != nullptr;
+    // (the caller's density may be aligned to single values: those one by one)
+    const bool single = reinterpret_cast<uintptr_t>(src0) % 8 != 0;
+    const int pieces = single ? 0 : tot / E;
     const int npc = want ? pieces : 0;
+    if (single && want)
+      for (int q = threadIdx.x; q < tot; q += blockDim.x) cp_async<sizeof(T)>(pin + q, src0 + off + q, true);
     for (int q = threadIdx.x; q < npc; q += blockDim.x) {
       cp_async<8>(pin + q * E, src0 + off + q * E, true);
       if (a.mode == 1) cp_async<8>(pin + (size_t)Rfull * n + q * E, a.d + off + q * E, true);
     }
-    if (want && pieces * E < tot && threadIdx.x == 0) {
+    if (want && !single && pieces * E < tot && threadIdx.x == 0) {
       const int q = tot - 1;                 // E = 2 and tot odd: the last float
       cp_async<sizeof(T)>(pin + q, src0 + off + q, true);
       if (a.mode == 1) cp_async<sizeof(T)>(pin + (size_t)Rfull * n + q, a.d + off + q, true);
