@@ -63,14 +63,15 @@ __device__ __forceinline__ void phases_part(const double* __restrict__ pos, int 
 // sum w f.y |SZ|^2 over the entries of rows with |G|^2 <= g2rows:
 //   f = (v~(G)/Omega per unit charge, (2 pi/Omega) exp(-G^2/(4 eta^2))/G^2) by m^2,
 // tabulated once per plan.  FP32 plans hold the first as two floats, so that V_loc
-// is the FP32 rounding of the exact product as before without FP64 conversions and
-// products (a third of the kernel's time on the FP64 pipe), and sum the second in
-// compensated FP32: |SZ|^2 carries 3e-7 already.
+// is the FP32 rounding of the exact product without FP64 conversions and products.
+// The Ewald sum is FP64 from weight to sum in every plan: it enters F directly, and
+// its size (thousands of hartree in a large cell) is far above that of its changes.
 // grid: (row tiles, kz tiles); CT threads along kz.
 template <typename T> struct SfEntry;
 template <> struct alignas(16) SfEntry<float> {
-  float v, vlo, e, pad;
-  static SfEntry make(double a, double b) { return {(float)a, (float)(a - (double)(float)a), (float)b, 0.f}; }
+  float v, vlo;
+  double e;
+  static SfEntry make(double a, double b) { return {(float)a, (float)(a - (double)(float)a), b}; }
   __device__ __forceinline__ float vloc(float z) const { return fmaf(v, z, vlo * z); }
 };
 template <> struct alignas(16) SfEntry<double> {
@@ -214,7 +215,7 @@ __global__ void __launch_bounds__(NT) k_struct(const cplx<T>* __restrict__ ph, c
     if (more) { store_rows(I0 + CH, buf ^ 1); cp_async_wait<0>(); }
     __syncthreads();
   }
-  Acc<T> ewa;
+  double ewa = 0;
 #pragma unroll
   for (int i = 0; i < TR; ++i) {
     const int r = blockIdx.x * RT + rt + RB * i;
@@ -230,7 +231,7 @@ __global__ void __launch_bounds__(NT) k_struct(const cplx<T>* __restrict__ ph, c
       const T(&x)[8] = acc[i][j];
       SfEntry<T> f{};
       if (inside) f = o.sf_tab[a * a + b * b + kz * kz];
-      const T w = (kz == 0 || 2 * kz == n) ? (T)1 : (T)2;
+      const double we = (kz == 0 || 2 * kz == n ? 1.0 : 2.0) * f.e;
       auto put = [&](int kx, int ky, T re, T im) {
         const size_t at = ((size_t)kx * n + ky) * nh + kz;
         const cplx<T> s = mk<T>(re, im);
@@ -242,7 +243,7 @@ __global__ void __launch_bounds__(NT) k_struct(const cplx<T>* __restrict__ ph, c
           o.SZ[at] = sz;
           if (inside) {
             o.vloc[at] = mk<T>(f.vloc(sz.x), f.vloc(sz.y));
-            ewa.add(w * f.e * (sz.x * sz.x + sz.y * sz.y));
+            ewa += we * ((double)sz.x * (double)sz.x + (double)sz.y * (double)sz.y);
           } else {
             o.vloc[at] = mk<T>((T)0, (T)0);
           }
@@ -254,7 +255,7 @@ __global__ void __launch_bounds__(NT) k_struct(const cplx<T>* __restrict__ ph, c
       if (ma && pb) put(n - a, b, x[4] + x[5], x[6] - x[7]);
     }
   }
-  double v[1] = {ewa.get()}, out[1];
+  double v[1] = {ewa}, out[1];
   block_sum<1>(v, red, out);
   if (tid == 0) o.ew[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = out[0];
   const int nb = gridDim.x * gridDim.y;
