@@ -174,7 +174,8 @@ class Engine : public IEngine {
   unsigned int* counters = nullptr;   // last-block arrival counters (0 between launches)
   double* pos_d = nullptr;
   double* Z_d = nullptr;
-  C* phases = nullptr;       // exp(-2 pi i m R / L) per ion and axis (k_phases)
+  typename Phase<T>::type* phases = nullptr;   // exp(-2 pi i m R / L) per ion and axis (phases_part)
+  C* phases_t = nullptr;                       // the same in the plan's type (FP64 plans: phases)
   // row pairs (a, b) of the structure factor without the full S(G), and whether
   // the entries outside their rows are zero
   int2* sf_rows = nullptr;
@@ -601,6 +602,8 @@ class Engine : public IEngine {
     if ((rc = alloc(&pos_d, (size_t)cs.Z.size() * 3))) return rc;
     if ((rc = alloc(&Z_d, cs.Z.size()))) return rc;
     if ((rc = alloc(&phases, (size_t)cs.Z.size() * 3 * n))) return rc;
+    if constexpr (sizeof(T) == 8) phases_t = phases;
+    else if ((rc = alloc(&phases_t, (size_t)cs.Z.size() * 3 * n))) return rc;
     OFDFT_CK(cudaMemcpyAsync(Z_d, cs.Z.data(), cs.Z.size() * sizeof(double), cudaMemcpyHostToDevice, st));
     // shared-memory limits
     if ((rc = raise_smem_limits())) return rc;
@@ -902,7 +905,7 @@ class Engine : public IEngine {
       const int g = (nrows + RT - 1) / RT;
       if (g * ctiles < least) return OFDFT_OK;
       const size_t sm = struct_smem<T, TR, TC, NT>(CT);
-      OFDFT_RUN("k_struct", st, (double)nrows * 4 * nh * sizeof(C) * 3.0, k_struct<T, TR, TC, NT><<<dim3(g, ctiles), NT, sm, st>>>(phases, zw, (int)cs.Z.size(), n, rows, nrows, CT, so));
+      OFDFT_RUN("k_struct", st, (double)nrows * 4 * nh * sizeof(C) * 3.0, k_struct<T, TR, TC, NT><<<dim3(g, ctiles), NT, sm, st>>>(phases, phases_t, zw, (int)cs.Z.size(), n, rows, nrows, CT, so));
       done = true;
       return OFDFT_OK;
     };
@@ -929,7 +932,7 @@ class Engine : public IEngine {
     const int gb = (int)std::min<long>(2L * nsm, (ncomb + 255) / 256);
     const int gp = std::min(4 * nsm, (nion * 3 + 7) / 8);
     double* real = partials + partials_cap - gb;         // behind k_struct's partials
-    OFDFT_RUN("k_ions", st, (double)nion * 3 * n * sizeof(C), k_ions<T><<<gb + gp, 256, 0, st>>>(pos_d, Z_d, nion, n, L, phases, eta, rcut, nimg_mi, gb, real));
+    OFDFT_RUN("k_ions", st, (double)nion * 3 * n * (16 + (sizeof(T) == 4 ? sizeof(C) : 0)), k_ions<T><<<gb + gp, 256, 0, st>>>(pos_d, Z_d, nion, n, L, phases, phases_t, eta, rcut, nimg_mi, gb, real));
     const int full = S_out != nullptr;
     // without the full S(G) only the rows inside sf_m2 are formed, the others
     // stay zero
@@ -1654,7 +1657,7 @@ int Engine<T>::forces(const void* rho, double* f_out_h, void* stream_) {
   constexpr int TI = sizeof(T) == 4 ? 4 : 2;
   const int ny = (nion + kForceWarps * TI - 1) / (kForceWarps * TI);
   const EwaldForceArgs wa{pos_d, Z_d, L, ew_eta, ew_rcut, ew_nimg, nsplit, partials};
-  OFDFT_RUN("k_forces_g", st, (double)f_nk * 128 * sizeof(C), k_forces_g<T, TI><<<f_ntile * ny + nion * nsplit, 32 * kForceWarps, 0, st>>>(f_qq, f_rows, f_nrows, f_tk, phases, nion, n, f_part, f_ntile, ny, wa));
+  OFDFT_RUN("k_forces_g", st, (double)f_nk * 128 * sizeof(C), k_forces_g<T, TI><<<f_ntile * ny + nion * nsplit, 32 * kForceWarps, 0, st>>>(f_qq, f_rows, f_nrows, f_tk, phases_t, nion, n, f_part, f_ntile, ny, wa));
   OFDFT_RUN("k_sum_force_parts", st, (double)nion * nsplit * 24, k_sum_force_parts<<<(3 * nion + 3) / 4, 128, 0, st>>>(f_part, f_ntile, Z_d, tp, partials, nion, nsplit, f_out));
   OFDFT_CK(cudaMemcpyAsync(f_out_h, f_out, (size_t)nion * 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
   OFDFT_CK(cudaStreamSynchronize(st));

@@ -9,37 +9,87 @@ namespace ofdft {
 // ---------------------------------------------------------------------------
 // Structure factor on the half spectrum.  Phases factorise per axis:
 // exp(-i G.R) = e_x(m_x) e_y(m_y) e_z(m_z) with e_d(m) = exp(-2 pi i m R_d / L);
-// ph[(I*3 + d)*n + k] holds them (k in FFT order), formed in FP64 and rounded to
-// the plan's type; one sine and cosine per |m|, the negative m by conjugation.
-// One warp per (ion, axis): its lanes evaluate e(0..15) and e(16 k), k = 0..15
-// (one FP64 sine and cosine each; 65 of them per axis at 128^3 kept the FP64 pipe
-// busy for 13 us with 300 ions), and e(16 k + l) = e(16 k) e(l).
+// ph[(I*3 + d)*n + k] holds them (k in FFT order): FP64 values, in FP32 plans as pairs
+// of floats (48 bits); pt the same rounded to the plan's type (FP64 plans: ph itself).
+// One sine and cosine per |m|, the negative m by conjugation; one warp per (ion, axis).
+// FP32 plans: its lanes evaluate e(0..15) and e(16 k), k = 0..15 (one FP64 sine and
+// cosine each; 65 of them per axis at 128^3 kept the FP64 pipe busy for 13 us with 300
+// ions), and e(16 k + l) = e(16 k) e(l), 3e-16 off, below the pairs' 2e-15.  FP64 plans
+// evaluate every m (1e-16).
+template <typename T> struct Phase;
+template <> struct Phase<double> {
+  using type = double2;
+  static __device__ __forceinline__ double2 make(double c, double s) { return make_double2(c, s); }
+  static __device__ __forceinline__ double2 conj(double2 e) { return make_double2(e.x, -e.y); }
+};
+template <> struct Phase<float> {
+  using type = float4;                   // cos, sin, and their remainders
+  static __device__ __forceinline__ float4 make(double c, double s) {
+    const float ch = (float)c, sh = (float)s;
+    return make_float4(ch, sh, (float)(c - (double)ch), (float)(s - (double)sh));
+  }
+  static __device__ __forceinline__ float4 conj(float4 e) { return make_float4(e.x, -e.y, e.z, -e.w); }
+};
+template <typename T> struct alignas(16) Quad { T a, b, c, d; };
+// The row products P = e_x e_y and M = e_x e_y*: (Re P, Im P, Re M, Im M), each rounded
+// to the plan's type once.  FP32: exact products of the leading floats (their remainders
+// by fma) and of leading with trailing ones, two-sums: 1e-14 before the rounding, in 48
+// FP32 operations (four FP64 products and sums per row and ion took 35 us of the FP64
+// pipe for 300 ions on 128^3).
+static __device__ __forceinline__ Quad<double> row_products(double2 x, double2 y, double z) {
+  const double xr = x.x * z, xi = x.y * z;
+  return Quad<double>{xr * y.x - xi * y.y, xr * y.y + xi * y.x, xr * y.x + xi * y.y, xi * y.x - xr * y.y};
+}
+static __device__ __forceinline__ float2 pair_product(float ah, float al, float bh, float bl) {
+  const float p = __fmul_rn(ah, bh);     // (never fused into a sum)
+  return make_float2(p, fmaf(ah, bl, fmaf(al, bh, fmaf(ah, bh, -p))));
+}
+static __device__ __forceinline__ float pair_sum(float2 a, float2 b) {
+  const float s = a.x + b.x, t = s - a.x;
+  return s + ((a.x - (s - t)) + (b.x - t) + (a.y + b.y));
+}
+static __device__ __forceinline__ Quad<float> row_products(float4 x, float4 y, float z) {
+  const float2 rr = pair_product(x.x, x.z, y.x, y.z), ii = pair_product(x.y, x.w, y.y, y.w);
+  const float2 ri = pair_product(x.x, x.z, y.y, y.w), ir = pair_product(x.y, x.w, y.x, y.z);
+  const float2 mi = make_float2(-ii.x, -ii.y), mri = make_float2(-ri.x, -ri.y);
+  return Quad<float>{z * pair_sum(rr, mi), z * pair_sum(ri, ir), z * pair_sum(rr, ii), z * pair_sum(ir, mri)};
+}
 template <typename T>
 __device__ __forceinline__ void phases_part(const double* __restrict__ pos, int n_ion, int n, double L,
-                                            cplx<T>* __restrict__ ph, int block, int blocks) {
+                                            typename Phase<T>::type* __restrict__ ph, cplx<T>* __restrict__ pt, int block,
+                                            int blocks) {
   const int h = n / 2 + 1, lane = threadIdx.x & 31;
   const int per = blockDim.x >> 5;
   for (int q = block * per + (threadIdx.x >> 5); q < n_ion * 3; q += blocks * per) {
     double f = pos[q] / L;
     f -= floor(f);                       // wrap into [0, 1)
-    // angle = -2 pi m f; reduce m f modulo 1 before the trig call
-    const int m0 = lane < 16 ? lane : (lane - 16) * 16;
-    double mf = (double)m0 * f;
-    mf -= rint(mf);
-    double s0, c0;
-    sincospi(-2.0 * mf, &s0, &c0);
-    cplx<T>* o = ph + (size_t)q * n;
+    // exp(-2 pi i m f), m f reduced modulo 1 before the trig call
+    auto phase = [&](int m, double& s, double& c) {
+      double mf = (double)m * f;
+      mf -= rint(mf);
+      sincospi(-2.0 * mf, &s, &c);
+    };
+    auto put = [&](int k, double c, double s) {
+      ph[(size_t)q * n + k] = Phase<T>::make(c, s);
+      if constexpr (sizeof(T) == 4) pt[(size_t)q * n + k] = mk<T>((T)c, (T)s);
+    };
+    double s0 = 0, c0 = 0;
+    if constexpr (sizeof(T) == 4) phase(lane < 16 ? lane : (lane - 16) * 16, s0, c0);
     for (int mb = 0; mb < h; mb += 32) {
       const int m = mb + lane;
-      const int k = min(m >> 4, 15), l = m - 16 * k;     // m <= 256: l = 16 only with k = 15
-      const int ll = l < 16 ? l : 17;
-      const double ck = __shfl_sync(0xffffffffu, c0, 16 + k), sk = __shfl_sync(0xffffffffu, s0, 16 + k);
-      const double cl = __shfl_sync(0xffffffffu, c0, ll & 31), sl = __shfl_sync(0xffffffffu, s0, ll & 31);
-      double c = cl, s = sl;
-      if (k > 0) { c = ck * cl - sk * sl; s = ck * sl + sk * cl; }
+      double c, s;
+      if constexpr (sizeof(T) == 4) {
+        const int k = min(m >> 4, 15), l = m - 16 * k;     // m <= 256: l = 16 only with k = 15
+        const int ll = l < 16 ? l : 17;
+        const double ck = __shfl_sync(0xffffffffu, c0, 16 + k), sk = __shfl_sync(0xffffffffu, s0, 16 + k);
+        const double cl = __shfl_sync(0xffffffffu, c0, ll & 31), sl = __shfl_sync(0xffffffffu, s0, ll & 31);
+        c = cl; s = sl;
+        if (k > 0) { c = ck * cl - sk * sl; s = ck * sl + sk * cl; }
+      }
       if (m >= h) continue;
-      if (2 * m < n) o[m] = mk<T>((T)c, (T)s);
-      if (m > 0) o[n - m] = mk<T>((T)c, (T)-s);          // m = n/2 of even n is stored as -n/2
+      if constexpr (sizeof(T) == 8) phase(m, s, c);
+      if (2 * m < n) put(m, c, s);
+      if (m > 0) put(n - m, c, -s);          // m = n/2 of even n is stored as -n/2
     }
   }
 }
@@ -54,7 +104,8 @@ __device__ __forceinline__ void phases_part(const double* __restrict__ pos, int 
 // on the full 128^3 half spectrum; the FP32 pipe needs 17 us for these sums.)
 // A thread owns TR row pairs (a, b) and TC kz; the ions go in chunks of CH whose
 // row products and kz phases are staged in shared memory, so a chunk's step
-// reads TR + TC/2 16-byte groups for 8 TR TC multiply-adds.  Two stages: the next
+// reads TR + TC/2 16-byte groups for 8 TR TC multiply-adds.  The row products are
+// rounded to the plan's type once (row_products).  Two stages: the next
 // chunk's kz phases are copied asynchronously and its row phases loaded before
 // the current chunk's sums, one barrier per chunk.
 // rows: (a, b) list, or nullptr for all 0 <= a, b <= n/2.
@@ -91,7 +142,6 @@ template <typename T> struct StructOut {
   const double* real; int nreal;
   unsigned int* counter;
 };
-template <typename T> struct alignas(16) Quad { T a, b, c, d; };
 template <typename T> struct StructCH { static constexpr int v = sizeof(T) == 4 ? 16 : 8; };   // ions per chunk
 // rows a lane of the staging holds: a block has at most 32 of these rows
 __host__ __device__ constexpr int struct_nr(int TR, int TC) { return TR * TC == 4 ? 2 : 1; }
@@ -103,8 +153,9 @@ constexpr size_t struct_smem(int CT) {
   return 2 * (size_t)StructCH<T>::v * ((size_t)CT * TC * sizeof(cplx<T>) + (size_t)(NT / CT) * TR * sizeof(Quad<T>));
 }
 template <typename T, int TR, int TC, int NT>
-__global__ void __launch_bounds__(NT) k_struct(const cplx<T>* __restrict__ ph, const double* __restrict__ zw, int n_ion,
-                                               int n, const int2* __restrict__ rows, int nrows, int CT, StructOut<T> o) {
+__global__ void __launch_bounds__(NT) k_struct(const typename Phase<T>::type* __restrict__ ph, const cplx<T>* __restrict__ pt,
+                                               const double* __restrict__ zw, int n_ion, int n,
+                                               const int2* __restrict__ rows, int nrows, int CT, StructOut<T> o) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[32];
   constexpr int CH = StructCH<T>::v;
@@ -143,20 +194,21 @@ __global__ void __launch_bounds__(NT) k_struct(const cplx<T>* __restrict__ ph, c
   const int ncol = min(CC, nh - col0);
   auto stage_z = [&](int I0, int buf) {
     for (int c = wid; c < CH && I0 + c < n_ion; c += NW) {
-      const cplx<T>* p = ph + ((size_t)(I0 + c) * 3 + 2) * n + col0;
+      const cplx<T>* p = pt + ((size_t)(I0 + c) * 3 + 2) * n + col0;
       cplx<T>* d = se + ((size_t)buf * CH + c) * CC;
       for (int k = lane; k < ncol; k += 32) cp_async_c(d + k, p + k, true);
     }
     cp_async_commit();
   };
   constexpr int CW = (CH + NW - 1) / NW;                 // ions per warp and chunk
-  cplx<T> vx[CW][NR], vy[CW][NR];
+  using Ph = typename Phase<T>::type;
+  Ph vx[CW][NR], vy[CW][NR];
   auto load_rows = [&](int I0) {
 #pragma unroll
     for (int w = 0; w < CW; ++w) {
       const int I = I0 + wid + NW * w;
       if (wid + NW * w >= CH || I >= n_ion) continue;
-      const cplx<T>* p = ph + (size_t)I * 3 * n;
+      const Ph* p = ph + (size_t)I * 3 * n;
 #pragma unroll
       for (int u = 0; u < NR; ++u)
         if (ra[u] >= 0) { vx[w][u] = p[ra[u]]; vy[w][u] = p[n + rb[u]]; }
@@ -171,12 +223,10 @@ __global__ void __launch_bounds__(NT) k_struct(const cplx<T>* __restrict__ ph, c
 #pragma unroll
       for (int u = 0; u < NR; ++u) {
         if (ra[u] < 0) continue;
-        cplx<T> ex = vx[w][u], ey = vy[w][u];
-        if (2 * ra[u] == n) ex.y = -ex.y;                // index n/2 holds -n/2
-        if (2 * rb[u] == n) ey.y = -ey.y;
-        ex.x *= z; ex.y *= z;
+        // (index n/2 holds -n/2)
         sr[((size_t)buf * CH + c) * RT + lane + 32 * u] =
-            Quad<T>{ex.x * ey.x - ex.y * ey.y, ex.x * ey.y + ex.y * ey.x, ex.x * ey.x + ex.y * ey.y, ex.y * ey.x - ex.x * ey.y};
+            row_products(2 * ra[u] == n ? Phase<T>::conj(vx[w][u]) : vx[w][u],
+                         2 * rb[u] == n ? Phase<T>::conj(vy[w][u]) : vy[w][u], z);
       }
     }
   };
@@ -379,10 +429,11 @@ static __device__ __forceinline__ void ewald_real_part(const double* __restrict_
 // latency that overlap).
 template <typename T>
 __global__ void __launch_bounds__(256) k_ions(const double* __restrict__ pos, const double* __restrict__ Z, int n_ion,
-                                              int n, double L, cplx<T>* __restrict__ ph, double eta, double rcut,
-                                              int nimg, int ne, double* __restrict__ partial) {
+                                              int n, double L, typename Phase<T>::type* __restrict__ ph,
+                                              cplx<T>* __restrict__ pt, double eta, double rcut, int nimg, int ne,
+                                              double* __restrict__ partial) {
   if ((int)blockIdx.x < ne) ewald_real_part(pos, Z, n_ion, L, eta, rcut, nimg, partial, blockIdx.x, ne);
-  else phases_part<T>(pos, n_ion, n, L, ph, blockIdx.x - ne, gridDim.x - ne);
+  else phases_part<T>(pos, n_ion, n, L, ph, pt, blockIdx.x - ne, gridDim.x - ne);
 }
 
 // ---------------------------------------------------------------------------
