@@ -253,6 +253,20 @@ __device__ __forceinline__ float2 tree_put(const Acc<float>& a) {
 }
 __device__ __forceinline__ double tree_put(const Acc<double>& a) { return a.get(); }
 
+// Products carried to the tree's values: pairs of floats (48 bits: exact products of
+// floats, their remainders by fma; __fmul_rn is never fused into a sum) or doubles.
+__device__ __forceinline__ float2 wide_mul(float a, float b) {
+  const float p = __fmul_rn(a, b);
+  return make_float2(p, fmaf(a, b, -p));
+}
+__device__ __forceinline__ double wide_mul(double a, double b) { return a * b; }
+__device__ __forceinline__ float2 wide_mul(float2 a, float2 b) {
+  const float p = __fmul_rn(a.x, b.x);
+  return make_float2(p, fmaf(a.x, b.y, fmaf(a.y, b.x, fmaf(a.x, b.x, -p))));
+}
+// a.x b.x + a.y b.y
+template <typename C> __device__ __forceinline__ auto wide_dot(C a, C b) { return tree_add(wide_mul(a.x, b.x), wide_mul(a.y, b.y)); }
+
 // Tree over values already parked in scr (column q at scr + q * (blockDim + 1));
 // afterwards column q's sum sits in scr[q * (blockDim + 1)].
 template <typename V>

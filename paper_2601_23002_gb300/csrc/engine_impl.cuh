@@ -196,10 +196,10 @@ class Engine : public IEngine {
   Quad<T>* f_qq = nullptr;
   double *f_part = nullptr, *f_out = nullptr;
   int f_nrows = -1, f_ntile = 0, f_nk = 0, f_m2 = 0;
-  // pressure: kernel tables on dilated cells and pnl(m^2) = (3 - 6a) K +
-  // dK/dlambda, built on the first call
+  // pressure: kernel tables on dilated cells, and by m^2 pnl = (3 - 6a) K + dK/dlambda
+  // and the local term's factor, built on the first call
   double* p_tab = nullptr;
-  T* p_pnl = nullptr;
+  PressureTab<T>* p_gtab = nullptr;
   bool p_ready = false;
   // |q| shells of the structure factors: CSR lists of half-spectrum entries
   // with Hermitian weights, kept for the last n_shells asked for
@@ -1671,8 +1671,21 @@ int Engine<T>::forces(const void* rho, double* f_out_h, void* stream_) {
 template <typename T>
 int Engine<T>::build_pressure_table(cudaStream_t st) {
   const int nm2 = 3 * h * h + 1;
+  const double tp = 2.0 * kPi / L;
   int rc;
-  if (!p_tab && ((rc = alloc(&p_tab, (size_t)4 * nm2 + 16)) || (rc = alloc(&p_pnl, nm2)))) return rc;
+  std::vector<double> pnl(nm2, 0.0);
+  std::vector<PressureTab<T>> tab(nm2);
+  auto upload = [&]() -> int {
+    for (int m = 0; m < nm2; ++m)
+      tab[m] = PressureTab<T>::make(pnl[m], m == 0 ? 3.0 : 1.0 - 0.5 * (tp * tp * (double)m) * (cs.rc * cs.rc));
+    if (!p_gtab && (rc = alloc(&p_gtab, nm2))) return rc;
+    OFDFT_CK(cudaMemcpyAsync(p_gtab, tab.data(), nm2 * sizeof(PressureTab<T>), cudaMemcpyHostToDevice, st));
+    OFDFT_CK(cudaStreamSynchronize(st));
+    p_ready = true;
+    return OFDFT_OK;
+  };
+  if (!use_na()) return upload();
+  if (!p_tab && (rc = alloc(&p_tab, (size_t)4 * nm2 + 16))) return rc;
   const double lam[4] = {1.002, 0.998, 1.001, 0.999};
   double* mp = p_tab + (size_t)4 * nm2;
   for (int i = 0; i < 4; ++i) {
@@ -1687,7 +1700,7 @@ int Engine<T>::build_pressure_table(cudaStream_t st) {
     KernArgs ka{L * lam[i], nbar / (lam[i] * lam[i] * lam[i]), Te, mph[4 * i + 1], mph[4 * i + 2], cs.alpha, nm2};
     OFDFT_RUN("k_kernel_table", st, (double)nm2 * 8, k_kernel_table<<<kernel_table_blocks(nm2), 32 * kKernWarps, 0, st>>>(ka, p_tab + (size_t)i * nm2));
   }
-  std::vector<double> tabs((size_t)4 * nm2), K0(nm2), pnl(nm2);
+  std::vector<double> tabs((size_t)4 * nm2), K0(nm2);
   OFDFT_CK(cudaMemcpyAsync(tabs.data(), p_tab, tabs.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
   OFDFT_CK(cudaMemcpyAsync(K0.data(), Kd, nm2 * sizeof(double), cudaMemcpyDeviceToHost, st));
   OFDFT_CK(cudaStreamSynchronize(st));
@@ -1696,11 +1709,7 @@ int Engine<T>::build_pressure_table(cudaStream_t st) {
     const double c2 = (tabs[(size_t)2 * nm2 + m] - tabs[(size_t)3 * nm2 + m]) / (2.0 * 1e-3);
     pnl[m] = (3.0 - 6.0 * cs.alpha) * K0[m] + (4.0 * c2 - c1) / 3.0;
   }
-  const std::vector<T> pt(pnl.begin(), pnl.end());
-  OFDFT_CK(cudaMemcpyAsync(p_pnl, pt.data(), nm2 * sizeof(T), cudaMemcpyHostToDevice, st));
-  OFDFT_CK(cudaStreamSynchronize(st));
-  p_ready = true;
-  return OFDFT_OK;
+  return upload();
 }
 
 // Pressure P = -dF/dOmega under a homogeneous dilation at fixed T (Results,
@@ -1712,7 +1721,7 @@ int Engine<T>::pressure(const void* rho, double* p_out_h, void* stream_) {
   cudaStream_t st = (cudaStream_t)stream_;
   int rc;
   const bool nl = use_na(), vw = use_psi();
-  if (nl && !p_ready && (rc = build_pressure_table(st))) return rc;
+  if (!p_ready && (rc = build_pressure_table(st))) return rc;
   // n~, (n^a)~ and (sqrt n)~ as needed; a = 1/2: one transform for the last two
   // (its mean is left out, and both terms' factors vanish at G = 0)
   const bool half = cs.alpha == 0.5;
@@ -1725,22 +1734,27 @@ int Engine<T>::pressure(const void* rho, double* p_out_h, void* stream_) {
   const int gb = 4 * nsm;
   const double cy = 9.8696044010893586188344909998762 / (1.4142135623730950488016887242097 * std::pow(Te, 1.5));
   OFDFT_RUN("k_pressure_r", st, (double)N * sizeof(T), k_pressure_r<T><<<gb, 256, 0, st>>>((const T*)rho, N, (T)cy, (T)Te, cs.terms, partials, cs.fd64 ? 1 : 0, cy, counters + 5, res_h));
+  const double tp = 2.0 * kPi / L;
+  // a power of two near 1 / N, exact where 1 / N is not; its ratio to 1 / N follows
+  const double sc = std::exp2(-std::floor(std::log2((double)N))), rN = 1.0 / (double)N / sc;
   if (nf) {
-    const double tp = 2.0 * kPi / L;
+    int m2cut = (int)std::min(3.0 * h * h, std::floor(g2cut_loc / (tp * tp)));
+    while (m2cut < 3 * h * h && tp * tp * (double)(m2cut + 1) <= g2cut_loc) ++m2cut;
+    while (m2cut >= 0 && tp * tp * (double)m2cut > g2cut_loc) --m2cut;
     const C* vl = (cs.terms & OFDFT_TERM_LOC) ? (view.planes ? vloc_pl : vloc) : nullptr;
-    OFDFT_RUN("k_pressure_g", st, (double)(nf + (vl != nullptr)) * NH * sizeof(C), k_pressure_g<T><<<gb, 256, 0, st>>>(use_n() ? spec[0] : nullptr, nl ? (half ? spec[2] : spec[1]) : nullptr, vw ? spec[2] : nullptr, view, vl, cou, p_pnl, (T)(tp * tp), (T)g2cut_loc, (T)(cs.rc * cs.rc), (T)(1.0 / (double)N), partials, counters + 5, res_h + 2));
+    OFDFT_RUN("k_pressure_g", st, (double)(nf + (vl != nullptr)) * NH * sizeof(C), k_pressure_g<T><<<gb, 256, 0, st>>>(use_n() ? spec[0] : nullptr, nl ? (half ? spec[2] : spec[1]) : nullptr, vw ? spec[2] : nullptr, view, vl, cou, p_gtab, (T)(tp * tp), m2cut, (T)sc, partials, counters + 5, res_h + 2));
   } else {
     std::memset(res_h + 2, 0, 4 * sizeof(double));
   }
   OFDFT_CK(cudaStreamSynchronize(st));
   double* P = p_out_h;
-  const double E_vW = 0.5 * Omega * res_h[5];
-  const double E_H = (cs.terms & OFDFT_TERM_HARTREE) ? 0.5 * Omega * res_h[4] : 0.0;
+  const double E_vW = 0.5 * Omega * rN * rN * res_h[5];
+  const double E_H = (cs.terms & OFDFT_TERM_HARTREE) ? 0.5 * Omega * rN * rN * res_h[4] : 0.0;
   P[0] = res_h[0] / (double)N;              // (1/Omega) dV sum n T p
   P[1] = 2.0 * E_vW / (3.0 * Omega);
-  P[2] = -res_h[3] / 3.0;
+  P[2] = -rN * rN * res_h[3] / 3.0;
   P[3] = E_H / (3.0 * Omega);
-  P[4] = res_h[2] / 3.0;
+  P[4] = rN * res_h[2] / 3.0;
   P[5] = res_h[1] / (double)N;
   P[6] = E_ion / (3.0 * Omega);
   P[7] = P[0] + P[1] + P[2] + P[3] + P[4] + P[5] + P[6];

@@ -40,17 +40,13 @@ static __device__ __forceinline__ Quad<double> row_products(double2 x, double2 y
   const double xr = x.x * z, xi = x.y * z;
   return Quad<double>{xr * y.x - xi * y.y, xr * y.y + xi * y.x, xr * y.x + xi * y.y, xi * y.x - xr * y.y};
 }
-static __device__ __forceinline__ float2 pair_product(float ah, float al, float bh, float bl) {
-  const float p = __fmul_rn(ah, bh);     // (never fused into a sum)
-  return make_float2(p, fmaf(ah, bl, fmaf(al, bh, fmaf(ah, bh, -p))));
-}
 static __device__ __forceinline__ float pair_sum(float2 a, float2 b) {
   const float s = a.x + b.x, t = s - a.x;
   return s + ((a.x - (s - t)) + (b.x - t) + (a.y + b.y));
 }
 static __device__ __forceinline__ Quad<float> row_products(float4 x, float4 y, float z) {
-  const float2 rr = pair_product(x.x, x.z, y.x, y.z), ii = pair_product(x.y, x.w, y.y, y.w);
-  const float2 ri = pair_product(x.x, x.z, y.y, y.w), ir = pair_product(x.y, x.w, y.x, y.z);
+  const float2 xr = make_float2(x.x, x.z), xi = make_float2(x.y, x.w), yr = make_float2(y.x, y.z), yi = make_float2(y.y, y.w);
+  const float2 rr = wide_mul(xr, yr), ii = wide_mul(xi, yi), ri = wide_mul(xr, yi), ir = wide_mul(xi, yr);
   const float2 mi = make_float2(-ii.x, -ii.y), mri = make_float2(-ri.x, -ri.y);
   return Quad<float>{z * pair_sum(rr, mi), z * pair_sum(ri, ir), z * pair_sum(rr, ii), z * pair_sum(ir, mri)};
 }
@@ -906,21 +902,37 @@ __global__ void __launch_bounds__(256) k_pressure_r(const T* __restrict__ rho, s
 //      |G|^2 <= g2cut, as in the energy)
 //   1: sum w |(n^a)~|^2 pnl(m^2),  pnl = (3 - 6a) K + dK/dlambda
 //   2: sum w 4 pi |n~|^2 / G^2      3: sum w G^2 |(sqrt n)~|^2
-// A warp takes a row of the layout at a time.  Products in the plan's precision,
-// compensated sums; the last block adds the blocks' partial[block][4] into out[].
+// with the spectra scaled by the power of two sc instead of 1 / N.  A warp takes a row
+// of the layout at a time.  0 and 1 (terms that cancel in the total) from the tables
+// tab[m^2] = (pnl, c) to the sums in FP64, which FP32 plans carry as pairs of floats (48
+// bits; FP64 products and sums took 200 of 573 us at 256^3); 2 and 3 as the evaluation's
+// energies: products in the plan's precision, compensated sums.  m2cut: |G|^2 <= g2cut.
+// The last block adds the blocks' partial[block][4] into out[].
+template <typename T> struct PressureTab;
+template <> struct PressureTab<double> {
+  double pnl, c;
+  static PressureTab make(double p, double c) { return {p, c}; }
+};
+template <> struct alignas(16) PressureTab<float> {
+  float2 pnl, c;
+  static float2 split(double v) { return make_float2((float)v, (float)(v - (double)(float)v)); }
+  static PressureTab make(double p, double c) { return {split(p), split(c)}; }
+};
 template <typename T>
 __global__ void __launch_bounds__(256) k_pressure_g(const cplx<T>* __restrict__ nt, const cplx<T>* __restrict__ wt,
                                                     const cplx<T>* __restrict__ pt, SpecView view,
                                                     const cplx<T>* __restrict__ vloc, const T* __restrict__ cou,
-                                                    const T* __restrict__ pnl, T tp2, T g2cut, T rc2, T invN,
+                                                    const PressureTab<T>* __restrict__ tab, T tp2, int m2cut, T sc,
                                                     double* __restrict__ partial, unsigned int* counter,
                                                     double* __restrict__ out) {
-  __shared__ typename TreeVal<T>::type scr[4 * 257];
+  using V = typename TreeVal<T>::type;
+  __shared__ V scr[4 * 257];
   const int n = view.n, nh = n / 2 + 1;
   const int len = view.planes ? n : nh, rows = view.planes ? nh * n : n * n;
   const int lane = threadIdx.x & 31;
   auto sgn = [&](int k) { return k <= (n - 1) / 2 ? k : k - n; };
-  Acc<T> acc[4];
+  V loc{}, nl{};
+  Acc<T> har, vw;
   for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < rows; r += (gridDim.x * blockDim.x) >> 5) {
     const int a = r / n, b = r - a * n;
     // plane layout: row (kz = a, px = b) over py; tiled: row (kx = a, ky = b) over kz
@@ -932,26 +944,26 @@ __global__ void __launch_bounds__(256) k_pressure_g(const cplx<T>* __restrict__ 
       const int m2 = m0 * m0 + my * my + kz * kz;
       const T w = (kz == 0 || 2 * kz == n) ? (T)1 : (T)2;
       const size_t q = (size_t)r * len + c;
-      const T G2 = tp2 * (T)m2;
       if (nt) {
-        const T x = nt[q].x * invN, y = nt[q].y * invN;
-        acc[2].add(w * cou[m2] * (x * x + y * y));
-        if (vloc && G2 <= g2cut) {
-          const cplx<T> v = vloc[q];
-          acc[0].add(w * (m2 == 0 ? (T)3 : (T)1 - (T)0.5 * G2 * rc2) * (x * v.x + y * v.y));
-        }
+        const cplx<T> f = cscale(nt[q], sc);
+        har.add(w * cou[m2] * (f.x * f.x + f.y * f.y));
+        if (vloc && m2 <= m2cut) loc = tree_add(loc, wide_mul(wide_dot(cscale(f, w), vloc[q]), tab[m2].c));
       }
       if (wt) {
-        const T x = wt[q].x * invN, y = wt[q].y * invN;
-        acc[1].add(w * (x * x + y * y) * pnl[m2]);
+        const cplx<T> f = cscale(wt[q], sc);
+        nl = tree_add(nl, wide_mul(wide_dot(cscale(f, w), f), tab[m2].pnl));
       }
       if (pt) {
-        const T x = pt[q].x * invN, y = pt[q].y * invN;
-        acc[3].add(w * G2 * (x * x + y * y));
+        const cplx<T> f = cscale(pt[q], sc);
+        vw.add(w * (tp2 * (T)m2) * (f.x * f.x + f.y * f.y));
       }
     }
   }
-  block_sum_tree<4, T>(acc, 4, partial + (size_t)blockIdx.x * 4, scr);
+  V* col = scr + threadIdx.x;
+  const int pitch = blockDim.x + 1;
+  col[0] = loc; col[pitch] = nl; col[2 * pitch] = tree_put(har); col[3 * pitch] = tree_put(vw);
+  block_tree_core(4, scr);
+  if (threadIdx.x < 4) partial[(size_t)blockIdx.x * 4 + threadIdx.x] = tree_get(scr[threadIdx.x * pitch]);
   if (arrive_last(counter)) {
     block_sum_columns(partial, gridDim.x, 4, out, nullptr);
     if (threadIdx.x == 0) *counter = 0u;

@@ -49,3 +49,36 @@ def test_ewald_sum_of_the_fp32_structure_factor(n, L, n_ion, Z):
     want = float((f * (A2[0] - A2[1])).sum())
     assert abs(want) > 1e-10 * float((f * A2[1]).sum())
     assert abs((E[0] - E[1]) - want) <= 1e-12 * float((f * A2[1]).sum())
+
+
+# Pressure, local part: of a uniform density 2^-4 the spectrum is n~(0) alone, exact in
+# FP32 where every butterfly is (2 and 3 points), and P_loc = n V_loc(0) with V_loc(0)
+# rounded to FP32: 3e-14 after a few operations on pairs of floats (48 bits).
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [16, 27, 72, 96])
+def test_local_pressure_of_a_uniform_density(n):
+    L, n_ion = 0.2 * n, 9
+    plan = Plan(L, n, np.full(n_ion, 2.0), 0.3, rc=1.1, precision="fp32")
+    plan.structure_factor(np.random.default_rng(n).uniform(0.0, L, (n_ion, 3)))
+    p = plan.pressure(torch.full((n ** 3,), 0.0625, dtype=torch.float32, device="cuda"))
+    plan.close()
+    v0 = float(np.float32(math.pi * 1.1 * 1.1 / L ** 3 * 2.0 * n_ion))
+    assert abs(p["loc"] - 0.0625 * v0) <= 3e-14 * 0.0625 * v0
+
+
+# Nonlocal part: planes of density 1/4 and 1/16 in turn, mean wave 1/4 (N_e / L^3 = 1/16): every
+# value of the transform of sqrt(n) is exact in FP32 and in FP64, and so is |n~|^2; the two
+# plans' pressures then differ by some roundings of FP64 and of pairs of floats (48 bits).
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [16, 32, 64])
+def test_nonlocal_pressure_of_an_exact_wave(n):
+    rho = torch.full((n, n, n), 0.25, dtype=torch.float64)
+    rho[1::2] = 0.0625
+    got = []
+    for precision in ("fp32", "fp64"):
+        plan = Plan(8.0, n, np.full(32, 1.0), 0.4, precision=precision)
+        plan.structure_factor(np.random.default_rng(n).uniform(0.0, 8.0, (32, 3)))
+        got.append(plan.pressure(rho.to(plan.dtype).cuda().reshape(-1))["nl"])
+        plan.close()
+    assert abs(got[1]) > 1e-6
+    assert abs(got[0] - got[1]) <= 1e-13 * abs(got[1])
