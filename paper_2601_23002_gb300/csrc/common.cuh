@@ -264,8 +264,23 @@ __device__ __forceinline__ float2 wide_mul(float2 a, float2 b) {
   const float p = __fmul_rn(a.x, b.x);
   return make_float2(p, fmaf(a.x, b.y, fmaf(a.y, b.x, fmaf(a.x, b.x, -p))));
 }
+__device__ __forceinline__ float2 wide_mul(float a, float2 b) { return wide_mul(make_float2(a, 0.0f), b); }
+// s += x without loss (floats: a two-sum; x must not be a product the compiler could fuse)
+__device__ __forceinline__ void wide_acc(float2& s, float x) {
+  const float t = s.x + x, b = t - s.x;
+  s.y += (s.x - (t - b)) + (x - b);
+  s.x = t;
+}
+__device__ __forceinline__ void wide_acc(double& s, double x) { s += x; }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return a * b; }
 // a.x b.x + a.y b.y
 template <typename C> __device__ __forceinline__ auto wide_dot(C a, C b) { return tree_add(wide_mul(a.x, b.x), wide_mul(a.y, b.y)); }
+
+__device__ __forceinline__ float2 shfl_xor_v(float2 v, int m) {
+  return make_float2(__shfl_xor_sync(0xffffffffu, v.x, m), __shfl_xor_sync(0xffffffffu, v.y, m));
+}
+__device__ __forceinline__ double shfl_xor_v(double v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
 
 // Tree over values already parked in scr (column q at scr + q * (blockDim + 1));
 // afterwards column q's sum sits in scr[q * (blockDim + 1)].

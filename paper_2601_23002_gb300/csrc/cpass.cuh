@@ -166,10 +166,6 @@ template <int N, bool D> struct CZ {
 // halves columns and lanes together (lane bits 4..2 choose the column, 7
 // additions), two more steps finish the warp, one barrier, and the first warp
 // adds the warps' sums.  Fixed order.  Floats as (hi, lo) pairs (tree_add).
-__device__ __forceinline__ float2 shfl_xor_v(float2 v, int m) {
-  return make_float2(__shfl_xor_sync(0xffffffffu, v.x, m), __shfl_xor_sync(0xffffffffu, v.y, m));
-}
-__device__ __forceinline__ double shfl_xor_v(double v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
 
 // scr: [warps][8]; dst[c] (c < ncol) by thread c of the first warp.  Begins
 // with a barrier (scr may alias data still being read); no barrier at the end.

@@ -1654,10 +1654,10 @@ int Engine<T>::forces(const void* rho, double* f_out_h, void* stream_) {
   int nsplit = (int)std::max<long>(1, std::min<long>({64, (4 * nsm + nion - 1) / nion, comb / 256}));
   while (nsplit > 1 && (size_t)nion * nsplit * 3 > partials_cap) --nsplit;
   if ((size_t)nion * nsplit * 3 > partials_cap) { set_error("forces: too many ions for the scratch"); return OFDFT_ERR_INVALID; }
-  constexpr int TI = sizeof(T) == 4 ? 4 : 2;
+  constexpr int TI = 2;
   const int ny = (nion + kForceWarps * TI - 1) / (kForceWarps * TI);
   const EwaldForceArgs wa{pos_d, Z_d, L, ew_eta, ew_rcut, ew_nimg, nsplit, partials};
-  OFDFT_RUN("k_forces_g", st, (double)f_nk * 128 * sizeof(C), k_forces_g<T, TI><<<f_ntile * ny + nion * nsplit, 32 * kForceWarps, 0, st>>>(f_qq, f_rows, f_nrows, f_tk, phases_t, nion, n, f_part, f_ntile, ny, wa));
+  OFDFT_RUN("k_forces_g", st, (double)f_nk * 128 * sizeof(C), k_forces_g<T, TI><<<f_ntile * ny + nion * nsplit, 32 * kForceWarps, 0, st>>>(f_qq, f_rows, f_nrows, f_tk, phases, phases_t, nion, n, f_part, f_ntile, ny, wa));
   OFDFT_RUN("k_sum_force_parts", st, (double)nion * nsplit * 24, k_sum_force_parts<<<(3 * nion + 3) / 4, 128, 0, st>>>(f_part, f_ntile, Z_d, tp, partials, nion, nsplit, f_out));
   OFDFT_CK(cudaMemcpyAsync(f_out_h, f_out, (size_t)nion * 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
   OFDFT_CK(cudaStreamSynchronize(st));

@@ -747,20 +747,19 @@ static __device__ __forceinline__ void ewald_force_part(const EwaldForceArgs& w,
 }
 
 // Block: one tile of 32 row pairs (a lane each) and NW TI ions (TI per warp).
-// Along kz (from the tile's largest down) a lane sums U = sum qq e_z and
-// V = sum kz qq e_z for its four rows (V by adding the running U after every
-// step kz >= 1), six operations per G and ion, against the tile's qq (registers,
-// read once per TI ions) and the ions' e_z (broadcast from shared memory); then
-// Im[P U] etc. times (a, b) and Im[P V], summed over the lanes.  (A gather of
-// three phases and two complex products per G and ion took 186 us for 128 ions
-// at 108^3.)  part[tile][ion][3], FP64, without the factor -Z_I 2 pi / L.
+// Along kz a lane sums U = sum qq e_z and V = sum m_z qq e_z for its four rows, the terms
+// rounded and added without loss (34 operations per G and ion in FP32), against the tile's qq (registers, read once per TI ions) and the ions' e_z (broadcast
+// from shared memory); then Im[P U] etc. times (a, b) and Im[P V], summed over the lanes.
+// (A gather of three phases and two complex products per
+// G and ion took 186 us for 128 ions at 108^3.)  part[tile][ion][3], FP64, without the factor -Z_I 2 pi / L.
 // grid.x: ntile tiles times ny ion groups, then n_ion nsplit blocks of the
 // Ewald real-space part, which overlap with them.
 constexpr int kForceWarps = 4;
 template <typename T, int TI>
 __global__ void __launch_bounds__(32 * kForceWarps) k_forces_g(const Quad<T>* __restrict__ qq, const int2* __restrict__ rows,
                                                                int nrows, const int* __restrict__ tk,
-                                                               const cplx<T>* __restrict__ ph, int n_ion, int n,
+                                                               const typename Phase<T>::type* __restrict__ ph,
+                                                               const cplx<T>* __restrict__ pt, int n_ion, int n,
                                                                double* __restrict__ part, int ntile, int ny,
                                                                EwaldForceArgs ewald) {
   constexpr int NI = kForceWarps * TI, KC = 32;
@@ -772,35 +771,32 @@ __global__ void __launch_bounds__(32 * kForceWarps) k_forces_g(const Quad<T>* __
   const int tile = blockIdx.x % ntile, I0 = blockIdx.x / ntile * NI;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int k0 = tk[tile], nk = tk[tile + 1] - k0;
-  cplx<T> U[TI][4], V[TI][4];
+  using V = typename TreeVal<T>::type;                   // FP64, or pairs of floats
+  V Ux[TI][4], Uy[TI][4], Vx[TI][4], Vy[TI][4];
 #pragma unroll
   for (int i = 0; i < TI; ++i)
 #pragma unroll
-    for (int s = 0; s < 4; ++s) { U[i][s] = mk<T>((T)0, (T)0); V[i][s] = mk<T>((T)0, (T)0); }
-  for (int kt = nk; kt > 0; kt -= KC) {                  // chunks [kb, kt), top first
+    for (int s = 0; s < 4; ++s) Ux[i][s] = Uy[i][s] = Vx[i][s] = Vy[i][s] = V{};
+  for (int kt = nk; kt > 0; kt -= KC) {                  // chunks [kb, kt), the small terms first
     const int kb = max(0, kt - KC);
     __syncthreads();
     for (int q = threadIdx.x; q < (kt - kb) * NI; q += 32 * kForceWarps) {
       const int i = q / (kt - kb), k = q - i * (kt - kb);
-      se[k][i] = I0 + i < n_ion ? ph[((size_t)(I0 + i) * 3 + 2) * n + kb + k] : mk<T>((T)0, (T)0);
+      se[k][i] = I0 + i < n_ion ? pt[((size_t)(I0 + i) * 3 + 2) * n + kb + k] : mk<T>((T)0, (T)0);
     }
     __syncthreads();
     for (int k = kt - 1; k >= kb; --k) {
       const Quad<T> q0 = qq[((size_t)(k0 + k) * 2) * 32 + lane], q1 = qq[((size_t)(k0 + k) * 2 + 1) * 32 + lane];
+      const T mz = (T)(2 * k == n ? -k : k);             // kz = n/2 is -n/2
 #pragma unroll
       for (int i = 0; i < TI; ++i) {
         const cplx<T> e = se[k - kb][warp * TI + i];
-        U[i][0].x = fma(q0.a, e.x, fma(-q0.b, e.y, U[i][0].x)); U[i][0].y = fma(q0.a, e.y, fma(q0.b, e.x, U[i][0].y));
-        U[i][1].x = fma(q0.c, e.x, fma(-q0.d, e.y, U[i][1].x)); U[i][1].y = fma(q0.c, e.y, fma(q0.d, e.x, U[i][1].y));
-        U[i][2].x = fma(q1.a, e.x, fma(-q1.b, e.y, U[i][2].x)); U[i][2].y = fma(q1.a, e.y, fma(q1.b, e.x, U[i][2].y));
-        U[i][3].x = fma(q1.c, e.x, fma(-q1.d, e.y, U[i][3].x)); U[i][3].y = fma(q1.c, e.y, fma(q1.d, e.x, U[i][3].y));
-        if (2 * k == n) {                                // kz = n/2 is -n/2: n/2 steps follow
+        const cplx<T> q[4] = {mk<T>(q0.a, q0.b), mk<T>(q0.c, q0.d), mk<T>(q1.a, q1.b), mk<T>(q1.c, q1.d)};
 #pragma unroll
-          for (int s = 0; s < 4; ++s) { V[i][s].x = (T)-n * U[i][s].x; V[i][s].y = (T)-n * U[i][s].y; }
-        }
-        if (k > 0) {
-#pragma unroll
-          for (int s = 0; s < 4; ++s) { V[i][s].x += U[i][s].x; V[i][s].y += U[i][s].y; }
+        for (int s = 0; s < 4; ++s) {
+          const T tx = fma(q[s].x, e.x, -(q[s].y * e.y)), ty = fma(q[s].x, e.y, q[s].y * e.x);
+          wide_acc(Ux[i][s], tx); wide_acc(Uy[i][s], ty);
+          wide_acc(Vx[i][s], mul_rn(mz, tx)); wide_acc(Vy[i][s], mul_rn(mz, ty));
         }
       }
     }
@@ -812,24 +808,26 @@ __global__ void __launch_bounds__(32 * kForceWarps) k_forces_g(const Quad<T>* __
   for (int i = 0; i < TI; ++i) {
     const int I = I0 + warp * TI + i;
     if (I >= n_ion) break;                               // the whole warp
-    const cplx<T>* p = ph + (size_t)I * 3 * n;
-    cplx<T> ex = p[a], ey = p[n + b];
-    if (2 * a == n) ex.y = -ex.y;
-    if (2 * b == n) ey.y = -ey.y;
-    const T Pr = ex.x * ey.x - ex.y * ey.y, Pi = ex.x * ey.y + ex.y * ey.x;
-    const T Mr = ex.x * ey.x + ex.y * ey.y, Mi = ex.y * ey.x - ex.x * ey.y;
-    // Im[P u], Im[P* u]
-    const T u0 = Pr * U[i][0].y + Pi * U[i][0].x, u1 = Pr * U[i][1].y - Pi * U[i][1].x;
-    const T u2 = Mr * U[i][2].y + Mi * U[i][2].x, u3 = Mr * U[i][3].y - Mi * U[i][3].x;
-    const T z0 = Pr * V[i][0].y + Pi * V[i][0].x, z1 = Pr * V[i][1].y - Pi * V[i][1].x;
-    const T z2 = Mr * V[i][2].y + Mi * V[i][2].x, z3 = Mr * V[i][3].y - Mi * V[i][3].x;
-    double f[3] = {(double)a * ((double)u0 - (double)u1 + (double)u2 - (double)u3),
-                   (double)b * ((double)u0 - (double)u1 - (double)u2 + (double)u3),
-                   (double)z0 + (double)z1 + (double)z2 + (double)z3};
+    const typename Phase<T>::type* p = ph + (size_t)I * 3 * n;
+    const auto ex = p[a], ey = p[n + b];
+    const Quad<T> pm = row_products(2 * a == n ? Phase<T>::conj(ex) : ex, 2 * b == n ? Phase<T>::conj(ey) : ey, (T)1);
+    // Im[P u] and Im[P* u] of the column sums
+    V u[4], z[4];
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      const T re = s < 2 ? pm.a : pm.c, im = s == 0 ? pm.b : s == 1 ? -pm.b : s == 2 ? pm.d : -pm.d;
+      const T sg = s & 1 ? (T)-1 : (T)1;                 // rows (-a, -b), (-a, +b): minus in the x component
+      u[s] = wide_mul(sg, tree_add(wide_mul(re, Uy[i][s]), wide_mul(im, Ux[i][s])));
+      z[s] = tree_add(wide_mul(re, Vy[i][s]), wide_mul(im, Vx[i][s]));
+    }
+    const V p01 = tree_add(u[0], u[1]), p23 = tree_add(u[2], u[3]);
+    V f[3] = {wide_mul((T)a, tree_add(p01, p23)), wide_mul((T)b, tree_add(p01, wide_mul((T)-1, p23))),
+              tree_add(tree_add(z[0], z[1]), tree_add(z[2], z[3]))};
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      const double s = warp_sum(f[d]);
-      if (lane == 0) part[((size_t)tile * n_ion + I) * 3 + d] = s;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) f[d] = tree_add(f[d], shfl_xor_v(f[d], o));
+      if (lane == 0) part[((size_t)tile * n_ion + I) * 3 + d] = tree_get(f[d]);
     }
   }
 }

@@ -1,12 +1,12 @@
-"""Sums that FP32 plans form in FP64: the Ewald energy's reciprocal part, the pressure's
-local and nonlocal parts."""
+"""Sums that FP32 plans form without FP32 rounding: the Ewald energy's reciprocal part, the
+pressure's local and nonlocal parts, the forces' sums over G."""
 import math
 
 import numpy as np
 import pytest
 import torch
 
-from paper_2601_23002_gb300 import Plan
+from paper_2601_23002_gb300 import Plan, TERM_LOC, TERMS_ALL
 
 
 def _m2(n):
@@ -82,3 +82,36 @@ def test_nonlocal_pressure_of_an_exact_wave(n):
         plan.close()
     assert abs(got[1]) > 1e-6
     assert abs(got[0] - got[1]) <= 1e-13 * abs(got[1])
+
+
+# Forces without the local term on an ion at the origin, whose phases are 1: the G sum is that
+# of the FP32 roundings of w efac Im S_Z (times m_z, rounded, for the z component), the
+# real-space part the FP64 plan's.  L = 0.6 n keeps every G of the grid in both plans' range.
+# 1e-12 of the sum of sizes: pairs of floats (48 bits) over at most 81 terms a row.
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,n_ion", [(24, 2), (45, 17), (96, 9), (160, 5)])
+def test_force_sums_of_the_fp32_structure_factor(n, n_ion):
+    L = 0.6 * n
+    pos = np.random.default_rng(n).uniform(0.0, L, (n_ion, 3))
+    pos[0] = 0.0
+    F, A = [], []
+    for precision, ct in (("fp32", torch.complex64), ("fp64", torch.complex128)):
+        S = torch.empty(n, n, n // 2 + 1, dtype=ct, device="cuda")
+        plan = Plan(L, n, np.ones(n_ion), 0.3, precision=precision, terms=TERMS_ALL & ~TERM_LOC)
+        plan.structure_factor(pos, S)
+        F.append(plan.forces(torch.full((n ** 3,), n_ion / L ** 3, dtype=plan.dtype, device="cuda"))[0])
+        A.append(torch.view_as_real(S)[..., 1].double())
+        plan.close()
+    tp = 2.0 * math.pi / L
+    G2 = tp ** 2 * _m2(n)
+    G2[0, 0, 0] = 1.0
+    eta2 = (math.pi * n / L) ** 2 / (4.0 * 39.0)
+    f = 4.0 * math.pi / L ** 3 * torch.exp(-G2 / (4.0 * eta2)) / G2 * _weights(n)
+    f[0, 0, 0] = 0.0
+    m = torch.tensor(np.rint(np.fft.fftfreq(n) * n), device="cuda")
+    t32, t64 = (f * A[0]).float(), f * A[1]
+    for d in range(3):
+        md = (m[:, None, None], m[None, :, None], m[None, None, :n // 2 + 1])[d].expand_as(t64)
+        a = (t32 * md.float()).double() if d == 2 else t32.double() * md
+        want = tp * float((a - t64 * md).sum())
+        assert abs((F[0][d] - F[1][d]) - want) <= 1e-12 * tp * float(a.abs().sum()), d
