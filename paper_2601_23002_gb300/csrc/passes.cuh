@@ -673,9 +673,11 @@ template <typename T, int KIND> struct EpiPoint {
     const T nf = fmax(nval, nmin);
     // FP32: one logarithm for TF and XC, of y = n cy itself: ln n + ln cy, with a
     // rounded constant, moved eta by the same 1e-7 at every point (F_TF off by 6e-8
-    // Ha/ion at 128^3, 1.6e-8 so)
+    // Ha/ion at 128^3, 5e-9 so).  Without a TF term in FP32 the logarithm is n's, and
+    // XC does not depend on the temperature (at 1e-27 Ha y overflows).
+    const bool own = !KIND && ((a.terms & 1) == 0 || a.fd64);
     T l2 = 0;
-    if constexpr (sizeof(T) == 4) l2 = __log2f(nf * cy);
+    if constexpr (sizeof(T) == 4) l2 = __log2f(own ? nf : nf * cy);
     T vrest = 0;
     if (KIND || (a.terms & 1)) {              // TF
       if (!KIND && sizeof(T) == 4 && a.fd64) {
@@ -695,7 +697,7 @@ template <typename T, int KIND> struct EpiPoint {
     }
     if (KIND || (a.terms & 8)) {              // XC
       T exc, vxc;
-      if constexpr (sizeof(T) == 4) pz81_l2(nf, l2, c3, lr, exc, vxc);
+      if constexpr (sizeof(T) == 4) pz81_l2(nf, l2, own ? 0.0f : c3, own ? kLnRs1 : lr, exc, vxc);
       else pz81(nf, exc, vxc);
       vrest += vxc;
       acc[1].add(nval * exc);
