@@ -329,12 +329,18 @@ __global__ void __launch_bounds__(NT) k_struct(const typename Phase<T>::type* __
 // ballots and a block prefix, in combination order), and only these, on dense
 // warps, are measured and evaluated in FP64 (partial[block]; fixed order).
 
-// Cells to shift a separation x by: nearest integer to x / L in FP32 where x is
-// good to 3e-4 bohr there (|x| < 4e3), else in FP64.  Screening and evaluation use
-// the same shift, so a pair at half a cell has one and the same image a = 0.
-static __device__ __forceinline__ float cell_shift(double x, double L, float iL) {
+// The minimum image of a separation x: x less L times the nearest integer to x / L,
+// found in FP32 where x is good to 3e-4 bohr there (|x| < 4e3), else in FP64.
+// Screening (FP32) and evaluation (FP64) use the same integer, so a pair at half a
+// cell has one and the same image a = 0.
+static __device__ __forceinline__ bool near_origin(double x) { return fabsf((float)x) < 4e3f; }
+static __device__ __forceinline__ float min_image_f(double x, double L, float Lf, float iL) {
   const float xf = (float)x;
-  return fabsf(xf) < 4e3f ? rintf(xf * iL) : (float)rint(x / L);
+  return near_origin(x) ? fmaf(-Lf, rintf(xf * iL), xf) : (float)(x - L * rint(x / L));
+}
+// the separation at image a in FP64
+static __device__ __forceinline__ double at_image(double x, double L, float iL, int a) {
+  return near_origin(x) ? x + L * (double)(a - rintf((float)x * iL)) : x - L * rint(x / L) + L * (double)a;
 }
 // The squared distance in FP32 at image (a, b, c), each axis good to 1e-3 bohr.
 static __device__ __forceinline__ bool maybe_inside(const double* p, const double* q, double L, float Lf, float iL,
@@ -343,10 +349,7 @@ static __device__ __forceinline__ bool maybe_inside(const double* p, const doubl
   float r2 = 0;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    const double x = p[d] - q[d];
-    const float k = cell_shift(x, L, iL), xf = (float)x;
-    const float v = fabsf(xf) < 4e3f ? fmaf(-Lf, k, xf) : (float)(x - L * (double)k);
-    const float u = v + (float)im[d] * Lf;
+    const float u = min_image_f(p[d] - q[d], L, Lf, iL) + (float)im[d] * Lf;
     r2 += u * u;
   }
   return r2 < rc2m;
@@ -354,9 +357,7 @@ static __device__ __forceinline__ bool maybe_inside(const double* p, const doubl
 // the displacement at that image in FP64
 static __device__ __forceinline__ double3 displacement(const double* p, const double* q, double L, float iL, int a,
                                                        int b, int c) {
-  const double x = p[0] - q[0], y = p[1] - q[1], z = p[2] - q[2];
-  return make_double3(x + L * (double)(a - cell_shift(x, L, iL)), y + L * (double)(b - cell_shift(y, L, iL)),
-                      z + L * (double)(c - cell_shift(z, L, iL)));
+  return make_double3(at_image(p[0] - q[0], L, iL, a), at_image(p[1] - q[1], L, iL, b), at_image(p[2] - q[2], L, iL, c));
 }
 // Slots, in thread order, of the threads with `in` among blockDim <= 256; the
 // count in total.  Between two block barriers.
