@@ -72,7 +72,7 @@ enum {
 /* The cell.  Z points to host memory and is copied by ofdft_plan_create. */
 typedef struct {
     double L;            /* cubic cell side, bohr (> 0)                                */
-    int n;               /* grid points per side: even, 2,3,5-smooth, 8 <= n <= 512    */
+    int n;               /* grid points per side: 2,3,5-smooth (odd or even), 8 to 512  */
     int n_ion;           /* number of ions (>= 1)                                      */
     const double* Z;     /* host [n_ion] valence charges (> 0); N_e = sum Z            */
     double rc;           /* Gaussian smoothing radius of the local ion potential, bohr */

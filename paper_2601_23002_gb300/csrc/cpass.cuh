@@ -924,8 +924,8 @@ template <typename T> struct CPass {
 // wave (160^3, 162 planes: 93 -> 64 us with 5).  Above 160 a plane takes several
 // blocks: 4 up to 200 (200^3: 147 us, 165 with 5), then 5 (216^3: 207, 213 with 4;
 // 240^3: 296, 379 with 8); the tiled chain took 264 us at 200^3, 332 at 216^3.  FP64: the
-// least dtime (two fields, before the radices were chosen with it: 96^3 277 us with
-// 1, 224 with 4; 45^3 69 with 1, 43 with 2).
+// least dtime of 1, 2 and 4 (two fields, before the radices were chosen with it: 96^3
+// 277 us with 1, 224 with 4; 45^3 69 with 1, 43 with 2, 36 to 46 with 3 to 8).
 template <typename T, int N> constexpr int cp_cluster(int nf) {
   const int planes = nf * (N / 2 + 1);
   if (sizeof(T) == 4)

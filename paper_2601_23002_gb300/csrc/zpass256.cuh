@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(256, 4) k_zfwd256(ProArgs<T> a, Spectra<T> sp,
 // instead of two.
 // KIND: see EpiPoint (3: mode 3).  Bound by instruction issue, half of it the
 // functional: 270 us (8 rows), 226 (16 rows), 197 (the functional specialised by
-// KIND, binade polynomials), 186 (block sums by warp halving).
+// KIND, its coefficients in one row per interval), 186 (block sums by warp halving).
 template <typename T, int R, int KIND>
 __global__ void __launch_bounds__(256, 3) k_zinv256(Spectra<T> sp, EpiArgs<T> a, const cplx<T>* __restrict__ tw_h,
                                                    const cplx<T>* __restrict__ tw_n) {
