@@ -748,8 +748,13 @@ static __device__ __forceinline__ void ewald_force_part(const EwaldForceArgs& w,
 }
 
 // Block: one tile of 32 row pairs (a lane each) and NW TI ions (TI per warp).
-// Along kz a lane sums U = sum qq e_z and V = sum m_z qq e_z for its four rows, the terms
-// rounded and added without loss (34 operations per G and ion in FP32), against the tile's qq (registers, read once per TI ions) and the ions' e_z (broadcast
+// Along kz (from the tile's largest down) a lane sums U = sum qq e_z and V = sum m_z qq e_z
+// for its four rows: KF kz at a time as running sums (V by adding U after every step), which
+// then go into sums without loss (U, and V + kz U).  In FP32, KF = 2, 21 operations per G
+// and ion (34 for every term without loss): the rounding of these sums and products
+// leaves (4.4, 4.4, 3.9)e-9 hartree/bohr on three ions in 27 bohr, compensated sums of
+// single terms with FP32 products (11.8, 11.6, 4.5)e-9, sums running over the whole column
+// (13.5, 11.8, 7.0)e-9.  Against the tile's qq (registers, read once per TI ions) and the ions' e_z (broadcast
 // from shared memory); then Im[P U] etc. times (a, b) and Im[P V], summed over the lanes.
 // (A gather of three phases and two complex products per
 // G and ion took 186 us for 128 ions at 108^3.)  part[tile][ion][3], FP64, without the factor -Z_I 2 pi / L.
@@ -773,11 +778,16 @@ __global__ void __launch_bounds__(32 * kForceWarps) k_forces_g(const Quad<T>* __
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int k0 = tk[tile], nk = tk[tile + 1] - k0;
   using V = typename TreeVal<T>::type;                   // FP64, or pairs of floats
+  constexpr int KF = sizeof(T) == 4 ? 2 : 16;
   V Ux[TI][4], Uy[TI][4], Vx[TI][4], Vy[TI][4];
+  cplx<T> u[TI][4], v[TI][4];
 #pragma unroll
   for (int i = 0; i < TI; ++i)
 #pragma unroll
-    for (int s = 0; s < 4; ++s) Ux[i][s] = Uy[i][s] = Vx[i][s] = Vy[i][s] = V{};
+    for (int s = 0; s < 4; ++s) {
+      Ux[i][s] = Uy[i][s] = Vx[i][s] = Vy[i][s] = V{};
+      u[i][s] = v[i][s] = mk<T>((T)0, (T)0);
+    }
   for (int kt = nk; kt > 0; kt -= KC) {                  // chunks [kb, kt), the small terms first
     const int kb = max(0, kt - KC);
     __syncthreads();
@@ -788,16 +798,31 @@ __global__ void __launch_bounds__(32 * kForceWarps) k_forces_g(const Quad<T>* __
     __syncthreads();
     for (int k = kt - 1; k >= kb; --k) {
       const Quad<T> q0 = qq[((size_t)(k0 + k) * 2) * 32 + lane], q1 = qq[((size_t)(k0 + k) * 2 + 1) * 32 + lane];
-      const T mz = (T)(2 * k == n ? -k : k);             // kz = n/2 is -n/2
 #pragma unroll
       for (int i = 0; i < TI; ++i) {
         const cplx<T> e = se[k - kb][warp * TI + i];
         const cplx<T> q[4] = {mk<T>(q0.a, q0.b), mk<T>(q0.c, q0.d), mk<T>(q1.a, q1.b), mk<T>(q1.c, q1.d)};
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
-          const T tx = fma(q[s].x, e.x, -(q[s].y * e.y)), ty = fma(q[s].x, e.y, q[s].y * e.x);
-          wide_acc(Ux[i][s], tx); wide_acc(Uy[i][s], ty);
-          wide_acc(Vx[i][s], mul_rn(mz, tx)); wide_acc(Vy[i][s], mul_rn(mz, ty));
+          u[i][s].x = fma(q[s].x, e.x, fma(-q[s].y, e.y, u[i][s].x));
+          u[i][s].y = fma(q[s].x, e.y, fma(q[s].y, e.x, u[i][s].y));
+        }
+        if (2 * k == n) {                                // (the first step) kz = n/2 is -n/2
+#pragma unroll
+          for (int s = 0; s < 4; ++s) {
+            wide_acc(Vx[i][s], mul_rn((T)-n, u[i][s].x)); wide_acc(Vy[i][s], mul_rn((T)-n, u[i][s].y));
+          }
+        }
+        if (k % KF != 0) {
+#pragma unroll
+          for (int s = 0; s < 4; ++s) { v[i][s].x += u[i][s].x; v[i][s].y += u[i][s].y; }
+        } else {
+#pragma unroll
+          for (int s = 0; s < 4; ++s) {
+            wide_acc(Ux[i][s], u[i][s].x); wide_acc(Uy[i][s], u[i][s].y);
+            wide_acc(Vx[i][s], fma((T)k, u[i][s].x, v[i][s].x)); wide_acc(Vy[i][s], fma((T)k, u[i][s].y, v[i][s].y));
+            u[i][s] = v[i][s] = mk<T>((T)0, (T)0);
+          }
         }
       }
     }
@@ -813,15 +838,15 @@ __global__ void __launch_bounds__(32 * kForceWarps) k_forces_g(const Quad<T>* __
     const auto ex = p[a], ey = p[n + b];
     const Quad<T> pm = row_products(2 * a == n ? Phase<T>::conj(ex) : ex, 2 * b == n ? Phase<T>::conj(ey) : ey, (T)1);
     // Im[P u] and Im[P* u] of the column sums
-    V u[4], z[4];
+    V w[4], z[4];
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
       const T re = s < 2 ? pm.a : pm.c, im = s == 0 ? pm.b : s == 1 ? -pm.b : s == 2 ? pm.d : -pm.d;
       const T sg = s & 1 ? (T)-1 : (T)1;                 // rows (-a, -b), (-a, +b): minus in the x component
-      u[s] = wide_mul(sg, tree_add(wide_mul(re, Uy[i][s]), wide_mul(im, Ux[i][s])));
+      w[s] = wide_mul(sg, tree_add(wide_mul(re, Uy[i][s]), wide_mul(im, Ux[i][s])));
       z[s] = tree_add(wide_mul(re, Vy[i][s]), wide_mul(im, Vx[i][s]));
     }
-    const V p01 = tree_add(u[0], u[1]), p23 = tree_add(u[2], u[3]);
+    const V p01 = tree_add(w[0], w[1]), p23 = tree_add(w[2], w[3]);
     V f[3] = {wide_mul((T)a, tree_add(p01, p23)), wide_mul((T)b, tree_add(p01, wide_mul((T)-1, p23))),
               tree_add(tree_add(z[0], z[1]), tree_add(z[2], z[3]))};
 #pragma unroll
