@@ -111,19 +111,23 @@ __device__ __forceinline__ void phases_part(const double* __restrict__ pos, int 
 //   f = (v~(G)/Omega per unit charge, (2 pi/Omega) exp(-G^2/(4 eta^2))/G^2) by m^2,
 // tabulated once per plan.  FP32 plans hold the first as two floats, so that V_loc
 // is the FP32 rounding of the exact product without FP64 conversions and products.
-// The Ewald sum is FP64 from weight to sum in every plan: it enters F directly, and
-// its size (thousands of hartree in a large cell) is far above that of its changes.
+// The Ewald sum loses nothing to FP32 from weight to sum, which FP32 plans carry as pairs
+// of floats (48 bits; FP64 products and sums took 6 us for 300 ions on 128^3): it enters F
+// directly, and its size (thousands of hartree in a large cell) is far above that of its changes.
 // grid: (row tiles, kz tiles); CT threads along kz.
 template <typename T> struct SfEntry;
 template <> struct alignas(16) SfEntry<float> {
-  float v, vlo;
-  double e;
-  static SfEntry make(double a, double b) { return {(float)a, (float)(a - (double)(float)a), b}; }
+  float v, vlo, e, elo;
+  static SfEntry make(double a, double b) {
+    return {(float)a, (float)(a - (double)(float)a), (float)b, (float)(b - (double)(float)b)};
+  }
+  __device__ __forceinline__ float2 weight(float w) const { return make_float2(w * e, w * elo); }   // w = 1, 2
   __device__ __forceinline__ float vloc(float z) const { return fmaf(v, z, vlo * z); }
 };
 template <> struct alignas(16) SfEntry<double> {
   double v, e;
   static SfEntry make(double a, double b) { return {a, b}; }
+  __device__ __forceinline__ double weight(double w) const { return w * e; }
   __device__ __forceinline__ double vloc(double z) const { return v * z; }
 };
 template <typename T> struct StructOut {
@@ -261,7 +265,8 @@ __global__ void __launch_bounds__(NT) k_struct(const typename Phase<T>::type* __
     if (more) { store_rows(I0 + CH, buf ^ 1); cp_async_wait<0>(); }
     __syncthreads();
   }
-  double ewa = 0;
+  using V = typename TreeVal<T>::type;
+  V ewa{};
 #pragma unroll
   for (int i = 0; i < TR; ++i) {
     const int r = blockIdx.x * RT + rt + RB * i;
@@ -277,7 +282,7 @@ __global__ void __launch_bounds__(NT) k_struct(const typename Phase<T>::type* __
       const T(&x)[8] = acc[i][j];
       SfEntry<T> f{};
       if (inside) f = o.sf_tab[a * a + b * b + kz * kz];
-      const double we = (kz == 0 || 2 * kz == n ? 1.0 : 2.0) * f.e;
+      V sz2{};
       auto put = [&](int kx, int ky, T re, T im) {
         const size_t at = ((size_t)kx * n + ky) * nh + kz;
         const cplx<T> s = mk<T>(re, im);
@@ -289,7 +294,7 @@ __global__ void __launch_bounds__(NT) k_struct(const typename Phase<T>::type* __
           o.SZ[at] = sz;
           if (inside) {
             o.vloc[at] = mk<T>(f.vloc(sz.x), f.vloc(sz.y));
-            ewa += we * ((double)sz.x * (double)sz.x + (double)sz.y * (double)sz.y);
+            sz2 = tree_add(sz2, wide_dot(sz, sz));
           } else {
             o.vloc[at] = mk<T>((T)0, (T)0);
           }
@@ -299,9 +304,10 @@ __global__ void __launch_bounds__(NT) k_struct(const typename Phase<T>::type* __
       if (ma && mb) put(n - a, n - b, x[0] + x[1], x[2] - x[3]);
       if (pa && mb) put(a, n - b, x[4] - x[5], x[6] + x[7]);
       if (ma && pb) put(n - a, b, x[4] + x[5], x[6] - x[7]);
+      ewa = tree_add(ewa, wide_mul(f.weight(kz == 0 || 2 * kz == n ? (T)1 : (T)2), sz2));
     }
   }
-  double v[1] = {ewa}, out[1];
+  double v[1] = {tree_get(ewa)}, out[1];
   block_sum<1>(v, red, out);
   if (tid == 0) o.ew[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = out[0];
   const int nb = gridDim.x * gridDim.y;
