@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(256, 4) k_zfwd256(ProArgs<T> a, Spectra<T> sp,
     // X[k] = (Z[k] + Z*[H-k])/2 - (i/2) W_N^k (Z[k] - Z*[H-k]), k = 0..H (Z[H] = Z[0]),
     // of the round's transforms; consecutive lanes take consecutive rows of one k, so
     // that plane layout's entries (k, row) at k N^2 + row fill whole lines (a team
-    // storing its own row moved 32 bytes per line: the load-store unit 65% busy)
+    // storing its own row moved 32 bytes per line)
     const int units = min(Z256::TEAMS, ntr - t0), lg = units > 16 ? 5 : units > 8 ? 4 : 3;
     const int nk = min(NH, a.nkz);
     for (int q = threadIdx.x; q < (nk << lg); q += 256) {
